@@ -445,7 +445,7 @@ bool tc_plan(int n, int h, int w, const dc_geom *g, int n_sm, TcParams *p) {
   if (g->groups != 1 || g->c_in % 8 || g->c_out % 8) return false;
   if (g->stride != 1 && g->stride != 2) return false;
   if (g->k > 7) return false;
-  if (g->stride == 2 && (w % 2 || g->k == 1)) return false;
+  if (g->stride == 2 && g->k == 1) return false;
   KOrder ko;
   dc_korder_init(&ko, g);
   if (ko.e_pad > 256 || ko.fold || ko.pair || ko.rows) return false;    // fold- and pair-order weights belong to their own kernels

@@ -443,6 +443,27 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
     assert_close(nchw(y), O.relu6(lin + r.transpose(0, 3, 1, 2)), TOL_BF16)
 
 
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w,kernel", [
+    (24, 24, 3, 1, 1, 3, 31, 23, "k_conv_tc_pairrows"),     # odd padding: the last pixel is the second of its output pair
+    (32, 32, 5, 1, 2, 2, 28, 29, "k_conv_tc_pairrows"),     # even padding: the last output pair has one pixel
+    (32, 32, 3, 1, 1, 51, 25, 25, "k_conv_tc_pairrows"),    # several tiles per CTA: more tiles than stages
+    (16, 8, 3, 1, 0, 2, 18, 41, "k_conv_tc_pairrows"),      # no padding
+    (8, 16, 3, 1, 1, 1, 6, 301, "k_conv_tc_pairrows"),      # three column strips: only the last one holds the column
+    (16, 16, 7, 1, 3, 3, 20, 21, "k_conv_tc_pairrows"),     # 7x7
+    (8, 8, 3, 1, 1, 200, 5, 3, "k_conv_tc_pairrows"),       # one whole pair per row
+    (32, 16, 1, 1, 0, 2, 33, 25, "k_conv_tc_pairrows"),     # 1x1
+    (16, 128, 3, 1, 1, 3, 12, 17, "k_conv_tc_pairrows"),    # two accumulator slots, run-time channel loop
+    (24, 32, 3, 2, 1, 3, 28, 29, "k_conv_tc_pairrows"),     # stride 2: the column in both row planes
+    (32, 16, 5, 2, 2, 2, 31, 45, "k_conv_tc_pairrows"),     # stride 2, even padding
+    (16, 24, 3, 2, 0, 4, 17, 37, "k_conv_tc_pairrows"),     # stride 2, no padding
+    (40, 32, 3, 2, 1, 2, 28, 29, "k_conv_tc"),              # stride 2 on parity planes
+    (96, 144, 5, 2, 2, 1, 57, 57, "k_conv_tc"),             # the same, several tiles per image
+    (24, 168, 3, 2, 1, 1, 49, 49, "k_conv_tc"),             # few channels, more outputs than the pair rows take
+])
+def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel)
+
+
 @pytest.mark.parametrize("c,k,s,p,n,h,w", [(64, 3, 1, 1, 2, 19, 21), (48, 3, 2, 1, 1, 20, 30), (32, 5, 1, 2, 1, 11, 13)])
 def test_dwconv_stencil_without_activation(dc, c, k, s, p, n, h, w):
     """The stencil's instantiations without ReLU6 (tile widths 32 and 16, widths that are no multiple of a
