@@ -4,13 +4,14 @@
 #include "common.cuh"
 
 // ----------------------------------------------------------------------------------------------
-// dense, fp32: one thread = one output pixel x 4 consecutive output channels.
+// dense, fp32, channel counts that are no multiple of 4 (conv_f32.cu takes the others): one thread =
+// one output pixel x 4 consecutive output channels.
 // weights fp32 [k][k][c_in][c_out]: threads of a pixel read consecutive output channels.
 // ----------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_conv_dense_f32(const float *__restrict__ x, const float *__restrict__ w,
-                                                        const float *__restrict__ bias,
-                                                        const float *__restrict__ residual, float *__restrict__ y,
-                                                        int n, int h, int wd, int ho, int wo, dc_geom g, int act) {
+__global__ void __launch_bounds__(128) k_conv_dense_f32_any(const float *__restrict__ x, const float *__restrict__ w,
+                                                            const float *__restrict__ bias,
+                                                            const float *__restrict__ residual, float *__restrict__ y,
+                                                            int n, int h, int wd, int ho, int wo, dc_geom g, int act) {
   const int noc = (g.c_out + 3) / 4;
   const long long total = (long long)n * ho * wo * noc;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -236,8 +237,10 @@ dc_status dc_launch_conv_simt(const void *x, int n, int h, int w, const dc_geom 
                               dc_dtype dtype, cudaStream_t stream) {
   const int ho = dc_out_extent(h, g->k, g->stride, g->pad), wo = dc_out_extent(w, g->k, g->stride, g->pad);
   if (dtype == DC_F32) {
+    const dc_status s = dc_launch_conv_f32(x, n, h, w, g, w_packed, bias, act, residual, y, stream);
+    if (s != DC_ERR_UNSUPPORTED) return s;
     long long total = (long long)n * ho * wo * ((g->c_out + 3) / 4);
-    k_conv_dense_f32<<<simt_blocks(total, 128, 148 * 64), 128, 0, stream>>>(
+    k_conv_dense_f32_any<<<simt_blocks(total, 128, 148 * 64), 128, 0, stream>>>(
         (const float *)x, (const float *)w_packed, bias, (const float *)residual, (float *)y, n, h, w, ho, wo, *g,
         (int)act);
   } else {

@@ -464,6 +464,43 @@ def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel)
 
 
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (32, 32, 5, 1, 2, 3, 28, 28),       # whole pixel tiles and a ragged last one
+    (8, 40, 3, 1, 1, 1, 7, 9),          # a K slice of 16 spans two taps; 40 channels per tile
+    (4, 20, 3, 2, 1, 2, 9, 11),         # four taps per slice, K no multiple of a slice, stride 2
+    (12, 33, 5, 1, 2, 1, 8, 8),         # ragged taps in a slice, channels no multiple of 8
+    (960, 160, 1, 1, 0, 1, 7, 7),       # K split over a cluster
+    (160, 320, 3, 1, 1, 1, 7, 7),       # the same with taps
+    (72, 16, 3, 1, 1, 1, 5, 5),         # a split whose last CTAs have fewer slices
+    (24, 24, 7, 1, 3, 1, 9, 9),
+    (16, 16, 1, 1, 0, 1, 1, 1),         # one pixel, one slice
+    (64, 72, 3, 2, 0, 1, 15, 17),       # stride 2, no padding
+    (40, 48, 3, 1, 1, 40, 25, 25),      # many tiles, none split
+    (6, 8, 3, 1, 1, 2, 9, 9),           # channels no multiple of 4: the kernel that takes any count
+])
+def test_dense_fp32_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    g = dc.geom(c_in, c_out, 1, k, s, p)
+    spec = I.make_layer(14, 0, c_in, c_out, k, s, p)
+    lay = dc.DeviceLayer(spec)
+    wf = torch.empty_like(lay.weight)
+    bf = torch.empty(c_out, device="cuda")
+    dc.fold_bn(lay, wf, bf)
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(wf, g, dc.F32, packed)
+    x = I.make_input(15, (n, h, w, c_in))
+    ho, wo = O.out_extent(h, k, s, p), O.out_extent(w, k, s, p)
+    r = I.normal(16, 99, (n, ho, wo, c_out))
+    Wf, bfo = O.fold_bn(spec)
+    lin = O.conv_direct(x.transpose(0, 3, 1, 2), Wf, bfo, k, s, p)
+    # fp32 sums of up to 1440 products: errors of about 1e-6 of the result's rms, a hundredth of the bounds
+    y = run_conv(dc, dev(x), g, packed, bf, dc.ACT_IDENTITY)
+    assert_close(nchw(y), lin, TOL_F32, bf16=False)
+    y = run_conv(dc, dev(x), g, packed, bf, dc.ACT_RELU6, residual=dev(r))
+    assert_close(nchw(y), O.relu6(lin + r.transpose(0, 3, 1, 2)), TOL_F32, bf16=False)
+    again = run_conv(dc, dev(x), g, packed, bf, dc.ACT_RELU6, residual=dev(r))
+    assert torch.equal(y, again)
+
+
 @pytest.mark.parametrize("c,k,s,p,n,h,w", [(64, 3, 1, 1, 2, 19, 21), (48, 3, 2, 1, 1, 20, 30), (32, 5, 1, 2, 1, 11, 13)])
 def test_dwconv_stencil_without_activation(dc, c, k, s, p, n, h, w):
     """The stencil's instantiations without ReLU6 (tile widths 32 and 16, widths that are no multiple of a
