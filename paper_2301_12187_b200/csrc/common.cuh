@@ -16,7 +16,7 @@
 
 static inline bool dc_aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static inline size_t dc_round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-static inline int dc_div_up(int a, int b) { return (a + b - 1) / b; }
+__host__ __device__ static inline int dc_div_up(int a, int b) { return (a + b - 1) / b; }
 static inline int dc_floor_div2(int a) { return (a >= 0) ? a / 2 : -((-a + 1) / 2); }
 
 // Per-device host state.  SM counts and function attributes belong to a device, not to the process:

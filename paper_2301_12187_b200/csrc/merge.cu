@@ -194,115 +194,6 @@ __global__ void __launch_bounds__(256) k_compose_dd_tiled(Piece first, Piece sec
   }
 }
 
-// dense 3x3 (stride 1) followed by dense 3x3, large channel counts (VGG-style runs): the result's
-// 5x5 kernel of one (o, i) pair is the sum over c of the full 2-D product of W2[o][c] (3x3) and
-// W1[c][i] (3x3), 81 multiply-adds per c, none of them with a structural zero -- the gathered GEMM
-// of the kernels above multiplies all 9 x 25 (tap, position) pairs, 64 % of which are zero.
-// CTA: 16 output channels x 32 input channels, 256 threads, a thread owns one o and two i (50
-// accumulators); slices of 8 intermediate channels are staged in shared memory with the next slice's
-// loads in flight (taps padded to 12 floats, read as three 16-byte vectors).  blockIdx.x walks the
-// tiles (i fastest); the blocks after them compute the bias.
-// At most 128 registers per thread, so that two CTAs share an SM and one's loads hide behind the other's
-// arithmetic (c = 512: 1.31 -> 0.97 ms).  Tiles of 8 output channels in CTAs of 128 threads, for results with
-// fewer tiles than two per SM, were measured and spill (c = 256: 209 -> 302 us): not kept.
-constexpr int kPolyC = 8;
-__global__ void __launch_bounds__(256, 2) k_compose_poly33(Piece first, Piece second, float *out, float *b_out, int gx, int gy) {
-  __shared__ __align__(16) float W2s[2][16][kPolyC][12];   // [o][c][tap]
-  __shared__ __align__(16) float W1s[2][kPolyC][32][12];   // [c][i][tap]
-  if ((int)blockIdx.x >= gx * gy) {
-    compose_bias_block(first, second, b_out, (int)blockIdx.x - gx * gy);
-    return;
-  }
-  const int c0 = first.c_in, c1 = first.c_out, c2 = second.c_out;
-  const int o0 = ((int)blockIdx.x / gx) * 16, i0 = ((int)blockIdx.x % gx) * 32;
-  const int t = threadIdx.x, ol = t >> 4, il = t & 15;       // this thread's o, and i = il, il + 16
-  // loads of a slice: W2: 16 o x 8 c x 9 = 1152 floats, W1: 8 c x 32 i x 9 = 2304 floats
-  constexpr int N2 = (16 * kPolyC * 9 + 255) / 256, N1 = (kPolyC * 32 * 9) / 256;
-  // fetch() only issues the loads and notes in bit masks what decides each element's value; the values are
-  // first touched in stage(), behind the arithmetic on the current slice (see k_compose_dd_tiled).
-  float r2[N2], r1[N1];
-  uint32_t ok2, id2, ok1, id1;
-  auto fetch = [&](int cs) {
-    ok2 = id2 = ok1 = id1 = 0u;
-#pragma unroll
-    for (int q = 0; q < N2; ++q) {
-      const int e = t + 256 * q;                 // (o, c, tap): taps of one (o, c) are contiguous in memory
-      const int tap = e % 9, oc = e / 9, cl = oc % kPolyC, o = o0 + oc / kPolyC, c = cs + cl;
-      const bool ok = e < 16 * kPolyC * 9 && o < c2 && c < c1;
-      r2[q] = second.w[ok ? ((size_t)o * c1 + c) * 9 + tap : 0];
-      ok2 |= (ok ? 1u : 0u) << q;
-      id2 |= ((ok && second.ident && o == c && tap == 4) ? 1u : 0u) << q;
-    }
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      const int e = t + 256 * q;                 // (c, i, tap)
-      const int tap = e % 9, ci = e / 9, i = i0 + ci % 32, c = cs + ci / 32;
-      const bool ok = c < c1 && i < c0;
-      r1[q] = first.w[ok ? ((size_t)c * c0 + i) * 9 + tap : 0];
-      ok1 |= (ok ? 1u : 0u) << q;
-      id1 |= ((ok && first.ident && c == i && tap == 4) ? 1u : 0u) << q;
-    }
-  };
-  auto stage = [&](int buf) {
-#pragma unroll
-    for (int q = 0; q < N2; ++q) {
-      const int e = t + 256 * q, tap = e % 9, oc = e / 9;
-      if (e < 16 * kPolyC * 9)
-        W2s[buf][oc / kPolyC][oc % kPolyC][tap] = ((ok2 >> q) & 1u) ? (((id2 >> q) & 1u) ? r2[q] + 1.f : r2[q]) : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < N1; ++q) {
-      const int e = t + 256 * q, tap = e % 9, ci = e / 9;
-      W1s[buf][ci / 32][ci % 32][tap] = ((ok1 >> q) & 1u) ? (((id1 >> q) & 1u) ? r1[q] + 1.f : r1[q]) : 0.f;
-    }
-  };
-  float acc[2][25] = {};
-  fetch(0);
-  stage(0);
-  __syncthreads();
-  int buf = 0;
-  for (int cs = 0; cs < c1; cs += kPolyC) {
-    const bool more = cs + kPolyC < c1;
-    if (more) fetch(cs + kPolyC);
-#pragma unroll 4
-    for (int cl = 0; cl < kPolyC; ++cl) {
-      float a[12], b[2][12];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        *reinterpret_cast<float4 *>(a + 4 * v) = *reinterpret_cast<const float4 *>(&W2s[buf][ol][cl][4 * v]);
-        *reinterpret_cast<float4 *>(b[0] + 4 * v) = *reinterpret_cast<const float4 *>(&W1s[buf][cl][il][4 * v]);
-        *reinterpret_cast<float4 *>(b[1] + 4 * v) = *reinterpret_cast<const float4 *>(&W1s[buf][cl][il + 16][4 * v]);
-      }
-#pragma unroll
-      for (int u2 = 0; u2 < 3; ++u2)
-#pragma unroll
-        for (int v2 = 0; v2 < 3; ++v2)
-#pragma unroll
-          for (int u1 = 0; u1 < 3; ++u1)
-#pragma unroll
-            for (int v1 = 0; v1 < 3; ++v1) {
-              acc[0][(u1 + u2) * 5 + v1 + v2] = fmaf(a[u2 * 3 + v2], b[0][u1 * 3 + v1], acc[0][(u1 + u2) * 5 + v1 + v2]);
-              acc[1][(u1 + u2) * 5 + v1 + v2] = fmaf(a[u2 * 3 + v2], b[1][u1 * 3 + v1], acc[1][(u1 + u2) * 5 + v1 + v2]);
-            }
-    }
-    if (more) stage(buf ^ 1);
-    __syncthreads();
-    buf ^= 1;
-  }
-  const int o = o0 + ol;
-  if (o < c2) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = i0 + il + 16 * h;
-      if (i < c0) {
-        float *dst = out + ((size_t)o * c0 + i) * 25;
-#pragma unroll
-        for (int e = 0; e < 25; ++e) dst[e] = acc[h][e];
-      }
-    }
-  }
-}
-
 // dense o dense for small results (the usual case: a merged kernel has a few thousand elements):
 // 8 x 32 output tile, one output per thread, so that even a 24 x 216 result spreads over 21 CTAs;
 // operands staged in shared memory a slice of up to kDdSmallSlice reduction rows at a time, all of
@@ -769,6 +660,454 @@ __global__ void __launch_bounds__(kBlockThreads) k_merge_block(const __grid_cons
 }
 
 // ----------------------------------------------------------------------------------------------
+// The same block step for 3x3 depthwise layers, tiled over (output, input) channels and split over the
+// hidden channels inside the CTA, and -- for a run that is one block -- with the delivery in the same
+// launch.
+//
+// For one hidden channel c the 3x3 kernel of a pair (o, i) grows by p = (W3[o][c] s[c]) W1[c][i] times
+// the nine taps D[c][.]: one multiplication and nine FMAs per pair, and W', with its 9 x c_hidden terms,
+// never exists in between.  A CTA owns 8 x 16 pairs, a thread of a warp 2 x 2 of them (36 sums); the
+// eight warps take an eighth of the hidden channels each, stage their own operands by cp.async four
+// slices of 16 channels deep (no CTA barrier until the sums meet in shared memory, in warp order), so
+// that narrow blocks are short chains and wide ones fill the chip: 160 -> 960 -> 160 has 200 tiles.
+// BN scales s = g1 g2 ride on W3, g3 on the result.
+//
+// Blocks behind the tiles compute the bias (8 output channels each); behind those, for a packed
+// result, the chunks of the packed copy that hold no weight are zeroed.
+//
+// Before, with one CTA per output channel that read every operand, then a delivery launch: 24 -> 144 -> 24
+// 9.4 us, 64 -> 384 -> 64 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  Here 6.5, 9.0 and 26.4 us (19 fp32
+// TFLOP/s: 200 tiles on 148 SMs, so a quarter of the SMs do two).
+// ----------------------------------------------------------------------------------------------
+constexpr int kMbO = 8, kMbI = 16, kMbWarps = 8, kMbSlice = 16, kMbStages = 4;
+constexpr int kMbThreads = kMbWarps * 32;
+constexpr int kMbW1 = kMbSlice * kMbI, kMbW3 = kMbO * kMbSlice, kMbD = kMbSlice * 9;   // floats of a slice's operands
+constexpr int kMbStage = kMbW1 + kMbW3 + kMbD;
+constexpr int kMbTile = kMbO * kMbI * 9;                          // sums of a CTA
+constexpr int kMbRing = kMbWarps * kMbStages * kMbStage * 4;      // bytes of the operand rings
+static_assert(kMbRing >= kMbWarps * kMbTile * 4, "the warps' sums reuse the rings");
+
+struct TiledBlocks {
+  BlockArgs blk[kBlockBatch];
+  int first[kBlockBatch + 1];    // first CTA of each block's tiles and bias groups
+  int n;
+};
+struct BlockDelivery {           // of a run that is one block; mode < 0: the block is a piece of a longer run
+  void *packed;
+  int mode;                      // 0: no packed copy, 1: fp32, 2: bf16 chunks
+  int ident;
+  KOrder ko;
+};
+
+__device__ __forceinline__ void mb_cp16(float *dst, const float *src, bool ok) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst), n = ok ? 16u : 0u;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n));
+}
+
+// true when chunk `idx8` of the packed bf16 copy holds weights (c_in is a multiple of 8: all of them or none)
+__device__ __forceinline__ bool packed_chunk_live(const KOrder &ko, int idx8, int c_out) {
+  int plane, o, pc, ccg, r, s;
+  dc_packed_unchunk(ko, idx8, &plane, &o);
+  const int grp = plane / ko.e_pad, e = plane - grp * ko.e_pad;
+  if (!dc_korder_decode(ko, e, &pc, &ccg, &r, &s)) return false;
+  if (ko.fold) {
+    s = o / ko.co8;
+    return s < ko.k && o - s * ko.co8 < c_out;
+  }
+  if (ko.pair >= 2) {
+    int px = 0;
+    if (ko.pair == 2) { px = o / ko.co8; o -= px * ko.co8; }
+    s = 2 * s + (ccg >= ko.cch ? 1 : 0) - (ko.pair == 2 ? px : (ko.pad & 1));
+    return px < 2 && o < c_out && s >= 0 && s < ko.k;
+  }
+  return o < c_out && (grp * ko.cg + ccg) * 8 < ko.c_in;
+}
+
+// The packed copy of a tile of OT output x IT input channels whose K x K kernels lie in shared memory as
+// [o][i][tap].  fp32: [tap][i][o].  bf16: one chunk of 8 input channels per (output channel, chunk, tap), written
+// where the forward kernels' K order wants it; pair rows hold every chunk twice, the second copy one pixel further on.
+template <int OT, int IT, int K>
+__device__ __forceinline__ void deliver_tile(const BlockDelivery &dv, const float *sums, int o0, int i0, int c0, int c2,
+                                             int tid, int threads) {
+  constexpr int KK = K * K;
+  if (dv.mode == 1) {
+    float *out = reinterpret_cast<float *>(dv.packed);
+    for (int e = tid; e < OT * IT * KK; e += threads) {
+      const int ow = e % OT, rest = e / OT, iw = rest % IT, t = rest / IT;
+      if (o0 + ow < c2 && i0 + iw < c0) out[((size_t)t * c0 + i0 + iw) * c2 + o0 + ow] = sums[(ow * IT + iw) * KK + t];
+    }
+    return;
+  }
+  uint4 *out = reinterpret_cast<uint4 *>(dv.packed);
+  for (int e = tid; e < OT * (IT / 8) * KK; e += threads) {
+    const int ow = e % OT, rest = e / OT, hf = rest % (IT / 8), t = rest / (IT / 8), o = o0 + ow, ch = i0 + hf * 8;
+    if (o >= c2 || ch >= c0) continue;
+    __align__(16) __nv_bfloat16 v8[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(sums[(ow * IT + hf * 8 + q) * KK + t]);
+    const uint4 v = *reinterpret_cast<const uint4 *>(v8);
+    const int r = t / K, sx = t - K * r;
+    out[dc_packed_chunk(dv.ko, dc_korder_encode(dv.ko, ch >> 3, r, sx), dc_korder_row(dv.ko, sx, o))] = v;
+    if (dv.ko.pair == 2) {
+      const int plane = (r * dv.ko.ns[0] + ((sx + 1) >> 1)) * 2 * dv.ko.cch + ((sx + 1) & 1) * dv.ko.cch + (ch >> 3);
+      out[dc_packed_chunk(dv.ko, plane, dv.ko.co8 + o)] = v;
+    }
+  }
+}
+
+// zeroes the chunks of the packed bf16 copy that hold no weight; CTA `cta` of `ctas`
+__device__ __forceinline__ void zero_dead_chunks(const BlockDelivery &dv, int c_out, int cta, int ctas) {
+  const int total8 = dv.ko.ng * dv.ko.e_pad * dv.ko.n_pad;
+  for (int e = cta * (int)blockDim.x + (int)threadIdx.x; e < total8; e += ctas * (int)blockDim.x)
+    if (!packed_chunk_live(dv.ko, e, c_out)) reinterpret_cast<uint4 *>(dv.packed)[e] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+__global__ void __launch_bounds__(kMbThreads, 2)
+k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ BlockDelivery dv) {
+  extern __shared__ __align__(16) float mb_smem[];
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  dc_pdl_enter();
+  if ((int)blockIdx.x >= tb.first[tb.n]) {
+    zero_dead_chunks(dv, tb.blk[0].c2, (int)blockIdx.x - tb.first[tb.n], (int)gridDim.x - tb.first[tb.n]);
+    return;
+  }
+  int bi = 0;
+  while ((int)blockIdx.x >= tb.first[bi + 1]) ++bi;
+  const BlockArgs &a = tb.blk[bi];
+  const int c0 = a.c0, c1 = a.c1, c2 = a.c2;
+  const int gi = dc_div_up(c0, kMbI), go = dc_div_up(c2, kMbO);
+  const int blk = (int)blockIdx.x - tb.first[bi];
+  if (blk >= gi * go) {
+    // ---- bias of 8 output channels: q[c] = b2~ + (sum of D~) b1~, then one dot product per warp
+    const int o = (blk - gi * go) * kMbO + warp;
+    float *q = mb_smem;                            // the host keeps c1 within the rings
+    for (int c = tid; c < c1; c += kMbThreads) {
+      const float g1 = raw_scale(a.l1, c), g2 = raw_scale(a.l2, c);
+      float dsum = 0.f;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) dsum += g2 * a.l2.w[(size_t)c * 9 + t];
+      q[c] = fmaf(dsum, raw_bias(a.l1, c, g1), raw_bias(a.l2, c, g2));
+    }
+    __syncthreads();
+    if (o < c2) {
+      const float g3 = raw_scale(a.l3, o);
+      float s = 0.f;
+#pragma unroll 4
+      for (int c = lane; c < c1; c += 32) s = fmaf(g3 * a.l3.w[(size_t)o * c1 + c], q[c], s);
+      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      if (lane == 0) a.b_out[o] = raw_bias(a.l3, o, g3) + s;
+    }
+    return;
+  }
+  // ---- 8 x 16 pairs
+  const int o0 = (blk / gi) * kMbO, i0 = (blk % gi) * kMbI;
+  const int per = ((c1 + kMbWarps - 1) / kMbWarps + 3) & ~3;       // hidden channels of a warp
+  const int cb = warp * per, ce = cb + per < c1 ? cb + per : c1;
+  const int nsl = ce > cb ? (ce - cb + kMbSlice - 1) / kMbSlice : 0;
+  float *ring = mb_smem + warp * (kMbStages * kMbStage);
+  auto fetch = [&](int sl, int buf) {
+    float *st = ring + buf * kMbStage;
+    const int c = cb + sl * kMbSlice;
+    // W1[c..c+15][i0..i0+15]: 64 pieces; W3[o0..o0+7][c..c+15]: 32; D[c..c+15][9]: 36 (channels and c1 are multiples of 4)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = lane + 32 * h, r = e >> 2, ii = i0 + (e & 3) * 4;
+      const bool ok = c + r < ce && ii < c0;
+      mb_cp16(st + e * 4, ok ? a.l1.w + (size_t)(c + r) * c0 + ii : a.l1.w, ok);
+    }
+    {
+      const int o = o0 + (lane >> 2), cc = c + (lane & 3) * 4;
+      const bool ok = o < c2 && cc < ce;
+      mb_cp16(st + kMbW1 + lane * 4, ok ? a.l3.w + (size_t)o * c1 + cc : a.l3.w, ok);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = lane + 32 * h;
+      const bool ok = e * 4 < (ce - c) * 9;
+      if (e < kMbD / 4) mb_cp16(st + kMbW1 + kMbW3 + e * 4, ok ? a.l2.w + (size_t)c * 9 + e * 4 : a.l2.w, ok);
+    }
+  };
+#pragma unroll
+  for (int sl = 0; sl < kMbStages - 1; ++sl) {
+    if (sl < nsl) fetch(sl, sl);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  const int ol = (lane >> 3) * 2, il = (lane & 7) * 2;             // this thread's pairs: o0 + ol + {0, 1}, i0 + il + {0, 1}
+  float acc[2][2][9] = {};
+  int buf = 0, fbuf = kMbStages - 1;
+  // BN scales of a slice's channels: lane l holds channel l & 15's.  Their operands are asked for a slice ahead and
+  // first touched behind the slice's arithmetic.
+  float bn[4] = {1.f, 1.f, 1.f, 1.f};
+  auto ask = [&](int sl) {
+    const int cs = cb + sl * kMbSlice + (lane & 15), c = cs < ce ? cs : cb;
+    if (a.l1.gamma) { bn[0] = a.l1.gamma[c]; bn[1] = a.l1.var[c]; }
+    if (a.l2.gamma) { bn[2] = a.l2.gamma[c]; bn[3] = a.l2.var[c]; }
+  };
+  auto scale = [&]() {
+    return (a.l1.gamma ? bn[0] / sqrtf(bn[1] + a.l1.eps) : 1.f) * (a.l2.gamma ? bn[2] / sqrtf(bn[3] + a.l2.eps) : 1.f);
+  };
+  float sc = 1.f;
+  if (nsl > 0) { ask(0); sc = scale(); }
+#pragma unroll 1
+  for (int sl = 0; sl < nsl; ++sl) {
+    ask(sl + 1);                                   // past the end: the warp's first channel, not used
+    asm volatile("cp.async.wait_group %0;" ::"n"(kMbStages - 2) : "memory");
+    __syncwarp();
+    if (sl + kMbStages - 1 < nsl) fetch(sl + kMbStages - 1, fbuf);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float *st = ring + buf * kMbStage;
+    auto four = [&](int q) {                       // channels q .. q + 3 of the slice
+      float w3[2][4], d[36];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<float4 *>(w3[h]) = *reinterpret_cast<const float4 *>(st + kMbW1 + (ol + h) * kMbSlice + q);
+#pragma unroll
+      for (int e = 0; e < 9; ++e)
+        *reinterpret_cast<float4 *>(d + 4 * e) = *reinterpret_cast<const float4 *>(st + kMbW1 + kMbW3 + q * 9 + 4 * e);
+#pragma unroll
+      for (int cl = 0; cl < 4; ++cl) {
+        const float s = __shfl_sync(0xffffffffu, sc, q + cl);
+        const float2 w1 = *reinterpret_cast<const float2 *>(st + (q + cl) * kMbI + il);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float ws = w3[h][cl] * s;
+          const float p0 = ws * w1.x, p1 = ws * w1.y;
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            acc[h][0][t] = fmaf(p0, d[cl * 9 + t], acc[h][0][t]);
+            acc[h][1][t] = fmaf(p1, d[cl * 9 + t], acc[h][1][t]);
+          }
+        }
+      }
+    };
+    const int left = ce - (cb + sl * kMbSlice);    // channels of the slice: a multiple of 4
+    if (left >= kMbSlice) {
+#pragma unroll
+      for (int q = 0; q < kMbSlice; q += 4) four(q);
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < left; q += 4) four(q);
+    }
+    sc = scale();
+    __syncwarp();                                  // the slice's buffer may be refilled
+    buf = buf + 1 == kMbStages ? 0 : buf + 1;
+    fbuf = fbuf + 1 == kMbStages ? 0 : fbuf + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // ---- the warps' sums meet: [warp][o][i][tap]
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
+#pragma unroll
+      for (int t = 0; t < 9; ++t) mb_smem[warp * kMbTile + ((ol + h) * kMbI + il + v) * 9 + t] = acc[h][v][t];
+  __syncthreads();
+  const bool last = dv.mode >= 0;
+  for (int e = tid; e < kMbTile; e += kMbThreads) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMbWarps; ++w) s += mb_smem[w * kMbTile + e];
+    const int oi = e / 9, t = e - oi * 9, o = o0 + oi / kMbI, i = i0 + oi % kMbI;
+    if (o < c2 && i < c0) {
+      s *= raw_scale(a.l3, o);
+      if (last && dv.ident && o == i && t == 4) s += 1.f;
+      a.w_out[((size_t)o * c0 + i) * 9 + t] = s;
+    }
+    if (last && dv.mode > 0) mb_smem[e] = s;       // element e of warp 0's sums is read by this thread alone
+  }
+  if (!last || dv.mode == 0) return;
+  __syncthreads();
+  deliver_tile<kMbO, kMbI, 3>(dv, mb_smem, o0, i0, c0, c2, tid, kMbThreads);
+}
+
+// ----------------------------------------------------------------------------------------------
+// dense 3x3 (stride 1) followed by dense 3x3: the result's 5x5 kernel of a pair (o, i) is the sum over the
+// intermediate channels c of the full 2-D product of W2[o][c] and W1[c][i], 81 multiply-adds per c and none of
+// them with a structural zero (a gathered GEMM multiplies all 9 x 25 tap/position pairs, 64 % of which are).
+//
+// What bounds it is the FMA pipes, so nothing else may: a CTA owns 8 x 8 pairs, a thread of a warp 2 x 1 of them
+// (50 sums, 162 FMAs per c for 27 shared-memory reads, conflict-free because nine floats apart); the eight
+// warps take an eighth of the channels each and stage their own operands by cp.async in slices of 4 channels
+// (whole 16-byte pieces: the taps of neighbouring channels are contiguous in both operands), three deep,
+// without a CTA barrier until their sums meet in shared memory in warp order.  Small results therefore spread
+// over the chip as well (32 -> 32 -> 32: 16 CTAs, four channels a warp).
+//
+// BN of layers taken as they are: the first's scale rides on its taps, the second's on the sums.  An identity
+// riding on a piece adds W2 or W1 itself (and 1) to the sums.  Blocks behind the tiles compute the bias (8 output
+// channels each); behind those, for a packed result, the chunks without weights are zeroed.
+//
+// Tiles of 16 x 32 pairs with CTA barriers per slice, a fold launch before and a delivery after: c = 64 50 us,
+// 256 141 us, 512 859 us.  Here 7.6, 86 and 587 us (37 useful fp32 TFLOP/s: two thirds of the issue slots are taken,
+// a quarter of them by the operand reads; what holds the rest is the register file, whose banks the compiler cannot
+// keep apart for 50 sums).  Packed FMAs over the two output channels measured 106 us at c = 256, 80 registers and
+// three CTAs per SM 98.
+// ----------------------------------------------------------------------------------------------
+constexpr int kP3O = 8, kP3I = 8, kP3Warps = 8, kP3Slice = 4, kP3Stages = 3;
+constexpr int kP3Threads = kP3Warps * 32;
+constexpr int kP3Op = kP3O * kP3Slice * 9;                        // floats of one operand's slice: [o][c][9] or [c][i][9]
+constexpr int kP3Stage = 2 * kP3Op;
+constexpr int kP3Tile = kP3O * kP3I * 25;
+constexpr int kP3Ring = kP3Warps * kP3Stages * kP3Stage * 4;
+static_assert(kP3Ring >= kP3Warps * kP3Tile * 4, "the warps' sums reuse the rings");
+
+struct Operand33 {
+  RawLayer l;                    // weights, bias, BN (none for a piece)
+  int ident;                     // the identity kernel is added
+};
+struct Compose33 {
+  Operand33 first, second;
+  int c0, c1, c2;
+  float *w_out, *b_out;
+  int gi, go;                    // tiles
+};
+
+__global__ void __launch_bounds__(kP3Threads, 2)
+k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDelivery dv) {
+  extern __shared__ __align__(16) float p3_smem[];
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = a.c0, c1 = a.c1, c2 = a.c2;
+  const RawLayer &l1 = a.first.l, &l2 = a.second.l;
+  int blk = (int)blockIdx.x;
+  dc_pdl_enter();
+  if (blk >= a.gi * a.go) {
+    blk -= a.gi * a.go;
+    if (blk >= a.go) {
+      zero_dead_chunks(dv, c2, blk - a.go, (int)gridDim.x - a.gi * a.go - a.go);
+      return;
+    }
+    // ---- bias: b'[o] = b2~[o] + sum_c (g2 sum of W2[o][c] (+ 1 where c == o and an identity rides)) b1~[c]; a warp per o
+    const int o = blk * kP3O + warp;
+    if (o >= c2) return;
+    const float g2 = raw_scale(l2, o);
+    float s = 0.f;
+#pragma unroll 2
+    for (int c = lane; c < c1; c += 32) {
+      const float b1 = raw_bias(l1, c, raw_scale(l1, c));
+      float ws = (a.second.ident && c == o) ? 1.f : 0.f;
+      float wt = 0.f;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) wt += l2.w[((size_t)o * c1 + c) * 9 + t];
+      s = fmaf(fmaf(g2, wt, ws), b1, s);
+    }
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if (lane == 0) a.b_out[o] = raw_bias(l2, o, g2) + s;
+    return;
+  }
+  const int o0 = (blk / a.gi) * kP3O, i0 = (blk % a.gi) * kP3I;
+  const int per = ((c1 + kP3Warps - 1) / kP3Warps + 3) & ~3;
+  const int cb = warp * per, ce = cb + per < c1 ? cb + per : c1;
+  const int nsl = ce > cb ? (ce - cb) / kP3Slice : 0;               // c1 is a multiple of 4
+  float *ring = p3_smem + warp * (kP3Stages * kP3Stage);
+  // 72 pieces of each operand per slice: W2 rows of 36 floats (4 channels of one o), W1 rows of 72 (8 i of one channel)
+  const float *src[5];
+  int step[5];
+#pragma unroll
+  for (int h = 0; h < 5; ++h) {
+    const int e = lane + 32 * h;
+    src[h] = nullptr;
+    step[h] = 0;
+    if (e < 72) {
+      const int o = e / 9, x = e - o * 9;
+      if (o0 + o < c2) { src[h] = l2.w + ((size_t)(o0 + o) * c1 + cb) * 9 + x * 4; step[h] = kP3Slice * 9; }
+    } else if (e < 144) {
+      const int f = e - 72, c = f / 18, x = f - c * 18;             // a piece lies inside one channel's 8 i: c0 is a multiple of 4
+      if (i0 * 9 + x * 4 < c0 * 9) { src[h] = l1.w + ((size_t)(cb + c) * c0 + i0) * 9 + x * 4; step[h] = kP3Slice * c0 * 9; }
+    }
+  }
+  auto fetch = [&](int buf) {
+    float *st = ring + buf * kP3Stage;
+#pragma unroll
+    for (int h = 0; h < 5; ++h) {
+      const int e = lane + 32 * h;
+      if (e < 144) mb_cp16(st + e * 4, src[h] ? src[h] : l2.w, src[h] != nullptr);
+      if (src[h]) src[h] += step[h];
+    }
+  };
+#pragma unroll
+  for (int sl = 0; sl < kP3Stages - 1; ++sl) {
+    if (sl < nsl) fetch(sl);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // BN scale of the first layer: lane l holds channel l & 3's of a slice, asked for a slice ahead
+  float bn_g = 1.f, bn_v = 1.f;
+  auto ask = [&](int sl) {
+    const int cs = cb + sl * kP3Slice + (lane & 3), c = cs < ce ? cs : cb;
+    if (l1.gamma) { bn_g = l1.gamma[c]; bn_v = l1.var[c]; }
+  };
+  auto scale = [&]() { return l1.gamma ? bn_g / sqrtf(bn_v + l1.eps) : 1.f; };
+  float sc = 1.f;
+  if (nsl > 0) { ask(0); sc = scale(); }
+  const int ol = (lane >> 3) * 2, il = lane & 7;
+  float acc[2][25] = {};
+  int buf = 0, fbuf = kP3Stages - 1;
+#pragma unroll 1
+  for (int sl = 0; sl < nsl; ++sl) {
+    ask(sl + 1);                                   // past the end: the warp's first channel, not used
+    asm volatile("cp.async.wait_group %0;" ::"n"(kP3Stages - 2) : "memory");
+    __syncwarp();
+    if (sl + kP3Stages - 1 < nsl) fetch(fbuf);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float *w2 = ring + buf * kP3Stage + ol * (kP3Slice * 9), *w1 = ring + buf * kP3Stage + kP3Op + il * 9;
+#pragma unroll
+    for (int c = 0; c < kP3Slice; ++c) {
+      const float s = __shfl_sync(0xffffffffu, sc, c);
+      float b[9], x[2][9];
+#pragma unroll
+      for (int t = 0; t < 9; ++t) {
+        b[t] = w1[c * (kP3I * 9) + t] * s;
+        x[0][t] = w2[c * 9 + t];
+        x[1][t] = w2[kP3Slice * 9 + c * 9 + t];
+      }
+#pragma unroll
+      for (int u2 = 0; u2 < 3; ++u2)
+#pragma unroll
+        for (int v2 = 0; v2 < 3; ++v2)
+#pragma unroll
+          for (int u1 = 0; u1 < 3; ++u1)
+#pragma unroll
+            for (int v1 = 0; v1 < 3; ++v1) {
+              acc[0][(u1 + u2) * 5 + v1 + v2] = fmaf(x[0][u2 * 3 + v2], b[u1 * 3 + v1], acc[0][(u1 + u2) * 5 + v1 + v2]);
+              acc[1][(u1 + u2) * 5 + v1 + v2] = fmaf(x[1][u2 * 3 + v2], b[u1 * 3 + v1], acc[1][(u1 + u2) * 5 + v1 + v2]);
+            }
+    }
+    sc = scale();
+    __syncwarp();                                  // the slice's buffer may be refilled
+    buf = buf + 1 == kP3Stages ? 0 : buf + 1;
+    fbuf = fbuf + 1 == kP3Stages ? 0 : fbuf + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int t = 0; t < 25; ++t) p3_smem[warp * kP3Tile + ((ol + h) * kP3I + il) * 25 + t] = acc[h][t];
+  __syncthreads();
+  const bool last = dv.mode >= 0;
+  for (int e = tid; e < kP3Tile; e += kP3Threads) {
+    float s = 0.f;
+#pragma unroll
+    for (int w = 0; w < kP3Warps; ++w) s += p3_smem[w * kP3Tile + e];
+    const int oi = e / 25, t = e - oi * 25, o = o0 + oi / kP3I, i = i0 + oi % kP3I;
+    if (o < c2 && i < c0) {
+      const float g2 = raw_scale(l2, o);
+      s *= g2;
+      const int u = t / 5 - 1, v = t - (t / 5) * 5 - 1;              // tap of the 3x3 kernel centred in the 5x5 one
+      if (u >= 0 && u < 3 && v >= 0 && v < 3) {
+        if (a.first.ident) s = fmaf(g2, l2.w[((size_t)o * c1 + i) * 9 + u * 3 + v], s);                       // W2 o I
+        if (a.second.ident) s = fmaf(raw_scale(l1, o), l1.w[((size_t)o * c0 + i) * 9 + u * 3 + v], s);        // I o W1
+      }
+      if (t == 12 && o == i) s += (a.first.ident && a.second.ident ? 1.f : 0.f) + (last && dv.ident ? 1.f : 0.f);
+      a.w_out[((size_t)o * c0 + i) * 25 + t] = s;
+    }
+    if (last && dv.mode > 0) p3_smem[e] = s;       // element e of warp 0's sums is read by this thread alone
+  }
+  if (!last || dv.mode == 0) return;
+  __syncthreads();
+  deliver_tile<kP3O, kP3I, 5>(dv, p3_smem, o0, i0, c0, c2, tid, kP3Threads);
+}
+
+// ----------------------------------------------------------------------------------------------
 // host: validation and geometry
 // ----------------------------------------------------------------------------------------------
 
@@ -854,8 +1193,31 @@ static inline int blocks_for(size_t total, int threads) {
   return (int)(b > 65535 ? 65535 : (b == 0 ? 1 : b));
 }
 
-// Composes second o first into a new piece; launches when `go`.
-static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool go, cudaStream_t st) {
+// CTAs that zero the chunks of a packed copy that hold no weight
+static int zero_ctas(const BlockDelivery &dv, const dc_geom &mg, int threads) {
+  const KOrder &ko = dv.ko;
+  if (dv.mode != 2) return 0;
+  const bool full = ko.fold == 0 && ko.pair == 0 && ko.n_pad == mg.c_out && ko.e == ko.e_pad && (!ko.rows || mg.c_in % 16 == 0);
+  return full ? 0 : dc_div_up(ko.ng * ko.e_pad * ko.n_pad, threads * 4);
+}
+
+// 3x3 after 3x3, 16-byte pieces of both operands
+static bool compose33_ok(int c_in, int c_mid, int k1, int s1, int k2) {
+  return k1 == 3 && s1 == 1 && k2 == 3 && c_in % 4 == 0 && c_mid % 4 == 0;
+}
+static void launch_compose33(const Operand33 &first, const Operand33 &second, int c0, int c1, int c2, float *w, float *b,
+                             const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st) {
+  const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
+  static unsigned char attr_done[kDcMaxDevices];
+  dc_set_max_smem_once(k_compose33, kP3Ring, attr_done);
+  (void)dc_launch_pdl(k_compose33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kP3Threads)), dim3(kP3Threads), kP3Ring, st, a, dv);
+}
+
+// Composes second o first into a new piece; launches when `go`.  With `dv`, the piece is the run's result: where the
+// kernel can deliver it itself it goes to w_final / b_final (and the packed copy) and *delivered is set.
+static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool go, cudaStream_t st,
+                     const BlockDelivery *dv = nullptr, const dc_geom *mg = nullptr, float *w_final = nullptr,
+                     float *b_final = nullptr, bool *delivered = nullptr) {
   Piece out;
   out.c_in = first.c_in; out.c_out = second.c_out;
   out.k = first.k + (second.k - 1) * first.stride;
@@ -868,7 +1230,13 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
   out.w = w; out.b = b;
   if (go) {
     const int nbias = bias_blocks(out.c_out, 256);
-    if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k > 1 &&
+    if (!first.diag && !second.diag && compose33_ok(first.c_in, first.c_out, first.k, first.stride, second.k)) {
+      auto operand = [](const Piece &p) { return Operand33{RawLayer{p.w, p.b, nullptr, nullptr, nullptr, nullptr, 0.f}, p.ident}; };
+      BlockDelivery piece{nullptr, -1, 0, KOrder{}};
+      if (dv) { out.w = w = w_final; out.b = b = b_final; *delivered = true; }
+      launch_compose33(operand(first), operand(second), first.c_in, first.c_out, second.c_out, w, b, dv ? *dv : piece,
+                       mg ? *mg : dc_geom{}, st);
+    } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k > 1 &&
         first.c_out * second.k * second.k <= kAfter1x1MaxFloats) {
       dim3 grid(dc_div_up(out.c_in * out.k * out.k, 256), out.c_out + 1);
       if ((int)grid.x < nbias) grid.x = nbias;
@@ -876,9 +1244,6 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
     } else if (!first.diag && !second.diag && elems <= (size_t)200000 && second.k <= 7) {
       const int gx = dc_div_up(out.c_in * out.k * out.k, 32), gy = dc_div_up(out.c_out, 8);
       k_compose_dd_small<<<gx * gy + nbias, 256, 0, st>>>(first, second, w, b, out.k, gx, gy);
-    } else if (!first.diag && !second.diag && first.k == 3 && second.k == 3 && first.stride == 1) {
-      const int gx = dc_div_up(out.c_in, 32), gy = dc_div_up(out.c_out, 16);
-      k_compose_poly33<<<gx * gy + nbias, 256, 0, st>>>(first, second, w, b, gx, gy);
     } else if (!first.diag && !second.diag) {
       // 128 x 64 tiles when they still give every SM two tiles, 64 x 64 otherwise
       const int gx = dc_div_up(out.c_in * out.k * out.k, 64);
@@ -902,19 +1267,24 @@ static int group_of(const dc_residual *res, int n_res, int idx) {
   return -1;
 }
 
-// Hidden channels k_merge_block stages per pass for this block (0: the block does not qualify).
+// How the block that starts at layer i is merged: kTiledBlock by k_merge_block33, a positive number by k_merge_block
+// (hidden channels it stages per pass), 0: the layers are no such block.
+constexpr int kTiledBlock = -1;
 static int block_chunk(const dc_layer *L, int n, const dc_residual *res, int n_res, int i) {
   if (i + 2 >= n) return 0;
   const dc_layer &e = L[i], &d = L[i + 1], &p = L[i + 2];
   if (e.groups != 1 || e.k != 1 || e.stride != 1 || e.pad != 0) return 0;
   if (d.groups == 1 || d.groups != d.c_in) return 0;
   if (p.groups != 1 || p.k != 1 || p.stride != 1 || p.pad != 0) return 0;
-  if (e.c_in * d.k * d.k > kBlockThreads * kBlockMaxPerThread) return 0;
-  // wide blocks are faster step by step: their compositions fill the GPU, one CTA per output channel does not
-  if ((long)e.c_out * e.c_in * d.k * d.k > 150000) return 0;
   const int g0 = group_of(res, n_res, i), g1 = group_of(res, n_res, i + 1), g2 = group_of(res, n_res, i + 2);
   const bool whole = g0 >= 0 && g0 == g1 && g1 == g2 && res[g0].first == i && res[g0].last == i + 2;
   if (!whole && (g0 >= 0 || g1 >= 0 || g2 >= 0)) return 0;
+  // 16-byte pieces of every operand; the bias blocks hold one float per hidden channel where the operand rings lie
+  if (d.k == 3 && e.c_in % 4 == 0 && e.c_out % 4 == 0 && e.c_out <= kMbRing / 4) return kTiledBlock;
+  if (e.c_in * d.k * d.k > kBlockThreads * kBlockMaxPerThread) return 0;
+  // wide blocks of other kernel sizes are faster step by step: their compositions fill the GPU, one CTA per output
+  // channel does not
+  if ((long)e.c_out * e.c_in * d.k * d.k > 150000) return 0;
   const int per = e.c_in + d.k * d.k + 1;
   int ch = (200 * 1024 / 4) / per;
   if (ch > e.c_out) ch = e.c_out;
@@ -937,12 +1307,33 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   if (merged) *merged = mg;
   Bump bump{go ? (char *)workspace : nullptr, 0};
 
+  // What the last launch delivers.  A run that is one block of the tiled kind, or two dense 3x3 layers, needs no launch of
+  // its own for that (nor, in the second case, for the BN): the kernel that merges it reads the layers as they are and
+  // writes the result and the packed copy (a chunk of which is 8 input channels).
+  const size_t elems = (size_t)mg.c_out * mg.c_in * mg.k * mg.k;
+  KOrder ko;
+  dc_korder_init(&ko, &mg);
+  const int mode = !w_packed ? 0 : (packed_dtype == DC_F32 ? 1 : 2);
+  if (go && !dc_aligned16(w_packed)) return DC_ERR_ALIGNMENT;
+  const bool can_pack = mode != 2 || mg.c_in % 8 == 0;
+  if (go && n == 2 && algo != DC_MERGE_STEPS && can_pack && layers[0].groups == 1 && layers[1].groups == 1 &&
+      compose33_ok(layers[0].c_in, layers[0].c_out, layers[0].k, layers[0].stride, layers[1].k)) {
+    int id[2] = {0, 0}, whole = 0;
+    for (int g = 0; g < n_res; ++g) {
+      if (res[g].first != res[g].last) whole = 1;
+      else id[res[g].first] = 1;
+    }
+    launch_compose33(Operand33{raw_of(layers[0]), id[0]}, Operand33{raw_of(layers[1]), id[1]}, mg.c_in, layers[0].c_out, mg.c_out,
+                     w_merged, b_merged, BlockDelivery{w_packed, mode, whole, ko}, mg, st);
+    return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+  }
+
   // 0. inverted-residual blocks (1x1, depthwise, 1x1) are merged in one step from the raw layers
   std::vector<int> chunk_at(n, 0), covered(n, 0);
   if (algo != DC_MERGE_STEPS)
     for (int i = 0; i + 2 < n;) {
       const int ch = block_chunk(layers, n, res, n_res, i);
-      if (ch > 0) { chunk_at[i] = ch; covered[i] = covered[i + 1] = covered[i + 2] = 1; i += 3; }
+      if (ch != 0) { chunk_at[i] = ch; covered[i] = covered[i + 1] = covered[i + 2] = 1; i += 3; }
       else ++i;
     }
 
@@ -980,11 +1371,26 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     flush();
   }
 
+  const bool at_once = n == 3 && chunk_at[0] == kTiledBlock && can_pack;
+
   // 2. compose: blocks and skip groups first (with their identity tap), then left to right
   BlockBatch batch;
   int n_batch = 0, batch_grid = 0;
   size_t batch_smem = 0;
+  TiledBlocks tiled;
+  tiled.n = 0;
+  tiled.first[0] = 0;
+  BlockDelivery dv{nullptr, -1, 0, ko};
+  bool delivered = false;
+  auto flush_tiled = [&]() {
+    if (tiled.n == 0) return;
+    static unsigned char attr_done[kDcMaxDevices];
+    dc_set_max_smem_once(k_merge_block33, kMbRing, attr_done);
+    (void)dc_launch_pdl(k_merge_block33, dim3(tiled.first[tiled.n] + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), kMbRing, st, tiled, dv);
+    tiled.n = 0;
+  };
   auto flush_blocks = [&]() {
+    flush_tiled();
     if (n_batch == 0) return;
     static unsigned char attr_done[kDcMaxDevices];
     dc_set_max_smem_once(k_merge_block, 200 * 1024, attr_done);
@@ -997,13 +1403,22 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   while (i < n) {
     Piece piece;
     int gi = find_group(res, n_res, i);
-    if (chunk_at[i] > 0) {
+    if (chunk_at[i] != 0) {
       const dc_layer &e = layers[i], &d = layers[i + 1], &p = layers[i + 2];
       piece = Piece{nullptr, nullptr, e.c_in, p.c_out, d.k, d.stride, 0, gi >= 0 ? 1 : 0};
       float *w = bump.take(piece_elems(piece.c_in, piece.c_out, piece.k, 0));
       float *b = bump.take(piece.c_out);
+      if (at_once) {
+        w = w_merged; b = b_merged;
+        dv.packed = w_packed; dv.mode = mode; dv.ident = piece.ident;
+      }
       piece.w = w; piece.b = b;
-      if (go) {
+      if (go && chunk_at[i] == kTiledBlock) {
+        const int t = tiled.n++;
+        tiled.blk[t] = BlockArgs{raw_of(e), raw_of(d), raw_of(p), e.c_in, e.c_out, p.c_out, d.k, 0, w, b};
+        tiled.first[t + 1] = tiled.first[t] + dc_div_up(e.c_in, kMbI) * dc_div_up(p.c_out, kMbO) + dc_div_up(p.c_out, kMbO);
+        if (tiled.n == kBlockBatch) flush_tiled();
+      } else if (go) {
         batch.blk[n_batch] = BlockArgs{raw_of(e), raw_of(d), raw_of(p), e.c_in, e.c_out, p.c_out, d.k, chunk_at[i], w, b};
         const size_t smem = (size_t)chunk_at[i] * (e.c_in + d.k * d.k + 1) * sizeof(float);
         if (smem > batch_smem) batch_smem = smem;
@@ -1026,24 +1441,20 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     if (!have) { acc = piece; have = true; }
     else {
       if (go) flush_blocks();
-      acc = compose(acc, piece, bump, go, st);
+      // the run's last composition: piece.ident is the second operand's, the result carries none
+      const BlockDelivery fin{w_packed, mode, 0, ko};
+      const bool last = i == n && go && can_pack;
+      acc = compose(acc, piece, bump, go, st, last ? &fin : nullptr, &mg, w_merged, b_merged, &delivered);
     }
   }
   if (need) *need = bump.off + 256;
   if (!go) return DC_OK;
   flush_blocks();
 
+  if (at_once || delivered) return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+
   // 3. deliver: dense fp32 result, bias, optional packed copy, in one launch
-  size_t elems = (size_t)mg.c_out * mg.c_in * mg.k * mg.k;
-  KOrder ko;
-  dc_korder_init(&ko, &mg);
-  int mode = 0;
-  size_t p_elems = 0;
-  if (w_packed) {
-    mode = packed_dtype == DC_F32 ? 1 : 2;
-    p_elems = mode == 1 ? elems : (size_t)ko.ng * ko.e_pad * ko.n_pad * 8;
-    if (!dc_aligned16(w_packed)) return DC_ERR_ALIGNMENT;
-  }
+  const size_t p_elems = mode == 2 ? (size_t)ko.ng * ko.e_pad * ko.n_pad * 8 : elems;
   const int chunked = mode == 2 && p_elems >= (size_t)262144;
   const int nb_w = blocks_for(elems, 256), nb_p = mode ? blocks_for(chunked ? p_elems / 8 : p_elems, 256) : 0;
   k_deliver<<<nb_w + 1 + nb_p, 256, 0, st>>>(acc, w_merged, b_merged, w_packed, mode, ko, nb_w, nb_p, chunked);
