@@ -180,10 +180,9 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
       g->c_in % 8 == 0 && g->c_out % 8 == 0) {
     const int n16 = (int)dc_round_up((size_t)g->c_out, 16);
     ko->rows = 1;
-    // output channels per pass: at most 128, fewer for 5x5 and 7x7 kernels, whose weight stage of one
-    // (plane, tap row) step (k * 8 chunk planes of n_tile rows) must fit the shared-memory ring twice
-    // beside two activation stages and the epilogue's turn-around buffers
-    const int n_tile_max = (g->k == 1 && g->c_in >= 512 && g->c_out > 256) ? 256 : (g->k <= 4 ? 128 : (g->k <= 5 ? 96 : 64));
+    // output channels per pass: at most 128 (two accumulator sets of two blocks in tensor memory; from 128 columns on
+    // the tensor core runs at its rate), 256 for deep 1x1 layers with many outputs
+    const int n_tile_max = (g->k == 1 && g->c_in >= 512 && g->c_out > 256) ? 256 : 128;
     ko->nnt = dc_div_up(n16, n_tile_max);
     ko->n_tile = (int)dc_round_up((size_t)dc_div_up(n16, ko->nnt), 16);
     ko->n_pad = ko->nnt * ko->n_tile;

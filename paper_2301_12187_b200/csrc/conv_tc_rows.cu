@@ -51,6 +51,7 @@ struct RowsParams {
   int mb;                      // blocks per tile
   int lines_img;               // rbox * wbox: GEMM rows per image of a tile
   uint32_t inv_lines, inv_wbox; // ceil(2^20 / lines_img), ceil(2^20 / wbox)
+  int partial;                       // weight stages of one tap column instead of a whole (plane, tap row) step
   int a_stage_bytes, a_box_bytes, b_stage_bytes;
   int sa, sb, nacc, act;
   int b_resident;              // all weights stay in shared memory (one copy per CTA)
@@ -89,8 +90,11 @@ struct Item {
 
 // RESIDENT: all weights of the layer (a single output-channel pass, at most 128 KB) stay in shared memory:
 // one copy per CTA instead of one stream per work item.  Compile-time, so that the streaming version's
-// loops carry no switches.
-template <bool RESIDENT>
+// loops carry no switches.  PARTIAL (streamed weights only): a weight stage holds one tap column of a (plane, tap row)
+// step instead of all of them, for layers whose whole step does not fit twice beside the activation planes (5x5 with
+// 128 outputs per pass: 82 KB).  Where it fits, the whole step is faster: half as many waits, and longer stretches of
+// instructions (160 -> 960 3x3: 26.0 us whole and two deep, 30.2 us by tap columns six deep).
+template <bool RESIDENT, bool PARTIAL>
 __global__ void __launch_bounds__(kThreads, 1)
 k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
                const void *__restrict__ w_packed, const float *__restrict__ bias,
@@ -165,19 +169,20 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           }
           if (++sa == p.sa) { sa = 0; pa ^= 1; }
           const int nsl = plane_steps(p, g);
-          const int nplanes = p.k * nsl * 2;     // chunk planes of one (g, r) step
+          const int nplanes = (PARTIAL ? 1 : p.k) * nsl * 2;       // chunk planes of one weight stage
+          const int nstages = PARTIAL ? p.k * p.k : p.k;
+          size_t plane0 = (size_t)g * p.k * p.k * 8;
 #pragma unroll 1
-          for (int r = 0; r < p.k && !RESIDENT; ++r) {
+          for (int r = 0; r < nstages && !RESIDENT; ++r, plane0 += nplanes) {
             if (!warp_wait(&sh.b_empty[sb], pb ^ 1, abort_flag, ws, 0x20000u | sb)) { ok = false; break; }
-            const uint32_t dst = b_base0 + (uint32_t)sb * (uint32_t)p.b_stage_bytes;
-            const size_t plane0 = (size_t)g * p.k * p.k * 8 + (size_t)r * nplanes;
-            if (lane == 0) mbar_arrive_expect_tx(&sh.b_full[sb], (uint32_t)(nplanes * p.n_tile * 16));
-            __syncwarp();
-            // the planes of a step are contiguous in the packed weights, with several passes too (there a
+            // the planes of a stage are contiguous in the packed weights, with several passes too (there a
             // pass's rows of all planes are stored together): one bulk copy
-            if (lane == 0)
-              bulk_load(dst, wsrc + ((size_t)q.nt * p.planes_all + plane0) * p.n_tile * 16, (uint32_t)(nplanes * p.n_tile * 16),
-                        &sh.b_full[sb]);
+            if (lane == 0) {
+              const uint32_t bytes = (uint32_t)(nplanes * p.n_tile * 16);
+              mbar_arrive_expect_tx(&sh.b_full[sb], bytes);
+              bulk_load(b_base0 + (uint32_t)sb * (uint32_t)p.b_stage_bytes,
+                        wsrc + ((size_t)q.nt * p.planes_all + plane0) * p.n_tile * 16, bytes, &sh.b_full[sb]);
+            }
             if (++sb == p.sb) { sb = 0; pb ^= 1; }
           }
         }
@@ -259,8 +264,11 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           tc_fence_after();
           const uint32_t a_stage = a_row0 + (uint32_t)sa * ((uint32_t)p.a_stage_bytes >> 4);
           const int nsl = plane_steps(p, g);
+          const int nstages = PARTIAL ? p.k * p.k : p.k;
+          uint32_t tap_off = 0;                            // of the stage's first tap, in 16-byte units; PARTIAL: its column
+          int col = 0;
 #pragma unroll 1
-          for (int r = 0; r < p.k; ++r) {
+          for (int r = 0; r < nstages; ++r) {
             uint32_t b_stage;
             if (RESIDENT) {
               b_stage = b_row0 + (uint32_t)((g * p.k * p.k * 8 + r * p.k * nsl * 2) * p.n_tile);   // planes before this step
@@ -279,12 +287,12 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const uint32_t d = tmem_base + (uint32_t)((set * p.mb + b) * p.n_tile);
                 // descriptors advance by adds only: +8 (one line) per tap column, +2 (32 bytes) per K step on
                 // the activation side, two chunk planes per instruction on the weight side
-                uint32_t a_lo = ((a_stage + (uint32_t)(b * 1024 + r * p.wbox * 8)) & 0x3FFFu) | (1u << 16);
+                uint32_t a_lo = ((a_stage + (uint32_t)(b * 1024) + tap_off) & 0x3FFFu) | (1u << 16);
                 uint32_t b_lo = (b_stage & 0x3FFFu) | ((uint32_t)p.n_tile << 16);
                 const uint32_t b_inc = 2u * (uint32_t)p.n_tile;
                 if (nsl == 4) {                  // a full plane of 64 channels
 #pragma unroll 1
-                  for (int s = 0; s < p.k; ++s, a_lo += 8u) {
+                  for (int s = 0; s < (PARTIAL ? 1 : p.k); ++s, a_lo += 8u) {
 #pragma unroll
                     for (int sl = 0; sl < 4; ++sl) {
                       umma_bf16(d, ((uint64_t)a_hi << 32) | (uint64_t)(a_lo + 2u * sl), ((uint64_t)b_hi << 32) | (uint64_t)b_lo, idesc, 1u);
@@ -293,7 +301,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                   }
                 } else {
 #pragma unroll 1
-                  for (int s = 0; s < p.k; ++s, a_lo += 8u) {
+                  for (int s = 0; s < (PARTIAL ? 1 : p.k); ++s, a_lo += 8u) {
 #pragma unroll 1
                     for (int sl = 0; sl < nsl; ++sl) {
                       umma_bf16(d, ((uint64_t)a_hi << 32) | (uint64_t)(a_lo + 2u * sl), ((uint64_t)b_hi << 32) | (uint64_t)b_lo, idesc, 1u);
@@ -307,6 +315,14 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             if (!RESIDENT) {
               if (leader) umma_commit(&sh.b_empty[sb]);    // this warp is done with the weight stage
               if (++sb == p.sb) { sb = 0; pb ^= 1; }
+            }
+            if (!PARTIAL) {
+              tap_off += (uint32_t)(p.wbox * 8);
+            } else if (++col == p.k) {
+              col = 0;
+              tap_off += (uint32_t)((p.wbox - p.k + 1) * 8);
+            } else {
+              tap_off += 8u;
             }
           }
           if (ok && leader) umma_commit(&sh.a_empty[sa]);  // ... and with the plane
@@ -349,7 +365,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll 1
         for (int b = blk_lo + par; b < blk_hi; b += 2) {
           const int pos = b * 128 + q * 32 + lane;
-          // pos < 512 and the divisors are at most 256: multiplying by the rounded-up reciprocal is exact
+          // pos < 256 and the divisors are below 2^12: multiplying by the rounded-up reciprocal is exact
           const int il = (int)(((uint32_t)pos * p.inv_lines) >> 20), rem = pos - il * p.lines_img;
           const int yy = (int)(((uint32_t)rem * p.inv_wbox) >> 20), xx = rem - yy * p.wbox;
           const bool valid = il < p.ni && iq.img0 + il < p.n_img && yy < th_valid && xx < tw_valid;
@@ -471,65 +487,96 @@ EncodeTiledFn get_encode_fn() {
 }
 
 constexpr int kSmemBudget = 220 * 1024;
-constexpr int kMaxLines = 128 * kMaxBlocks;      // GEMM rows of a tile
 constexpr int kSlack = 1024;
+
+// Shared memory in front of the rings: constant operand, bias rows and zero rows, the epilogue warps' buffers.
+int rows_fixed_bytes(const KOrder &ko, int *off_stage) {
+  *off_stage = (int)dc_round_up((size_t)1024 + (size_t)(ko.n_pad + ko.n_tile) * 16, 128);
+  return (int)dc_round_up((size_t)*off_stage + kEpiWarps * 32 * kStagePitch, 1024);
+}
 
 bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   KOrder ko;
   dc_korder_init(&ko, g);
   if (!ko.rows) return false;
+  if ((long long)n * h * w * g->c_in >= (1ll << 40) || (long long)n * h * w >= (1ll << 31)) return false;
+  // a 1x1 layer does not know rows or images: its pixels are one run, which tiles cut without a remainder per row
+  if (g->k == 1 && g->pad == 0) { w *= n * h; n = 1; h = 1; }
   const int ho = dc_out_extent(h, g->k, 1, g->pad), wo = dc_out_extent(w, g->k, 1, g->pad);
-  if (ho <= 0 || wo <= 0) return false;
-  if ((long long)n * h * w * g->c_in >= (1ll << 40) || (long long)n * ho * wo >= (1ll << 31)) return false;
+  if (ho <= 0 || wo <= 0 || (long long)n * ho * wo >= (1ll << 31)) return false;
   p->n_img = n; p->h = h; p->w = w; p->ho = ho; p->wo = wo;
   p->c_in = g->c_in; p->c_out = g->c_out;
   p->k = g->k; p->pad = g->pad;
   p->planes = dc_div_up(g->c_in, 64);
   p->n_tile = ko.n_tile; p->nnt = ko.nnt; p->n_pad = ko.n_pad;
   p->planes_all = ko.e_pad;
-  // tile: as many rows as fit kMaxLines GEMM rows; whole small images several at a time.  Rows may be cut into
-  // strips: of the first few strip counts that fit, the one with the fewest tiles per image wins (28 x 28 with a
-  // 3 x 3 kernel: two strips of 14 columns x 14 rows make 4 tiles where full rows x 6 make 5)
-  int nxt0 = 1;
-  while (dc_div_up(wo, nxt0) + g->k - 1 > kMaxLines / g->k) ++nxt0;       // at least one output row per tile
-  int th = 0, best_tiles = 0;
+  p->off_bias = 0;
+  p->off_a = rows_fixed_bytes(ko, &p->off_stage);
+  // A tile's GEMM rows are the patch pixels from its first to its last output, halo columns included: at most two
+  // 128-row blocks.  Its patch (rows and halo) must fit the activation ring twice beside three weight stages.
+  const long long tap_bytes = 8ll * p->n_tile * 16;        // weights of one tap column of a (plane, tap row) step
+  const long long max_a = (kSmemBudget - 1024 - p->off_a - kSlack - (3 * tap_bytes > 26 * 1024 ? 3 * tap_bytes : 26 * 1024)) / 2;
+  // Tile: the least estimated time of the CTA with the most work.  An item costs its tensor-core instructions (cycles as
+  // measured for 128 x N x 16) or the bytes it takes in from L2 (20 per cycle and SM), whichever is more, and a chain of
+  // waits; several items overlap only in part.  Candidates: every strip count that leaves rows of at most 256 pixels, with
+  // as many rows as give two blocks or one, evened out over the height; whole small images several at a time.
+  const int cyc = 36 + p->n_tile / 4 > p->n_tile / 2 ? 36 + p->n_tile / 4 : p->n_tile / 2;
+  const double per_block = (double)g->k * g->k * dc_div_up(g->c_in, 16) * cyc;
+  const double w_item = (double)ko.e_pad * p->n_tile * 16;
+  double best = 0.0;
   p->nxt = 0;
-  for (int cand = nxt0; cand <= nxt0 + 3 && cand <= wo; ++cand) {
-    const int tw_c = dc_div_up(wo, cand), nxt_c = dc_div_up(wo, tw_c);
-    int th_c = kMaxLines / (tw_c + g->k - 1) - (g->k - 1);
-    if (th_c < 1) continue;
-    if (th_c > ho) th_c = ho;
-    const int tiles_c = nxt_c * dc_div_up(ho, th_c);
-    if (p->nxt == 0 || tiles_c < best_tiles) { p->nxt = nxt_c; p->tw = tw_c; th = th_c; best_tiles = tiles_c; }
+  auto consider = [&](int tw, int th, int ni) {
+    const int wbox = tw + g->k - 1, rbox = th + g->k - 1;
+    if (wbox > 256 || rbox > 256) return;
+    const int lines = rbox * wbox;
+    if ((long long)dc_round_up((size_t)ni * lines * 128, 1024) > max_a) return;
+    const int mb = dc_div_up((ni - 1) * lines + (th - 1) * wbox + tw, 128);
+    if (mb > kMaxBlocks) return;
+    const int nxt = dc_div_up(wo, tw);
+    const long long items = (long long)dc_div_up(n, ni) * nxt * dc_div_up(ho, th) * p->nnt;
+    const long long per_cta = (items + n_sm - 1) / n_sm, blocks = (items * mb + n_sm - 1) / n_sm;
+    const double mma = (double)(blocks < per_cta * mb ? blocks : per_cta * mb) * per_block;
+    const double intake = (double)per_cta * ((double)ni * lines * 128 * p->planes + w_item) / 20.0;
+    const double all = (double)items * ((double)ni * lines * 128 * p->planes + w_item) / 3000.0;      // what L2 gives all SMs together
+    const double mem = intake > all ? intake : all;
+    const double cost = (mma > mem ? mma + 0.2 * mem : mem + 0.2 * mma) + 1500.0 * (double)per_cta + lines * 2.0;
+    if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; }
+  };
+  int nxt0 = 1;
+  while (dc_div_up(wo, nxt0) + g->k - 1 > 256) nxt0 = nxt0 < 64 ? nxt0 + 1 : nxt0 + nxt0 / 32;
+  if (ho == 1 && g->k == 1) {
+    // one run of pixels: full tiles, or as many as there are CTAs to take them
+    consider(wo < 256 ? wo : 256, 1, 1);
+    consider(wo < 128 ? wo : 128, 1, 1);
+    for (int r = 1; r <= 4; ++r) {
+      const long long tiles = (long long)r * n_sm / p->nnt;
+      const long long tw = tiles > 0 ? (wo + tiles - 1) / tiles : 0;
+      if (tw >= 1 && tw <= 256) consider((int)tw, 1, 1);
+    }
+  } else {
+    for (int cand = nxt0; cand <= nxt0 + 5 && cand <= wo; ++cand) {
+      const int tw = dc_div_up(wo, cand);
+      int last_th = 0;
+      for (int mb = kMaxBlocks; mb >= 1; --mb) {
+        if (mb * 128 < tw) break;
+        int th = (mb * 128 - tw) / (tw + g->k - 1) + 1;
+        if (th > ho) th = ho;
+        if (th != last_th) consider(tw, th, 1);
+        last_th = th;
+        const int even = dc_div_up(ho, dc_div_up(ho, th));
+        if (even != th) consider(tw, even, 1);
+      }
+    }
+    if (nxt0 == 1)
+      for (int ni = 2; ni <= 8 && ni <= n; ++ni) consider(wo, ho, ni);
   }
   if (p->nxt == 0) return false;
+  const int th = p->th;
   p->wbox = p->tw + g->k - 1;
-  p->th = th;
   p->rbox = th + g->k - 1;
   p->lines_img = p->rbox * p->wbox;
   p->inv_lines = ((1u << 20) + (uint32_t)p->lines_img - 1) / (uint32_t)p->lines_img;
   p->inv_wbox = ((1u << 20) + (uint32_t)p->wbox - 1) / (uint32_t)p->wbox;
-  p->ni = 1;
-  if (th == ho && p->nxt == 1) {
-    int ni_max = kMaxLines / p->lines_img;
-    if (ni_max > n) ni_max = n;
-    if (ni_max > 8) ni_max = 8;
-    if (ni_max < 1) ni_max = 1;
-    // Fewer images per tile where that fills the machine: a work item takes in its activation planes and its
-    // pass's weights from L2, and the launch lasts as long as the CTA with the most items.  Cost of a choice =
-    // items per CTA x (bytes of an item + 64 KB for the item's own chain of waits); a smaller count must win
-    // by a tenth.  960 -> 160, 1 x 1, 128 images of 7 x 7: two images per tile (128 items) instead of five (52).
-    const long long w_item = (long long)ko.e_pad * p->n_tile * 16;
-    long long best_cost = 0;
-    p->ni = ni_max;
-    for (int c = ni_max; c >= 1; --c) {
-      const long long items_c = (long long)dc_div_up(n, c) * p->nnt;
-      const long long per_cta = (items_c + n_sm - 1) / n_sm;
-      const long long cost = per_cta * ((long long)c * p->lines_img * 128 * p->planes + w_item + 64 * 1024);
-      if (c == ni_max || cost * 10 < best_cost * 9) { best_cost = cost; p->ni = c; }
-    }
-  }
-  if (p->wbox > 256 || p->rbox > 256) return false;
   p->tiles_y = dc_div_up(ho, th);
   p->img_groups = dc_div_up(n, p->ni);
   const int last = (p->ni - 1) * p->lines_img + (th - 1) * p->wbox + p->tw;    // GEMM rows up to the last valid one
@@ -562,13 +609,9 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   }
   p->a_box_bytes = p->ni * p->lines_img * 128;
   p->a_stage_bytes = (int)dc_round_up((size_t)p->a_box_bytes, 1024);
-  p->b_stage_bytes = (int)dc_round_up((size_t)g->k * 4 * 2 * p->n_tile * 16, 1024);
   // Layout: bias, activation stages, weight stages.  A block's 128 GEMM rows plus the tap shift may
   // reach up to ~200 lines (25 KB) past its stage; behind the last activation stage that lands in
   // the weight stages, which are larger (what is read there only feeds rows that are dropped).
-  p->off_bias = 0;
-  p->off_stage = (int)dc_round_up((size_t)1024 + (size_t)(p->n_pad + p->n_tile) * 16, 128);   // constant operand, bias rows, zero rows
-  p->off_a = (int)dc_round_up((size_t)p->off_stage + kEpiWarps * 32 * kStagePitch, 1024);
   // rings: weights first (they are the larger stream), then activation planes
   int sa = 2, sb = 2;
   // Small weights of a single pass stay resident where a work item would otherwise stream more weight than
@@ -577,12 +620,19 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   // version measured no faster.)
   const long long b_all = (long long)dc_round_up((size_t)ko.e_pad * p->n_tile * 16, 1024);
   p->b_resident = (p->nnt == 1 && b_all <= 128 * 1024 && (p->planes >= 3 || b_all >= 2ll * p->a_stage_bytes)) ? 1 : 0;
+  // a weight stage is a whole (plane, tap row) step where that fits twice
+  p->partial = 0;
+  p->b_stage_bytes = (int)dc_round_up((size_t)(g->k * tap_bytes), 1024);
   auto total = [&](int a, int b) {
     const long long wbytes = p->b_resident ? b_all : (long long)b * p->b_stage_bytes;
     const long long tail = wbytes >= 26 * 1024 ? kSlack : 26 * 1024 - wbytes + kSlack;   // room for the overrun
     return 1024ll + p->off_a + wbytes + (long long)a * p->a_stage_bytes + tail;
   };
   if (p->b_resident && total(sa, sb) > kSmemBudget) p->b_resident = 0;
+  if (!p->b_resident && total(sa, sb) > kSmemBudget) {
+    p->partial = 1;
+    p->b_stage_bytes = (int)dc_round_up((size_t)tap_bytes, 1024);
+  }
   if (total(sa, sb) > kSmemBudget) return false;
   while (!p->b_resident && sb < kFirstB && total(sa, sb + 1) <= kSmemBudget) ++sb;
   while (sa < kFirstA && total(sa + 1, sb) <= kSmemBudget) ++sa;
@@ -619,8 +669,8 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
   CUtensorMap map_a;
   {
     const cuuint64_t C = (cuuint64_t)g->c_in;
-    cuuint64_t gdim[4] = {C, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
-    cuuint64_t gstr[3] = {2 * C, (cuuint64_t)w * C * 2, (cuuint64_t)h * w * C * 2};
+    cuuint64_t gdim[4] = {C, (cuuint64_t)p.w, (cuuint64_t)p.h, (cuuint64_t)p.n_img};
+    cuuint64_t gstr[3] = {2 * C, (cuuint64_t)p.w * C * 2, (cuuint64_t)p.h * p.w * C * 2};
     cuuint32_t box[4] = {64, (cuuint32_t)p.wbox, (cuuint32_t)p.rbox, (cuuint32_t)p.ni};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = encode(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(x), gdim, gstr, box, es,
@@ -628,11 +678,12 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return DC_ERR_CUDA;
   }
-  static unsigned char attr_done[kDcMaxDevices];
-  static unsigned char attr_done_r[kDcMaxDevices];
-  DC_CUDA_OK(p.b_resident ? dc_set_max_smem_once(k_conv_tc_rows<true>, kSmemBudget, attr_done_r)
-                          : dc_set_max_smem_once(k_conv_tc_rows<false>, kSmemBudget, attr_done));
-  const cudaError_t le = dc_launch_pdl(p.b_resident ? k_conv_tc_rows<true> : k_conv_tc_rows<false>, dim3(p.grid), dim3(kThreads), (size_t)p.smem_bytes, stream, map_a, p,
+  using Kernel = decltype(&k_conv_tc_rows<false, false>);
+  static constexpr Kernel kernels[3] = {k_conv_tc_rows<false, false>, k_conv_tc_rows<true, false>, k_conv_tc_rows<false, true>};
+  static unsigned char attr_done[3][kDcMaxDevices];
+  const int which = p.b_resident ? 1 : (p.partial ? 2 : 0);
+  DC_CUDA_OK(dc_set_max_smem_once(kernels[which], kSmemBudget, attr_done[which]));
+  const cudaError_t le = dc_launch_pdl(kernels[which], dim3(p.grid), dim3(kThreads), (size_t)p.smem_bytes, stream, map_a, p,
                                        w_packed, bias, (const __nv_bfloat16 *)residual, (__nv_bfloat16 *)y,
                                        (DcWsHeader *)workspace);
   return le == cudaSuccess && cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;

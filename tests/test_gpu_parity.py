@@ -465,6 +465,21 @@ def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, several column strips and row tiles
+    (72, 200, 5, 1, 2, 2, 11, 13),       # the same in two passes, a partial plane of channels
+    (40, 48, 7, 1, 3, 1, 16, 40),        # 7x7
+    (64, 64, 3, 1, 1, 2, 9, 120),        # wide rows: a tile of two output rows
+    (64, 64, 3, 1, 1, 40, 5, 5),         # several small images per tile
+    (64, 64, 1, 1, 0, 1, 3, 5),          # 1x1: one short run of pixels
+    (96, 576, 1, 1, 0, 3, 13, 13),       # 1x1: pixels of several images in a tile, a ragged last tile
+    (64, 384, 1, 1, 0, 64, 14, 14),      # 1x1: more tiles than CTAs
+    (32, 96, 1, 1, 0, 1, 1, 1),          # one pixel
+])
+def test_rows_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (32, 32, 5, 1, 2, 3, 28, 28),       # whole pixel tiles and a ragged last one
     (8, 40, 3, 1, 1, 1, 7, 9),          # a K slice of 16 spans two taps; 40 channels per tile
     (4, 20, 3, 2, 1, 2, 9, 11),         # four taps per slice, K no multiple of a slice, stride 2
