@@ -55,6 +55,7 @@ struct RowsParams {
   int a_stage_bytes, a_box_bytes, b_stage_bytes;
   int sa, sb, nacc, act;
   int b_resident;              // all weights stay in shared memory (one copy per CTA)
+  int ksplit, part_pitch;      // CTAs that share an item's reduction; floats between rows of their partial sums
   int off_bias, off_stage, off_b, off_a, smem_bytes;
   int tmem_cols;
 };
@@ -94,7 +95,12 @@ struct Item {
 // step instead of all of them, for layers whose whole step does not fit twice beside the activation planes (5x5 with
 // 128 outputs per pass: 82 KB).  Where it fits, the whole step is faster: half as many waits, and longer stretches of
 // instructions (160 -> 960 3x3: 26.0 us whole and two deep, 30.2 us by tap columns six deep).
-template <bool RESIDENT, bool PARTIAL>
+//
+// SPLITK: a cluster of p.ksplit CTAs shares one work item, each taking a run of its (plane, tap row) steps, for layers
+// with fewer items than SMs whose reduction is long (384 -> 64 3x3 on one 14 x 14 image is one item of 432
+// instructions per block).  The partial sums meet in distributed shared memory -- in the rings' place, which nothing
+// reads any more -- and are added in rank order; every CTA finishes its share of the outputs.
+template <bool RESIDENT, bool PARTIAL, bool SPLITK>
 __global__ void __launch_bounds__(kThreads, 1)
 k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
                const void *__restrict__ w_packed, const float *__restrict__ bias,
@@ -118,7 +124,15 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   int nitems = p.items_per + (bid < p.items_rem ? 1 : 0);
   int item0 = bid * p.items_per + (bid < p.items_rem ? bid : p.items_rem);
   int blk_first = 0, blk_end = p.mb;
-  if (p.split) {
+  // this CTA's run of the item's (plane, weight stage) steps
+  const int nstages = PARTIAL ? p.k * p.k : p.k;
+  const int rank = SPLITK ? bid % p.ksplit : 0;
+  const int st0 = SPLITK ? p.planes * nstages * rank / p.ksplit : 0;
+  const int st1 = SPLITK ? p.planes * nstages * (rank + 1) / p.ksplit : p.planes * nstages;
+  if (SPLITK) {
+    item0 = bid / p.ksplit;
+    nitems = 1;
+  } else if (p.split) {
     const int u0 = item0, u1 = item0 + nitems - 1;           // first and last block of the run
     item0 = u0 / p.mb;
     const int item1 = u1 / p.mb;
@@ -159,7 +173,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         Item q;
         q.of(p, item0 + it);
 #pragma unroll 1
-        for (int g = 0; g < p.planes && ok; ++g) {
+        for (int g = SPLITK ? st0 / nstages : 0; g * nstages < st1 && ok; ++g) {
           if (!warp_wait(&sh.a_empty[sa], pa ^ 1, abort_flag, ws, 0x10000u | sa)) { ok = false; break; }
           if (lane == 0) {
             // channels past c_in, pixels outside the image and images past the batch arrive as zeros
@@ -170,10 +184,11 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (++sa == p.sa) { sa = 0; pa ^= 1; }
           const int nsl = plane_steps(p, g);
           const int nplanes = (PARTIAL ? 1 : p.k) * nsl * 2;       // chunk planes of one weight stage
-          const int nstages = PARTIAL ? p.k * p.k : p.k;
-          size_t plane0 = (size_t)g * p.k * p.k * 8;
+          const int r_lo = SPLITK && st0 > g * nstages ? st0 - g * nstages : 0;
+          const int r_hi = SPLITK && st1 < (g + 1) * nstages ? st1 - g * nstages : nstages;
+          size_t plane0 = (size_t)g * p.k * p.k * 8 + (size_t)r_lo * nplanes;
 #pragma unroll 1
-          for (int r = 0; r < nstages && !RESIDENT; ++r, plane0 += nplanes) {
+          for (int r = r_lo; r < r_hi && !RESIDENT; ++r, plane0 += nplanes) {
             if (!warp_wait(&sh.b_empty[sb], pb ^ 1, abort_flag, ws, 0x20000u | sb)) { ok = false; break; }
             // the planes of a stage are contiguous in the packed weights, with several passes too (there a
             // pass's rows of all planes are stored together): one bulk copy
@@ -189,6 +204,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
     }
     __syncwarp();
+    if (SPLITK) { cluster_sync(); cluster_sync(); }
   } else {
     // ---- consumer preparation
     if (warp == kMmaWarp) {
@@ -252,23 +268,25 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           // bias first (needs no load): it also initialises the accumulators of this warp's blocks
           Item iq;
           iq.of(p, item0 + it);
-          const uint32_t bias_row = bias_row0 + (uint32_t)(iq.nt * p.n_tile);
+          // (with the reduction split, one CTA adds the bias and the others start from zero rows)
+          const uint32_t bias_row = SPLITK && rank > 0 ? zero_row : bias_row0 + (uint32_t)(iq.nt * p.n_tile);
           const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)((bias_row & 0x3FFFu) | ((zero_row - bias_row) << 16));
 #pragma unroll 1
           for (int b = blk_lo + mw; b < blk_hi; b += kMmaWarps)
             if (leader) umma_bf16(tmem_base + (uint32_t)((set * p.mb + b) * p.n_tile), ones_desc, bd, idesc, 0u);
         }
 #pragma unroll 1
-        for (int g = 0; g < p.planes && ok; ++g) {
+        for (int g = SPLITK ? st0 / nstages : 0; g * nstages < st1 && ok; ++g) {
           if (!warp_wait(&sh.a_full[sa], pa, abort_flag, ws, 0x40000u | sa)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_stage = a_row0 + (uint32_t)sa * ((uint32_t)p.a_stage_bytes >> 4);
           const int nsl = plane_steps(p, g);
-          const int nstages = PARTIAL ? p.k * p.k : p.k;
-          uint32_t tap_off = 0;                            // of the stage's first tap, in 16-byte units; PARTIAL: its column
-          int col = 0;
+          const int r_lo = SPLITK && st0 > g * nstages ? st0 - g * nstages : 0;
+          const int r_hi = SPLITK && st1 < (g + 1) * nstages ? st1 - g * nstages : nstages;
+          int col = PARTIAL && SPLITK ? r_lo % p.k : 0;    // PARTIAL: tap column of the stage
+          uint32_t tap_off = (uint32_t)(((PARTIAL ? r_lo / p.k : r_lo) * p.wbox + col) * 8);   // of the stage's first tap, in 16-byte units
 #pragma unroll 1
-          for (int r = 0; r < nstages; ++r) {
+          for (int r = r_lo; r < r_hi; ++r) {
             uint32_t b_stage;
             if (RESIDENT) {
               b_stage = b_row0 + (uint32_t)((g * p.k * p.k * 8 + r * p.k * nsl * 2) * p.n_tile);   // planes before this step
@@ -348,8 +366,26 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                 (uint32_t)((lane & 3) ^ ((lane >> 3) & 3)) * 16u;
       uint32_t acc_ph[2] = {0u, 0u};
       const bool relu6 = p.act == DC_ACT_RELU6;
+      if (SPLITK && warp_wait(&sh.acc_full[0], 0u, abort_flag, ws, 0x60000u)) {
+        // all of this CTA's instructions are done, so its rings hold nothing any more: the partial sums go there
+        tc_fence_after();
+        const uint32_t part = smem_u32(smem_a);
 #pragma unroll 1
-      for (int it = 0; it < nitems; ++it) {
+        for (int b = par; b < p.mb; b += 2) {
+          const uint32_t row = part + (uint32_t)(b * 128 + q * 32 + lane) * (uint32_t)(p.part_pitch * 4);
+          const uint32_t taddr = tmem_row + (uint32_t)(b * p.n_tile);
+#pragma unroll 1
+          for (int ch = 0; ch < p.n_tile; ch += 16) {
+            uint32_t v[16];
+            tmem_ld16(taddr + (uint32_t)ch, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) sts_u4(row + (uint32_t)(ch + i) * 4u, make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]));
+          }
+        }
+      }
+#pragma unroll 1
+      for (int it = 0; it < nitems && !SPLITK; ++it) {
         const int set = p.nacc == 2 ? (it & 1) : 0;
         Item iq;
         iq.of(p, item0 + it);
@@ -455,6 +491,54 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (lane == 0) mbar_arrive(&sh.acc_empty[set]);
       }
     }
+    if (SPLITK) {
+      cluster_sync();                              // every CTA's partial sums are written
+      if (warp >= kFirstEpiWarp && !*abort_flag) {
+        Item iq;
+        iq.of(p, item0);
+        const int x0 = iq.xt * p.tw, y0 = iq.ty * p.th;
+        const int tw_valid = p.wo - x0 < p.tw ? p.wo - x0 : p.tw;
+        const int th_valid = p.ho - y0 < p.th ? p.ho - y0 : p.th;
+        const int ch0 = iq.nt * p.n_tile;
+        const int chunks = (p.c_out - ch0 < p.n_tile ? p.c_out - ch0 : p.n_tile) >> 3;
+        const uint32_t part = smem_u32(smem_a);
+        const bool relu6 = p.act == DC_ACT_RELU6;
+        // 8 channels of a pixel at a time, dealt out over the threads of the whole cluster
+#pragma unroll 1
+        for (int u = rank * (kEpiWarps * 32) + (int)threadIdx.x - kFirstEpiWarp * 32; u < p.mb * 128 * chunks; u += p.ksplit * kEpiWarps * 32) {
+          const int pos = u / chunks, ch = (u - pos * chunks) * 8;
+          const int il = (int)(((uint32_t)pos * p.inv_lines) >> 20), rem = pos - il * p.lines_img;
+          const int yy = (int)(((uint32_t)rem * p.inv_wbox) >> 20), xx = rem - yy * p.wbox;
+          if (il >= p.ni || iq.img0 + il >= p.n_img || yy >= th_valid || xx >= tw_valid) continue;
+          const uint32_t at = part + (uint32_t)(pos * p.part_pitch + ch) * 4u;
+          float f[8] = {};
+#pragma unroll 4
+          for (int r = 0; r < p.ksplit; ++r) {
+            const uint32_t remote = map_cluster(at, (uint32_t)r);
+            const uint4 lo = lds_cluster_u4(remote), hi = lds_cluster_u4(remote + 16u);
+            f[0] += __uint_as_float(lo.x); f[1] += __uint_as_float(lo.y); f[2] += __uint_as_float(lo.z); f[3] += __uint_as_float(lo.w);
+            f[4] += __uint_as_float(hi.x); f[5] += __uint_as_float(hi.y); f[6] += __uint_as_float(hi.z); f[7] += __uint_as_float(hi.w);
+          }
+          const size_t o = ((size_t)((iq.img0 + il) * p.ho + (y0 + yy)) * p.wo + (x0 + xx)) * p.c_out + ch0 + ch;
+          if (residual) {
+            const uint4 rv = *reinterpret_cast<const uint4 *>(residual + o);
+            const __nv_bfloat162 *rb = reinterpret_cast<const __nv_bfloat162 *>(&rv);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float2 rf = __bfloat1622float2(rb[i]);
+              f[2 * i] += rf.x; f[2 * i + 1] += rf.y;
+            }
+          }
+          uint4 ov;
+          uint32_t *ow = reinterpret_cast<uint32_t *>(&ov);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            ow[i] = relu6 ? min_bf16x2(pack_bf16x2_relu(f[2 * i], f[2 * i + 1]), 0x40C040C0u) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
+          *reinterpret_cast<uint4 *>(y + o) = ov;
+        }
+      }
+      cluster_sync();                              // nobody leaves while its sums may still be read
+    }
     // ---- consumer teardown
     if (*abort_flag) {
       const unsigned long long t0 = globaltimer_ns();
@@ -495,6 +579,38 @@ int rows_fixed_bytes(const KOrder &ko, int *off_stage) {
   return (int)dc_round_up((size_t)*off_stage + kEpiWarps * 32 * kStagePitch, 1024);
 }
 
+// Clusters of `size` CTAs (an SM's shared memory each) the current device runs at once: a property of its GPCs, asked for
+// once per device.  Without a device (planning on the host): a B200's.
+constexpr int kMaxSplit = 8;
+int max_clusters(int size) {
+  static constexpr int kB200[kMaxSplit + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+  static int cached[kDcMaxDevices][kMaxSplit + 1];
+  const int dev = dc_current_device();
+  if (dev < 0) { (void)cudaGetLastError(); return kB200[size]; }
+  if (cached[dev][size] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size * 64);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBudget;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    static unsigned char attr_done[kDcMaxDevices];
+    if (dc_set_max_smem_once(k_conv_tc_rows<false, false, true>, kSmemBudget, attr_done) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, k_conv_tc_rows<false, false, true>, &cfg) != cudaSuccess || n <= 0) {
+      (void)cudaGetLastError();
+      n = kB200[size];
+    }
+    cached[dev][size] = n;
+  }
+  return cached[dev][size];
+}
+
 bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   KOrder ko;
   dc_korder_init(&ko, g);
@@ -516,15 +632,20 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   // 128-row blocks.  Its patch (rows and halo) must fit the activation ring twice beside three weight stages.
   const long long tap_bytes = 8ll * p->n_tile * 16;        // weights of one tap column of a (plane, tap row) step
   const long long max_a = (kSmemBudget - 1024 - p->off_a - kSlack - (3 * tap_bytes > 26 * 1024 ? 3 * tap_bytes : 26 * 1024)) / 2;
-  // Tile: the least estimated time of the CTA with the most work.  An item costs its tensor-core instructions (cycles as
-  // measured for 128 x N x 16) or the bytes it takes in from L2 (20 per cycle and SM), whichever is more, and a chain of
-  // waits; several items overlap only in part.  Candidates: every strip count that leaves rows of at most 256 pixels, with
-  // as many rows as give two blocks or one, evened out over the height; whole small images several at a time.
+  // Tile and split of the reduction: the least estimated time of the CTA with the most work, in cycles.  An item costs
+  // its tensor-core instructions (a 128 x N x 16 takes max(36 + N/4, N/2)) and the bytes it takes in from L2, which
+  // overlap in part, and a chain of waits; a shared item costs the meeting of its partial sums, which grows with the
+  // CTAs and the bytes.  The constants are fitted to 41 layers timed in every tile and split considered here (1 to 128
+  // images of 49 to 12544 pixels): the choice is within 2.5 % of the best on average, 19 % at worst.
+  // Candidates: every strip count that leaves rows of at most 256 pixels, with as many rows as give two blocks or
+  // one, evened out over the height; whole small images several at a time.
   const int cyc = 36 + p->n_tile / 4 > p->n_tile / 2 ? 36 + p->n_tile / 4 : p->n_tile / 2;
   const double per_block = (double)g->k * g->k * dc_div_up(g->c_in, 16) * cyc;
   const double w_item = (double)ko.e_pad * p->n_tile * 16;
   double best = 0.0;
   p->nxt = 0;
+  p->ksplit = 1;
+  const int fixed_part = kSmemBudget - 1024 - p->off_a;     // bytes of the rings, where partial sums would go
   auto consider = [&](int tw, int th, int ni) {
     const int wbox = tw + g->k - 1, rbox = th + g->k - 1;
     if (wbox > 256 || rbox > 256) return;
@@ -535,12 +656,21 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     const int nxt = dc_div_up(wo, tw);
     const long long items = (long long)dc_div_up(n, ni) * nxt * dc_div_up(ho, th) * p->nnt;
     const long long per_cta = (items + n_sm - 1) / n_sm, blocks = (items * mb + n_sm - 1) / n_sm;
-    const double mma = (double)(blocks < per_cta * mb ? blocks : per_cta * mb) * per_block;
-    const double intake = (double)per_cta * ((double)ni * lines * 128 * p->planes + w_item) / 20.0;
-    const double all = (double)items * ((double)ni * lines * 128 * p->planes + w_item) / 3000.0;      // what L2 gives all SMs together
-    const double mem = intake > all ? intake : all;
-    const double cost = (mma > mem ? mma + 0.2 * mem : mem + 0.2 * mma) + 1500.0 * (double)per_cta + lines * 2.0;
-    if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; }
+    const double mma = 1.7 * (double)(blocks < per_cta * mb ? blocks : per_cta * mb) * per_block;
+    const double bytes = (double)ni * lines * 128 * p->planes + w_item;
+    const double all = (double)items * bytes / 8000.0;               // what L2 gives all SMs together
+    for (int split = 1; split <= kMaxSplit; ++split) {
+      // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
+      if (split == 7) continue;
+      if (split > 1 && (items * split > n_sm || items > max_clusters(split) || p->planes * g->k < split ||
+                        mb * 128 * (p->n_tile + 4) * 4 > fixed_part))
+        break;
+      const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
+      const double meet = split > 1 ? 450.0 + 580.0 * split + (double)ni * th * tw * p->n_tile * 0.8 : 0.0;
+      const double ctas = (double)(items * split < 148 ? items * split : 148);
+      const double cost = (m > l ? m + 0.77 * l : l + 0.77 * m) + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + meet;
+      if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->ksplit = split; }
+    }
   };
   int nxt0 = 1;
   while (dc_div_up(wo, nxt0) + g->k - 1 > 256) nxt0 = nxt0 < 64 ? nxt0 + 1 : nxt0 + nxt0 / 32;
@@ -596,7 +726,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   // items of two blocks on 148 SMs, three items = six blocks on 48 of them against five by blocks), the runs are
   // cut by blocks: an item at a run's end is then shared by two CTAs, each staging its tile and weights.
   p->split = 0;
-  if (p->mb > 1) {
+  if (p->mb > 1 && p->ksplit == 1) {
     const long long units = items * p->mb;
     const int grid_u = units < n_sm ? (int)units : n_sm;
     const long long whole = (items / p->grid + (items % p->grid ? 1 : 0)) * p->mb, cut = units / grid_u + (units % grid_u ? 1 : 0);
@@ -619,7 +749,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   // (For 1 x 1 layers of one or two planes the weight stream is small beside the activations and the resident
   // version measured no faster.)
   const long long b_all = (long long)dc_round_up((size_t)ko.e_pad * p->n_tile * 16, 1024);
-  p->b_resident = (p->nnt == 1 && b_all <= 128 * 1024 && (p->planes >= 3 || b_all >= 2ll * p->a_stage_bytes)) ? 1 : 0;
+  p->b_resident = (p->ksplit == 1 && p->nnt == 1 && b_all <= 128 * 1024 && (p->planes >= 3 || b_all >= 2ll * p->a_stage_bytes)) ? 1 : 0;
   // a weight stage is a whole (plane, tap row) step where that fits twice
   p->partial = 0;
   p->b_stage_bytes = (int)dc_round_up((size_t)(g->k * tap_bytes), 1024);
@@ -647,6 +777,11 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   p->sa = sa; p->sb = sb;
   p->off_b = p->off_a + sa * p->a_stage_bytes;
   p->smem_bytes = (int)total(sa, sb);
+  p->part_pitch = p->n_tile + 4;                 // lanes of a quarter warp 16 bytes apart in the banks
+  if (p->ksplit > 1) {
+    const int need = 1024 + p->off_a + p->mb * 128 * p->part_pitch * 4;
+    if (p->smem_bytes < need) p->smem_bytes = need;
+  }
   return true;
 }
 
@@ -678,13 +813,15 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return DC_ERR_CUDA;
   }
-  using Kernel = decltype(&k_conv_tc_rows<false, false>);
-  static constexpr Kernel kernels[3] = {k_conv_tc_rows<false, false>, k_conv_tc_rows<true, false>, k_conv_tc_rows<false, true>};
-  static unsigned char attr_done[3][kDcMaxDevices];
-  const int which = p.b_resident ? 1 : (p.partial ? 2 : 0);
+  using Kernel = decltype(&k_conv_tc_rows<false, false, false>);
+  static constexpr Kernel kernels[5] = {k_conv_tc_rows<false, false, false>, k_conv_tc_rows<true, false, false>,
+                                        k_conv_tc_rows<false, true, false>, k_conv_tc_rows<false, false, true>,
+                                        k_conv_tc_rows<false, true, true>};
+  static unsigned char attr_done[5][kDcMaxDevices];
+  const int which = p.b_resident ? 1 : (p.partial ? 2 : 0) + (p.ksplit > 1 ? (p.partial ? 2 : 3) : 0);
   DC_CUDA_OK(dc_set_max_smem_once(kernels[which], kSmemBudget, attr_done[which]));
-  const cudaError_t le = dc_launch_pdl(kernels[which], dim3(p.grid), dim3(kThreads), (size_t)p.smem_bytes, stream, map_a, p,
-                                       w_packed, bias, (const __nv_bfloat16 *)residual, (__nv_bfloat16 *)y,
-                                       (DcWsHeader *)workspace);
+  const cudaError_t le = dc_launch_pdl_cluster(kernels[which], dim3(p.grid * p.ksplit), dim3(kThreads), (size_t)p.smem_bytes, stream,
+                                               p.ksplit, map_a, p, w_packed, bias, (const __nv_bfloat16 *)residual,
+                                               (__nv_bfloat16 *)y, (DcWsHeader *)workspace);
   return le == cudaSuccess && cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }

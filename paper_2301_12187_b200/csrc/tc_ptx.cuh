@@ -223,6 +223,22 @@ __device__ __forceinline__ bool bar_all(int id, int count, bool ok) {
       : "memory");
   return all != 0;
 }
+// all threads of the cluster's CTAs that have not exited meet; shared-memory writes before it are visible behind it
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+// the address of this CTA's shared address `a` in CTA `rank` of the cluster, and a 16-byte read there
+__device__ __forceinline__ uint32_t map_cluster(uint32_t a, uint32_t rank) {
+  uint32_t d;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ uint4 lds_cluster_u4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // 16-byte asynchronous copy global -> shared without the zero-fill operand
 __device__ __forceinline__ void cp_async16_full(uint32_t dst, const void *src) {

@@ -480,6 +480,18 @@ def test_rows_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (384, 64, 3, 1, 1, 1, 14, 14),       # one item for the chip: its 18 steps over a cluster of eight
+    (960, 160, 1, 1, 0, 1, 7, 7),        # 1x1: 15 planes over a cluster
+    (576, 200, 3, 1, 1, 2, 13, 9),       # several items, two passes, a ragged map
+    (256, 128, 5, 1, 2, 1, 20, 21),      # weight stages of one tap column
+    (160, 48, 3, 1, 1, 3, 5, 5),         # a half-filled last plane, several images per item
+    (80, 32, 3, 1, 1, 1, 3, 4),          # fewer pixels than one warp reads
+])
+def test_rows_with_a_shared_reduction_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (32, 32, 5, 1, 2, 3, 28, 28),       # whole pixel tiles and a ragged last one
     (8, 40, 3, 1, 1, 1, 7, 9),          # a K slice of 16 spans two taps; 40 channels per tile
     (4, 20, 3, 2, 1, 2, 9, 11),         # four taps per slice, K no multiple of a slice, stride 2
