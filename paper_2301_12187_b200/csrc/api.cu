@@ -26,7 +26,7 @@ extern "C" const char *dc_conv_kernel_name(int n, int h, int w, const dc_geom *g
   if (dtype == DC_F32) return "k_conv_dense_f32";
   if (dtype != DC_BF16) return nullptr;
   if (dc_conv_pairrows_supported(n, h, w, g)) return "k_conv_tc_pairrows";
-  if (dc_conv_rows_supported(n, h, w, g)) return "k_conv_tc_rows";
+  if (dc_conv_rows_supported(n, h, w, g)) return g->stride == 2 ? "k_conv_tc" : "k_conv_tc_rows";
   if (dc_conv_fold_supported(n, h, w, g)) return "k_conv_tc_fold";
   if (dc_conv_tc_supported(n, h, w, g)) return "k_conv_tc";
   if (dc_conv_stem_s2_supported(n, h, w, g) && dc_conv_stem_supported(n, h, w, g)) return "k_conv_stem_s2";

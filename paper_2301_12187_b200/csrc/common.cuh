@@ -174,15 +174,20 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   // 37 us on the general kernel).  Chunk planes are
   // ordered (plane g of 64 channels, tap row r, tap column s, 16-channel step, half): the planes of
   // one (g, r) step are contiguous, which is the unit the kernel streams.
-  if (g->groups == 1 && g->stride == 1 && g->k <= 7 &&
-      (ko->cch >= 5 ? g->c_out >= 32
-                    : ((g->k == 1 && ko->cch >= 2 && g->c_out >= 48) || (g->k >= 3 && ko->cch >= 2 && ko->co8 > 128))) &&
+  // Stride 2 (k >= 3; what the pair rows do not take) has the taps of a plane ordered by the parity of the patch row and
+  // column they read, class by class, so that one class reads one sub-tile of every second row and column.
+  const bool rows_s2 = g->stride == 2 && g->k >= 3 && ko->cch >= 2;
+  if (g->groups == 1 && g->k <= 7 && (g->stride == 1 || rows_s2) &&
+      (rows_s2 || (ko->cch >= 5 ? g->c_out >= 32
+                    : ((g->k == 1 && ko->cch >= 2 && g->c_out >= 48) || (g->k >= 3 && ko->cch >= 2 && ko->co8 > 128)))) &&
       g->c_in % 8 == 0 && g->c_out % 8 == 0) {
     const int n16 = (int)dc_round_up((size_t)g->c_out, 16);
     ko->rows = 1;
     // output channels per pass: at most 128 (two accumulator sets of two blocks in tensor memory; from 128 columns on
-    // the tensor core runs at its rate), 256 for deep 1x1 layers with many outputs
-    const int n_tile_max = (g->k == 1 && g->c_in >= 512 && g->c_out > 256) ? 256 : 128;
+    // the tensor core runs at its rate), 256 for deep 1x1 layers with many outputs, and for stride 2, whose four
+    // sub-tiles are then staged once
+    const int n_tile_max = (g->stride == 2 || (g->k == 1 && g->c_in >= 512 && g->c_out > 256)) ? 256 : 128;
+    ko->pcs = 1;
     ko->nnt = dc_div_up(n16, n_tile_max);
     ko->n_tile = (int)dc_round_up((size_t)dc_div_up(n16, ko->nnt), 16);
     ko->n_pad = ko->nnt * ko->n_tile;
@@ -215,6 +220,19 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   ko->e_pad = (ko->e + 1) & ~1;
 }
 
+// Rows order, stride 2: taps before class (py, px) of a k x k kernel, class rows then class columns even first ...
+__host__ __device__ static inline int dc_s2_base(int k, int py, int px) {
+  const int e = (k + 1) >> 1, o = k >> 1;        // even and odd tap rows (or columns)
+  return py ? e * k + (px ? o * e : 0) : (px ? e * e : 0);
+}
+// ... and the class of tap position `tap`: returns its base, its parities and its number of columns
+__host__ __device__ static inline int dc_s2_class(int k, int tap, int *py, int *px, int *nc) {
+  *py = tap >= dc_s2_base(k, 1, 0);
+  *px = tap >= dc_s2_base(k, *py, 1);
+  *nc = (k + 1 - *px) >> 1;
+  return dc_s2_base(k, *py, *px);
+}
+
 // entry index within a group -> (pc, ccg, r, s); returns false for the zero padding entry
 __host__ __device__ static inline bool dc_korder_decode(const KOrder &ko, int e, int *pc, int *ccg,
                                                         int *r, int *s) {
@@ -227,8 +245,15 @@ __host__ __device__ static inline bool dc_korder_decode(const KOrder &ko, int e,
     const int nsl = left >= 64 ? 4 : (left + 15) / 16;
     const int half = rem & 1, q = rem >> 1;
     const int sl = q % nsl, tap = q / nsl;
-    *r = tap / ko.k;
-    *s = tap - *r * ko.k;
+    if (ko.stride == 2) {
+      int py, px, nc;
+      const int rest = tap - dc_s2_class(ko.k, tap, &py, &px, &nc);
+      *r = 2 * (rest / nc) + py;
+      *s = 2 * (rest % nc) + px;
+    } else {
+      *r = tap / ko.k;
+      *s = tap - *r * ko.k;
+    }
     *ccg = gpl * 8 + sl * 2 + half;
     *pc = 0;
     return true;
@@ -288,7 +313,8 @@ __host__ __device__ static inline int dc_korder_encode(const KOrder &ko, int cc,
   if (ko.rows) {
     const int gpl = cc >> 3, left = ko.c_in - 64 * gpl;
     const int nsl = left >= 64 ? 4 : (left + 15) / 16;
-    return gpl * ko.k * ko.k * 8 + ((r * ko.k + s) * nsl + ((cc & 7) >> 1)) * 2 + (cc & 1);
+    const int tap = ko.stride == 2 ? dc_s2_base(ko.k, r & 1, s & 1) + (r >> 1) * ((ko.k + 1 - (s & 1)) >> 1) + (s >> 1) : r * ko.k + s;
+    return gpl * ko.k * ko.k * 8 + (tap * nsl + ((cc & 7) >> 1)) * 2 + (cc & 1);
   }
   if (ko.pair == 2)            // the copy for the first pixel of the pair: dx = s, pixel s & 1 of shift s >> 1
     return (r * ko.ns[0] + (s >> 1)) * 2 * ko.cch + (s & 1) * ko.cch + cc;

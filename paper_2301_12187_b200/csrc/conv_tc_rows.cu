@@ -41,7 +41,7 @@ constexpr int kStagePitch = 64;                  // bytes per pixel in an epilog
 
 struct RowsParams {
   int n_img, h, w, ho, wo, c_in, c_out;
-  int k, pad, planes;          // planes of 64 input channels
+  int k, stride, pad, planes;  // planes of 64 input channels
   int tw, th, nxt, wbox, rbox, ni;   // tile: outputs per row, rows, strips per row, patch width / rows, images
   int tiles_y, img_groups;
   int grid, items_per, items_rem;    // CTAs; CTA b takes items_per (+1 if b < items_rem) work items
@@ -75,6 +75,23 @@ __device__ __forceinline__ int plane_steps(const RowsParams &p, int g) {
   return left >= 64 ? 4 : (left + 15) >> 4;
 }
 
+// Activation plane v of an item: 64 channels of the patch, or for stride 2 one of the four sub-tiles of those, with the
+// taps that read it: kr rows x kc columns, the first at position tap0 of the plane's taps in the packed weights.
+struct Plane {
+  int g, py, px, kr, kc, tap0;
+  __device__ __forceinline__ Plane(const RowsParams &p, int v, bool s2) {
+    g = v; py = 0; px = 0; kr = p.k; kc = p.k; tap0 = 0;
+    if (s2) {
+      g = v >> 2;
+      py = (v >> 1) & 1;
+      px = v & 1;
+      kr = (p.k + 1 - py) >> 1;
+      kc = (p.k + 1 - px) >> 1;
+      tap0 = dc_s2_base(p.k, py, px);
+    }
+  }
+};
+
 // work item -> (pass, image group, column strip, row tile); items are ordered (tile, pass)
 struct Item {
   int nt, img0, xt, ty;
@@ -100,11 +117,18 @@ struct Item {
 // with fewer items than SMs whose reduction is long (384 -> 64 3x3 on one 14 x 14 image is one item of 432
 // instructions per block).  The partial sums meet in distributed shared memory -- in the rings' place, which nothing
 // reads any more -- and are added in rank order; every CTA finishes its share of the outputs.
-template <bool RESIDENT, bool PARTIAL, bool SPLITK>
-__global__ void __launch_bounds__(kThreads, 1)
-k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
-               const void *__restrict__ w_packed, const float *__restrict__ bias,
-               const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
+//
+// S2: stride 2.  A plane of 64 channels is four sub-tiles of every second row and column of the patch (tensor map with
+// element strides 2, one load each), and tap (r, s) reads sub-tile (r & 1, s & 1) at row r >> 1, column s >> 1: each
+// sub-tile is a plane of its own with a smaller kernel, and GEMM rows are output pixels as before.  Gathered by 16-byte
+// cp.async (conv_tc.cu, which had these layers before), an SM took in 16 KB of patch per microsecond: 96 -> 144 5x5 to
+// 28 x 28, 128 images 77 us there, 70 here; 20 images of 50 x 50 53 and 15.5; 40 -> 32 3x3, 64 images of 28 x 28, 14.0
+// and 6.0; 160 -> 96 3x3, 64 images of 14 x 14, 23.6 and 11.0.
+template <bool RESIDENT, bool PARTIAL, bool SPLITK, bool S2>
+__device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsParams &p,
+                                          const void *__restrict__ w_packed, const float *__restrict__ bias,
+                                          const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y,
+                                          DcWsHeader *ws) {
   extern __shared__ __align__(1024) uint8_t smem_raw_base[];
   __shared__ __align__(8) Shared sh;
 
@@ -124,11 +148,14 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   int nitems = p.items_per + (bid < p.items_rem ? 1 : 0);
   int item0 = bid * p.items_per + (bid < p.items_rem ? bid : p.items_rem);
   int blk_first = 0, blk_end = p.mb;
-  // this CTA's run of the item's (plane, weight stage) steps
-  const int nstages = PARTIAL ? p.k * p.k : p.k;
+  // Activation planes (S2: four sub-tiles of each), and this CTA's share of the item: a run of (plane, weight stage)
+  // steps -- whole sub-tiles for S2, whose stages are not all alike.
+  const int nv = p.planes * (S2 ? 4 : 1);
+  const int unit = S2 ? 1 : (PARTIAL ? p.k * p.k : p.k);
   const int rank = SPLITK ? bid % p.ksplit : 0;
-  const int st0 = SPLITK ? p.planes * nstages * rank / p.ksplit : 0;
-  const int st1 = SPLITK ? p.planes * nstages * (rank + 1) / p.ksplit : p.planes * nstages;
+  const int st0 = SPLITK ? nv * unit * rank / p.ksplit : 0;
+  const int st1 = SPLITK ? nv * unit * (rank + 1) / p.ksplit : nv * unit;
+  const int v_lo = SPLITK ? st0 / unit : 0, v_hi = SPLITK ? (st1 + unit - 1) / unit : nv;
   if (SPLITK) {
     item0 = bid / p.ksplit;
     nitems = 1;
@@ -173,20 +200,22 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         Item q;
         q.of(p, item0 + it);
 #pragma unroll 1
-        for (int g = SPLITK ? st0 / nstages : 0; g * nstages < st1 && ok; ++g) {
+        for (int v = v_lo; v < v_hi && ok; ++v) {
+          const Plane pl(p, v, S2);
           if (!warp_wait(&sh.a_empty[sa], pa ^ 1, abort_flag, ws, 0x10000u | sa)) { ok = false; break; }
           if (lane == 0) {
             // channels past c_in, pixels outside the image and images past the batch arrive as zeros
             mbar_arrive_expect_tx(&sh.a_full[sa], (uint32_t)p.a_box_bytes);
-            tma_load_4d(a_base0 + (uint32_t)sa * (uint32_t)p.a_stage_bytes, &map_a, &sh.a_full[sa], 64 * g,
-                        q.xt * p.tw - p.pad, q.ty * p.th - p.pad, q.img0);
+            tma_load_4d(a_base0 + (uint32_t)sa * (uint32_t)p.a_stage_bytes, &map_a, &sh.a_full[sa], 64 * pl.g,
+                        (S2 ? 2 : 1) * q.xt * p.tw - p.pad + pl.px, (S2 ? 2 : 1) * q.ty * p.th - p.pad + pl.py, q.img0);
           }
           if (++sa == p.sa) { sa = 0; pa ^= 1; }
-          const int nsl = plane_steps(p, g);
-          const int nplanes = (PARTIAL ? 1 : p.k) * nsl * 2;       // chunk planes of one weight stage
-          const int r_lo = SPLITK && st0 > g * nstages ? st0 - g * nstages : 0;
-          const int r_hi = SPLITK && st1 < (g + 1) * nstages ? st1 - g * nstages : nstages;
-          size_t plane0 = (size_t)g * p.k * p.k * 8 + (size_t)r_lo * nplanes;
+          const int nsl = plane_steps(p, pl.g);
+          const int nplanes = (PARTIAL ? 1 : pl.kc) * nsl * 2;     // chunk planes of one weight stage
+          const int nstages = PARTIAL ? pl.kr * pl.kc : pl.kr;
+          const int r_lo = SPLITK && !S2 && st0 > v * unit ? st0 - v * unit : 0;
+          const int r_hi = SPLITK && !S2 && st1 < (v + 1) * unit ? st1 - v * unit : nstages;
+          size_t plane0 = (size_t)pl.g * p.k * p.k * 8 + (size_t)(pl.tap0 * nsl * 2) + (size_t)r_lo * nplanes;
 #pragma unroll 1
           for (int r = r_lo; r < r_hi && !RESIDENT; ++r, plane0 += nplanes) {
             if (!warp_wait(&sh.b_empty[sb], pb ^ 1, abort_flag, ws, 0x20000u | sb)) { ok = false; break; }
@@ -276,20 +305,22 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             if (leader) umma_bf16(tmem_base + (uint32_t)((set * p.mb + b) * p.n_tile), ones_desc, bd, idesc, 0u);
         }
 #pragma unroll 1
-        for (int g = SPLITK ? st0 / nstages : 0; g * nstages < st1 && ok; ++g) {
+        for (int v = v_lo; v < v_hi && ok; ++v) {
+          const Plane pl(p, v, S2);
           if (!warp_wait(&sh.a_full[sa], pa, abort_flag, ws, 0x40000u | sa)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_stage = a_row0 + (uint32_t)sa * ((uint32_t)p.a_stage_bytes >> 4);
-          const int nsl = plane_steps(p, g);
-          const int r_lo = SPLITK && st0 > g * nstages ? st0 - g * nstages : 0;
-          const int r_hi = SPLITK && st1 < (g + 1) * nstages ? st1 - g * nstages : nstages;
-          int col = PARTIAL && SPLITK ? r_lo % p.k : 0;    // PARTIAL: tap column of the stage
-          uint32_t tap_off = (uint32_t)(((PARTIAL ? r_lo / p.k : r_lo) * p.wbox + col) * 8);   // of the stage's first tap, in 16-byte units
+          const int nsl = plane_steps(p, pl.g);
+          const int nstages = PARTIAL ? pl.kr * pl.kc : pl.kr;
+          const int r_lo = SPLITK && !S2 && st0 > v * unit ? st0 - v * unit : 0;
+          const int r_hi = SPLITK && !S2 && st1 < (v + 1) * unit ? st1 - v * unit : nstages;
+          int col = PARTIAL && SPLITK ? r_lo % pl.kc : 0;          // PARTIAL: tap column of the stage
+          uint32_t tap_off = (uint32_t)(((PARTIAL ? r_lo / pl.kc : r_lo) * p.wbox + col) * 8);   // of the stage's first tap, in 16-byte units
 #pragma unroll 1
           for (int r = r_lo; r < r_hi; ++r) {
             uint32_t b_stage;
             if (RESIDENT) {
-              b_stage = b_row0 + (uint32_t)((g * p.k * p.k * 8 + r * p.k * nsl * 2) * p.n_tile);   // planes before this step
+              b_stage = b_row0 + (uint32_t)((pl.g * p.k * p.k * 8 + (pl.tap0 + r * pl.kc) * nsl * 2) * p.n_tile);   // planes before this step
             } else {
               if (!warp_wait(&sh.b_full[sb], pb, abort_flag, ws, 0x50000u | sb)) { ok = false; break; }
               tc_fence_after();
@@ -310,7 +341,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const uint32_t b_inc = 2u * (uint32_t)p.n_tile;
                 if (nsl == 4) {                  // a full plane of 64 channels
 #pragma unroll 1
-                  for (int s = 0; s < (PARTIAL ? 1 : p.k); ++s, a_lo += 8u) {
+                  for (int s = 0; s < (PARTIAL ? 1 : pl.kc); ++s, a_lo += 8u) {
 #pragma unroll
                     for (int sl = 0; sl < 4; ++sl) {
                       umma_bf16(d, ((uint64_t)a_hi << 32) | (uint64_t)(a_lo + 2u * sl), ((uint64_t)b_hi << 32) | (uint64_t)b_lo, idesc, 1u);
@@ -319,7 +350,7 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                   }
                 } else {
 #pragma unroll 1
-                  for (int s = 0; s < (PARTIAL ? 1 : p.k); ++s, a_lo += 8u) {
+                  for (int s = 0; s < (PARTIAL ? 1 : pl.kc); ++s, a_lo += 8u) {
 #pragma unroll 1
                     for (int sl = 0; sl < nsl; ++sl) {
                       umma_bf16(d, ((uint64_t)a_hi << 32) | (uint64_t)(a_lo + 2u * sl), ((uint64_t)b_hi << 32) | (uint64_t)b_lo, idesc, 1u);
@@ -336,9 +367,9 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             if (!PARTIAL) {
               tap_off += (uint32_t)(p.wbox * 8);
-            } else if (++col == p.k) {
+            } else if (++col == pl.kc) {
               col = 0;
-              tap_off += (uint32_t)((p.wbox - p.k + 1) * 8);
+              tap_off += (uint32_t)((p.wbox - pl.kc + 1) * 8);
             } else {
               tap_off += 8u;
             }
@@ -553,6 +584,22 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
 }
 
+template <bool RESIDENT, bool PARTIAL, bool SPLITK>
+__global__ void __launch_bounds__(kThreads, 1)
+k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
+               const void *__restrict__ w_packed, const float *__restrict__ bias,
+               const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
+  rows_body<RESIDENT, PARTIAL, SPLITK, false>(map_a, p, w_packed, bias, residual, y, ws);
+}
+// the general kernel's stride-2 layers, fed the same way
+template <bool RESIDENT, bool PARTIAL, bool SPLITK>
+__global__ void __launch_bounds__(kThreads, 1)
+k_conv_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
+          const void *__restrict__ w_packed, const float *__restrict__ bias,
+          const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
+  rows_body<RESIDENT, PARTIAL, SPLITK, true>(map_a, p, w_packed, bias, residual, y, ws);
+}
+
 // ------------------------------------------------------------------------------------------ host
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -618,11 +665,12 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   if ((long long)n * h * w * g->c_in >= (1ll << 40) || (long long)n * h * w >= (1ll << 31)) return false;
   // a 1x1 layer does not know rows or images: its pixels are one run, which tiles cut without a remainder per row
   if (g->k == 1 && g->pad == 0) { w *= n * h; n = 1; h = 1; }
-  const int ho = dc_out_extent(h, g->k, 1, g->pad), wo = dc_out_extent(w, g->k, 1, g->pad);
+  const int S = g->stride, ho = dc_out_extent(h, g->k, S, g->pad), wo = dc_out_extent(w, g->k, S, g->pad);
+  const int halo = S == 2 ? (g->k - 1) / 2 : g->k - 1, subs = S == 2 ? 4 : 1;      // of a plane (sub-tile); sub-tiles per plane
   if (ho <= 0 || wo <= 0 || (long long)n * ho * wo >= (1ll << 31)) return false;
   p->n_img = n; p->h = h; p->w = w; p->ho = ho; p->wo = wo;
   p->c_in = g->c_in; p->c_out = g->c_out;
-  p->k = g->k; p->pad = g->pad;
+  p->k = g->k; p->stride = S; p->pad = g->pad;
   p->planes = dc_div_up(g->c_in, 64);
   p->n_tile = ko.n_tile; p->nnt = ko.nnt; p->n_pad = ko.n_pad;
   p->planes_all = ko.e_pad;
@@ -647,8 +695,8 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   p->ksplit = 1;
   const int fixed_part = kSmemBudget - 1024 - p->off_a;     // bytes of the rings, where partial sums would go
   auto consider = [&](int tw, int th, int ni) {
-    const int wbox = tw + g->k - 1, rbox = th + g->k - 1;
-    if (wbox > 256 || rbox > 256) return;
+    const int wbox = tw + halo, rbox = th + halo;
+    if (S * wbox > 256 || S * rbox > 256) return;
     const int lines = rbox * wbox;
     if ((long long)dc_round_up((size_t)ni * lines * 128, 1024) > max_a) return;
     const int mb = dc_div_up((ni - 1) * lines + (th - 1) * wbox + tw, 128);
@@ -657,12 +705,12 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     const long long items = (long long)dc_div_up(n, ni) * nxt * dc_div_up(ho, th) * p->nnt;
     const long long per_cta = (items + n_sm - 1) / n_sm, blocks = (items * mb + n_sm - 1) / n_sm;
     const double mma = 1.7 * (double)(blocks < per_cta * mb ? blocks : per_cta * mb) * per_block;
-    const double bytes = (double)ni * lines * 128 * p->planes + w_item;
+    const double bytes = (double)ni * lines * 128 * p->planes * subs + w_item;
     const double all = (double)items * bytes / 8000.0;               // what L2 gives all SMs together
     for (int split = 1; split <= kMaxSplit; ++split) {
       // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
       if (split == 7) continue;
-      if (split > 1 && (items * split > n_sm || items > max_clusters(split) || p->planes * g->k < split ||
+      if (split > 1 && (items * split > n_sm || items > max_clusters(split) || p->planes * (S == 2 ? 4 : g->k) < split ||
                         mb * 128 * (p->n_tile + 4) * 4 > fixed_part))
         break;
       const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
@@ -673,7 +721,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     }
   };
   int nxt0 = 1;
-  while (dc_div_up(wo, nxt0) + g->k - 1 > 256) nxt0 = nxt0 < 64 ? nxt0 + 1 : nxt0 + nxt0 / 32;
+  while (S * (dc_div_up(wo, nxt0) + halo) > 256) nxt0 = nxt0 < 64 ? nxt0 + 1 : nxt0 + nxt0 / 32;
   if (ho == 1 && g->k == 1) {
     // one run of pixels: full tiles, or as many as there are CTAs to take them
     consider(wo < 256 ? wo : 256, 1, 1);
@@ -689,7 +737,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
       int last_th = 0;
       for (int mb = kMaxBlocks; mb >= 1; --mb) {
         if (mb * 128 < tw) break;
-        int th = (mb * 128 - tw) / (tw + g->k - 1) + 1;
+        int th = (mb * 128 - tw) / (tw + halo) + 1;
         if (th > ho) th = ho;
         if (th != last_th) consider(tw, th, 1);
         last_th = th;
@@ -702,8 +750,8 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   }
   if (p->nxt == 0) return false;
   const int th = p->th;
-  p->wbox = p->tw + g->k - 1;
-  p->rbox = th + g->k - 1;
+  p->wbox = p->tw + halo;
+  p->rbox = th + halo;
   p->lines_img = p->rbox * p->wbox;
   p->inv_lines = ((1u << 20) + (uint32_t)p->lines_img - 1) / (uint32_t)p->lines_img;
   p->inv_wbox = ((1u << 20) + (uint32_t)p->wbox - 1) / (uint32_t)p->wbox;
@@ -752,7 +800,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   p->b_resident = (p->ksplit == 1 && p->nnt == 1 && b_all <= 128 * 1024 && (p->planes >= 3 || b_all >= 2ll * p->a_stage_bytes)) ? 1 : 0;
   // a weight stage is a whole (plane, tap row) step where that fits twice
   p->partial = 0;
-  p->b_stage_bytes = (int)dc_round_up((size_t)(g->k * tap_bytes), 1024);
+  p->b_stage_bytes = (int)dc_round_up((size_t)((S == 2 ? (g->k + 1) / 2 : g->k) * tap_bytes), 1024);
   auto total = [&](int a, int b) {
     const long long wbytes = p->b_resident ? b_all : (long long)b * p->b_stage_bytes;
     const long long tail = wbytes >= 26 * 1024 ? kSlack : 26 * 1024 - wbytes + kSlack;   // room for the overrun
@@ -806,19 +854,23 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
     const cuuint64_t C = (cuuint64_t)g->c_in;
     cuuint64_t gdim[4] = {C, (cuuint64_t)p.w, (cuuint64_t)p.h, (cuuint64_t)p.n_img};
     cuuint64_t gstr[3] = {2 * C, (cuuint64_t)p.w * C * 2, (cuuint64_t)p.h * p.w * C * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)p.wbox, (cuuint32_t)p.rbox, (cuuint32_t)p.ni};
-    cuuint32_t es[4] = {1, 1, 1, 1};
+    // stride 2: the box spans 2 wbox x 2 rbox pixels and takes every second column and row
+    const cuuint32_t S = (cuuint32_t)p.stride;
+    cuuint32_t box[4] = {64, S * (cuuint32_t)p.wbox, S * (cuuint32_t)p.rbox, (cuuint32_t)p.ni};
+    cuuint32_t es[4] = {1, S, S, 1};
     CUresult r = encode(&map_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(x), gdim, gstr, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return DC_ERR_CUDA;
   }
   using Kernel = decltype(&k_conv_tc_rows<false, false, false>);
-  static constexpr Kernel kernels[5] = {k_conv_tc_rows<false, false, false>, k_conv_tc_rows<true, false, false>,
-                                        k_conv_tc_rows<false, true, false>, k_conv_tc_rows<false, false, true>,
-                                        k_conv_tc_rows<false, true, true>};
-  static unsigned char attr_done[5][kDcMaxDevices];
-  const int which = p.b_resident ? 1 : (p.partial ? 2 : 0) + (p.ksplit > 1 ? (p.partial ? 2 : 3) : 0);
+  static constexpr Kernel kernels[10] = {
+      k_conv_tc_rows<false, false, false>, k_conv_tc_rows<true, false, false>, k_conv_tc_rows<false, true, false>,
+      k_conv_tc_rows<false, false, true>,  k_conv_tc_rows<false, true, true>,  k_conv_tc<false, false, false>,
+      k_conv_tc<true, false, false>,       k_conv_tc<false, true, false>,      k_conv_tc<false, false, true>,
+      k_conv_tc<false, true, true>};
+  static unsigned char attr_done[10][kDcMaxDevices];
+  const int which = (p.stride == 2 ? 5 : 0) + (p.b_resident ? 1 : (p.partial ? 2 : 0) + (p.ksplit > 1 ? (p.partial ? 2 : 3) : 0));
   DC_CUDA_OK(dc_set_max_smem_once(kernels[which], kSmemBudget, attr_done[which]));
   const cudaError_t le = dc_launch_pdl_cluster(kernels[which], dim3(p.grid * p.ksplit), dim3(kThreads), (size_t)p.smem_bytes, stream,
                                                p.ksplit, map_a, p, w_packed, bias, (const __nv_bfloat16 *)residual,

@@ -492,6 +492,21 @@ def test_rows_with_a_shared_reduction_against_the_oracle(dc, c_in, c_out, k, s, 
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (96, 144, 5, 2, 2, 9, 57, 50),       # several tiles per image and per CTA, odd height
+    (96, 144, 5, 2, 2, 1, 20, 20),       # the reduction shared by a cluster
+    (40, 32, 3, 2, 1, 40, 28, 28),       # weights resident
+    (48, 64, 7, 2, 3, 2, 31, 44),        # 7x7: classes of 16, 12, 12 and 9 taps
+    (72, 200, 3, 2, 0, 1, 17, 150),      # no padding, column strips, a partial last plane
+    (64, 264, 3, 2, 1, 2, 21, 19),       # two passes
+    (160, 256, 5, 2, 1, 3, 15, 9),       # padding 1, 256 outputs: weight stages of one tap
+    (24, 168, 3, 2, 1, 30, 9, 9),        # few channels, several images per tile
+    (384, 24, 3, 2, 1, 1, 7, 7),         # few outputs
+])
+def test_stride_2_by_sub_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (32, 32, 5, 1, 2, 3, 28, 28),       # whole pixel tiles and a ragged last one
     (8, 40, 3, 1, 1, 1, 7, 9),          # a K slice of 16 spans two taps; 40 channels per tile
     (4, 20, 3, 2, 1, 2, 9, 11),         # four taps per slice, K no multiple of a slice, stride 2
