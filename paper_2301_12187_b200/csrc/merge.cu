@@ -1108,6 +1108,84 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
 }
 
 // ----------------------------------------------------------------------------------------------
+// A dense 1x1 and a 3x3 depthwise layer, in either order, as a run of its own: every element of the result is one
+// product, W'[o][i][t] = W~[o][i] D~[c][t] with c = o (1x1 first) or c = i (depthwise first), so the run is bound by
+// writing its result (160 -> 960: 5.5 MB and its packed copy) and by its launches.  One launch reads the layers as they
+// are and delivers tiles of 8 x 16 channel pairs; blocks behind the tiles compute the bias (a warp per output channel)
+// and zero the packed chunks without weights.  As fold, composition and delivery, three launches with the result
+// written and read in between: 160 -> 960 then depthwise 27.6 us, depthwise then 576 -> 96 27.1, 384 -> 64 17.3; here
+// 9.6, 7.6 and 5.3 us.
+// ----------------------------------------------------------------------------------------------
+struct Outer33 {
+  RawLayer dense, dw;
+  int ident_dense, ident_dw;     // identity kernels riding on the layers
+  int dw_first;
+  int c0, c2;                    // input and output channels of the run
+  float *w_out, *b_out;
+  int gi, go;
+};
+
+__global__ void __launch_bounds__(kMbThreads)
+k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ BlockDelivery dv) {
+  __shared__ float wv[kMbO * kMbI], dd[kMbI * 9], out[kMbTile];
+  const int tid = (int)threadIdx.x, lane = tid & 31;
+  const int c0 = a.c0, c2 = a.c2;
+  int blk = (int)blockIdx.x;
+  dc_pdl_enter();
+  if (blk >= a.gi * a.go) {
+    blk -= a.gi * a.go;
+    if (blk >= a.go) {
+      zero_dead_chunks(dv, c2, blk - a.go, (int)gridDim.x - a.gi * a.go - a.go);
+      return;
+    }
+    const int o = blk * kMbO + (tid >> 5);
+    if (o >= c2) return;
+    float s = 0.f;
+    if (a.dw_first) {                              // b2~ + sum_c W~[o][c] b1~[c]
+      const float g2 = raw_scale(a.dense, o);
+#pragma unroll 4
+      for (int c = lane; c < c0; c += 32) {
+        const float w = fmaf(g2, a.dense.w[(size_t)o * c0 + c], a.ident_dense && c == o ? 1.f : 0.f);
+        s = fmaf(w, raw_bias(a.dw, c, raw_scale(a.dw, c)), s);
+      }
+      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      if (lane == 0) a.b_out[o] = raw_bias(a.dense, o, g2) + s;
+    } else {                                       // b2~ + (sum_t D~[o][t]) b1~[o]
+      const float g2 = raw_scale(a.dw, o);
+      s = lane < 9 ? g2 * a.dw.w[(size_t)o * 9 + lane] : 0.f;
+      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      if (lane == 0)
+        a.b_out[o] = fmaf(s + (a.ident_dw ? 1.f : 0.f), raw_bias(a.dense, o, raw_scale(a.dense, o)), raw_bias(a.dw, o, g2));
+    }
+    return;
+  }
+  const int o0 = (blk / a.gi) * kMbO, i0 = (blk % a.gi) * kMbI;
+  if (tid < kMbO * kMbI) {
+    const int o = o0 + tid / kMbI, i = i0 + tid % kMbI;
+    wv[tid] = o < c2 && i < c0 ? fmaf(raw_scale(a.dense, o), a.dense.w[(size_t)o * c0 + i], a.ident_dense && o == i ? 1.f : 0.f) : 0.f;
+  }
+  const int d0 = a.dw_first ? i0 : o0, nd = a.dw_first ? kMbI : kMbO, cd = a.dw_first ? c0 : c2;
+  if (tid < nd * 9) {
+    const int c = d0 + tid / 9, t = tid % 9;
+    dd[tid] = c < cd ? fmaf(raw_scale(a.dw, c), a.dw.w[(size_t)c * 9 + t], a.ident_dw && t == 4 ? 1.f : 0.f) : 0.f;
+  }
+  __syncthreads();
+  for (int e = tid; e < kMbTile; e += kMbThreads) {
+    const int oi = e / 9, t = e - oi * 9, ow = oi / kMbI, iw = oi % kMbI, o = o0 + ow, i = i0 + iw;
+    float v = wv[oi] * dd[(a.dw_first ? iw : ow) * 9 + t];
+    if (dv.ident && o == i && t == 4) v += 1.f;
+    if (o < c2 && i < c0) a.w_out[((size_t)o * c0 + i) * 9 + t] = v;
+    out[e] = v;
+  }
+  if (dv.mode == 0) return;
+  __syncthreads();
+  deliver_tile<kMbO, kMbI, 3>(dv, out, o0, i0, c0, c2, tid, kMbThreads);
+}
+
+// the bias of a composition on its own
+__global__ void k_compose_bias(Piece first, Piece second, float *b_out) { compose_bias_block(first, second, b_out, (int)blockIdx.x); }
+
+// ----------------------------------------------------------------------------------------------
 // host: validation and geometry
 // ----------------------------------------------------------------------------------------------
 
@@ -1213,6 +1291,14 @@ static void launch_compose33(const Operand33 &first, const Operand33 &second, in
   (void)dc_launch_pdl(k_compose33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kP3Threads)), dim3(kP3Threads), kP3Ring, st, a, dv);
 }
 
+// A 1x1 after a large dense kernel is a plain matrix product: the fp32 convolution's kernel runs it as a 1x1 layer whose
+// pixels are the second layer's rows and whose weights are the first layer as stored (960 -> 320 -> 1280: 81 us with the
+// gathered product, 59.9 us).  False: a shape outside that kernel's range, nothing was launched.
+static bool compose_as_product(const Piece &first, const Piece &second, float *out, cudaStream_t st) {
+  const dc_geom g = {first.c_out, first.c_in * first.k * first.k, 1, 1, 1, 0};
+  return dc_launch_conv_f32(second.w, 1, 1, second.c_out, &g, first.w, nullptr, DC_ACT_IDENTITY, nullptr, out, st) != DC_ERR_UNSUPPORTED;
+}
+
 // Composes second o first into a new piece; launches when `go`.  With `dv`, the piece is the run's result: where the
 // kernel can deliver it itself it goes to w_final / b_final (and the packed copy) and *delivered is set.
 static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool go, cudaStream_t st,
@@ -1244,6 +1330,9 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
     } else if (!first.diag && !second.diag && elems <= (size_t)200000 && second.k <= 7) {
       const int gx = dc_div_up(out.c_in * out.k * out.k, 32), gy = dc_div_up(out.c_out, 8);
       k_compose_dd_small<<<gx * gy + nbias, 256, 0, st>>>(first, second, w, b, out.k, gx, gy);
+    } else if (!first.diag && !second.diag && second.k == 1 && !first.ident && !second.ident &&
+               compose_as_product(first, second, w, st)) {
+      k_compose_bias<<<nbias, 256, 0, st>>>(first, second, b);
     } else if (!first.diag && !second.diag) {
       // 128 x 64 tiles when they still give every SM two tiles, 64 x 64 otherwise
       const int gx = dc_div_up(out.c_in * out.k * out.k, 64);
@@ -1326,6 +1415,24 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     launch_compose33(Operand33{raw_of(layers[0]), id[0]}, Operand33{raw_of(layers[1]), id[1]}, mg.c_in, layers[0].c_out, mg.c_out,
                      w_merged, b_merged, BlockDelivery{w_packed, mode, whole, ko}, mg, st);
     return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+  }
+
+  if (go && n == 2 && algo != DC_MERGE_STEPS && can_pack) {
+    const dc_layer &l1 = layers[0], &l2 = layers[1];
+    const bool dw_first = l1.groups != 1;
+    const dc_layer &de = dw_first ? l2 : l1, &dw = dw_first ? l1 : l2;
+    if (de.groups == 1 && de.k == 1 && dw.groups != 1 && dw.k == 3 && (dw_first || de.stride == 1)) {
+      int id[2] = {0, 0}, whole = 0;
+      for (int g = 0; g < n_res; ++g) {
+        if (res[g].first != res[g].last) whole = 1;
+        else id[res[g].first] = 1;
+      }
+      const Outer33 a{raw_of(de), raw_of(dw), id[dw_first ? 1 : 0], id[dw_first ? 0 : 1], dw_first ? 1 : 0, mg.c_in, mg.c_out,
+                      w_merged, b_merged, dc_div_up(mg.c_in, kMbI), dc_div_up(mg.c_out, kMbO)};
+      const BlockDelivery dv{w_packed, mode, whole, ko};
+      (void)dc_launch_pdl(k_merge_outer33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), 0, st, a, dv);
+      return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+    }
   }
 
   // 0. inverted-residual blocks (1x1, depthwise, 1x1) are merged in one step from the raw layers

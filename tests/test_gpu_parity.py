@@ -216,6 +216,52 @@ def test_block_step_edge_cases(dc, case):
     assert O.rel_l2(wm2.cpu().numpy(), W) <= TOL_W and O.rel_l2(bm2.cpu().numpy(), b) <= TOL_W
 
 
+@pytest.mark.parametrize("case", ["expand_dw", "dw_project", "dw_s2_project", "dw_skip_project", "expand_skip_dw", "whole_skip",
+                                  "no_bn", "narrow", "dense_pair_skips", "dense_pair_ragged", "block_ragged", "block_k5",
+                                  "wide_1x1_pair"])
+def test_runs_delivered_by_one_launch(dc, case):
+    """Runs whose merge and delivery are one launch (a block, two dense 3x3 layers, a 1x1 and a depthwise layer), at ragged
+    tile edges, with identities on one layer or on the whole run, and the fp32 packed copy as well."""
+    mk = I.make_layer
+    res = []
+    if case == "expand_dw":
+        specs = [mk(51, 0, 24, 104, 1, 1, 0), mk(51, 1, 104, 104, 3, 2, 1, depthwise=True)]
+    elif case == "dw_project":
+        specs = [mk(52, 0, 136, 136, 3, 1, 1, depthwise=True), mk(52, 1, 136, 40, 1, 1, 0)]
+    elif case == "dw_s2_project":
+        specs = [mk(53, 0, 56, 56, 3, 2, 1, depthwise=True), mk(53, 1, 56, 264, 1, 1, 0)]
+    elif case == "dw_skip_project":
+        specs, res = [mk(54, 0, 48, 48, 3, 1, 1, depthwise=True), mk(54, 1, 48, 24, 1, 1, 0)], [(0, 0)]
+    elif case == "expand_skip_dw":
+        specs, res = [mk(55, 0, 40, 40, 1, 1, 0), mk(55, 1, 40, 40, 3, 1, 1, depthwise=True)], [(0, 0), (1, 1)]
+    elif case == "whole_skip":
+        specs, res = [mk(56, 0, 72, 72, 3, 1, 1, depthwise=True), mk(56, 1, 72, 72, 1, 1, 0)], [(0, 1)]
+    elif case == "no_bn":
+        specs = [mk(57, 0, 16, 32, 1, 1, 0, with_bn=False, with_bias=True), mk(57, 1, 32, 32, 3, 1, 1, depthwise=True, with_bn=False)]
+    elif case == "narrow":           # channels that are no multiple of a packed chunk
+        specs = [mk(58, 0, 6, 20, 1, 1, 0), mk(58, 1, 20, 20, 3, 1, 1, depthwise=True)]
+    elif case == "dense_pair_skips":
+        specs, res = [mk(59, 0, 24, 24, 3, 1, 1), mk(59, 1, 24, 24, 3, 1, 1)], [(0, 0), (1, 1)]
+    elif case == "dense_pair_ragged":
+        specs, res = [mk(60, 0, 20, 44, 3, 1, 1), mk(60, 1, 44, 13, 3, 2, 1, with_bn=False)], []
+    elif case == "block_ragged":
+        specs = [mk(61, 0, 40, 92, 1, 1, 0), mk(61, 1, 92, 92, 3, 2, 1, depthwise=True), mk(61, 2, 92, 21, 1, 1, 0)]
+    elif case == "block_k5":
+        specs = [mk(62, 0, 24, 64, 1, 1, 0), mk(62, 1, 64, 64, 5, 1, 2, depthwise=True), mk(62, 2, 64, 24, 1, 1, 0)]
+        res = [(0, 2)]
+    else:
+        specs = [mk(63, 0, 320, 96, 1, 1, 0), mk(63, 1, 96, 640, 1, 1, 0)]
+    W, b, k, s, p = O.merge_formula(specs, res)
+    for code in (dc.BF16, dc.F32):
+        g, wm, bm, packed = run_merge(dc, specs, res, packed_dtype=code)
+        assert (g.k, g.stride, g.pad) == (k, s, p)
+        assert O.rel_l2(wm.cpu().numpy(), W) <= TOL_W and O.rel_l2(bm.cpu().numpy(), b) <= TOL_W
+        again = torch.full_like(packed, 7)
+        dc.pack_weights(wm, g, code, again)
+        torch.cuda.synchronize()
+        assert torch.equal(packed, again)
+
+
 @pytest.mark.parametrize("c,n,h,w", [(64, 2, 28, 28), (128, 2, 14, 14), (256, 1, 14, 14), (512, 1, 14, 14)])
 def test_vgg_style_dense_merge(dc, c, n, h, w):
     """Two dense 3x3 layers (VGG-style, c -> c -> c) merged into one 5x5 layer: merged weights against
