@@ -1,5 +1,6 @@
-// Dense stride-1 convolution with many input channels as an implicit GEMM over PIXEL ROWS fed
-// straight from TMA tiles (see KOrder, "rows" order).
+// Dense convolution with many input channels as an implicit GEMM over PIXEL ROWS fed straight from
+// TMA tiles (see KOrder, "rows" order): stride 1, and stride 2 with a plane held as four sub-tiles
+// (S2 below).  1x1 layers see their pixels as one run, whatever image or row they lie in.
 //
 // A shared-memory line (128 bytes) holds 64 channels of one pixel; the input channels are cut into
 // planes of 64 (the last one zero filled by the TMA unit), and a GEMM row is a pixel of the haloed
@@ -13,13 +14,13 @@
 // The reduction runs over (plane g, tap row r) steps.  Each step needs k * nsl(g) * 2 chunk planes
 // of weights ([n_tile rows][8] bf16, no swizzle), which stream through their own ring: a layer such
 // as 160 -> 960, 3x3 has 2.8 MB of weights, 40x the activations of an image.  Output channels go in
-// passes of n_tile <= 128; accumulators (blocks of 128 rows x n_tile columns) live in tensor memory,
+// passes of n_tile <= 128 (256 for deep wide 1x1 layers and stride 2); accumulators (blocks of 128 rows x n_tile columns) live in tensor memory,
 // two sets when they fit so that the epilogue of one work item overlaps the MMAs of the next.
 //
 // Roles (352 threads): warp 0 producer (issues TMA / bulk loads in consumption order),
 // warps 1-2 MMA issue (blocks alternate between them), warps 3-10 epilogue (two per tensor-memory
 // lane quadrant, blocks alternate).  A work item is (tile, output-channel pass); CTAs (one per SM)
-// take contiguous runs of items.  All waits are bounded (tc::mbar_wait).
+// take contiguous runs of items, or a cluster of them shares one item (SPLITK below).  All waits are bounded (tc::mbar_wait).
 #include <type_traits>
 #include "tc_ptx.cuh"
 
