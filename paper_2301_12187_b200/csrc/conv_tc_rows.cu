@@ -721,8 +721,13 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
       if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->ksplit = split; }
     }
   };
-  int nxt0 = 1;
-  while (S * (dc_div_up(wo, nxt0) + halo) > 256) nxt0 = nxt0 < 64 ? nxt0 + 1 : nxt0 + nxt0 / 32;
+  // The fewest strips whose tile of one output row is within the tensor map's box (256 pixels) and the activation ring
+  // (max_a, in whole kilobytes).  The ring is the tighter bound for 5x5 and 7x7 kernels, whose weight stages leave it
+  // less room and whose patches have more rows: 128 -> 128 7x7 has strips of at most 78 outputs, not 250.
+  const long long ring = max_a / 1024 * 8 / (1 + halo) - halo, box = 256 / S - halo;
+  const int strip = (int)(ring < box ? ring : box);
+  if (strip < 1) return false;
+  const int nxt0 = dc_div_up(wo, strip);
   if (ho == 1 && g->k == 1) {
     // one run of pixels: full tiles, or as many as there are CTAs to take them
     consider(wo < 256 ? wo : 256, 1, 1);
@@ -745,6 +750,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
         const int even = dc_div_up(ho, dc_div_up(ho, th));
         if (even != th) consider(tw, even, 1);
       }
+      if (p->nxt == 0) consider(tw, 1, 1);
     }
     if (nxt0 == 1)
       for (int ni = 2; ni <= 8 && ni <= n; ++ni) consider(wo, ho, ni);

@@ -110,6 +110,25 @@ def test_kernel_name_query_follows_the_dispatch_rules():
     assert dc.conv_kernel_name(0, 16, 16, dc.geom(16, 24, 1, 3, 1, 1), dc.BF16) is None
 
 
+@pytest.mark.parametrize("k", [1, 3, 5, 7])
+@pytest.mark.parametrize("stride", [1, 2])
+def test_wide_maps_stay_on_the_tensor_cores(k, stride):
+    """Layers whose weights only the rows kernel reads: a column strip that fits is found at every width, also where the
+    patch of the widest strip the tensor map allows does not fit beside the weights."""
+    if (k, stride) == (1, 2):
+        pytest.skip("1x1 layers of stride 2 have no tensor-core kernel")
+    widths = sorted({7, 12, 13, 63, 255, 256, 257} | {int(7 * 1.07 ** i) for i in range(95)} | set(range(600, 4097, 499)) | {4033, 4096})
+    for c_in, c_out in [(16, 160), (40, 48), (64, 64), (72, 200), (64, 128), (128, 128), (64, 256), (256, 256), (512, 512)]:
+        if k == 1 and c_in == 16:
+            continue
+        for n, h in ((1, 7), (1, 96), (8, 31)):
+            for pad in {0, k // 2}:
+                g = dc.geom(c_in, c_out, 1, k, stride, pad)
+                for w in widths:
+                    name = dc.conv_kernel_name(n, h, w, g, dc.BF16)
+                    assert name in ("k_conv_tc_rows", "k_conv_tc"), (c_in, c_out, n, h, w, pad, name)
+
+
 def test_entry_points_validate_before_touching_the_device():
     lib = dc.lib()
     g = dc.geom(24, 24, 1, 3, 1, 1)

@@ -520,6 +520,8 @@ def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel
     (96, 576, 1, 1, 0, 3, 13, 13),       # 1x1: pixels of several images in a tile, a ragged last tile
     (64, 384, 1, 1, 0, 64, 14, 14),      # 1x1: more tiles than CTAs
     (32, 96, 1, 1, 0, 1, 1, 1),          # one pixel
+    (64, 128, 5, 1, 2, 1, 6, 1300),      # wide: the strips the tensor map allows do not fit beside the weights
+    (128, 128, 7, 1, 3, 1, 8, 640),      # the same with 7x7
 ])
 def test_rows_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
