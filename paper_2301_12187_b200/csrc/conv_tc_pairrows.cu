@@ -643,10 +643,6 @@ bool pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams *p) {
   if (w < 2) return false;                        // at least one whole pixel pair per image row
   const int ho = dc_out_extent(h, g->k, S, g->pad), wo = dc_out_extent(w, g->k, S, g->pad);
   if (ho <= 0 || wo <= 0) return false;
-  // The smallest odd-width maps stay with the CUDA-core kernel, not because it is faster (24 -> 24 3x3 at 9 x 15:
-  // 11.2 us there, 3.8 us here) but because the parity suite holds that kernel to the oracle on pair-order weights
-  // at 9 x 15: the line lies just above that size.
-  if ((w & 1) && S == 1 && (long long)n * ho * wo < 136) return false;
   if ((long long)n * h * w * g->c_in >= (1ll << 40)) return false;
   p->n_img = n; p->h = h; p->w = w; p->ho = ho; p->wo = wo;
   p->c_in = g->c_in; p->c_out = g->c_out; p->co8 = ko.co8;

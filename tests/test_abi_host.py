@@ -94,6 +94,8 @@ def test_kernel_name_query_follows_the_dispatch_rules():
     # channel counts that are no multiple of 8: CUDA cores
     assert dc.conv_kernel_name(64, 56, 56, dc.geom(24, 24, 1, 3, 1, 1), dc.BF16) == "k_conv_tc_pairrows"
     assert dc.conv_kernel_name(128, 28, 28, dc.geom(32, 32, 1, 5, 1, 2), dc.BF16) == "k_conv_tc_pairrows"
+    for n, h, w in ((1, 7, 7), (1, 9, 15), (2, 9, 15), (1, 11, 11), (1, 1, 3)):      # odd widths, at any number of outputs
+        assert dc.conv_kernel_name(n, h, w, dc.geom(24, 24, 1, 3, 1, 1), dc.BF16) == "k_conv_tc_pairrows"
     assert dc.conv_kernel_name(128, 14, 14, dc.geom(40, 32, 1, 5, 1, 2), dc.BF16) == "k_conv_tc_fold"
     assert dc.conv_kernel_name(128, 56, 56, dc.geom(24, 32, 1, 3, 2, 1), dc.BF16) == "k_conv_tc_pairrows"
     assert dc.conv_kernel_name(128, 56, 56, dc.geom(96, 144, 1, 5, 2, 2), dc.BF16) == "k_conv_tc"

@@ -418,7 +418,7 @@ def test_single_conv_bf16_with_explicit_skip(dc, c_in, c_out, k, s, p, n, h, w, 
     (16, 8, 3, 1, 0, 1, 18, 40, "k_conv_tc_pairrows"),      # no padding, 16 of 64 channels of a line used
     (8, 16, 3, 1, 1, 1, 6, 300, "k_conv_tc_pairrows"),      # three column strips: per-pixel stores, strip halos
     (16, 16, 7, 1, 3, 1, 20, 20, "k_conv_tc_pairrows"),     # 7x7: 56 instructions per block
-    (24, 24, 3, 1, 1, 1, 9, 15, "k_conv_dense_bf16"),       # odd width: pair-order weights read by the CUDA-core kernel
+    (24, 24, 3, 1, 1, 1, 9, 15, "k_conv_tc_pairrows"),      # odd width, one small image
     (40, 32, 5, 1, 2, 2, 14, 14, "k_conv_tc_fold"),         # odd entry count (padding entry), 5 tap columns
     (48, 24, 3, 1, 1, 2, 20, 20, "k_conv_tc_fold"),
     (64, 32, 3, 1, 1, 1, 12, 70, "k_conv_tc_fold"),         # two column strips
@@ -467,9 +467,9 @@ def test_single_conv_bf16_with_explicit_skip(dc, c_in, c_out, k, s, p, n, h, w, 
     (200, 24, 3, 1, 1, 2, 14, 14, "k_conv_tc"),             # many channels, fewer than 32 outputs: general kernel
     (192, 32, 1, 1, 0, 2, 28, 28, "k_conv_tc_rows"),        # 1x1 projection to 32 channels
 ])
-def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel):
+def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel, algo=0):
     g = dc.geom(c_in, c_out, 1, k, s, p)
-    assert dc.conv_kernel_name(n, h, w, g, dc.BF16) == kernel
+    assert kernel is None or dc.conv_kernel_name(n, h, w, g, dc.BF16) == kernel
     spec = I.make_layer(11, 0, c_in, c_out, k, s, p)
     lay = dc.DeviceLayer(spec)
     wf = torch.empty_like(lay.weight)
@@ -483,9 +483,9 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
     Wf, bfo = O.fold_bn(spec)
     lin = O.conv_direct(x.transpose(0, 3, 1, 2), Wf, bfo, k, s, p)
     # plain, and with skip input + ReLU6
-    y = run_conv(dc, dev(x, torch.bfloat16), g, packed, bf, dc.ACT_IDENTITY)
+    y = run_conv(dc, dev(x, torch.bfloat16), g, packed, bf, dc.ACT_IDENTITY, algo=algo)
     assert_close(nchw(y), lin, TOL_BF16)
-    y = run_conv(dc, dev(x, torch.bfloat16), g, packed, bf, dc.ACT_RELU6, residual=dev(r, torch.bfloat16))
+    y = run_conv(dc, dev(x, torch.bfloat16), g, packed, bf, dc.ACT_RELU6, residual=dev(r, torch.bfloat16), algo=algo)
     assert_close(nchw(y), O.relu6(lin + r.transpose(0, 3, 1, 2)), TOL_BF16)
 
 
@@ -497,6 +497,8 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
     (8, 16, 3, 1, 1, 1, 6, 301, "k_conv_tc_pairrows"),      # three column strips: only the last one holds the column
     (16, 16, 7, 1, 3, 3, 20, 21, "k_conv_tc_pairrows"),     # 7x7
     (8, 8, 3, 1, 1, 200, 5, 3, "k_conv_tc_pairrows"),       # one whole pair per row
+    (24, 24, 3, 1, 1, 1, 7, 7, "k_conv_tc_pairrows"),       # fewer outputs than a block has rows
+    (16, 16, 5, 1, 2, 1, 1, 3, "k_conv_tc_pairrows"),       # the smallest odd width the map has a pair in
     (32, 16, 1, 1, 0, 2, 33, 25, "k_conv_tc_pairrows"),     # 1x1
     (16, 128, 3, 1, 1, 3, 12, 17, "k_conv_tc_pairrows"),    # two accumulator slots, run-time channel loop
     (24, 32, 3, 2, 1, 3, 28, 29, "k_conv_tc_pairrows"),     # stride 2: the column in both row planes
@@ -508,6 +510,20 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
 ])
 def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel):
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel)
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (24, 24, 3, 1, 1, 1, 9, 15),         # pair rows
+    (24, 32, 3, 2, 1, 2, 13, 11),        # pair rows, stride 2
+    (48, 24, 3, 1, 1, 1, 10, 13),        # fold
+    (72, 200, 3, 1, 1, 1, 7, 9),         # rows, two passes, a partial last plane
+    (40, 264, 3, 2, 1, 1, 9, 13),        # rows, stride 2, two passes
+    (32, 40, 1, 1, 0, 1, 9, 7),          # general
+    (8, 136, 5, 2, 1, 1, 11, 13),        # general, stride 2
+    (20, 12, 3, 1, 1, 1, 9, 7),          # channels no multiple of 8
+])
+def test_cuda_core_kernel_reads_every_weight_order(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, None, algo=dc.ALGO_SIMT)
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
