@@ -23,10 +23,10 @@ extern "C" size_t dc_conv_workspace_bytes(void) { return sizeof(DcWsHeader); }
 
 extern "C" const char *dc_conv_kernel_name(int n, int h, int w, const dc_geom *g, dc_dtype dtype) {
   if (dc_validate_geom(g) != DC_OK || g->groups != 1 || n <= 0 || h <= 0 || w <= 0) return nullptr;
-  if (dtype == DC_F32) return "k_conv_dense_f32";
+  if (dtype == DC_F32) return dc_conv_f32_supported(n, h, w, g) ? "k_conv_dense_f32" : "k_conv_dense_f32_any";
   if (dtype != DC_BF16) return nullptr;
   if (dc_conv_pairrows_supported(n, h, w, g)) return "k_conv_tc_pairrows";
-  if (dc_conv_rows_supported(n, h, w, g)) return g->stride == 2 ? "k_conv_tc" : "k_conv_tc_rows";
+  if (dc_conv_rows_supported(n, h, w, g)) return g->stride == 2 ? "k_conv_tc_rows_s2" : "k_conv_tc_rows";
   if (dc_conv_fold_supported(n, h, w, g)) return "k_conv_tc_fold";
   if (dc_conv_tc_supported(n, h, w, g)) return "k_conv_tc";
   if (dc_conv_stem_s2_supported(n, h, w, g) && dc_conv_stem_supported(n, h, w, g)) return "k_conv_stem_s2";

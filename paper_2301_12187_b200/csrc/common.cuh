@@ -418,7 +418,8 @@ struct DcWsHeader {
 dc_status dc_launch_conv_simt(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                               const float *bias, dc_act act, const void *residual, void *y,
                               dc_dtype dtype, cudaStream_t stream);
-// fp32; DC_ERR_UNSUPPORTED: a shape for the kernel that takes any channel count
+// fp32, channels in multiples of 4; false and DC_ERR_UNSUPPORTED: a shape for the kernel that takes any count
+bool dc_conv_f32_supported(int n, int h, int w, const dc_geom *g);
 dc_status dc_launch_conv_f32(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                              const float *bias, dc_act act, const void *residual, void *y, cudaStream_t stream);
 dc_status dc_launch_conv_tc(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,

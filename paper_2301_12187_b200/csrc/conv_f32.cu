@@ -320,6 +320,11 @@ bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *pl) {
 
 }  // namespace
 
+bool dc_conv_f32_supported(int n, int h, int w, const dc_geom *g) {
+  F32Plan pl;
+  return f32_plan(n, h, w, g, dc_sm_count(), &pl);
+}
+
 dc_status dc_launch_conv_f32(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                              const float *bias, dc_act act, const void *residual, void *y, cudaStream_t stream) {
   F32Plan pl;

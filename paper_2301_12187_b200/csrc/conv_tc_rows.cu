@@ -592,12 +592,12 @@ k_conv_tc_rows(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
   rows_body<RESIDENT, PARTIAL, SPLITK, false>(map_a, p, w_packed, bias, residual, y, ws);
 }
-// the general kernel's stride-2 layers, fed the same way
+// stride 2
 template <bool RESIDENT, bool PARTIAL, bool SPLITK>
 __global__ void __launch_bounds__(kThreads, 1)
-k_conv_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
-          const void *__restrict__ w_packed, const float *__restrict__ bias,
-          const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
+k_conv_tc_rows_s2(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ RowsParams p,
+                  const void *__restrict__ w_packed, const float *__restrict__ bias,
+                  const __nv_bfloat16 *__restrict__ residual, __nv_bfloat16 *__restrict__ y, DcWsHeader *ws) {
   rows_body<RESIDENT, PARTIAL, SPLITK, true>(map_a, p, w_packed, bias, residual, y, ws);
 }
 
@@ -872,10 +872,10 @@ dc_status dc_launch_conv_rows(const void *x, int n, int h, int w, const dc_geom 
   }
   using Kernel = decltype(&k_conv_tc_rows<false, false, false>);
   static constexpr Kernel kernels[10] = {
-      k_conv_tc_rows<false, false, false>, k_conv_tc_rows<true, false, false>, k_conv_tc_rows<false, true, false>,
-      k_conv_tc_rows<false, false, true>,  k_conv_tc_rows<false, true, true>,  k_conv_tc<false, false, false>,
-      k_conv_tc<true, false, false>,       k_conv_tc<false, true, false>,      k_conv_tc<false, false, true>,
-      k_conv_tc<false, true, true>};
+      k_conv_tc_rows<false, false, false>,    k_conv_tc_rows<true, false, false>,    k_conv_tc_rows<false, true, false>,
+      k_conv_tc_rows<false, false, true>,     k_conv_tc_rows<false, true, true>,     k_conv_tc_rows_s2<false, false, false>,
+      k_conv_tc_rows_s2<true, false, false>,  k_conv_tc_rows_s2<false, true, false>, k_conv_tc_rows_s2<false, false, true>,
+      k_conv_tc_rows_s2<false, true, true>};
   static unsigned char attr_done[10][kDcMaxDevices];
   const int which = (p.stride == 2 ? 5 : 0) + (p.b_resident ? 1 : (p.partial ? 2 : 0) + (p.ksplit > 1 ? (p.partial ? 2 : 3) : 0));
   DC_CUDA_OK(dc_set_max_smem_once(kernels[which], kSmemBudget, attr_done[which]));

@@ -98,7 +98,7 @@ def test_kernel_name_query_follows_the_dispatch_rules():
         assert dc.conv_kernel_name(n, h, w, dc.geom(24, 24, 1, 3, 1, 1), dc.BF16) == "k_conv_tc_pairrows"
     assert dc.conv_kernel_name(128, 14, 14, dc.geom(40, 32, 1, 5, 1, 2), dc.BF16) == "k_conv_tc_fold"
     assert dc.conv_kernel_name(128, 56, 56, dc.geom(24, 32, 1, 3, 2, 1), dc.BF16) == "k_conv_tc_pairrows"
-    assert dc.conv_kernel_name(128, 56, 56, dc.geom(96, 144, 1, 5, 2, 2), dc.BF16) == "k_conv_tc"
+    assert dc.conv_kernel_name(128, 56, 56, dc.geom(96, 144, 1, 5, 2, 2), dc.BF16) == "k_conv_tc_rows_s2"
     assert dc.conv_kernel_name(128, 14, 14, dc.geom(96, 576, 1, 1, 1, 0), dc.BF16) == "k_conv_tc_rows"
     assert dc.conv_kernel_name(128, 7, 7, dc.geom(160, 960, 1, 3, 1, 1), dc.BF16) == "k_conv_tc_rows"
     assert dc.conv_kernel_name(128, 28, 28, dc.geom(144, 32, 1, 3, 1, 1), dc.BF16) == "k_conv_tc_rows"
@@ -107,7 +107,9 @@ def test_kernel_name_query_follows_the_dispatch_rules():
     assert dc.conv_kernel_name(2, 17, 33, dc.geom(3, 40, 1, 3, 2, 1), dc.BF16) == "k_conv_stem_tc"
     assert dc.conv_kernel_name(1, 20, 20, dc.geom(3, 264, 1, 3, 2, 1), dc.BF16) == "k_conv_smallcin_bf16"
     assert dc.conv_kernel_name(128, 56, 56, dc.geom(20, 12, 1, 3, 1, 1), dc.BF16) == "k_conv_dense_bf16"
+    assert dc.conv_kernel_name(2, 16, 17, dc.geom(8, 136, 1, 3, 2, 1), dc.BF16) == "k_conv_tc"
     assert dc.conv_kernel_name(2, 16, 16, dc.geom(16, 24, 1, 3, 1, 1), dc.F32) == "k_conv_dense_f32"
+    assert dc.conv_kernel_name(2, 16, 16, dc.geom(6, 24, 1, 3, 1, 1), dc.F32) == "k_conv_dense_f32_any"
     assert dc.conv_kernel_name(2, 16, 16, dc.geom(16, 16, 16, 3, 1, 1), dc.BF16) is None
     assert dc.conv_kernel_name(0, 16, 16, dc.geom(16, 24, 1, 3, 1, 1), dc.BF16) is None
 
@@ -128,7 +130,7 @@ def test_wide_maps_stay_on_the_tensor_cores(k, stride):
                 g = dc.geom(c_in, c_out, 1, k, stride, pad)
                 for w in widths:
                     name = dc.conv_kernel_name(n, h, w, g, dc.BF16)
-                    assert name in ("k_conv_tc_rows", "k_conv_tc"), (c_in, c_out, n, h, w, pad, name)
+                    assert name in ("k_conv_tc_rows", "k_conv_tc_rows_s2"), (c_in, c_out, n, h, w, pad, name)
 
 
 def test_entry_points_validate_before_touching_the_device():

@@ -438,11 +438,11 @@ def test_single_conv_bf16_with_explicit_skip(dc, c_in, c_out, k, s, p, n, h, w, 
     (24, 32, 3, 2, 1, 2, 28, 28, "k_conv_tc_pairrows"),     # stride 2: one output per line, even/odd row boxes
     (32, 16, 5, 2, 2, 1, 30, 44, "k_conv_tc_pairrows"),     # stride 2, even padding, 5x5
     (16, 24, 3, 2, 0, 2, 17, 36, "k_conv_tc_pairrows"),     # stride 2, no padding, odd height
-    (40, 32, 3, 2, 1, 2, 28, 28, "k_conv_tc"),              # stride 2 on parity planes (more than 32 channels)
-    (96, 144, 5, 2, 2, 1, 56, 56, "k_conv_tc"),             # the widest stride-2 merged layer of the network: several tiles per image
-    (48, 64, 7, 2, 3, 1, 31, 44, "k_conv_tc"),              # 7x7 stride 2, odd height: four even and three odd tap rows
-    (48, 24, 5, 2, 1, 2, 22, 26, "k_conv_tc"),              # 5x5 stride 2 with padding 1: odd tap columns lead
-    (72, 48, 3, 2, 0, 1, 17, 150, "k_conv_tc"),             # stride 2 without padding, two column strips
+    (40, 32, 3, 2, 1, 2, 28, 28, "k_conv_tc_rows_s2"),       # stride 2 by sub-tiles (more than 32 channels)
+    (96, 144, 5, 2, 2, 1, 56, 56, "k_conv_tc_rows_s2"),      # the widest stride-2 merged layer of the network: several tiles per image
+    (48, 64, 7, 2, 3, 1, 31, 44, "k_conv_tc_rows_s2"),       # 7x7 stride 2, odd height: four even and three odd tap rows
+    (48, 24, 5, 2, 1, 2, 22, 26, "k_conv_tc_rows_s2"),       # 5x5 stride 2 with padding 1: odd tap columns lead
+    (72, 48, 3, 2, 0, 1, 17, 150, "k_conv_tc_rows_s2"),      # stride 2 without padding, two column strips
     (32, 16, 1, 1, 0, 2, 20, 24, "k_conv_tc_pairrows"),     # 1x1: one instruction per 32-byte K step
     (32, 96, 1, 1, 0, 2, 20, 24, "k_conv_tc_rows"),         # 1x1 expansion from few channels: one half-filled plane
     (16, 96, 1, 1, 0, 1, 40, 112, "k_conv_tc_rows"),        # 1x1 expansion from 16 channels, row tiles
@@ -504,9 +504,9 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
     (24, 32, 3, 2, 1, 3, 28, 29, "k_conv_tc_pairrows"),     # stride 2: the column in both row planes
     (32, 16, 5, 2, 2, 2, 31, 45, "k_conv_tc_pairrows"),     # stride 2, even padding
     (16, 24, 3, 2, 0, 4, 17, 37, "k_conv_tc_pairrows"),     # stride 2, no padding
-    (40, 32, 3, 2, 1, 2, 28, 29, "k_conv_tc"),              # stride 2 on parity planes
-    (96, 144, 5, 2, 2, 1, 57, 57, "k_conv_tc"),             # the same, several tiles per image
-    (24, 168, 3, 2, 1, 1, 49, 49, "k_conv_tc"),             # few channels, more outputs than the pair rows take
+    (40, 32, 3, 2, 1, 2, 28, 29, "k_conv_tc_rows_s2"),       # stride 2 by sub-tiles
+    (96, 144, 5, 2, 2, 1, 57, 57, "k_conv_tc_rows_s2"),      # the same, several tiles per image
+    (24, 168, 3, 2, 1, 1, 49, 49, "k_conv_tc_rows_s2"),      # few channels, more outputs than the pair rows take
 ])
 def test_odd_widths_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel):
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, kernel)
@@ -567,6 +567,18 @@ def test_rows_with_a_shared_reduction_against_the_oracle(dc, c_in, c_out, k, s, 
     (384, 24, 3, 2, 1, 1, 7, 7),         # few outputs
 ])
 def test_stride_2_by_sub_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows_s2")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (8, 136, 3, 2, 1, 2, 28, 28),        # even width
+    (8, 136, 3, 2, 1, 3, 27, 29),        # odd sides: the last column is in one parity plane only
+    (8, 144, 5, 2, 2, 2, 22, 25),        # 5x5, even padding
+    (8, 136, 5, 2, 1, 1, 31, 26),        # 5x5, odd tap columns lead
+    (8, 200, 3, 2, 0, 1, 17, 151),       # no padding, two column strips
+    (8, 264, 3, 2, 1, 2, 15, 13),        # two passes
+])
+def test_stride_2_on_parity_planes_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc")
 
 
