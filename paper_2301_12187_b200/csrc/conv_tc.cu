@@ -107,8 +107,8 @@ k_conv_tc(const void *__restrict__ w_packed, const __grid_constant__ TcParams p,
   uint8_t *smem_a = smem + p.off_a;
   uint8_t *smem_out = smem + p.off_out;
   uint8_t *smem_zero = smem_a + (size_t)p.stages * p.a_stage_bytes;   // always-zero plane + slack
-  uint8_t *smem_ones = smem + p.off_bias;        // 8 GEMM rows of the constant operand: (1, 1, 0, ..) in 16 bytes each
-  uint8_t *smem_bias = smem_ones + 128;          // [nnt * n_tile][16 bytes]: bias as two bf16 terms, then n_tile zero rows
+  uint8_t *smem_ones = smem + p.off_bias;        // 8 GEMM rows of the constant operand: (1, 1, 1, 0, ..) in 16 bytes each
+  uint8_t *smem_bias = smem_ones + 128;          // [nnt * n_tile][16 bytes]: bias as three bf16 terms, then n_tile zero rows
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile uint32_t *abort_flag = &abort_s;
@@ -132,20 +132,12 @@ k_conv_tc(const void *__restrict__ w_packed, const __grid_constant__ TcParams p,
   if (threadIdx.x >= 5 * 32) {
     const int t = threadIdx.x - 5 * 32;
     // The bias is added by the tensor core: one instruction per block multiplies a constant operand (1.0 in
-    // the first two K elements of every GEMM row; one 8-row group read sixteen times, group stride 0; its
-    // second K chunk is the zero plane) with [bias as bf16, its bf16 remainder, 0, ...] per output channel
-    // (exact to 16 mantissa bits) before the block's other instructions accumulate.
-    if (t < 8) reinterpret_cast<uint4 *>(smem_ones)[t] = make_uint4(0x3F803F80u, 0u, 0u, 0u);
-    for (int i = t; i < (p.nnt + 1) * p.n_tile; i += 128) {
-      uint32_t w0 = 0u;
-      if (bias && i < p.c_out) {
-        const float b = bias[i];
-        const __nv_bfloat16 hi = __float2bfloat16_rn(b);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
-        w0 = (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16);
-      }
-      reinterpret_cast<uint4 *>(smem_bias)[i] = make_uint4(w0, 0u, 0u, 0u);
-    }
+    // the first three K elements of every GEMM row; one 8-row group read sixteen times, group stride 0; its
+    // second K chunk is the zero plane) with the bias of each output channel as three bf16 terms before the
+    // block's other instructions accumulate.
+    if (t < 8) reinterpret_cast<uint4 *>(smem_ones)[t] = bias_ones();
+    for (int i = t; i < (p.nnt + 1) * p.n_tile; i += 128)
+      reinterpret_cast<uint4 *>(smem_bias)[i] = bias && i < p.c_out ? bias_terms(bias[i]) : make_uint4(0u, 0u, 0u, 0u);
     // the zero plane: second chunk of the padding entry, and the landing zone of reads past the last stage
     uint4 *z = reinterpret_cast<uint4 *>(smem_zero);
     for (int i = t; i < (p.mb * 2048 + 1024) / 16; i += 128) z[i] = make_uint4(0u, 0u, 0u, 0u);

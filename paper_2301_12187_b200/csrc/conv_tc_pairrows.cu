@@ -389,7 +389,7 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
   uint8_t *smem_a = smem + p.off_a;              // 1024-byte aligned stages (the swizzle pattern repeats every 1024 bytes)
   uint8_t *smem_out = smem + p.off_out;
   uint8_t *smem_ones = smem + p.off_bias;        // 8 lines of the constant operand (1024-byte aligned)
-  uint8_t *smem_bias = smem_ones + 1024;         // [n_pad][16 bytes]: bias as two bf16 terms, then n_pad zero rows
+  uint8_t *smem_bias = smem_ones + 1024;         // [n_pad][16 bytes]: bias as three bf16 terms, then n_pad zero rows
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile uint32_t *abort_flag = &sh.abort;
@@ -504,25 +504,17 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
       tmem_relinquish();
     } else if (warp >= kFirstEpiWarp) {
       // The bias is added by the tensor core: one instruction per block multiplies a constant operand
-      // (1.0 in the first two K elements of every line) with [bias as bf16, its bf16 remainder, 0, ...]
-      // per accumulator column (exact to 16 mantissa bits) before the block's other instructions
-      // accumulate.  The constant operand is one 8-line group read sixteen times (group stride 0); with
-      // the 128-byte swizzle the first 16-byte chunk of line r sits at chunk r.  Column n belongs to
-      // output channel n mod co8 (the second pixel's columns follow the first's).
+      // (1.0 in the first three K elements of every line) with each accumulator column's bias as three bf16
+      // terms before the block's other instructions accumulate.  The constant operand is one 8-line group read
+      // sixteen times (group stride 0); with the 128-byte swizzle the first 16-byte chunk of line r sits at
+      // chunk r.  Column n belongs to output channel n mod co8 (the second pixel's columns follow the first's).
       const int t0 = (int)threadIdx.x - kFirstEpiWarp * 32;
       const int ncol = (p.stride == 1 ? 2 : 1) * p.co8;
       for (int t = t0; t < 64; t += kEpiWarps * 32)
-        reinterpret_cast<uint4 *>(smem_ones)[t] = make_uint4((t & 7) == (t >> 3) ? 0x3F803F80u : 0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(smem_ones)[t] = (t & 7) == (t >> 3) ? bias_ones() : make_uint4(0u, 0u, 0u, 0u);
       for (int t = t0; t < 2 * p.n_pad; t += kEpiWarps * 32) {
-        uint32_t w0 = 0u;
         const int ch = t < ncol ? (t >= p.co8 ? t - p.co8 : t) : p.c_out;
-        if (bias && ch < p.c_out) {
-          const float b = bias[ch];
-          const __nv_bfloat16 hi = __float2bfloat16_rn(b);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
-          w0 = (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16);
-        }
-        reinterpret_cast<uint4 *>(smem_bias)[t] = make_uint4(w0, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(smem_bias)[t] = bias && ch < p.c_out ? bias_terms(bias[ch]) : make_uint4(0u, 0u, 0u, 0u);
       }
       fence_proxy_async();                       // both are read by the tensor core (async proxy)
     }

@@ -526,6 +526,62 @@ def test_cuda_core_kernel_reads_every_weight_order(dc, c_in, c_out, k, s, p, n, 
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, None, algo=dc.ALGO_SIMT)
 
 
+BIAS_CASES = [
+    (32, 32, 3, 1, 1, 2, 9, 15),         # pair rows, odd width
+    (24, 24, 3, 1, 1, 2, 10, 16),        # pair rows, even width
+    (24, 32, 3, 2, 1, 2, 13, 11),        # pair rows, stride 2
+    (144, 32, 3, 1, 1, 8, 28, 28),       # rows, resident weights
+    (384, 64, 3, 1, 1, 1, 14, 14),       # rows, a shared reduction
+    (128, 128, 5, 1, 2, 4, 30, 33),      # rows, weight stages of one tap column
+    (40, 32, 3, 2, 1, 2, 28, 29),        # rows, stride 2
+    (48, 24, 3, 1, 1, 1, 20, 20),        # fold
+    (200, 24, 3, 1, 1, 1, 14, 14),       # general
+    (8, 136, 3, 2, 1, 1, 13, 15),        # general, stride 2
+]
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", BIAS_CASES)
+def test_bias_keeps_its_32_bits(dc, c_in, c_out, k, s, p, n, h, w):
+    """A bias that the products cancel down to its last 8 bits: y = b - hi - mid with hi and mid the two bf16 values that
+    hold its first 16.  A few roundings of an fp32 sum are at most 2^-21 |b|; a bias held as two bf16 terms is off by 2^-17."""
+    gen = torch.Generator().manual_seed(17)
+    b = (torch.randn(c_out, generator=gen) * 2.0 ** torch.randint(-6, 7, (c_out,), generator=gen)).float()
+    cut = lambda v: (v.view(torch.int32) & -65536).view(torch.float32)
+    hi = cut(b)
+    mid = cut(b - hi)
+    w4 = torch.zeros(c_out, c_in, k, k)
+    w4[:, 0, p, p], w4[:, 1, p, p] = -hi, -mid           # the centre tap: inside the image for every output
+    x = torch.zeros(n, h, w, c_in)
+    x[..., :2] = 1.0
+    want = (b.double() - hi.double() - mid.double()).expand(n, *[O.out_extent(e, k, s, p) for e in (h, w)], c_out)
+    g = dc.geom(c_in, c_out, 1, k, s, p)
+    packed = torch.empty(dc.packed_bytes(g, dc.BF16), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(w4.cuda(), g, dc.BF16, packed)
+    for algo in (dc.ALGO_AUTO, dc.ALGO_SIMT):
+        y = run_conv(dc, x.cuda().bfloat16(), g, packed, b.cuda(), dc.ACT_IDENTITY, algo=algo).double().cpu()
+        assert float(((y - want).abs() / b.double().abs()).max()) <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", BIAS_CASES)
+def test_bias_that_is_not_finite(dc, c_in, c_out, k, s, p, n, h, w):
+    """Infinities and NaN in the bias, and a finite value that rounds to a bf16 infinity, come out as from the CUDA-core
+    kernel, and only in their own channels."""
+    b = torch.linspace(-1, 1, c_out)
+    b[:4] = torch.tensor([float("inf"), -float("inf"), float("nan"), 3.4e38])
+    g = dc.geom(c_in, c_out, 1, k, s, p)
+    packed = torch.empty(dc.packed_bytes(g, dc.BF16), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(torch.zeros(c_out, c_in, k, k).cuda(), g, dc.BF16, packed)
+    x, ws = torch.ones(n, h, w, c_in, device="cuda", dtype=torch.bfloat16), torch.zeros(dc.conv_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    out = []
+    for algo in (dc.ALGO_AUTO, dc.ALGO_SIMT):
+        y = torch.empty(n, O.out_extent(h, k, s, p), O.out_extent(w, k, s, p), c_out, device="cuda", dtype=torch.bfloat16)
+        dc.conv_forward(x, g, packed, b.cuda(), dc.ACT_IDENTITY, None, y, ws, algo=algo)
+        assert dc.workspace_status(ws) == dc.OK
+        out.append(y.float())
+    assert torch.equal(torch.nan_to_num(out[0], nan=7e7), torch.nan_to_num(out[1], nan=7e7))
+    assert bool(out[0][..., 2].isnan().all()) and not bool(out[0][..., 3:].isnan().any())
+
+
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, several column strips and row tiles
     (72, 200, 5, 1, 2, 2, 11, 13),       # the same in two passes, a partial plane of channels
