@@ -53,6 +53,8 @@ typedef enum {
 } dc_status;
 
 typedef enum { DC_F32 = 0, DC_BF16 = 1 } dc_dtype;
+/* DC_ACT_RELU6 is min(max(v, 0), 6).  A NaN becomes 0, except in k_conv_stem_s2 and in the bf16 depthwise stencil, where it
+ * becomes 6. */
 typedef enum { DC_ACT_IDENTITY = 0, DC_ACT_RELU6 = 1 } dc_act;
 typedef enum { DC_ALGO_AUTO = 0, DC_ALGO_TCGEN05 = 1, DC_ALGO_SIMT = 2 } dc_algo;
 

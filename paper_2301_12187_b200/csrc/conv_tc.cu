@@ -374,12 +374,9 @@ k_conv_tc(const void *__restrict__ w_packed, const __grid_constant__ TcParams p,
                   }
                   uint4 ov;
                   uint32_t *ow = reinterpret_cast<uint32_t *>(&ov);
-                  // ReLU6: the conversion clamps at zero itself, one packed minimum against (6, 6) does the rest
-                  // (the same values as clamping before rounding, since 0 and 6 are bf16 values)
 #pragma unroll
                   for (int i = 0; i < 4; ++i)
-                    ow[i] = decltype(RELU)::value ? min_bf16x2(pack_bf16x2_relu(f[2 * i], f[2 * i + 1]), 0x40C040C0u)
-                                                  : pack_bf16x2(f[2 * i], f[2 * i + 1]);
+                    ow[i] = decltype(RELU)::value ? relu6_bf16x2(f[2 * i], f[2 * i + 1]) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
                   *reinterpret_cast<uint4 *>(pdst + ch * 2) = ov;
                 }
               }

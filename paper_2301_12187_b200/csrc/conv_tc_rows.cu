@@ -451,13 +451,9 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
             }
             uint4 ov;
             uint32_t *ow = reinterpret_cast<uint32_t *>(&ov);
-            // ReLU6 on the rounded pairs: 0 and 6 are bf16 values and rounding is monotonic, so clamping in and
-            // after the conversion gives the same values as clamping before it: the conversion clamps at zero
-            // itself, one packed minimum against (6, 6) does the rest
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-              ow[i] = decltype(RELU)::value ? min_bf16x2(pack_bf16x2_relu(f[2 * i], f[2 * i + 1]), 0x40C040C0u)
-                                            : pack_bf16x2(f[2 * i], f[2 * i + 1]);
+              ow[i] = decltype(RELU)::value ? relu6_bf16x2(f[2 * i], f[2 * i + 1]) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
             return ov;
           };
           // 32 accumulator columns per read while they last.  A thread owns a pixel, so stored directly
@@ -557,7 +553,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
           uint32_t *ow = reinterpret_cast<uint32_t *>(&ov);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            ow[i] = relu6 ? min_bf16x2(pack_bf16x2_relu(f[2 * i], f[2 * i + 1]), 0x40C040C0u) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
+            ow[i] = relu6 ? relu6_bf16x2(f[2 * i], f[2 * i + 1]) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
           *reinterpret_cast<uint4 *>(y + o) = ov;
         }
       }

@@ -211,6 +211,18 @@ __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
   return d;
 }
 
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// ReLU6 of two floats as packed bf16: 0 and 6 are bf16 values and rounding is monotonic, so clamping behind the
+// conversion gives the same values as before it.  The maximum comes first, so that a NaN becomes 0 as in dc_act_apply
+// (clamped at zero by the conversion itself, which keeps NaN, it would come out of the minimum as 6).
+__device__ __forceinline__ uint32_t relu6_bf16x2(float lo, float hi) {
+  return min_bf16x2(max_bf16x2(pack_bf16x2(lo, hi), 0u), 0x40C040C0u);
+}
+
 // named barrier `id` over `count` threads
 // 16-byte shared-memory accesses by 32-bit shared address (no generic-address arithmetic)
 __device__ __forceinline__ void sts_u4(uint32_t a, uint4 v) {

@@ -580,6 +580,11 @@ def test_bias_that_is_not_finite(dc, c_in, c_out, k, s, p, n, h, w):
         out.append(y.float())
     assert torch.equal(torch.nan_to_num(out[0], nan=7e7), torch.nan_to_num(out[1], nan=7e7))
     assert bool(out[0][..., 2].isnan().all()) and not bool(out[0][..., 3:].isnan().any())
+    # ReLU6 clamps them: a NaN becomes 0 in every kernel
+    for algo in (dc.ALGO_AUTO, dc.ALGO_SIMT):
+        dc.conv_forward(x, g, packed, b.cuda(), dc.ACT_RELU6, None, y, ws, algo=algo)
+        assert [float(v) for v in y[..., :4].float().amax((0, 1, 2))] == [6.0, 0.0, 0.0, 6.0]
+        assert [float(v) for v in y[..., :4].float().amin((0, 1, 2))] == [6.0, 0.0, 0.0, 6.0]
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
