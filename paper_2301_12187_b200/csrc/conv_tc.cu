@@ -137,7 +137,7 @@ k_conv_tc(const void *__restrict__ w_packed, const __grid_constant__ TcParams p,
     // block's other instructions accumulate.
     if (t < 8) reinterpret_cast<uint4 *>(smem_ones)[t] = bias_ones();
     for (int i = t; i < (p.nnt + 1) * p.n_tile; i += 128)
-      reinterpret_cast<uint4 *>(smem_bias)[i] = bias && i < p.c_out ? bias_terms(bias[i]) : make_uint4(0u, 0u, 0u, 0u);
+      reinterpret_cast<uint4 *>(smem_bias)[i] = bias_terms(bias && i < p.c_out ? bias[i] : 0.f);
     // the zero plane: second chunk of the padding entry, and the landing zone of reads past the last stage
     uint4 *z = reinterpret_cast<uint4 *>(smem_zero);
     for (int i = t; i < (p.mb * 2048 + 1024) / 16; i += 128) z[i] = make_uint4(0u, 0u, 0u, 0u);

@@ -514,7 +514,7 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
         reinterpret_cast<uint4 *>(smem_ones)[t] = (t & 7) == (t >> 3) ? bias_ones() : make_uint4(0u, 0u, 0u, 0u);
       for (int t = t0; t < 2 * p.n_pad; t += kEpiWarps * 32) {
         const int ch = t < ncol ? (t >= p.co8 ? t - p.co8 : t) : p.c_out;
-        reinterpret_cast<uint4 *>(smem_bias)[t] = bias && ch < p.c_out ? bias_terms(bias[ch]) : make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && ch < p.c_out ? bias[ch] : 0.f);
       }
       fence_proxy_async();                       // both are read by the tensor core (async proxy)
     }

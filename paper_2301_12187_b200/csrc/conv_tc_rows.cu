@@ -252,7 +252,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
         reinterpret_cast<uint4 *>(smem_ones)[t] = c == r ? bias_ones() : make_uint4(0u, 0u, 0u, 0u);
       }
       for (int t = t0; t < p.n_pad + p.n_tile; t += kEpiWarps * 32)
-        reinterpret_cast<uint4 *>(smem_bias)[t] = bias && t < p.c_out ? bias_terms(bias[t]) : make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && t < p.c_out ? bias[t] : 0.f);
       fence_proxy_async();                       // both are read by the tensor core (async proxy)
     }
     tc_fence_before();
