@@ -1283,25 +1283,39 @@ static int zero_ctas(const BlockDelivery &dv, const dc_geom &mg, int threads) {
 static bool compose33_ok(int c_in, int c_mid, int k1, int s1, int k2) {
   return k1 == 3 && s1 == 1 && k2 == 3 && c_in % 4 == 0 && c_mid % 4 == 0;
 }
+// The first status of a merge's launches that is not DC_OK.  A launch in <<<>>> form leaves its error with
+// cudaGetLastError, and it is asked for behind each of them: asked once at the end of the merge it may be gone (the fp32
+// convolution asks, and clears, it too; a run whose refused launch was followed by one of those returned DC_OK).
+struct MergeStatus {
+  dc_status s = DC_OK;
+  void note(dc_status t) { if (s == DC_OK) s = t; }
+  void note(cudaError_t e) { note(e == cudaSuccess ? DC_OK : DC_ERR_CUDA); }
+  void launched() { note(cudaGetLastError()); }
+};
+
 static void launch_compose33(const Operand33 &first, const Operand33 &second, int c0, int c1, int c2, float *w, float *b,
-                             const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st) {
+                             const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
   static unsigned char attr_done[kDcMaxDevices];
-  dc_set_max_smem_once(k_compose33, kP3Ring, attr_done);
-  (void)dc_launch_pdl(k_compose33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kP3Threads)), dim3(kP3Threads), kP3Ring, st, a, dv);
+  status.note(dc_set_max_smem_once(k_compose33, kP3Ring, attr_done));
+  status.note(dc_launch_pdl(k_compose33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kP3Threads)), dim3(kP3Threads), kP3Ring, st, a, dv));
+  status.launched();
 }
 
 // A 1x1 after a large dense kernel is a plain matrix product: the fp32 convolution's kernel runs it as a 1x1 layer whose
 // pixels are the second layer's rows and whose weights are the first layer as stored (960 -> 320 -> 1280: 81 us with the
 // gathered product, 59.9 us).  False: a shape outside that kernel's range, nothing was launched.
-static bool compose_as_product(const Piece &first, const Piece &second, float *out, cudaStream_t st) {
+static bool compose_as_product(const Piece &first, const Piece &second, float *out, cudaStream_t st, MergeStatus &status) {
   const dc_geom g = {first.c_out, first.c_in * first.k * first.k, 1, 1, 1, 0};
-  return dc_launch_conv_f32(second.w, 1, 1, second.c_out, &g, first.w, nullptr, DC_ACT_IDENTITY, nullptr, out, st) != DC_ERR_UNSUPPORTED;
+  const dc_status s = dc_launch_conv_f32(second.w, 1, 1, second.c_out, &g, first.w, nullptr, DC_ACT_IDENTITY, nullptr, out, st);
+  if (s == DC_ERR_UNSUPPORTED) return false;
+  status.note(s);
+  return true;
 }
 
 // Composes second o first into a new piece; launches when `go`.  With `dv`, the piece is the run's result: where the
 // kernel can deliver it itself it goes to w_final / b_final (and the packed copy) and *delivered is set.
-static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool go, cudaStream_t st,
+static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool go, cudaStream_t st, MergeStatus &status,
                      const BlockDelivery *dv = nullptr, const dc_geom *mg = nullptr, float *w_final = nullptr,
                      float *b_final = nullptr, bool *delivered = nullptr) {
   Piece out;
@@ -1321,7 +1335,7 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       BlockDelivery piece{nullptr, -1, 0, KOrder{}};
       if (dv) { out.w = w = w_final; out.b = b = b_final; *delivered = true; }
       launch_compose33(operand(first), operand(second), first.c_in, first.c_out, second.c_out, w, b, dv ? *dv : piece,
-                       mg ? *mg : dc_geom{}, st);
+                       mg ? *mg : dc_geom{}, st, status);
     } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k > 1 &&
         first.c_out * second.k * second.k <= kAfter1x1MaxFloats) {
       dim3 grid(dc_div_up(out.c_in * out.k * out.k, 256), out.c_out + 1);
@@ -1331,7 +1345,7 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       const int gx = dc_div_up(out.c_in * out.k * out.k, 32), gy = dc_div_up(out.c_out, 8);
       k_compose_dd_small<<<gx * gy + nbias, 256, 0, st>>>(first, second, w, b, out.k, gx, gy);
     } else if (!first.diag && !second.diag && second.k == 1 && !first.ident && !second.ident &&
-               compose_as_product(first, second, w, st)) {
+               compose_as_product(first, second, w, st, status)) {
       k_compose_bias<<<nbias, 256, 0, st>>>(first, second, b);
     } else if (!first.diag && !second.diag) {
       // 128 x 64 tiles when they still give every SM two tiles, 64 x 64 otherwise
@@ -1345,6 +1359,7 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       const int nb = blocks_for(elems, 256);
       k_compose_diag<<<nb + nbias, 256, 0, st>>>(first, second, w, b, out.k, (int)elems, nb);
     }
+    status.launched();
   }
   return out;
 }
@@ -1395,6 +1410,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   if (s != DC_OK) return s;
   if (merged) *merged = mg;
   Bump bump{go ? (char *)workspace : nullptr, 0};
+  MergeStatus status;
 
   // What the last launch delivers.  A run that is one block of the tiled kind, or two dense 3x3 layers, needs no launch of
   // its own for that (nor, in the second case, for the BN): the kernel that merges it reads the layers as they are and
@@ -1413,8 +1429,8 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
       else id[res[g].first] = 1;
     }
     launch_compose33(Operand33{raw_of(layers[0]), id[0]}, Operand33{raw_of(layers[1]), id[1]}, mg.c_in, layers[0].c_out, mg.c_out,
-                     w_merged, b_merged, BlockDelivery{w_packed, mode, whole, ko}, mg, st);
-    return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+                     w_merged, b_merged, BlockDelivery{w_packed, mode, whole, ko}, mg, st, status);
+    return status.s;
   }
 
   if (go && n == 2 && algo != DC_MERGE_STEPS && can_pack) {
@@ -1430,8 +1446,9 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
       const Outer33 a{raw_of(de), raw_of(dw), id[dw_first ? 1 : 0], id[dw_first ? 0 : 1], dw_first ? 1 : 0, mg.c_in, mg.c_out,
                       w_merged, b_merged, dc_div_up(mg.c_in, kMbI), dc_div_up(mg.c_out, kMbO)};
       const BlockDelivery dv{w_packed, mode, whole, ko};
-      (void)dc_launch_pdl(k_merge_outer33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), 0, st, a, dv);
-      return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+      status.note(dc_launch_pdl(k_merge_outer33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), 0, st, a, dv));
+      status.launched();
+      return status.s;
     }
   }
 
@@ -1457,6 +1474,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
         int bx = blocks_for(max_total, 256);
         dim3 grid(bx > 1024 ? 1024 : bx, cnt);       // a few elements per thread: the launch is short beside its chain
         k_fold_bn<<<grid, 256, 0, st>>>(t);
+        status.launched();
       }
       cnt = 0;
       max_total = 1;
@@ -1492,16 +1510,18 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   auto flush_tiled = [&]() {
     if (tiled.n == 0) return;
     static unsigned char attr_done[kDcMaxDevices];
-    dc_set_max_smem_once(k_merge_block33, kMbRing, attr_done);
-    (void)dc_launch_pdl(k_merge_block33, dim3(tiled.first[tiled.n] + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), kMbRing, st, tiled, dv);
+    status.note(dc_set_max_smem_once(k_merge_block33, kMbRing, attr_done));
+    status.note(dc_launch_pdl(k_merge_block33, dim3(tiled.first[tiled.n] + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), kMbRing, st, tiled, dv));
+    status.launched();
     tiled.n = 0;
   };
   auto flush_blocks = [&]() {
     flush_tiled();
     if (n_batch == 0) return;
     static unsigned char attr_done[kDcMaxDevices];
-    dc_set_max_smem_once(k_merge_block, 200 * 1024, attr_done);
+    status.note(dc_set_max_smem_once(k_merge_block, 200 * 1024, attr_done));
     k_merge_block<<<dim3(batch_grid, n_batch), kBlockThreads, batch_smem, st>>>(batch);
+    status.launched();
     n_batch = 0; batch_grid = 0; batch_smem = 0;
   };
   Piece acc{};
@@ -1541,7 +1561,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     } else {
       piece = folded[res[gi].first];
       if (go) flush_blocks();
-      for (int j = res[gi].first + 1; j <= res[gi].last; ++j) piece = compose(piece, folded[j], bump, go, st);
+      for (int j = res[gi].first + 1; j <= res[gi].last; ++j) piece = compose(piece, folded[j], bump, go, st, status);
       piece.ident = 1;          // f(x) + x: the identity kernel rides along as a flag
       i = res[gi].last + 1;
     }
@@ -1551,21 +1571,22 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
       // the run's last composition: piece.ident is the second operand's, the result carries none
       const BlockDelivery fin{w_packed, mode, 0, ko};
       const bool last = i == n && go && can_pack;
-      acc = compose(acc, piece, bump, go, st, last ? &fin : nullptr, &mg, w_merged, b_merged, &delivered);
+      acc = compose(acc, piece, bump, go, st, status, last ? &fin : nullptr, &mg, w_merged, b_merged, &delivered);
     }
   }
   if (need) *need = bump.off + 256;
   if (!go) return DC_OK;
   flush_blocks();
 
-  if (at_once || delivered) return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+  if (at_once || delivered) return status.s;
 
   // 3. deliver: dense fp32 result, bias, optional packed copy, in one launch
   const size_t p_elems = mode == 2 ? (size_t)ko.ng * ko.e_pad * ko.n_pad * 8 : elems;
   const int chunked = mode == 2 && p_elems >= (size_t)262144;
   const int nb_w = blocks_for(elems, 256), nb_p = mode ? blocks_for(chunked ? p_elems / 8 : p_elems, 256) : 0;
   k_deliver<<<nb_w + 1 + nb_p, 256, 0, st>>>(acc, w_merged, b_merged, w_packed, mode, ko, nb_w, nb_p, chunked);
-  return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+  status.launched();
+  return status.s;
 }
 
 // Workspace bytes that cover either launch form.

@@ -262,6 +262,26 @@ def test_runs_delivered_by_one_launch(dc, case):
         assert torch.equal(packed, again)
 
 
+def test_a_launch_that_is_refused_is_reported(dc):
+    """A 3x3 layer with 65536 outputs after a 1x1 layer needs a grid the device does not have (the runtime refuses the
+    launch, nothing runs).  The 1x1 layer after it is composed by the fp32 convolution, whose launch succeeds: the merge
+    must report the refused one all the same.  Asked once more, the library has no error left over."""
+    z = lambda *s: torch.zeros(*s, device="cuda")
+    shapes = [(64, 4, 1, 0), (4, 65536, 3, 1), (65536, 352, 1, 0)]
+    keep = [z(co, ci, k, k) for ci, co, k, _ in shapes]
+    layers = [dc.Layer(ci, co, 1, k, 1, p, w.data_ptr(), None, None, None, None, None, 0.0) for (ci, co, k, p), w in zip(shapes, keep)]
+    g, ws_bytes = dc.merge_query(layers, [])
+    wm, bm, ws = z(g.c_out, g.c_in, 3, 3), z(g.c_out), torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda")
+    with pytest.raises(dc.DcError) as e:
+        dc.merge_chain(layers, [], wm, bm, None, dc.F32, ws)
+    assert e.value.status == dc.ERR_CUDA
+    torch.cuda.synchronize()
+    del keep, layers, wm, bm, ws
+    specs, res = small_chain("t1")
+    g, wm, bm, _ = run_merge(dc, specs, res)
+    assert O.rel_l2(wm.cpu().numpy(), O.merge_formula(specs, res)[0]) <= TOL_W
+
+
 @pytest.mark.parametrize("c,n,h,w", [(64, 2, 28, 28), (128, 2, 14, 14), (256, 1, 14, 14), (512, 1, 14, 14)])
 def test_vgg_style_dense_merge(dc, c, n, h, w):
     """Two dense 3x3 layers (VGG-style, c -> c -> c) merged into one 5x5 layer: merged weights against
