@@ -123,7 +123,8 @@ dc_status dc_packed_bytes(const dc_geom *g, dc_dtype dtype, size_t *bytes);
  *   W'[o,i,u1+s1*u2,v1+s1*v2] += W2[o,c,u2,v2] * W1[c,i,u1,v1],  b' = b2 + (sum_taps W2) b1.
  * Outputs (device): w_merged fp32 [c_out][c_in][k'][k'], b_merged fp32 [c_out]; if w_packed is
  * not NULL also the packed copy for packed_dtype (size from dc_packed_bytes).  workspace: device,
- * at least the bytes dc_merge_query reports.  fp32 FMA arithmetic throughout.
+ * at least the bytes dc_merge_query reports; it overlaps nothing else.  The outputs may overlap the
+ * layers' arrays (which then do not survive the call), not one another.  fp32 FMA arithmetic throughout.
  */
 dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
                          float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,

@@ -1399,6 +1399,27 @@ static RawLayer raw_of(const dc_layer &L) {
   return RawLayer{L.weight, L.bias, L.bn_gamma, L.bn_beta, L.bn_mean, L.bn_var, L.bn_eps};
 }
 
+// True when an output of the merge shares memory with an array of its layers.  The kernels that merge and deliver in one
+// launch write the result while other CTAs still read the layers, so such a merge goes through the workspace and delivers in
+// a launch behind them.
+static bool writes_into_layers(const dc_layer *layers, int n, const float *w, size_t w_bytes, const float *b, size_t b_bytes,
+                               const void *packed, size_t packed_bytes) {
+  auto shares = [](const void *p, size_t np, const void *q, size_t nq) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), c = reinterpret_cast<uintptr_t>(q);
+    return p && q && a < c + nq && c < a + np;
+  };
+  for (int i = 0; i < n; ++i) {
+    const dc_layer &L = layers[i];
+    const size_t per_channel = (size_t)L.c_out * sizeof(float);
+    const void *arr[6] = {L.weight, L.bias, L.bn_gamma, L.bn_beta, L.bn_mean, L.bn_var};
+    for (int j = 0; j < 6; ++j) {
+      const size_t bytes = j == 0 ? piece_elems(L.c_in, L.c_out, L.k, L.groups != 1) * sizeof(float) : per_channel;
+      if (shares(arr[j], bytes, w, w_bytes) || shares(arr[j], bytes, b, b_bytes) || shares(arr[j], bytes, packed, packed_bytes)) return true;
+    }
+  }
+  return false;
+}
+
 // One walk drives both the size query (go == false: nothing is dereferenced or launched) and the
 // launches (go == true: the caller has already checked workspace_bytes against the query).
 static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *res, int n_res,
@@ -1421,7 +1442,10 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   const int mode = !w_packed ? 0 : (packed_dtype == DC_F32 ? 1 : 2);
   if (go && !dc_aligned16(w_packed)) return DC_ERR_ALIGNMENT;
   const bool can_pack = mode != 2 || mg.c_in % 8 == 0;
-  if (go && n == 2 && algo != DC_MERGE_STEPS && can_pack && layers[0].groups == 1 && layers[1].groups == 1 &&
+  const size_t p_bytes = mode == 2 ? (size_t)ko.ng * ko.e_pad * ko.n_pad * 16 : elems * sizeof(float);
+  const bool direct = go && n <= 3 && algo != DC_MERGE_STEPS && can_pack &&
+                      !writes_into_layers(layers, n, w_merged, elems * sizeof(float), b_merged, mg.c_out * sizeof(float), w_packed, p_bytes);
+  if (direct && n == 2 && layers[0].groups == 1 && layers[1].groups == 1 &&
       compose33_ok(layers[0].c_in, layers[0].c_out, layers[0].k, layers[0].stride, layers[1].k)) {
     int id[2] = {0, 0}, whole = 0;
     for (int g = 0; g < n_res; ++g) {
@@ -1433,7 +1457,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     return status.s;
   }
 
-  if (go && n == 2 && algo != DC_MERGE_STEPS && can_pack) {
+  if (direct && n == 2) {
     const dc_layer &l1 = layers[0], &l2 = layers[1];
     const bool dw_first = l1.groups != 1;
     const dc_layer &de = dw_first ? l2 : l1, &dw = dw_first ? l1 : l2;
@@ -1496,7 +1520,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     flush();
   }
 
-  const bool at_once = n == 3 && chunk_at[0] == kTiledBlock && can_pack;
+  const bool at_once = direct && n == 3 && chunk_at[0] == kTiledBlock;
 
   // 2. compose: blocks and skip groups first (with their identity tap), then left to right
   BlockBatch batch;

@@ -262,6 +262,38 @@ def test_runs_delivered_by_one_launch(dc, case):
         assert torch.equal(packed, again)
 
 
+@pytest.mark.parametrize("case", ["block", "dense_pair", "expand_dw"])
+@pytest.mark.parametrize("alias", ["weights", "bias", "packed"])
+def test_merge_into_its_layers_arrays(dc, case, alias):
+    """Outputs that lie where the layers' arrays lie: the same result as into buffers of their own."""
+    mk = I.make_layer
+    specs = {"block": [mk(71, 0, 40, 240, 1, 1, 0), mk(71, 1, 240, 240, 3, 1, 1, depthwise=True), mk(71, 2, 240, 40, 1, 1, 0)],
+             "dense_pair": [mk(72, 0, 64, 64, 3, 1, 1), mk(72, 1, 64, 64, 3, 1, 1)],
+             "expand_dw": [mk(73, 0, 96, 96, 1, 1, 0), mk(73, 1, 96, 96, 3, 1, 1, depthwise=True)]}[case]
+    g, wm, bm, packed = run_merge(dc, specs, [], packed_dtype=dc.BF16)
+    layers = [dc.DeviceLayer(s) for s in specs]
+    _, ws_bytes = dc.merge_query(layers, [])
+    ws = torch.zeros(ws_bytes, dtype=torch.uint8, device="cuda")
+    out = {"weights": torch.empty_like(wm), "bias": torch.empty_like(bm), "packed": torch.empty_like(packed)}
+    # the layer's array lies at the start of the output's buffer
+    last = layers[-1] if alias == "bias" and case == "block" else layers[0]
+    src = last.bn[1] if alias == "bias" else last.weight
+    flat = out[alias].reshape(-1).view(torch.uint8).view(torch.float32)
+    assert flat.numel() >= src.numel()
+    flat[:src.numel()].copy_(src.reshape(-1))
+    if alias == "bias":
+        last.c.bn_beta = flat.data_ptr()
+    else:
+        last.c.weight = flat.data_ptr()
+    dc.merge_chain(layers, [], out["weights"], out["bias"], out["packed"], dc.BF16, ws)
+    torch.cuda.synchronize()
+    # two walks of the same fp32 sums: a few units of the last place apart
+    assert O.rel_l2(out["weights"].cpu().numpy(), wm.cpu().numpy()) <= 1e-6 and O.rel_l2(out["bias"].cpu().numpy(), bm.cpu().numpy()) <= 1e-6
+    again = torch.empty_like(packed)
+    dc.pack_weights(out["weights"], g, dc.BF16, again)
+    assert torch.equal(out["packed"], again)
+
+
 def test_a_launch_that_is_refused_is_reported(dc):
     """A 3x3 layer with 65536 outputs after a 1x1 layer needs a grid the device does not have (the runtime refuses the
     launch, nothing runs).  The 1x1 layer after it is composed by the fp32 convolution, whose launch succeeds: the merge
