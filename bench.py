@@ -7,8 +7,9 @@ convolution forward over the batch (dc_conv_forward).  Headline workload: the Mo
 inverted-residual block at 56x56, batch 64, bf16 (1x1 24->144, dw3x3, 1x1 144->24, skip folded ->
 one 3x3 conv 24->24).  The default run also measures the stride-2 merge (cfg2), the cross-block
 merge (cfg3) and the full depth-compressed MobileNetV2-1.0 (cfg4: with every valid span of a seeded
-pattern merged, and cut by Algorithm 1 over the latency table measured on the spot) and reports them
-under `per_config` of the same JSON line.
+pattern merged, and cut by Algorithm 1 over the latency table measured on the spot) and reports their
+main figures under `per_config` of the same JSON line; everything measured about them, the network's table
+of launch groups included, goes to stderr, one JSON line per workload.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload all|cfg1|cfg2|cfg3|cfg4|vgg] [--impl reference]
 
@@ -585,6 +586,13 @@ def chain_entry(cb, figs, e2e_ms, e2e_info, world, cpu):
     return out
 
 
+def brief(entry):
+    """The main figures of a per_config entry: what fits into the headline's line."""
+    fwd = entry["forward_ms"]["median"] * 1e3 if "forward_ms" in entry else entry["conv_forward_us"]["median"]
+    return {"forward_us": round(fwd, 2), "merge_us": round(entry["merge_latency_us"]["median"], 2),
+            "step_us": round(entry["ms_per_step"] * 1e3, 2), "frac": round(entry["roofline"]["frac"], 4)}
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -713,7 +721,12 @@ def run_ours(args):
         args_lat = copy.copy(args)
         args_lat.plan = "latency"
         per["cfg4_latency_plan"] = measure_network(args_lat, peaks, peak_src)[0]
-        out["per_config"] = per
+        for name, entry in per.items():
+            print(json.dumps({"detail": name, **entry}), file=sys.stderr)
+        out["per_config"] = {name: brief(entry) for name, entry in per.items()}
+        roof = {k: v for k, v in out["roofline"].items()
+                if k not in ("nominal", "roofline_us", "us_min", "us_max", "replays", "launches_per_replay")}     # in cfg1's detail
+        out["roofline"] = roof
     print(json.dumps(out))
 
 

@@ -698,13 +698,13 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     const double all = (double)items * bytes / 8000.0;               // what L2 gives all SMs together
     for (int split = 1; split <= kMaxSplit; ++split) {
       // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
-      if (split == 7) continue;
+      if (split == 7) continue;                  // no more clusters of seven than of eight run at once (15 each)
       if (split > 1 && (items * split > n_sm || items > max_clusters(split) || p->planes * (S == 2 ? 4 : g->k) < split ||
                         mb * 128 * (p->n_tile + 4) * 4 > fixed_part))
         break;
       const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
       const double meet = split > 1 ? 450.0 + 580.0 * split + (double)ni * th * tw * p->n_tile * 0.8 : 0.0;
-      const double ctas = (double)(items * split < 148 ? items * split : 148);
+      const double ctas = (double)(items * split < n_sm ? items * split : n_sm);
       const double cost = (m > l ? m + 0.77 * l : l + 0.77 * m) + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + meet;
       if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->ksplit = split; }
     }
@@ -782,9 +782,10 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   }
   p->a_box_bytes = p->ni * p->lines_img * 128;
   p->a_stage_bytes = (int)dc_round_up((size_t)p->a_box_bytes, 1024);
-  // Layout: bias, activation stages, weight stages.  A block's 128 GEMM rows plus the tap shift may
-  // reach up to ~200 lines (25 KB) past its stage; behind the last activation stage that lands in
-  // the weight stages, which are larger (what is read there only feeds rows that are dropped).
+  // Layout: bias, activation stages, weight stages.  The last block's 128 GEMM rows plus the tap shift reach at most 127
+  // lines (16 KB) past its stage, because the patch holds the halo of its last output; behind the last activation stage
+  // that lands in the weight stages or in room kept free for it (what is read there only feeds rows that are dropped).
+  // (26 KB are kept: the constants of the estimate above were fitted with that.)
   // rings: weights first (they are the larger stream), then activation planes
   int sa = 2, sb = 2;
   // Small weights of a single pass stay resident where a work item would otherwise stream more weight than
