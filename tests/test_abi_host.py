@@ -114,13 +114,10 @@ def test_kernel_name_query_follows_the_dispatch_rules():
     assert dc.conv_kernel_name(0, 16, 16, dc.geom(16, 24, 1, 3, 1, 1), dc.BF16) is None
 
 
-@pytest.mark.parametrize("k", [1, 3, 5, 7])
-@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("k,stride", [(1, 1), (3, 1), (5, 1), (7, 1), (3, 2), (5, 2), (7, 2)])
 def test_wide_maps_stay_on_the_tensor_cores(k, stride):
     """Layers whose weights only the rows kernel reads: a column strip that fits is found at every width, also where the
     patch of the widest strip the tensor map allows does not fit beside the weights."""
-    if (k, stride) == (1, 2):
-        pytest.skip("1x1 layers of stride 2 have no tensor-core kernel")
     widths = sorted({7, 12, 13, 63, 255, 256, 257} | {int(7 * 1.07 ** i) for i in range(95)} | set(range(600, 4097, 499)) | {4033, 4096})
     for c_in, c_out in [(16, 160), (40, 48), (64, 64), (72, 200), (64, 128), (128, 128), (64, 256), (256, 256), (512, 512)]:
         if k == 1 and c_in == 16:
@@ -197,3 +194,14 @@ def test_vgg_style_cases_have_the_shapes_of_their_stage():
         assert case.x_shape == (2, hw, hw, c) and case.dtype == "bf16" and case.residuals == []
         assert [(s.c_in, s.c_out, s.k, s.stride, s.pad, s.groups, s.act) for s in case.layers] == [(c, c, 3, 1, 1, 1, None)] * 2
         assert O.compose_geometry(case.layers) == (5, 1, 2)
+
+
+def test_bench_line_holds_main_figures_only():
+    """The headline's per_config entry of a workload: four numbers, from a chain's entry or a network's (whose table of launch
+    groups stays out of the line)."""
+    import bench
+    chain = {"conv_forward_us": {"median": 8.5}, "merge_latency_us": {"median": 6.25}, "ms_per_step": 0.016, "roofline": {"frac": 0.34567}}
+    net = {"forward_ms": {"median": 0.667}, "merge_latency_us": {"median": 128.0}, "ms_per_step": 0.815, "roofline": {"frac": 0.5357},
+           "groups": [{}] * 27}
+    assert bench.brief(chain) == {"forward_us": 8.5, "merge_us": 6.25, "step_us": 16.0, "frac": 0.3457}
+    assert bench.brief(net) == {"forward_us": 667.0, "merge_us": 128.0, "step_us": 815.0, "frac": 0.5357}

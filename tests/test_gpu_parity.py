@@ -492,30 +492,30 @@ def test_single_conv_bf16_with_explicit_skip(dc, c_in, c_out, k, s, p, n, h, w, 
     (16, 24, 3, 2, 0, 2, 17, 36, "k_conv_tc_pairrows"),     # stride 2, no padding, odd height
     (40, 32, 3, 2, 1, 2, 28, 28, "k_conv_tc_rows_s2"),       # stride 2 by sub-tiles (more than 32 channels)
     (96, 144, 5, 2, 2, 1, 56, 56, "k_conv_tc_rows_s2"),      # the widest stride-2 merged layer of the network: several tiles per image
-    (48, 64, 7, 2, 3, 1, 31, 44, "k_conv_tc_rows_s2"),       # 7x7 stride 2, odd height: four even and three odd tap rows
-    (48, 24, 5, 2, 1, 2, 22, 26, "k_conv_tc_rows_s2"),       # 5x5 stride 2 with padding 1: odd tap columns lead
-    (72, 48, 3, 2, 0, 1, 17, 150, "k_conv_tc_rows_s2"),      # stride 2 without padding, two column strips
+    (48, 64, 7, 2, 3, 1, 31, 44, "k_conv_tc_rows_s2"),       # 7x7 stride 2, odd height
+    (48, 24, 5, 2, 1, 2, 22, 26, "k_conv_tc_rows_s2"),       # 5x5 stride 2 with padding 1
+    (72, 48, 3, 2, 0, 1, 17, 150, "k_conv_tc_rows_s2"),      # stride 2 without padding, four column strips
     (32, 16, 1, 1, 0, 2, 20, 24, "k_conv_tc_pairrows"),     # 1x1: one instruction per 32-byte K step
     (32, 96, 1, 1, 0, 2, 20, 24, "k_conv_tc_rows"),         # 1x1 expansion from few channels: one half-filled plane
-    (16, 96, 1, 1, 0, 1, 40, 112, "k_conv_tc_rows"),        # 1x1 expansion from 16 channels, row tiles
-    (32, 192, 3, 1, 1, 2, 28, 28, "k_conv_tc_rows"),        # 3x3 from few channels to more outputs than the pair rows take: two column strips, 110 KB of resident weights
+    (16, 96, 1, 1, 0, 1, 40, 112, "k_conv_tc_rows"),        # 1x1 expansion from 16 channels: one run of pixels, runs cut by blocks
+    (32, 192, 3, 1, 1, 2, 28, 28, "k_conv_tc_rows"),        # 3x3 from few channels to more outputs than the pair rows take: two column strips, two passes
     (16, 136, 5, 1, 2, 1, 12, 20, "k_conv_tc_rows"),        # the same with 16 channels and a 5x5 kernel, two passes
     (32, 40, 1, 1, 0, 2, 20, 24, "k_conv_tc"),              # 1x1 with 40 outputs: general kernel
     (16, 128, 3, 1, 1, 1, 12, 16, "k_conv_tc_pairrows"),    # N = 256: two accumulator slots, run-time channel loop
     (32, 64, 3, 2, 1, 1, 28, 28, "k_conv_tc_pairrows"),     # stride 2, 64 output channels
-    (160, 200, 3, 1, 1, 5, 7, 7, "k_conv_tc_rows"),         # three planes (the last half full), two passes; few images: one per tile
-    (96, 64, 1, 1, 0, 7, 7, 7, "k_conv_tc_rows"),           # 1x1 at 7 x 7, few images: one per tile
-    (96, 64, 1, 1, 0, 733, 7, 7, "k_conv_tc_rows"),         # 1x1, a machine's worth of images: five per tile (147 tiles), the last group of three
+    (160, 200, 3, 1, 1, 5, 7, 7, "k_conv_tc_rows"),         # three planes (the last half full), two passes; few images: one per tile, two strips, the reduction shared by three CTAs
+    (96, 64, 1, 1, 0, 7, 7, 7, "k_conv_tc_rows"),           # 1x1 at 7 x 7, few images: a run of 343 pixels in three tiles
+    (96, 64, 1, 1, 0, 733, 7, 7, "k_conv_tc_rows"),         # 1x1, a run of 35917 pixels: 141 tiles of 256, whatever image they lie in
     (160, 200, 3, 1, 1, 300, 7, 7, "k_conv_tc_rows"),       # 3x3 at 7 x 7 with more items than CTAs: three images per tile, two passes, runs cut by blocks (items shared by two CTAs)
-    (960, 160, 1, 1, 0, 128, 7, 7, "k_conv_tc_rows"),       # deep projection of the network: two images per tile fill the machine (five would leave two thirds idle)
+    (960, 160, 1, 1, 0, 128, 7, 7, "k_conv_tc_rows"),       # deep projection of the network: tiles of 128 pixels, two passes of 80 channels
     (512, 512, 1, 1, 0, 6, 7, 7, "k_conv_tc_rows"),          # deep 1x1 with more than 256 outputs: two passes of 256 channels, one accumulator set
-    (64, 48, 5, 1, 2, 1, 20, 70, "k_conv_tc_rows"),         # 5x5, two column strips, row tiles
-    (384, 64, 3, 1, 1, 2, 14, 14, "k_conv_tc_rows"),        # six planes, whole image per tile
-    (128, 128, 5, 1, 2, 2, 14, 14, "k_conv_tc_rows"),       # 5x5 with 128 outputs: two passes of 64 (weight stage limit)
-    (96, 96, 7, 1, 3, 1, 14, 14, "k_conv_tc_rows"),         # 7x7: passes of at most 80 output channels
-    (144, 32, 3, 1, 1, 1, 28, 28, "k_conv_tc_rows"),        # many channels, 32 outputs: rows kernel with resident weights, two strips of 14 x 14
-    (80, 48, 3, 1, 1, 2, 14, 27, "k_conv_tc_rows"),         # ragged strips (14 + 13 columns), whole height per tile
-    (64, 64, 3, 1, 1, 1, 33, 45, "k_conv_tc_rows"),         # three strips of 15 columns, row tiles of 13, 13 and 7
+    (64, 48, 5, 1, 2, 1, 20, 70, "k_conv_tc_rows"),         # 5x5, tiles of one output row, the reduction shared by three CTAs
+    (384, 64, 3, 1, 1, 2, 14, 14, "k_conv_tc_rows"),        # six planes, the reduction shared by five CTAs
+    (128, 128, 5, 1, 2, 2, 14, 14, "k_conv_tc_rows"),       # 5x5 with 128 outputs in one pass, the reduction shared by six CTAs
+    (96, 96, 7, 1, 3, 1, 14, 14, "k_conv_tc_rows"),         # 7x7: weight stages of one tap column, the reduction shared by eight CTAs
+    (144, 32, 3, 1, 1, 1, 28, 28, "k_conv_tc_rows"),        # many channels, 32 outputs: the reduction shared by three CTAs
+    (80, 48, 3, 1, 1, 2, 14, 27, "k_conv_tc_rows"),         # three strips of nine columns, resident weights
+    (64, 64, 3, 1, 1, 1, 33, 45, "k_conv_tc_rows"),         # five strips of nine columns, row tiles of 11, resident weights
     (200, 24, 3, 1, 1, 2, 14, 14, "k_conv_tc"),             # many channels, fewer than 32 outputs: general kernel
     (192, 32, 1, 1, 0, 2, 28, 28, "k_conv_tc_rows"),        # 1x1 projection to 32 channels
 ])
@@ -640,10 +640,12 @@ def test_bias_that_is_not_finite(dc, c_in, c_out, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
-    (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, several column strips and row tiles
-    (72, 200, 5, 1, 2, 2, 11, 13),       # the same in two passes, a partial plane of channels
+    (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, row tiles, a shared reduction
+    (72, 200, 5, 1, 2, 2, 11, 13),       # 5x5 in two passes, a partial plane of channels, a shared reduction
+    (64, 200, 5, 1, 2, 24, 28, 28),      # weight stages of one tap column, two passes, more items than CTAs, runs cut by blocks
+    (16, 200, 7, 1, 3, 16, 30, 30),      # the same with 7x7
     (40, 48, 7, 1, 3, 1, 16, 40),        # 7x7
-    (64, 64, 3, 1, 1, 2, 9, 120),        # wide rows: a tile of two output rows
+    (64, 64, 3, 1, 1, 2, 9, 120),        # wide rows: strips of 20 columns, whole height
     (64, 64, 3, 1, 1, 40, 5, 5),         # several small images per tile
     (64, 64, 1, 1, 0, 1, 3, 5),          # 1x1: one short run of pixels
     (96, 576, 1, 1, 0, 3, 13, 13),       # 1x1: pixels of several images in a tile, a ragged last tile
@@ -671,7 +673,8 @@ def test_rows_with_a_shared_reduction_against_the_oracle(dc, c_in, c_out, k, s, 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (96, 144, 5, 2, 2, 9, 57, 50),       # several tiles per image and per CTA, odd height
     (96, 144, 5, 2, 2, 1, 20, 20),       # the reduction shared by a cluster
-    (40, 32, 3, 2, 1, 40, 28, 28),       # weights resident
+    (40, 32, 3, 2, 1, 40, 28, 28),       # one image per tile, runs cut by blocks
+    (40, 48, 3, 2, 1, 160, 21, 21),      # weights resident, more items than CTAs
     (48, 64, 7, 2, 3, 2, 31, 44),        # 7x7: classes of 16, 12, 12 and 9 taps
     (72, 200, 3, 2, 0, 1, 17, 150),      # no padding, column strips, a partial last plane
     (64, 264, 3, 2, 1, 2, 21, 19),       # two passes
