@@ -31,6 +31,8 @@ COUNTERS = [
     ("gpu__dram_throughput.avg.pct_of_peak_sustained_elapsed", "DRAM throughput, % of peak"),
     ("lts__t_sector_hit_rate.pct", "L2 sector hit rate, %"),
     ("sm__pipe_tensor_cycles_active.avg.pct_of_peak_sustained_elapsed", "tensor pipe active, % of elapsed"),
+    ("sm__inst_executed_pipe_fma.avg.pct_of_peak_sustained_active", "FMA pipe, % of peak"),
+    ("smsp__issue_active.avg.pct_of_peak_sustained_active", "issue slots taken, %"),
     ("sm__inst_executed.avg.per_cycle_elapsed", "warp instructions per cycle per SM"),
     ("smsp__inst_executed.sum", "warp instructions executed"),
     ("sm__warps_active.avg.per_cycle_active", "warps resident per SM (avg)"),
@@ -46,6 +48,7 @@ COUNTERS = [
     ("smsp__average_warps_issue_stalled_no_instruction_per_issue_active.ratio", "stall: no instruction"),
     ("smsp__average_warps_issue_stalled_math_pipe_throttle_per_issue_active.ratio", "stall: math pipe throttle"),
     ("smsp__average_warps_issue_stalled_lg_throttle_per_issue_active.ratio", "stall: LSU queue (lg throttle)"),
+    ("smsp__average_warps_issue_stalled_dispatch_stall_per_issue_active.ratio", "stall: dispatch"),
 ]
 
 UNIT_BYTES = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}
