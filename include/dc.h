@@ -132,12 +132,16 @@ dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual
 
 /*
  * How dc_merge_chain walks a run.  DC_MERGE_STEPS: fold every layer, then compose the pieces
- * pairwise (one launch per step).  DC_MERGE_AUTO (what dc_merge_chain uses): as above, except
- * that every inverted-residual block inside the run -- dense 1x1 with stride 1, depthwise k x k,
- * dense 1x1 with stride 1, either a whole skip group or outside any -- is merged in one launch
- * straight from the raw layers (BN folded on the fly, the 6x wider intermediate kernel never
- * written): W'[o,i,t] = sum_c W3~[o,c] D~[c,t] W1~[c,i], which is Eq. 1 applied twice.  Both
- * forms evaluate the same formula in fp32; they differ in rounding order only.
+ * pairwise and deliver (a launch per step; the last composition of two 3x3 kernels delivers itself).
+ * DC_MERGE_AUTO (what dc_merge_chain uses): as above, except that runs and parts of runs of these
+ * kinds are merged straight from the raw layers, BN folded on the fly, in one launch:
+ *   - an inverted-residual block -- dense 1x1 with stride 1, depthwise k x k, dense 1x1 with
+ *     stride 1, either a whole skip group or outside any; the 6x wider intermediate kernel is never
+ *     written: W'[o,i,t] = sum_c W3~[o,c] D~[c,t] W1~[c,i], which is Eq. 1 applied twice;
+ *   - a run of two dense 3x3 layers, the first with stride 1;
+ *   - a run of a dense 1x1 layer and a 3x3 depthwise one, in either order.
+ * Where such a part with a 3x3 kernel is the whole run, the same launch writes the result and the packed copy.
+ * Both forms evaluate the same formula in fp32; they differ in rounding order only.
  */
 typedef enum { DC_MERGE_AUTO = 0, DC_MERGE_STEPS = 1 } dc_merge_algo;
 

@@ -12,14 +12,14 @@
 //  * slices of 16 K are staged by cp.async several deep in 16-byte pieces, straight from the feature
 //    map (zero filled outside it) and the weights.  With 4-byte pieces (weights turned to [channel][K],
 //    so that packed FMAs could take pairs of K) the copies cost as many shared-memory cycles as the
-//    reads: 30 instead of 38 TFLOP/s with the chip full;
+//    reads: 30 instead of 38 TFLOP/s with the chip full and the best tile;
 //  * TN follows the output channels (16 to 64 per tile), so that 24 or 40 of them do not run as 32 or 64;
 //  * K is split over a cluster of up to eight CTAs where the tiles alone would leave SMs idle (one
 //    image of a deep layer): the partial tiles meet in distributed shared memory and are added in rank
 //    order, so the result does not depend on timing.
 //
 // Before, with four outputs per thread and both operands from L1: 32 -> 32, 5x5, 32 images of 28 x 28
-// 162 us, here 46 (28 TFLOP/s; 38 on 256 images, where the tiles fill the SMs evenly); 160 -> 160, 3x3, one
+// 162 us, here 46 (28 TFLOP/s; 33 on 256 images with the plan below, 38 with the best one); 160 -> 160, 3x3, one
 // 7 x 7 image 255, here 7.8; 960 -> 160, 1x1, the same image 175, here 5.8.
 #include <cooperative_groups.h>
 
@@ -300,7 +300,8 @@ bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *pl) {
   // Least estimated time, in cycles of the SM with the most CTAs.  Per slice an SM needs the FMAs of its CTAs (16 x
   // TM x TN cycles of a CTA at full rate) but never less than a slice's own chain; a round of resident CTAs costs a
   // start-up, a cluster its meeting.  The constants are fitted to 15 layers (one pixel tile to eight rounds of them)
-  // timed in every configuration and split: the choice is on average within a tenth of the best.
+  // timed in every configuration and split.  Timed again on 15 layers: the choice is 10 % above the
+  // best on average, 43 % at worst (24 -> 32 3x3 of stride 2, 16 images of 56 x 56).
   int best_config = -1, best_split = 0;
   double best = 0.0;
   for (int cfg = 0; cfg < (int)(sizeof(kF32Configs) / sizeof(kF32Configs[0])); ++cfg)

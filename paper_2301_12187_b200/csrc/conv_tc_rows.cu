@@ -673,7 +673,8 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   // its tensor-core instructions (a 128 x N x 16 takes max(36 + N/4, N/2)) and the bytes it takes in from L2, which
   // overlap in part, and a chain of waits; a shared item costs the meeting of its partial sums, which grows with the
   // CTAs and the bytes.  The constants are fitted to 41 layers timed in every tile and split considered here (1 to 128
-  // images of 49 to 12544 pixels): the choice is within 2.5 % of the best on average, 19 % at worst.
+  // images of 49 to 12544 pixels).  Timed again on 32 layers: the choice is 2 % above the best on
+  // average, 21 % at worst (160 -> 96 3x3 of stride 2, 64 images of 14 x 14).
   // Candidates: every strip count that leaves rows of at most 256 pixels, with as many rows as give two blocks or
   // one, evened out over the height; whole small images several at a time.
   const int cyc = 36 + p->n_tile / 4 > p->n_tile / 2 ? 36 + p->n_tile / 4 : p->n_tile / 2;
