@@ -667,7 +667,10 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   p->off_a = rows_fixed_bytes(ko, &p->off_stage);
   // A tile's GEMM rows are the patch pixels from its first to its last output, halo columns included: at most two
   // 128-row blocks.  Its patch (rows and halo) must fit the activation ring twice beside three weight stages.
-  const long long tap_bytes = 8ll * p->n_tile * 16;        // weights of one tap column of a (plane, tap row) step
+  // weights of one tap column of a (plane, tap row) step: two chunk planes for each 16 channels of the widest plane.
+  // (Counted as eight for every plane, the steps of 16 to 48 channels seemed not to fit and ran by tap columns of one to
+  // three instructions: 32 -> 224 5x5, 10 images of 23 x 23 10.8 us, now 6.8.)
+  const long long tap_bytes = (g->c_in >= 64 ? 8ll : 2ll * dc_div_up(g->c_in, 16)) * p->n_tile * 16;
   const long long max_a = (kSmemBudget - 1024 - p->off_a - kSlack - (3 * tap_bytes > 26 * 1024 ? 3 * tap_bytes : 26 * 1024)) / 2;
   // Tile and split of the reduction: the least estimated time of the CTA with the most work, in cycles.  An item costs
   // its tensor-core instructions (a 128 x N x 16 takes max(36 + N/4, N/2)) and the bytes it takes in from L2, which

@@ -656,7 +656,8 @@ def test_bias_that_is_not_finite(dc, c_in, c_out, k, s, p, n, h, w):
     (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, row tiles, a shared reduction
     (72, 200, 5, 1, 2, 2, 11, 13),       # 5x5 in two passes, a partial plane of channels, a shared reduction
     (64, 200, 5, 1, 2, 24, 28, 28),      # weight stages of one tap column, two passes, more items than CTAs, runs cut by blocks
-    (16, 200, 7, 1, 3, 16, 30, 30),      # the same with 7x7
+    (16, 200, 7, 1, 3, 16, 30, 30),      # 16 channels, 7x7: whole steps of a quarter of a full plane's weights
+    (48, 136, 7, 1, 3, 4, 26, 31),       # 48 channels, 7x7: tap columns of three instructions
     (40, 48, 7, 1, 3, 1, 16, 40),        # 7x7
     (64, 64, 3, 1, 1, 2, 9, 120),        # wide rows: strips of 20 columns, whole height
     (64, 64, 3, 1, 1, 40, 5, 5),         # several small images per tile
