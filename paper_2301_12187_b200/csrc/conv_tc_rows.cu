@@ -700,6 +700,13 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     const double mma = 1.7 * (double)(blocks < per_cta * mb ? blocks : per_cta * mb) * per_block;
     const double bytes = (double)ni * lines * 128 * p->planes * subs + w_item;
     const double all = (double)items * bytes / 8000.0;               // what L2 gives all SMs together
+    // Where a whole step does not fit twice beside two planes the weights come by tap columns, each with a wait of its own
+    // behind a handful of instructions: 150 cycles a column.  Of 1500 random 3x3, 5x5 and 7x7 layers 33 became 1.06 to 1.5
+    // times as fast (72 -> 64 7x7, 29 images of 28 x 55: 51.3 -> 34.4 us), three 1.08 times slower.  Not at stride 2, whose
+    // steps are short and where five became slower (176 -> 104 7x7, 6 images of 76 x 76: 24.5 -> 30.9 us) and none faster.
+    const long long whole = (long long)dc_round_up((size_t)(g->k * tap_bytes), 1024);
+    const bool columns = S == 1 && g->k > 1 && 2048 + p->off_a + 2 * whole + 2 * (long long)dc_round_up((size_t)ni * lines * 128, 1024) > kSmemBudget;
+    const double waits = columns ? 150.0 * (double)per_cta * p->planes * g->k * g->k : 0.0;
     for (int split = 1; split <= kMaxSplit; ++split) {
       // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
       if (split == 7) continue;                  // no more clusters of seven than of eight run at once (15 each)
@@ -709,7 +716,7 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
       const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
       const double meet = split > 1 ? 450.0 + 580.0 * split + (double)ni * th * tw * p->n_tile * 0.8 : 0.0;
       const double ctas = (double)(items * split < n_sm ? items * split : n_sm);
-      const double cost = (m > l ? m + 0.77 * l : l + 0.77 * m) + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + meet;
+      const double cost = (m > l ? m + 0.77 * l : l + 0.77 * m) + waits / split + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + meet;
       if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->ksplit = split; }
     }
   };

@@ -597,7 +597,7 @@ BIAS_CASES = [
     (24, 32, 3, 2, 1, 2, 13, 11),        # pair rows, stride 2
     (144, 32, 3, 1, 1, 8, 28, 28),       # rows, resident weights
     (384, 64, 3, 1, 1, 1, 14, 14),       # rows, a shared reduction
-    (128, 128, 5, 1, 2, 4, 30, 33),      # rows, weight stages of one tap column
+    (128, 128, 5, 1, 2, 4, 30, 33),      # rows, 128 outputs of a 5x5 kernel
     (40, 32, 3, 2, 1, 2, 28, 29),        # rows, stride 2
     (48, 24, 3, 1, 1, 1, 20, 20),        # fold
     (200, 24, 3, 1, 1, 1, 14, 14),       # general
@@ -653,11 +653,13 @@ def test_bias_that_is_not_finite(dc, c_in, c_out, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
-    (128, 128, 5, 1, 2, 4, 30, 33),      # weight stages of one tap column, row tiles, a shared reduction
+    (128, 128, 5, 1, 2, 4, 30, 33),      # narrow strips whose whole steps fit, a shared reduction
     (72, 200, 5, 1, 2, 2, 11, 13),       # 5x5 in two passes, a partial plane of channels, a shared reduction
-    (64, 200, 5, 1, 2, 24, 28, 28),      # weight stages of one tap column, two passes, more items than CTAs, runs cut by blocks
+    (64, 200, 5, 1, 2, 24, 28, 28),      # two passes, more items than CTAs
     (16, 200, 7, 1, 3, 16, 30, 30),      # 16 channels, 7x7: whole steps of a quarter of a full plane's weights
-    (48, 136, 7, 1, 3, 4, 26, 31),       # 48 channels, 7x7: tap columns of three instructions
+    (72, 128, 5, 1, 2, 12, 50, 50),      # weight stages of one tap column, more items than CTAs
+    (128, 256, 5, 1, 2, 6, 28, 28),      # the same in two passes, a shared reduction
+    (48, 136, 7, 1, 3, 4, 26, 31),       # 48 channels, 7x7: two passes, runs cut by blocks
     (40, 48, 7, 1, 3, 1, 16, 40),        # 7x7
     (64, 64, 3, 1, 1, 2, 9, 120),        # wide rows: strips of 20 columns, whole height
     (64, 64, 3, 1, 1, 40, 5, 5),         # several small images per tile
