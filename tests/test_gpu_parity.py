@@ -675,6 +675,18 @@ def test_rows_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (160, 136, 3, 1, 1, 131, 7, 7),      # two or four images per tile, a ragged last group
+    (64, 64, 5, 1, 2, 150, 5, 5),        # halo of two columns and rows
+    (72, 48, 7, 1, 3, 151, 4, 6),        # halo of three: as wide as half a map
+    (48, 144, 3, 1, 1, 153, 1, 3),       # one-row maps: every row between two images is halo
+    (64, 64, 3, 1, 2, 150, 6, 6),        # padding that is not half the kernel: nothing is shared
+    (96, 64, 3, 1, 1, 40, 28, 28),       # whole rows of one image: halo columns only
+])
+def test_rows_with_shared_halos_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (384, 64, 3, 1, 1, 1, 14, 14),       # one item for the chip: its 18 steps over a cluster of eight
     (960, 160, 1, 1, 0, 1, 7, 7),        # 1x1: 15 planes over a cluster
     (576, 200, 3, 1, 1, 2, 13, 9),       # several items, two passes, a ragged map
