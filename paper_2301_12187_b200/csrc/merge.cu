@@ -676,16 +676,23 @@ __global__ void __launch_bounds__(kBlockThreads) k_merge_block(const __grid_cons
 // result, the chunks of the packed copy that hold no weight are zeroed.
 //
 // Before, with one CTA per output channel that read every operand, then a delivery launch: 24 -> 144 -> 24
-// 9.4 us, 64 -> 384 -> 64 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  Here 6.5, 9.0 and 26.4 us (19 fp32
-// TFLOP/s: 200 tiles on 148 SMs, so a quarter of the SMs do two).
+// 9.4 us, 64 -> 384 -> 64 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  With eight warps 6.5, 9.0 and 25.9 us (200 tiles
+// of 8 x 16 on 148 SMs: 52 of them had two, the others eight warps with no second tile to hide their latency); by sixteen warps in 140 tiles of 8 x 24 20.7
+// us, 120 -> 720 -> 120 (120 tiles) 19.0 -> 12.9, 88 -> 528 -> 88 15.0 -> 11.3.  Halved runs of the sums are nearer to 64 bits as well
+// (160 channels: 1.6e-7 -> 1.35e-7).
 // ----------------------------------------------------------------------------------------------
-constexpr int kMbO = 8, kMbI = 16, kMbWarps = 8, kMbSlice = 16, kMbStages = 4;
-constexpr int kMbThreads = kMbWarps * 32;
-constexpr int kMbW1 = kMbSlice * kMbI, kMbW3 = kMbO * kMbSlice, kMbD = kMbSlice * 9;   // floats of a slice's operands
-constexpr int kMbStage = kMbW1 + kMbW3 + kMbD;
-constexpr int kMbTile = kMbO * kMbI * 9;                          // sums of a CTA
-constexpr int kMbRing = kMbWarps * kMbStages * kMbStage * 4;      // bytes of the operand rings
-static_assert(kMbRing >= kMbWarps * kMbTile * 4, "the warps' sums reuse the rings");
+constexpr int kMbO = 8, kMbI = 16, kMbSlice = 16, kMbStages = 4;
+constexpr int kMbThreads = 256;
+constexpr int kMbTile = kMbO * kMbI * 9;                          // sums of a CTA of 8 x 16 pairs
+// A form of the kernel: IT input channels of a tile, W warps that share the hidden channels.
+template <int IT, int W>
+struct MbForm {
+  static constexpr int W1 = kMbSlice * IT, W3 = kMbO * kMbSlice, D = kMbSlice * 9;   // floats of a slice's operands
+  static constexpr int STAGE = W1 + W3 + D, TILE = kMbO * IT * 9;
+  static constexpr int RING = W * kMbStages * STAGE * 4;                             // bytes of the operand rings
+  static_assert(RING >= W * TILE * 4, "the warps' sums reuse the rings");
+};
+constexpr int kMbRing = MbForm<kMbI, 8>::RING;                    // the smallest form's
 
 struct TiledBlocks {
   BlockArgs blk[kBlockBatch];
@@ -762,8 +769,11 @@ __device__ __forceinline__ void zero_dead_chunks(const BlockDelivery &dv, int c_
     if (!packed_chunk_live(dv.ko, e, c_out)) reinterpret_cast<uint4 *>(dv.packed)[e] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-__global__ void __launch_bounds__(kMbThreads, 2)
+template <int IT, int W>
+__global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1)
 k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ BlockDelivery dv) {
+  using F = MbForm<IT, W>;
+  constexpr int NI = IT / 8;                       // input channels of a thread
   extern __shared__ __align__(16) float mb_smem[];
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   dc_pdl_enter();
@@ -775,13 +785,13 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
   while ((int)blockIdx.x >= tb.first[bi + 1]) ++bi;
   const BlockArgs &a = tb.blk[bi];
   const int c0 = a.c0, c1 = a.c1, c2 = a.c2;
-  const int gi = dc_div_up(c0, kMbI), go = dc_div_up(c2, kMbO);
+  const int gi = dc_div_up(c0, IT), go = dc_div_up(c2, kMbO);
   const int blk = (int)blockIdx.x - tb.first[bi];
   if (blk >= gi * go) {
     // ---- bias of 8 output channels: q[c] = b2~ + (sum of D~) b1~, then one dot product per warp
     const int o = (blk - gi * go) * kMbO + warp;
     float *q = mb_smem;                            // the host keeps c1 within the rings
-    for (int c = tid; c < c1; c += kMbThreads) {
+    for (int c = tid; c < c1; c += W * 32) {
       const float g1 = raw_scale(a.l1, c), g2 = raw_scale(a.l2, c);
       float dsum = 0.f;
 #pragma unroll
@@ -789,7 +799,7 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
       q[c] = fmaf(dsum, raw_bias(a.l1, c, g1), raw_bias(a.l2, c, g2));
     }
     __syncthreads();
-    if (o < c2) {
+    if (warp < kMbO && o < c2) {
       const float g3 = raw_scale(a.l3, o);
       float s = 0.f;
 #pragma unroll 4
@@ -800,31 +810,31 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
     return;
   }
   // ---- 8 x 16 pairs
-  const int o0 = (blk / gi) * kMbO, i0 = (blk % gi) * kMbI;
-  const int per = ((c1 + kMbWarps - 1) / kMbWarps + 3) & ~3;       // hidden channels of a warp
+  const int o0 = (blk / gi) * kMbO, i0 = (blk % gi) * IT;
+  const int per = ((c1 + W - 1) / W + 3) & ~3;       // hidden channels of a warp
   const int cb = warp * per, ce = cb + per < c1 ? cb + per : c1;
   const int nsl = ce > cb ? (ce - cb + kMbSlice - 1) / kMbSlice : 0;
-  float *ring = mb_smem + warp * (kMbStages * kMbStage);
+  float *ring = mb_smem + warp * (kMbStages * F::STAGE);
   auto fetch = [&](int sl, int buf) {
-    float *st = ring + buf * kMbStage;
+    float *st = ring + buf * F::STAGE;
     const int c = cb + sl * kMbSlice;
-    // W1[c..c+15][i0..i0+15]: 64 pieces; W3[o0..o0+7][c..c+15]: 32; D[c..c+15][9]: 36 (channels and c1 are multiples of 4)
+    // W1[c..c+15][i0..i0+IT-1]: 64 or 96 pieces; W3[o0..o0+7][c..c+15]: 32; D[c..c+15][9]: 36 (channels and c1 are multiples of 4)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int e = lane + 32 * h, r = e >> 2, ii = i0 + (e & 3) * 4;
+    for (int h = 0; h < NI; ++h) {
+      const int e = lane + 32 * h, r = e / (IT / 4), ii = i0 + (e % (IT / 4)) * 4;
       const bool ok = c + r < ce && ii < c0;
       mb_cp16(st + e * 4, ok ? a.l1.w + (size_t)(c + r) * c0 + ii : a.l1.w, ok);
     }
     {
       const int o = o0 + (lane >> 2), cc = c + (lane & 3) * 4;
       const bool ok = o < c2 && cc < ce;
-      mb_cp16(st + kMbW1 + lane * 4, ok ? a.l3.w + (size_t)o * c1 + cc : a.l3.w, ok);
+      mb_cp16(st + F::W1 + lane * 4, ok ? a.l3.w + (size_t)o * c1 + cc : a.l3.w, ok);
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int e = lane + 32 * h;
       const bool ok = e * 4 < (ce - c) * 9;
-      if (e < kMbD / 4) mb_cp16(st + kMbW1 + kMbW3 + e * 4, ok ? a.l2.w + (size_t)c * 9 + e * 4 : a.l2.w, ok);
+      if (e < F::D / 4) mb_cp16(st + F::W1 + F::W3 + e * 4, ok ? a.l2.w + (size_t)c * 9 + e * 4 : a.l2.w, ok);
     }
   };
 #pragma unroll
@@ -832,8 +842,8 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
     if (sl < nsl) fetch(sl, sl);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  const int ol = (lane >> 3) * 2, il = (lane & 7) * 2;             // this thread's pairs: o0 + ol + {0, 1}, i0 + il + {0, 1}
-  float acc[2][2][9] = {};
+  const int ol = (lane >> 3) * 2, il = (lane & 7) * NI;            // this thread's pairs: o0 + ol + {0, 1}, i0 + il + {0 .. NI - 1}
+  float acc[2][NI][9] = {};
   int buf = 0, fbuf = kMbStages - 1;
   // BN scales of a slice's channels: lane l holds channel l & 15's.  Their operands are asked for a slice ahead and
   // first touched behind the slice's arithmetic.
@@ -855,28 +865,33 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
     __syncwarp();
     if (sl + kMbStages - 1 < nsl) fetch(sl + kMbStages - 1, fbuf);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const float *st = ring + buf * kMbStage;
+    const float *st = ring + buf * F::STAGE;
     auto four = [&](int q) {                       // channels q .. q + 3 of the slice
       float w3[2][4], d[36];
 #pragma unroll
       for (int h = 0; h < 2; ++h)
-        *reinterpret_cast<float4 *>(w3[h]) = *reinterpret_cast<const float4 *>(st + kMbW1 + (ol + h) * kMbSlice + q);
+        *reinterpret_cast<float4 *>(w3[h]) = *reinterpret_cast<const float4 *>(st + F::W1 + (ol + h) * kMbSlice + q);
 #pragma unroll
       for (int e = 0; e < 9; ++e)
-        *reinterpret_cast<float4 *>(d + 4 * e) = *reinterpret_cast<const float4 *>(st + kMbW1 + kMbW3 + q * 9 + 4 * e);
+        *reinterpret_cast<float4 *>(d + 4 * e) = *reinterpret_cast<const float4 *>(st + F::W1 + F::W3 + q * 9 + 4 * e);
 #pragma unroll
       for (int cl = 0; cl < 4; ++cl) {
         const float s = __shfl_sync(0xffffffffu, sc, q + cl);
-        const float2 w1 = *reinterpret_cast<const float2 *>(st + (q + cl) * kMbI + il);
+        float w1[NI];
+        if (NI == 2) *reinterpret_cast<float2 *>(w1) = *reinterpret_cast<const float2 *>(st + (q + cl) * IT + il);
+        else
+#pragma unroll
+          for (int v = 0; v < NI; ++v) w1[v] = st[(q + cl) * IT + il + v];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float ws = w3[h][cl] * s;
-          const float p0 = ws * w1.x, p1 = ws * w1.y;
+          float pr[NI];
 #pragma unroll
-          for (int t = 0; t < 9; ++t) {
-            acc[h][0][t] = fmaf(p0, d[cl * 9 + t], acc[h][0][t]);
-            acc[h][1][t] = fmaf(p1, d[cl * 9 + t], acc[h][1][t]);
-          }
+          for (int v = 0; v < NI; ++v) pr[v] = ws * w1[v];
+#pragma unroll
+          for (int t = 0; t < 9; ++t)
+#pragma unroll
+            for (int v = 0; v < NI; ++v) acc[h][v][t] = fmaf(pr[v], d[cl * 9 + t], acc[h][v][t]);
         }
       }
     };
@@ -899,16 +914,16 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
 #pragma unroll
   for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int v = 0; v < 2; ++v)
+    for (int v = 0; v < NI; ++v)
 #pragma unroll
-      for (int t = 0; t < 9; ++t) mb_smem[warp * kMbTile + ((ol + h) * kMbI + il + v) * 9 + t] = acc[h][v][t];
+      for (int t = 0; t < 9; ++t) mb_smem[warp * F::TILE + ((ol + h) * IT + il + v) * 9 + t] = acc[h][v][t];
   __syncthreads();
   const bool last = dv.mode >= 0;
-  for (int e = tid; e < kMbTile; e += kMbThreads) {
+  for (int e = tid; e < F::TILE; e += W * 32) {
     float s = 0.f;
 #pragma unroll
-    for (int w = 0; w < kMbWarps; ++w) s += mb_smem[w * kMbTile + e];
-    const int oi = e / 9, t = e - oi * 9, o = o0 + oi / kMbI, i = i0 + oi % kMbI;
+    for (int w = 0; w < W; ++w) s += mb_smem[w * F::TILE + e];
+    const int oi = e / 9, t = e - oi * 9, o = o0 + oi / IT, i = i0 + oi % IT;
     if (o < c2 && i < c0) {
       s *= raw_scale(a.l3, o);
       if (last && dv.ident && o == i && t == 4) s += 1.f;
@@ -918,7 +933,7 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
   }
   if (!last || dv.mode == 0) return;
   __syncthreads();
-  deliver_tile<kMbO, kMbI, 3>(dv, mb_smem, o0, i0, c0, c2, tid, kMbThreads);
+  deliver_tile<kMbO, IT, 3>(dv, mb_smem, o0, i0, c0, c2, tid, W * 32);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -1182,6 +1197,263 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
   deliver_tile<kMbO, kMbI, 3>(dv, out, o0, i0, c0, c2, tid, kMbThreads);
 }
 
+// ----------------------------------------------------------------------------------------------
+// Two dense 1x1 layers as a run of their own: W' = (g2 W2 + I2) (g1 W1 + I1), a plain matrix product [c2][c1] x [c1][c0], from
+// the layers as they are to the delivered result in one launch.
+//
+// A CTA owns BO x BI results; its 256 threads are G groups that take the 16-channel slices of the reduction in turn, each
+// with operands of its own in shared memory (double buffered through registers, where W2 is turned to [channel][output] and
+// W1 gets its BN scale) and a barrier of its own; a thread owns TO x 4 results, TO / 4 + 1 16-byte reads for 4 TO FMAs.  The
+// groups' sums meet in shared memory in group order.  Tiles of 64 or 48 x 64 where they give the chip enough of them,
+// otherwise 32 x 32 by four groups, whose reductions are shorter chains.  Blocks behind the tiles compute the bias (a warp per
+// output) and zero the packed chunks without weights.
+//
+// As fold, product, bias and delivery, four launches with the product written and read in between: 960 -> 320 -> 1280 60.7 us,
+// now 37.8; 32 -> 16 -> 96 7.5, now 4.1; 160 -> 160 -> 160 15.0, now 6.0.
+// ----------------------------------------------------------------------------------------------
+struct Merge11 {
+  RawLayer l1, l2;
+  int ident1, ident2;            // identity kernels riding on the layers
+  int c0, c1, c2;
+  float *w_out, *b_out;
+  int gi, go;
+};
+
+template <int BO, int BI, int TO, int G>
+__global__ void __launch_bounds__(256, 3)
+k_merge_11(const __grid_constant__ Merge11 a, const __grid_constant__ BlockDelivery dv) {
+  constexpr int VA = TO % 4 == 0 ? 4 : 2;          // channels of W2 per read
+  constexpr int T = 256 / G, KS = 16, PA = BO + 4, PB = BI + 4, STAGE = KS * (PA + PB);
+  constexpr int PIECES = BO * KS / 4, NA = (PIECES + T - 1) / T, NB = BI * KS / 4 / T;     // 16-byte pieces a thread stages
+  static_assert(T == (BO / TO) * (BI / 4) && NA >= 1 && NB >= 1 && G * 2 * STAGE >= G * BO * BI / 2, "tile");
+  __shared__ __align__(16) float sm[G * 2 * STAGE < G * BO * BI ? G * BO * BI : G * 2 * STAGE];
+  const int tid = (int)threadIdx.x, lane = tid & 31, g = tid / T, t = tid % T;
+  const int c0 = a.c0, c1 = a.c1, c2 = a.c2;
+  int blk = (int)blockIdx.x;
+  dc_pdl_enter();
+  if (blk >= a.gi * a.go) {
+    blk -= a.gi * a.go;
+    const int nb = dc_div_up(c2, 8);
+    if (blk >= nb) {
+      zero_dead_chunks(dv, c2, blk - nb, (int)gridDim.x - a.gi * a.go - nb);
+      return;
+    }
+    const int o = blk * 8 + (tid >> 5);            // b2~ + sum_c (g2 W2[o][c] + I2) b1~[c]
+    if (o >= c2) return;
+    const float g2 = raw_scale(a.l2, o);
+    float s = 0.f;
+#pragma unroll 4
+    for (int c = lane; c < c1; c += 32)
+      s = fmaf(fmaf(g2, a.l2.w[(size_t)o * c1 + c], a.ident2 && c == o ? 1.f : 0.f), raw_bias(a.l1, c, raw_scale(a.l1, c)), s);
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if (lane == 0) a.b_out[o] = raw_bias(a.l2, o, g2) + s;
+    return;
+  }
+  const int o0 = (blk / a.gi) * BO, i0 = (blk % a.gi) * BI;
+  float *mine = sm + g * 2 * STAGE;
+  const int slices = (c1 + KS - 1) / KS, my = (slices - g + G - 1) / G;      // slices g, g + G, ...
+  float4 va[NA], vb[NB];
+  float gm[NB], vr[NB];                            // BN of W1's channels; first touched when staged, like the weights
+  auto fetch = [&](int sl) {                       // out-of-range pieces read element 0 and are zeroed when staged
+    const int cs = (g + sl * G) * KS;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = t + q * T, o = o0 + e / 4, c = cs + (e & 3) * 4;
+      va[q] = *reinterpret_cast<const float4 *>(a.l2.w + (e < PIECES && o < c2 && c < c1 ? (size_t)o * c1 + c : 0));
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = t + q * T, c = cs + e / (BI / 4), i = i0 + (e % (BI / 4)) * 4;
+      const bool ok = c < c1 && i < c0;
+      vb[q] = *reinterpret_cast<const float4 *>(a.l1.w + (ok ? (size_t)c * c0 + i : 0));
+      gm[q] = a.l1.gamma ? a.l1.gamma[ok ? c : 0] : 1.f;
+      vr[q] = a.l1.gamma ? a.l1.var[ok ? c : 0] : 1.f;
+    }
+  };
+  auto stage = [&](int sl, int buf) {
+    float *A = mine + buf * STAGE, *B = A + KS * PA;
+    const int cs = (g + sl * G) * KS;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int e = t + q * T, o = o0 + e / 4, c = (e & 3) * 4;
+      const bool ok = o < c2 && cs + c < c1;
+      if (e >= PIECES) continue;
+      A[(c + 0) * PA + e / 4] = ok ? va[q].x : 0.f;
+      A[(c + 1) * PA + e / 4] = ok ? va[q].y : 0.f;
+      A[(c + 2) * PA + e / 4] = ok ? va[q].z : 0.f;
+      A[(c + 3) * PA + e / 4] = ok ? va[q].w : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int e = t + q * T, c = cs + e / (BI / 4), i = i0 + (e % (BI / 4)) * 4;
+      const bool ok = c < c1 && i < c0;
+      const float sc = a.l1.gamma ? gm[q] / sqrtf(vr[q] + a.l1.eps) : 1.f;
+      *reinterpret_cast<float4 *>(B + (e / (BI / 4)) * PB + (e % (BI / 4)) * 4) =
+          ok ? make_float4(vb[q].x * sc, vb[q].y * sc, vb[q].z * sc, vb[q].w * sc) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  const int ty = t / (BI / 4), tx = t % (BI / 4);
+  float acc[TO][4] = {};
+  if (my > 0) { fetch(0); stage(0, 0); }
+  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(T) : "memory");
+#pragma unroll 1
+  for (int sl = 0; sl < my; ++sl) {
+    if (sl + 1 < my) fetch(sl + 1);
+    const float *A = mine + (sl & 1) * STAGE + ty * TO, *B = mine + (sl & 1) * STAGE + KS * PA + tx * 4;
+#pragma unroll
+    for (int k = 0; k < KS; ++k) {
+      float x[TO];
+#pragma unroll
+      for (int q = 0; q < TO; q += VA) {
+        if (VA == 4) *reinterpret_cast<float4 *>(x + q) = *reinterpret_cast<const float4 *>(A + k * PA + q);
+        else *reinterpret_cast<float2 *>(x + q) = *reinterpret_cast<const float2 *>(A + k * PA + q);
+      }
+      const float4 b = *reinterpret_cast<const float4 *>(B + k * PB);
+#pragma unroll
+      for (int q = 0; q < TO; ++q) {
+        acc[q][0] = fmaf(x[q], b.x, acc[q][0]);
+        acc[q][1] = fmaf(x[q], b.y, acc[q][1]);
+        acc[q][2] = fmaf(x[q], b.z, acc[q][2]);
+        acc[q][3] = fmaf(x[q], b.w, acc[q][3]);
+      }
+    }
+    if (sl + 1 < my) stage(sl + 1, (sl + 1) & 1);
+    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(T) : "memory");
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < TO; ++q)
+    *reinterpret_cast<float4 *>(sm + (g * BO + ty * TO + q) * BI + tx * 4) = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+  __syncthreads();
+  for (int e = tid; e < BO * BI; e += 256) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < G; ++q) s += sm[q * BO * BI + e];
+    const int o = o0 + e / BI, i = i0 + e % BI;
+    if (o < c2 && i < c0) {
+      const float g2 = raw_scale(a.l2, o);
+      s *= g2;
+      if (a.ident1) s = fmaf(g2, a.l2.w[(size_t)o * c1 + i], s);                        // g2 W2 I1: c0 == c1
+      if (a.ident2) s = fmaf(raw_scale(a.l1, o), a.l1.w[(size_t)o * c0 + i], s);        // I2 g1 W1: c1 == c2
+      if (o == i) s += (a.ident1 && a.ident2 ? 1.f : 0.f) + (dv.ident ? 1.f : 0.f);
+      a.w_out[(size_t)o * c0 + i] = s;
+    }
+    sm[e] = s;                                     // element e of group 0's sums is read by this thread alone
+  }
+  if (dv.mode == 0) return;
+  __syncthreads();
+  deliver_tile<BO, BI, 1>(dv, sm, o0, i0, c0, c2, tid, 256);
+}
+
+// ----------------------------------------------------------------------------------------------
+// A dense 3x3 piece after a dense 1x1 one with stride 1: every tap sum has one term,
+//   W'[o][i][t] = sum_c (W2[o][c][t] + I2) (W1[c][i] + I1),
+// a product of [o, t][c] with [c][i].  A CTA owns 8 output channels x nine taps x 32 input channels; a thread the taps of one
+// output channel for four of the input channels (nine broadcast values of W2 with four of W1: 36 FMAs for ten reads), and
+// the 256 threads are four groups that share the channels of every slice of 32.  Slices come in by cp.async, two deep.  The sums
+// meet in shared memory in group order and leave as the piece or, for a run's last composition, delivered.  Blocks
+// behind the tiles compute the bias, and zero the packed chunks without weights.
+//
+// With a thread per result that walked the channels from L2, and a delivery launch behind it, the merge 384 -> 96 -> (576) -> 96
+// took 38.0 us, now 21.8; 144 -> 32 -> (192) -> 32 13.9, now 13.3.  (The same for 5x5 pieces, two input channels a thread, was
+// faster from 64 channels on but took 9.6 us instead of 7.4 at 24 -> 8 -> 80, and its longer sums were further from 64 bits.)
+// ----------------------------------------------------------------------------------------------
+struct After11 {
+  Piece first, second;
+  float *w_out, *b_out;
+  int gi, go;
+};
+constexpr int kA1O = 8, kA1I = 32, kA1C = 32;    // results of a CTA: output and input channels; channels of a slice
+constexpr int kA1N = 4, kA1G = 256 / (kA1O * kA1I / kA1N);        // input channels of a thread, groups
+constexpr int kA1P = kA1C * 9 + 4;               // floats between output channels of a slice
+constexpr int kA1Stage = kA1O * kA1P + kA1C * kA1I, kA1Tile = kA1O * kA1I * 9;
+constexpr int kA1Smem = 4 * (2 * kA1Stage > kA1G * kA1Tile ? 2 * kA1Stage : kA1G * kA1Tile);
+
+__global__ void __launch_bounds__(256, 2)
+k_compose_after_11(const __grid_constant__ After11 a, const __grid_constant__ BlockDelivery dv) {
+  constexpr int K = 3, KK = 9, NI = kA1N, T = kA1O * kA1I / NI, G = kA1G, CTR = 4, PO = kA1P, STAGE = kA1Stage, TILE = kA1Tile;
+  extern __shared__ __align__(16) float a1_smem[];
+  const int tid = (int)threadIdx.x, g = tid / T, t = tid % T;
+  const Piece &p1 = a.first, &p2 = a.second;
+  const int c0 = p1.c_in, c1 = p1.c_out, c2 = p2.c_out;
+  int blk = (int)blockIdx.x;
+  dc_pdl_enter();
+  if (blk >= a.gi * a.go) {
+    blk -= a.gi * a.go;
+    if (blk >= a.go) {
+      zero_dead_chunks(dv, c2, blk - a.go, (int)gridDim.x - a.gi * a.go - a.go);
+      return;
+    }
+    compose_bias_block(p1, p2, a.b_out, blk);      // eight warps, eight output channels
+    return;
+  }
+  const int o0 = (blk / a.gi) * kA1O, i0 = (blk % a.gi) * kA1I;
+  const int slices = (c1 + kA1C - 1) / kA1C;
+  auto fetch = [&](int sl) {
+    float *A = a1_smem + (sl & 1) * STAGE, *B = A + kA1O * PO;
+    const int cs = sl * kA1C, left = c1 - cs < kA1C ? c1 - cs : kA1C;      // a multiple of 4
+    for (int e = tid; e < kA1O * (kA1C * KK / 4); e += 256) {
+      const int o = e / (kA1C * KK / 4), x = e - o * (kA1C * KK / 4);
+      const bool ok = o0 + o < c2 && x * 4 < left * KK;
+      mb_cp16(A + o * PO + x * 4, ok ? p2.w + ((size_t)(o0 + o) * c1 + cs) * KK + x * 4 : p2.w, ok);
+    }
+    for (int e = tid; e < kA1C * kA1I / 4; e += 256) {
+      const int c = e / (kA1I / 4), i = i0 + (e % (kA1I / 4)) * 4;
+      const bool ok = c < left && i < c0;
+      mb_cp16(B + e * 4, ok ? p1.w + (size_t)(cs + c) * c0 + i : p1.w, ok);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int ol = t / (kA1I / NI), il = (t % (kA1I / NI)) * NI;
+  float acc[NI][KK] = {};
+  fetch(0);
+#pragma unroll 1
+  for (int sl = 0; sl < slices; ++sl) {
+    if (sl + 1 < slices) {
+      fetch(sl + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const float *A = a1_smem + (sl & 1) * STAGE + ol * PO, *B = a1_smem + (sl & 1) * STAGE + kA1O * PO + il;
+#pragma unroll 4
+    for (int c = g; c < kA1C; c += G) {            // channels dealt in turn: short runs keep their sums in parts too
+      float b[NI];
+#pragma unroll
+      for (int q = 0; q < NI; ++q) b[q] = B[c * kA1I + q];
+#pragma unroll
+      for (int u = 0; u < KK; ++u) {
+        const float w = A[c * KK + u];
+#pragma unroll
+        for (int q = 0; q < NI; ++q) acc[q][u] = fmaf(w, b[q], acc[q][u]);
+      }
+    }
+    __syncthreads();                               // the slice's buffer is refilled in the next turn
+  }
+#pragma unroll
+  for (int q = 0; q < NI; ++q)
+#pragma unroll
+    for (int u = 0; u < KK; ++u) a1_smem[g * TILE + (ol * kA1I + il + q) * KK + u] = acc[q][u];
+  __syncthreads();
+  const bool last = dv.mode >= 0;
+  for (int e = tid; e < TILE; e += 256) {
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < G; ++q) s += a1_smem[q * TILE + e];
+    const int oi = e / KK, u = e - oi * KK, o = o0 + oi / kA1I, i = i0 + oi % kA1I;
+    if (o < c2 && i < c0) {
+      if (p1.ident) s += p2.w[((size_t)o * c1 + i) * KK + u];                          // W2 o I: c0 == c1
+      if (p2.ident && u == CTR) s += p1.w[(size_t)o * c0 + i];                         // I o W1: c1 == c2
+      if (u == CTR && o == i) s += (p1.ident && p2.ident ? 1.f : 0.f) + (last && dv.ident ? 1.f : 0.f);
+      a.w_out[((size_t)o * c0 + i) * KK + u] = s;
+    }
+    if (last && dv.mode > 0) a1_smem[e] = s;       // element e of group 0's sums is read by this thread alone
+  }
+  if (!last || dv.mode == 0) return;
+  __syncthreads();
+  deliver_tile<kA1O, kA1I, K>(dv, a1_smem, o0, i0, c0, c2, tid, 256);
+}
 // the bias of a composition on its own
 __global__ void k_compose_bias(Piece first, Piece second, float *b_out) { compose_bias_block(first, second, b_out, (int)blockIdx.x); }
 
@@ -1302,6 +1574,34 @@ static void launch_compose33(const Operand33 &first, const Operand33 &second, in
   status.launched();
 }
 
+template <int IT, int W>
+static void launch_block33_form(TiledBlocks &tb, const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
+  tb.first[0] = 0;
+  for (int i = 0; i < tb.n; ++i) {
+    const int go = dc_div_up(tb.blk[i].c2, kMbO);
+    tb.first[i + 1] = tb.first[i] + (dc_div_up(tb.blk[i].c0, IT) + 1) * go;       // tiles and bias groups
+  }
+  static unsigned char attr_done[kDcMaxDevices];
+  status.note(dc_set_max_smem_once(k_merge_block33<IT, W>, MbForm<IT, W>::RING, attr_done));
+  status.note(dc_launch_pdl(k_merge_block33<IT, W>, dim3(tb.first[tb.n] + zero_ctas(dv, mg, W * 32)), dim3(W * 32), MbForm<IT, W>::RING, st, tb, dv));
+  status.launched();
+}
+// Tiles of 8 x 16 pairs by eight warps; by sixteen, one CTA to an SM, for long reductions: of 8 x 16 where that gives no SM a
+// second tile, of 8 x 24 where it leaves the SM with the most pairs fewer of them.
+static void launch_block33(TiledBlocks &tb, const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
+  int tiles16 = 0, tiles24 = 0, hidden = 0;
+  for (int i = 0; i < tb.n; ++i) {
+    tiles16 += dc_div_up(tb.blk[i].c0, 16) * dc_div_up(tb.blk[i].c2, kMbO);
+    tiles24 += dc_div_up(tb.blk[i].c0, 24) * dc_div_up(tb.blk[i].c2, kMbO);
+    if (tb.blk[i].c1 > hidden) hidden = tb.blk[i].c1;
+  }
+  const int n_sm = dc_sm_count(), most16 = dc_div_up(tiles16, n_sm) * 16, most24 = dc_div_up(tiles24, n_sm) * 24;
+  if (hidden < 320) launch_block33_form<16, 8>(tb, dv, mg, st, status);
+  else if (tiles16 <= n_sm) launch_block33_form<16, 16>(tb, dv, mg, st, status);
+  else if (most24 < most16) launch_block33_form<24, 16>(tb, dv, mg, st, status);
+  else launch_block33_form<16, 8>(tb, dv, mg, st, status);
+}
+
 // A 1x1 after a large dense kernel is a plain matrix product: the fp32 convolution's kernel runs it as a 1x1 layer whose
 // pixels are the second layer's rows and whose weights are the first layer as stored (960 -> 320 -> 1280: 81 us with the
 // gathered product, 59.9 us).  False: a shape outside that kernel's range, nothing was launched.
@@ -1336,6 +1636,16 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       if (dv) { out.w = w = w_final; out.b = b = b_final; *delivered = true; }
       launch_compose33(operand(first), operand(second), first.c_in, first.c_out, second.c_out, w, b, dv ? *dv : piece,
                        mg ? *mg : dc_geom{}, st, status);
+    } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k == 3 && first.c_in % 4 == 0 &&
+               first.c_out % 4 == 0 && first.c_out >= 32 && second.c_out < 65535) {
+      // From 32 intermediate channels on, a whole slice (96 -> 24 -> 24 inside a longer run took 2.3 us more here).  More output
+      // channels than 65534 are left to the kernel below, whose grid the runtime refuses.
+      After11 a{first, second, w, b, dc_div_up(first.c_in, kA1I), dc_div_up(second.c_out, kA1O)};
+      BlockDelivery piece{nullptr, -1, 0, KOrder{}};
+      if (dv) { out.w = a.w_out = w_final; out.b = a.b_out = b_final; *delivered = true; piece = *dv; }
+      static unsigned char attr_done[kDcMaxDevices];
+      status.note(dc_set_max_smem_once(k_compose_after_11, kA1Smem, attr_done));
+      status.note(dc_launch_pdl(k_compose_after_11, dim3(a.gi * a.go + a.go + zero_ctas(piece, mg ? *mg : dc_geom{}, 256)), dim3(256), kA1Smem, st, a, piece));
     } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k > 1 &&
         first.c_out * second.k * second.k <= kAfter1x1MaxFloats) {
       dim3 grid(dc_div_up(out.c_in * out.k * out.k, 256), out.c_out + 1);
@@ -1476,6 +1786,37 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     }
   }
 
+  if (direct && n == 2 && layers[0].groups == 1 && layers[1].groups == 1 && layers[0].k == 1 && layers[1].k == 1 &&
+      layers[0].stride == 1 && layers[0].c_in % 4 == 0 && layers[0].c_out % 4 == 0) {
+    int id[2] = {0, 0}, whole = 0;
+    for (int g = 0; g < n_res; ++g) {
+      if (res[g].first != res[g].last) whole = 1;
+      else id[res[g].first] = 1;
+    }
+    Merge11 a{raw_of(layers[0]), raw_of(layers[1]), id[0], id[1], mg.c_in, layers[0].c_out, mg.c_out, w_merged, b_merged, 0, 0};
+    const BlockDelivery dv{w_packed, mode, whole, ko};
+    // 32 x 32 until tiles of 64 columns give most SMs one; of those the height that leaves the SM with the most tiles the least
+    // (960 -> 320 -> 1280: 300 tiles of 64 x 64 are three on four SMs and two on the others, 45.9 us)
+    const int n_sm = dc_sm_count(), wide[2] = {64, 48};
+    int bo = 32, bi = 32;
+    if (dc_div_up(a.c2, 64) * dc_div_up(a.c0, 64) >= 100) {
+      bi = 64;
+      long long best = 0;
+      for (int h : wide) {
+        const long long rows = (long long)dc_div_up(dc_div_up(a.c2, h) * dc_div_up(a.c0, 64), n_sm) * h;
+        if (bo == 32 || rows < best) { best = rows; bo = h; }
+      }
+    }
+    a.gi = dc_div_up(a.c0, bi);
+    a.go = dc_div_up(a.c2, bo);
+    const dim3 grid(a.gi * a.go + dc_div_up(a.c2, 8) + zero_ctas(dv, mg, 256));
+    if (bo == 64) status.note(dc_launch_pdl(k_merge_11<64, 64, 8, 2>, grid, dim3(256), 0, st, a, dv));
+    else if (bo == 48) status.note(dc_launch_pdl(k_merge_11<48, 64, 6, 2>, grid, dim3(256), 0, st, a, dv));
+    else status.note(dc_launch_pdl(k_merge_11<32, 32, 4, 4>, grid, dim3(256), 0, st, a, dv));
+    status.launched();
+    return status.s;
+  }
+
   // 0. inverted-residual blocks (1x1, depthwise, 1x1) are merged in one step from the raw layers
   std::vector<int> chunk_at(n, 0), covered(n, 0);
   if (algo != DC_MERGE_STEPS)
@@ -1533,10 +1874,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
   bool delivered = false;
   auto flush_tiled = [&]() {
     if (tiled.n == 0) return;
-    static unsigned char attr_done[kDcMaxDevices];
-    status.note(dc_set_max_smem_once(k_merge_block33, kMbRing, attr_done));
-    status.note(dc_launch_pdl(k_merge_block33, dim3(tiled.first[tiled.n] + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), kMbRing, st, tiled, dv));
-    status.launched();
+    launch_block33(tiled, dv, mg, st, status);
     tiled.n = 0;
   };
   auto flush_blocks = [&]() {
@@ -1567,7 +1905,6 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
       if (go && chunk_at[i] == kTiledBlock) {
         const int t = tiled.n++;
         tiled.blk[t] = BlockArgs{raw_of(e), raw_of(d), raw_of(p), e.c_in, e.c_out, p.c_out, d.k, 0, w, b};
-        tiled.first[t + 1] = tiled.first[t] + dc_div_up(e.c_in, kMbI) * dc_div_up(p.c_out, kMbO) + dc_div_up(p.c_out, kMbO);
         if (tiled.n == kBlockBatch) flush_tiled();
       } else if (go) {
         batch.blk[n_batch] = BlockArgs{raw_of(e), raw_of(d), raw_of(p), e.c_in, e.c_out, p.c_out, d.k, chunk_at[i], w, b};

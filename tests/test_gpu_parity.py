@@ -262,6 +262,56 @@ def test_runs_delivered_by_one_launch(dc, case):
         assert torch.equal(packed, again)
 
 
+@pytest.mark.parametrize("channels,res,bn", [
+    ((8, 4, 8), [], True),                     # one piece of four channels: three of four groups have no slice
+    ((36, 20, 44), [], True),                  # nothing a multiple of a tile or of a slice
+    ((40, 40, 40), [(0, 0)], True),            # an identity on the first layer, ...
+    ((40, 40, 40), [(0, 0), (1, 1)], False),   # ... on both, ...
+    ((72, 24, 72), [(0, 1)], True),            # ... on the run
+    ((648, 72, 712), [], True),                # tiles of 64 columns, ragged ones last
+    ((960, 320, 1280), [], True),              # the network's last merge: tiles of 48 rows
+])
+def test_two_1x1_layers_delivered_by_one_launch(dc, channels, res, bn):
+    a, m, o = channels
+    specs = [I.make_layer(81, 0, a, m, 1, 1, 0, with_bn=bn), I.make_layer(81, 1, m, o, 1, 1, 0)]
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32) if a % 8 == 0 and o % 8 == 0 else (dc.F32,))
+
+
+@pytest.mark.parametrize("c0,c1,c2,s,res", [
+    (40, 36, 24, 1, []),                       # a slice of 4 channels last, ragged tiles
+    (32, 32, 32, 1, [(0, 0)]),                 # an identity on the 1x1 layer, ...
+    (32, 32, 32, 1, [(0, 0), (1, 1)]),         # ... and on the 3x3 one
+    (384, 96, 100, 2, []),                     # three slices, stride 2
+    (72, 200, 9, 1, []),                       # one output channel more than a tile
+])
+@pytest.mark.parametrize("tail", [False, True])
+def test_3x3_after_1x1_against_the_oracle(dc, c0, c1, c2, s, res, tail):
+    """As a run's last composition, delivered by its own launch, and as a piece that a depthwise layer is composed with."""
+    specs = [I.make_layer(82, 0, c0, c1, 1, 1, 0), I.make_layer(82, 1, c1, c2, 3, s, 1)]
+    if tail:
+        specs.append(I.make_layer(82, 2, c2, c2, 3, 1, 1, depthwise=True))
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32))
+
+
+def _check_delivery(dc, specs, res, codes):
+    W, b, k, s, p = O.merge_formula(specs, res)
+    for code in codes:
+        g, wm, bm, packed = run_merge(dc, specs, res, packed_dtype=code)
+        assert (g.k, g.stride, g.pad) == (k, s, p)
+        assert O.rel_l2(wm.cpu().numpy(), W) <= TOL_W and O.rel_l2(bm.cpu().numpy(), b) <= TOL_W
+        again = torch.full_like(packed, 7)
+        dc.pack_weights(wm, g, code, again)
+        torch.cuda.synchronize()
+        assert torch.equal(packed, again)
+
+
+@pytest.mark.parametrize("c,hidden", [(24, 320), (136, 820), (160, 960), (200, 1000)])
+def test_blocks_by_sixteen_warps_against_the_oracle(dc, c, hidden):
+    """Long reductions: tiles of 8 x 16 and of 8 x 24 pairs, warps whose last slice is short or that have none."""
+    _check_delivery(dc, [I.make_layer(83, 0, c, hidden, 1, 1, 0), I.make_layer(83, 1, hidden, hidden, 3, 1, 1, depthwise=True),
+                         I.make_layer(83, 2, hidden, c, 1, 1, 0)], [(0, 2)], (dc.BF16, dc.F32))
+
+
 @pytest.mark.parametrize("case", ["block", "dense_pair", "expand_dw"])
 @pytest.mark.parametrize("alias", ["weights", "bias", "packed"])
 def test_merge_into_its_layers_arrays(dc, case, alias):
