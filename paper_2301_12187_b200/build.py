@@ -1,15 +1,18 @@
-"""Builds libdepthc.so (sm_100a) next to this file with nvcc.  `python -m paper_2301_12187_b200.build`."""
+"""Builds libdepthc.so (sm_100a, nvcc) and the Python module _dccall.so (gcc) next to this file.  `python -m paper_2301_12187_b200.build`."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdepthc.so")
+CALL_SRC = os.path.join(CSRC, "dccall.c")
+CALL_LIB = os.path.join(HERE, "_dccall.so")     # marshals the forward calls of dc.py
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -29,7 +32,17 @@ def needs_build() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_call(force: bool = False) -> None:
+    if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_LIB) >= os.path.getmtime(CALL_SRC):
+        return
+    tmp = CALL_LIB + ".tmp.%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp,
+                           CALL_SRC])
+    os.replace(tmp, CALL_LIB)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_call(force)
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

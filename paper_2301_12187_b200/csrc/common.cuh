@@ -50,6 +50,42 @@ static inline cudaError_t dc_set_max_smem_once(K kernel, int bytes, unsigned cha
   return e;
 }
 
+// Plans that a thread made lately, by shape: choosing tiles is a search of 1 to 3 us on the host, as long as a small launch
+// itself takes, and a network's layers come round again.  Per thread, so without locks; 64 shapes, a later one in a place
+// takes it over; nothing of a call's buffers is in it.  `make` fills a plan and answers whether the shape is in range.
+template <typename Plan>
+struct DcPlans {
+  struct Entry {
+    int key[12];
+    bool used, ok;
+    Plan plan;
+  };
+  Entry at[64] = {};
+  template <typename Make>
+  bool get(const int (&key)[12], Plan *plan, Make make) {
+    uint32_t hash = 2166136261u;
+    for (int i = 0; i < 12; ++i) hash = (hash ^ (uint32_t)key[i]) * 16777619u;
+    Entry &e = at[(hash ^ (hash >> 15)) & 63u];
+    bool same = e.used;
+    for (int i = 0; i < 12 && same; ++i) same = e.key[i] == key[i];
+    if (!same) {
+      e.used = false;
+      e.ok = make(&e.plan);
+      for (int i = 0; i < 12; ++i) e.key[i] = key[i];
+      e.used = true;
+    }
+    if (e.ok) *plan = e.plan;
+    return e.ok;
+  }
+};
+static inline int dc_plan_device() {               // a plan may depend on its device: SMs, clusters that run at once
+  const int dev = dc_current_device();
+  if (dev < 0) (void)cudaGetLastError();
+  return dev;
+}
+#define DC_PLAN_KEY(n, h, w, g, n_sm) \
+  {n, h, w, (g)->c_in, (g)->c_out, (g)->groups, (g)->k, (g)->stride, (g)->pad, n_sm, dc_plan_device(), 0}
+
 static inline int dc_out_extent(int h, int k, int s, int p) {
   int a = h + 2 * p - k;
   return a < 0 ? 0 : a / s + 1;

@@ -295,7 +295,7 @@ bool f32_grid(F32Plan *pl, int config, int split) {
   return true;
 }
 
-bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *pl) {
+bool make_f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *pl) {
   if (!f32_shape(n, h, w, g, &pl->p)) return false;
   // Least estimated time, in cycles of the SM with the most CTAs.  Per slice an SM needs the FMAs of its CTAs (16 x
   // TM x TN cycles of a CTA at full rate) but never less than a slice's own chain; a round of resident CTAs costs a
@@ -317,6 +317,11 @@ bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *pl) {
       if (best_config < 0 || cost < best) { best = cost; best_config = cfg; best_split = split; }
     }
   return best_config >= 0 && f32_grid(pl, best_config, best_split);
+}
+
+bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *p) {
+  static thread_local DcPlans<F32Plan> plans;
+  return plans.get(DC_PLAN_KEY(n, h, w, g, n_sm), p, [&](F32Plan *q) { return make_f32_plan(n, h, w, g, n_sm, q); });
 }
 
 }  // namespace

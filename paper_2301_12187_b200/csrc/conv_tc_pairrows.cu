@@ -627,7 +627,7 @@ constexpr int kSmemBudget = 220 * 1024;
 constexpr int kStageLimit = 48 * 1024;
 constexpr int kSlack = 17 * 1024;   // a block's 128 rows may reach this far past the last stage
 
-bool pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams *p) {
+bool make_pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams *p) {
   KOrder ko;
   dc_korder_init(&ko, g);
   if (ko.pair != 2 && ko.pair != 3) return false;
@@ -737,6 +737,11 @@ bool pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams *p) {
         p->a_lo[j] = (off >> 4) | (1u << 16);    // leading-dimension field: 1 (unused for swizzled K-major)
       }
   return true;
+}
+
+bool pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams *p) {
+  static thread_local DcPlans<PairParams> plans;
+  return plans.get(DC_PLAN_KEY(n, h, w, g, n_sm), p, [&](PairParams *q) { return make_pair_plan(n, h, w, g, n_sm, q); });
 }
 
 }  // namespace

@@ -658,7 +658,7 @@ int max_clusters(int size) {
   return cached[dev][size];
 }
 
-bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
+bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
   KOrder ko;
   dc_korder_init(&ko, g);
   if (!ko.rows) return false;
@@ -862,6 +862,11 @@ bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
     if (p->smem_bytes < need) p->smem_bytes = need;
   }
   return true;
+}
+
+bool rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams *p) {
+  static thread_local DcPlans<RowsParams> plans;
+  return plans.get(DC_PLAN_KEY(n, h, w, g, n_sm), p, [&](RowsParams *q) { return make_rows_plan(n, h, w, g, n_sm, q); });
 }
 
 }  // namespace

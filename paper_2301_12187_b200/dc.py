@@ -1,5 +1,6 @@
 """ctypes binding of libdepthc (include/dc.h).  Argument marshalling only: every step of the
-path runs in the library's CUDA kernels.  torch is used for device memory and streams.
+path runs in the library's CUDA kernels.  torch is used for device memory and streams.  The three
+forward calls are marshalled natively (csrc/dccall.c); the ctypes form behind them takes what that does not read.
 
 The functions carry the names of the C entry points without the `dc_` prefix.  Importing this
 module does not load the library; the first call does, and raises if it cannot.
@@ -109,6 +110,7 @@ EXPORTS = {
 }
 
 _lib = None
+_native = None
 
 
 class DcError(RuntimeError):
@@ -124,7 +126,7 @@ class DcError(RuntimeError):
 def lib():
     """Load libdepthc.so (building it with nvcc first if it is missing or stale).  Never falls
     back to anything else: without the library every call raises."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         from . import build as _build
         try:
@@ -136,8 +138,20 @@ def lib():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
+        import torch
+        from . import _dccall
+        at = lambda name: C.cast(getattr(L, name), C.c_void_p).value
+        _dccall.bind(at("dc_conv_forward_algo"), at("dc_dwconv_forward"), at("dc_block_forward"), torch.float32, torch.bfloat16,
+                     Geom, Block, getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device),
+                     getattr(torch._C, "_cuda_getCurrentRawStream", None))
+        _native = _dccall
         _lib = L
     return _lib
+
+
+def _load_native():
+    lib()
+    return _native
 
 
 def _check(st: int, what: str):
@@ -384,6 +398,11 @@ def conv_kernel_name(n: int, h: int, w: int, g: Geom, dtype: int) -> Optional[st
 
 
 def conv_forward(x, g: Geom, w_packed, bias, act, residual, y, workspace, stream=None, algo=ALGO_AUTO):
+    st = (_native or _load_native()).conv(x, g, w_packed, bias, act, residual, y, workspace, stream, algo)
+    if st == OK:
+        return
+    if st is not None:
+        raise DcError(st, "dc_conv_forward")
     n, h, w, _ = x.shape
     _check(lib().dc_conv_forward_algo(_ptr(x), n, h, w, C.byref(g), _ptr(w_packed), _ptr(bias), act,
                                       _ptr(residual), _ptr(y), dtype_code(x.dtype), _ptr(workspace),
@@ -392,6 +411,11 @@ def conv_forward(x, g: Geom, w_packed, bias, act, residual, y, workspace, stream
 
 
 def dwconv_forward(x, k, stride, pad, w_packed, bias, act, y, stream=None):
+    st = (_native or _load_native()).dwconv(x, k, stride, pad, w_packed, bias, act, y, stream)
+    if st == OK:
+        return
+    if st is not None:
+        raise DcError(st, "dc_dwconv_forward")
     n, h, w, c = x.shape
     _check(lib().dc_dwconv_forward(_ptr(x), n, h, w, c, k, stride, pad, _ptr(w_packed), _ptr(bias), act,
                                    _ptr(y), dtype_code(x.dtype), _stream(stream)), "dc_dwconv_forward")
@@ -409,6 +433,11 @@ def block_workspace_bytes(n, h, w, blk: Block, dtype: int) -> int:
 
 
 def block_forward(x, blk: Block, y, workspace, stream=None):
+    st = (_native or _load_native()).block(x, blk, y, workspace, stream)
+    if st == OK:
+        return
+    if st is not None:
+        raise DcError(st, "dc_block_forward")
     n, h, w, _ = x.shape
     _check(lib().dc_block_forward(_ptr(x), n, h, w, C.byref(blk), _ptr(y), dtype_code(x.dtype),
                                   _ptr(workspace), workspace.numel() * workspace.element_size(),

@@ -205,3 +205,44 @@ def test_bench_line_holds_main_figures_only():
            "groups": [{}] * 27}
     assert bench.brief(chain) == {"forward_us": 8.5, "merge_us": 6.25, "step_us": 16.0, "frac": 0.3457}
     assert bench.brief(net) == {"forward_us": 667.0, "merge_us": 128.0, "step_us": 815.0, "frac": 0.5357}
+
+
+class _NoNative:
+    """Stands for the native marshalling when it cannot read the arguments: the call then goes through ctypes."""
+    conv = dwconv = block = staticmethod(lambda *a: None)
+
+
+@pytest.mark.parametrize("change", ["none", "dtype", "three_dims", "float_act", "huge_act", "no_geom", "empty_batch", "short_workspace", "null_y"])
+def test_native_marshalling_reports_what_ctypes_reports(monkeypatch, change):
+    """Forward calls that are refused on the host: the same exception, status and message on both routes."""
+    import torch
+
+    class Stream:
+        cuda_stream = 0
+
+    x = torch.zeros(0 if change == "empty_batch" else 1, 4, 4, 8, dtype=torch.float16 if change == "dtype" else torch.bfloat16)
+    if change == "three_dims":
+        x = x[0]
+    y = None if change == "null_y" else torch.zeros(1, 4, 4, 8, dtype=torch.bfloat16)
+    ws = torch.zeros(16 if change == "short_workspace" else 256, dtype=torch.uint8)
+    w, b = torch.zeros(64), torch.zeros(8)
+    act = {"float_act": 0.5, "huge_act": 1 << 40}.get(change, 7)            # 7: no activation, refused by the library
+    g = None if change == "no_geom" else dc.geom(8, 8, 1, 1, 1, 0)
+    blk = None if change == "no_geom" else dc.Block(8, 48, 8, 0, 2, 1, 1, 0, 1, 1, None, None, 16, None, 16, None)
+    calls = [lambda: dc.conv_forward(x, g, w, b, act, None, y, ws, stream=Stream),
+             lambda: dc.dwconv_forward(x, 3, 1, 1, w, b, act, y, stream=Stream),
+             lambda: dc.block_forward(x, blk, y, ws, stream=Stream)]
+
+    def outcomes():
+        out = []
+        for call in calls:
+            try:
+                call()
+                out.append("returned")
+            except Exception as e:                # noqa: BLE001 -- what is compared is the exception
+                out.append((type(e).__name__, getattr(e, "status", None), str(e)))
+        return out
+
+    native = outcomes()
+    monkeypatch.setattr(dc, "_native", _NoNative)
+    assert native == outcomes() and "returned" not in native
