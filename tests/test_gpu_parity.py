@@ -868,6 +868,22 @@ def test_dwconv(dc, dtype, c, k, s, p, n, h, w):
     assert_close(nchw(y), ref, TOL_F32 if dtype == "f32" else TOL_BF16, bf16=(dtype == "bf16"))
 
 
+@pytest.mark.parametrize("c,k,s,p,n,h,w", [
+    (40, 3, 1, 1, 2, 9, 9),              # a partly filled last tile of channels
+    (72, 3, 2, 1, 3, 15, 13),            # the same, stride 2, odd sides
+    (8, 5, 1, 2, 1, 7, 7),               # eight channels, one tile
+    (152, 3, 1, 1, 1, 27, 24),           # one output row per thread
+    (360, 3, 1, 1, 70, 7, 7),            # two rows per thread of an odd height, several images per tile
+    (48, 3, 1, 1, 32, 56, 56),           # two rows per thread, more tiles than CTAs at once
+    (104, 5, 2, 2, 9, 21, 23),           # 5x5 of stride 2
+    (8, 5, 2, 2, 1, 6, 252),             # widest maps of the load unit's box: the last items read past their row
+    (16, 3, 1, 1, 1, 5, 254),
+])
+def test_dwconv_stencil_tiles(dc, c, k, s, p, n, h, w):
+    test_dwconv_stencil_without_activation(dc, c, k, s, p, n, h, w)
+    test_dwconv(dc, "bf16", c, k, s, p, n, h, w)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("c_in,c_out,t,s,n,h,w", [(24, 24, 6, 1, 2, 14, 14), (16, 24, 6, 2, 1, 16, 16),
                                                   (32, 16, 1, 1, 1, 12, 12)])
