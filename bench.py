@@ -418,7 +418,7 @@ def measure_network(args, peaks, peak_src):
         else:
             f = sum(2.0 * n * (ho * wo if s.role != "expand" else h * w) * s.c_out * (s.c_in // s.groups) * s.k * s.k for s in specs)
             b = 2.0 * (n * h * w * c + n * ho * wo * co)
-            kern = "block (3 launches)"
+            kern = "block"
         t = max(b / (peaks["hbm_gbs"] * 1e9), f / (peaks["bf16_tflops"] * 1e12))
         roof_s += t
         roof_nom_s += max(b / (NOMINAL_PEAKS["hbm_gbs"] * 1e9), f / (NOMINAL_PEAKS["bf16_tflops"] * 1e12))

@@ -53,8 +53,8 @@ typedef enum {
 } dc_status;
 
 typedef enum { DC_F32 = 0, DC_BF16 = 1 } dc_dtype;
-/* DC_ACT_RELU6 is min(max(v, 0), 6).  A NaN becomes 0, except in k_conv_stem_s2 and in the bf16 depthwise stencil, where it
- * becomes 6. */
+/* DC_ACT_RELU6 is min(max(v, 0), 6).  A NaN becomes 0, except in k_conv_stem_s2 and in bf16 depthwise layers (a block's
+ * too), where it becomes 6. */
 typedef enum { DC_ACT_IDENTITY = 0, DC_ACT_RELU6 = 1 } dc_act;
 typedef enum { DC_ALGO_AUTO = 0, DC_ALGO_TCGEN05 = 1, DC_ALGO_SIMT = 2 } dc_algo;
 
@@ -243,7 +243,9 @@ dc_status dc_block_workspace_bytes(int n, int h, int w, const dc_block *blk, dc_
 /*
  * Forward pass of one unmerged inverted-residual block: expand 1x1 + act, depthwise + act,
  * project 1x1, plus the block input when has_residual (the skip addition that stays explicit
- * when the block is not merged into a single convolution, App. E.1).
+ * when the block is not merged into a single convolution, App. E.1).  DC_BF16 blocks with both ReLU6, a 3x3 depthwise layer
+ * of padding 1 and channels in multiples of 8 (hidden ones of 16) run as one launch where that is faster; the hidden maps are
+ * then never written, and otherwise lie in the workspace.  y may be x: such a call goes through the workspace.
  */
 dc_status dc_block_forward(const void *x, int n, int h, int w, const dc_block *blk, void *y,
                            dc_dtype dtype, void *workspace, size_t workspace_bytes,

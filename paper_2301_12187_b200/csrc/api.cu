@@ -132,6 +132,26 @@ extern "C" dc_status dc_block_workspace_bytes(int n, int h, int w, const dc_bloc
   return DC_OK;
 }
 
+// The one-launch block kernel reads its operands as long as it writes y, and 16 bytes at a time: pointers that are not
+// aligned (which the launches of the three layers report) and outputs that overlap an input go through the workspace.
+static bool one_launch_block(const void *x, int n, int h, int w, int ho, int wo, const dc_block *b, const void *y) {
+  if (!b->has_expand) return false;
+  const dc_geom g1 = {b->c_in, b->c_hidden, 1, 1, 1, 0}, g3 = {b->c_hidden, b->c_out, 1, 1, 1, 0};
+  size_t bytes1 = 0, bytes3 = 0;
+  if (dc_packed_bytes(&g1, DC_BF16, &bytes1) != DC_OK || dc_packed_bytes(&g3, DC_BF16, &bytes3) != DC_OK) return false;
+  const struct { const void *at; size_t bytes; } in[] = {
+      {x, (size_t)n * h * w * b->c_in * 2}, {b->w_expand, bytes1}, {b->b_expand, (size_t)b->c_hidden * 4},
+      {b->w_dw, (size_t)b->dw_k * b->dw_k * b->c_hidden * 4}, {b->b_dw, (size_t)b->c_hidden * 4},
+      {b->w_project, bytes3}, {b->b_project, (size_t)b->c_out * 4}};
+  const char *y0 = (const char *)y, *y1 = y0 + (size_t)n * ho * wo * b->c_out * 2;
+  if (!dc_aligned16(y)) return false;
+  for (const auto &a : in) {
+    const char *a0 = (const char *)a.at;
+    if (a0 && (!dc_aligned16(a0) || (a0 < y1 && y0 < a0 + a.bytes))) return false;
+  }
+  return true;
+}
+
 extern "C" dc_status dc_block_forward(const void *x, int n, int h, int w, const dc_block *b, void *y,
                                       dc_dtype dtype, void *workspace, size_t workspace_bytes,
                                       dc_stream stream) {
@@ -143,6 +163,10 @@ extern "C" dc_status dc_block_forward(const void *x, int n, int h, int w, const 
   if (!dc_aligned16(workspace)) return DC_ERR_ALIGNMENT;
   const size_t es = dtype == DC_F32 ? 4 : 2;
   const int ho = dc_out_extent(h, b->dw_k, b->dw_stride, b->dw_pad), wo = dc_out_extent(w, b->dw_k, b->dw_stride, b->dw_pad);
+  if (dtype == DC_BF16 && one_launch_block(x, n, h, w, ho, wo, b, y)) {
+    s = dc_launch_block_tc(x, n, h, w, b, y, workspace, (cudaStream_t)stream);
+    if (s != DC_ERR_UNSUPPORTED) return s;
+  }
   char *ws = (char *)workspace;
   char *t_exp = ws + sizeof(DcWsHeader);
   char *t_dw = t_exp + (b->has_expand ? dc_round_up((size_t)n * h * w * b->c_hidden * es, 256) : 0);

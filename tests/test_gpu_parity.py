@@ -884,6 +884,76 @@ def test_dwconv_stencil_tiles(dc, c, k, s, p, n, h, w):
     test_dwconv(dc, "bf16", c, k, s, p, n, h, w)
 
 
+@pytest.mark.parametrize("c_in,hidden,c_out,s,n,h,w,biases,one_launch", [
+    (16, 96, 16, 1, 3, 9, 11, True, True),       # two groups of warps, a ragged map
+    (64, 384, 64, 1, 5, 14, 14, True, True),     # six chunks of 64 hidden channels
+    (40, 240, 232, 2, 1, 25, 26, True, True),    # stride 2, odd height, two passes of output channels
+    (24, 80, 32, 1, 2, 13, 12, False, True),     # chunks of 48 and 32, no biases
+    (24, 96, 8, 1, 2, 13, 12, True, True),       # eight outputs
+    (24, 80, 8, 1, 2, 13, 12, True, False),      # projection weights in groups of five chunks, padded to six: three launches
+    (72, 432, 40, 1, 1, 33, 34, True, True),     # a last pass of hidden channels that is shorter than the others
+    (16, 96, 24, 2, 1, 40, 112, True, True),     # several strips of columns
+    (24, 144, 24, 1, 40, 20, 20, True, True),    # several tiles per CTA
+    (32, 192, 32, 1, 77, 10, 10, False, True),   # several images per tile or tiles of one image, more of them than SMs
+    (16, 96, 264, 1, 1, 12, 12, True, False),    # more than 256 outputs: three launches
+    (24, 72, 24, 1, 1, 12, 12, True, False),     # hidden channels no multiple of 16: three launches
+])
+def test_block_in_one_launch_against_the_oracle(dc, c_in, hidden, c_out, s, n, h, w, biases, one_launch):
+    mk = I.make_layer
+    specs = [mk(91, 0, c_in, hidden, 1, 1, 0, act="relu6", with_bn=False, with_bias=biases),
+             mk(91, 1, hidden, hidden, 3, s, 1, depthwise=True, act="relu6", with_bn=False, with_bias=biases),
+             mk(91, 2, hidden, c_out, 1, 1, 0, with_bn=False, with_bias=biases)]
+    res = s == 1 and c_in == c_out
+    keep, ptrs = [], []
+    for spec, code in zip(specs, (dc.BF16, dc.F32, dc.BF16)):
+        lay = dc.DeviceLayer(spec)
+        g = dc.geom(spec.c_in, spec.c_out, spec.groups, spec.k, spec.stride, spec.pad)
+        packed = torch.empty(dc.packed_bytes(g, code), dtype=torch.uint8, device="cuda")
+        dc.pack_weights(lay.weight, g, code, packed)
+        keep.append((lay, packed))
+        ptrs += [packed.data_ptr(), lay.bias.data_ptr() if biases else None]
+    blk = dc.Block(c_in, hidden, c_out, 1, 3, s, 1, int(res), dc.ACT_RELU6, dc.ACT_RELU6, *ptrs)
+    x = I.make_input(92, (n, h, w, c_in), bf16=True)
+    gy = Guarded(torch, (n, O.out_extent(h, 3, s, 1), O.out_extent(w, 3, s, 1), c_out), torch.bfloat16, fill=float("nan"))
+    gws = Guarded(torch, (dc.block_workspace_bytes(n, h, w, blk, dc.BF16),), torch.uint8, fill=0)
+    dc.block_forward(dev(x, torch.bfloat16), blk, gy.t, gws.t)
+    assert dc.workspace_status(gws.t) == dc.OK
+    gy.check("block output")
+    gws.check("block workspace")
+    assert (not bool(gws.t[256:].any())) == one_launch          # the hidden maps were never in the workspace
+    cur = x.transpose(0, 3, 1, 2).astype(np.float64)
+    skip = cur
+    for spec in specs:
+        Wf, bfo = O.fold_bn(spec)
+        cur = O.conv_direct(cur, Wf, bfo, spec.k, spec.stride, spec.pad, spec.groups)
+        cur = O.relu6(cur) if spec.act == "relu6" else cur
+    assert_close(nchw(gy.t), cur + skip if res else cur, 3 * TOL_BF16, scale=3.0)      # as for three launches: the same roundings
+
+
+def test_block_in_place(dc):
+    """An output on the block's own input goes through the workspace, and gives what a separate one gives."""
+    n, h, w, c, m = 3, 14, 14, 24, 144
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *shape: torch.randn(*shape, generator=gen, device="cuda")
+    ptrs, keep = [], []
+    for wt, (ci, co, groups, k), code in ((rnd(m, c, 1, 1) / c ** 0.5, (c, m, 1, 1), dc.BF16), (rnd(m, 1, 3, 3) / 3, (m, m, m, 3), dc.F32),
+                                          (rnd(c, m, 1, 1) / m ** 0.5, (m, c, 1, 1), dc.BF16)):
+        g = dc.geom(ci, co, groups, k, 1, k // 2)
+        packed = torch.empty(dc.packed_bytes(g, code), dtype=torch.uint8, device="cuda")
+        dc.pack_weights(wt, g, code, packed)
+        keep += [packed, rnd(co)]
+        ptrs += [packed.data_ptr(), keep[-1].data_ptr()]
+    blk = dc.Block(c, m, c, 1, 3, 1, 1, 1, dc.ACT_RELU6, dc.ACT_RELU6, *ptrs)
+    x = rnd(n, h, w, c).bfloat16()
+    ws = torch.zeros(dc.block_workspace_bytes(n, h, w, blk, dc.BF16), dtype=torch.uint8, device="cuda")
+    y = torch.empty_like(x)
+    dc.block_forward(x, blk, y, ws)
+    assert not bool(ws[256:].any())
+    dc.block_forward(x, blk, x, ws)
+    assert bool(ws[256:].any())
+    assert torch.allclose(x.float(), y.float(), rtol=2.0 ** -7, atol=2.0 ** -6)      # one bf16 step, sums in another order
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("c_in,c_out,t,s,n,h,w", [(24, 24, 6, 1, 2, 14, 14), (16, 24, 6, 2, 1, 16, 16),
                                                   (32, 16, 1, 1, 1, 12, 12)])
