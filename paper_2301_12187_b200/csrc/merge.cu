@@ -678,7 +678,8 @@ __global__ void __launch_bounds__(kBlockThreads) k_merge_block(const __grid_cons
 // Before, with one CTA per output channel that read every operand, then a delivery launch: 24 -> 144 -> 24
 // 9.4 us, 64 -> 384 -> 64 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  With eight warps 6.5, 9.0 and 25.9 us (200 tiles
 // of 8 x 16 on 148 SMs: 52 of them had two, the others eight warps with no second tile to hide their latency); by sixteen warps in 140 tiles of 8 x 24 20.7
-// us, 120 -> 720 -> 120 (120 tiles) 19.0 -> 12.9, 88 -> 528 -> 88 15.0 -> 11.3.  Halved runs of the sums are nearer to 64 bits as well
+// us, 120 -> 720 -> 120 (120 tiles) 19.0 -> 12.9, 88 -> 528 -> 88 15.0 -> 11.3.  With the sums added 16 bytes at a time and the third
+// layer's scales asked for in front (behind the sums they were a chain of their own) 24 -> 144 -> 24 6.4 -> 6.0, 160 -> 960 -> 160 19.7.  Halved runs of the sums are nearer to 64 bits as well
 // (160 channels: 1.6e-7 -> 1.35e-7).
 // ----------------------------------------------------------------------------------------------
 constexpr int kMbO = 8, kMbI = 16, kMbSlice = 16, kMbStages = 4;
@@ -811,6 +812,8 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
   }
   // ---- 8 x 16 pairs
   const int o0 = (blk / gi) * kMbO, i0 = (blk % gi) * IT;
+  __shared__ float g3s[kMbO];                      // BN scales of the tile's output channels
+  if (tid < kMbO) g3s[tid] = o0 + tid < c2 ? raw_scale(a.l3, o0 + tid) : 0.f;
   const int per = ((c1 + W - 1) / W + 3) & ~3;       // hidden channels of a warp
   const int cb = warp * per, ce = cb + per < c1 ? cb + per : c1;
   const int nsl = ce > cb ? (ce - cb + kMbSlice - 1) / kMbSlice : 0;
@@ -919,17 +922,29 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
       for (int t = 0; t < 9; ++t) mb_smem[warp * F::TILE + ((ol + h) * IT + il + v) * 9 + t] = acc[h][v][t];
   __syncthreads();
   const bool last = dv.mode >= 0;
-  for (int e = tid; e < F::TILE; e += W * 32) {
-    float s = 0.f;
+  // four elements of the warps' sums at a time: rows of IT input channels are whole pieces, and so are 4 channels of them
+  for (int e = tid; e < F::TILE / 4; e += W * 32) {
+    float4 *p = reinterpret_cast<float4 *>(mb_smem) + e;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int w = 0; w < W; ++w) s += mb_smem[w * F::TILE + e];
-    const int oi = e / 9, t = e - oi * 9, o = o0 + oi / IT, i = i0 + oi % IT;
-    if (o < c2 && i < c0) {
-      s *= raw_scale(a.l3, o);
-      if (last && dv.ident && o == i && t == 4) s += 1.f;
-      a.w_out[((size_t)o * c0 + i) * 9 + t] = s;
+    for (int w = 0; w < W; ++w) {
+      const float4 q = p[w * (F::TILE / 4)];
+      s.x += q.x; s.y += q.y; s.z += q.z; s.w += q.w;
     }
-    if (last && dv.mode > 0) mb_smem[e] = s;       // element e of warp 0's sums is read by this thread alone
+    const int oi = e / (IT * 9 / 4), x = (e - oi * (IT * 9 / 4)) * 4, o = o0 + oi;
+    if (o < c2 && i0 + x / 9 < c0) {
+      const float g3 = g3s[oi];
+      s.x *= g3; s.y *= g3; s.z *= g3; s.w *= g3;
+      if (last && dv.ident) {                      // 1 at tap 4 of channel o
+        const int at = (o - i0) * 9 + 4 - x;
+        if (at == 0) s.x += 1.f;
+        if (at == 1) s.y += 1.f;
+        if (at == 2) s.z += 1.f;
+        if (at == 3) s.w += 1.f;
+      }
+      *reinterpret_cast<float4 *>(a.w_out + ((size_t)o * c0 + i0) * 9 + x) = s;
+    }
+    if (last && dv.mode > 0) *p = s;               // these elements of warp 0's sums are read by this thread alone
   }
   if (!last || dv.mode == 0) return;
   __syncthreads();
@@ -942,29 +957,35 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
 // them with a structural zero (a gathered GEMM multiplies all 9 x 25 tap/position pairs, 64 % of which are).
 //
 // What bounds it is the FMA pipes, so nothing else may: a CTA owns 8 x 8 pairs, a thread of a warp 2 x 1 of them
-// (50 sums, 162 FMAs per c for 27 shared-memory reads, conflict-free because nine floats apart); the eight
-// warps take an eighth of the channels each and stage their own operands by cp.async in slices of 4 channels
-// (whole 16-byte pieces: the taps of neighbouring channels are contiguous in both operands), three deep,
-// without a CTA barrier until their sums meet in shared memory in warp order.  Small results therefore spread
-// over the chip as well (32 -> 32 -> 32: 16 CTAs, four channels a warp).
+// (50 sums, 162 FMAs per c for 27 shared-memory reads, conflict-free because nine floats apart).  The reduction
+// is cut into eight parts, one for each of eight warps or two for each of four (see the rule at the launch); a warp
+// stages its own operands by cp.async in slices of 4 channels (whole 16-byte pieces: the taps of neighbouring channels
+// are contiguous in both operands), three deep, without a CTA barrier until the parts' sums meet in shared memory, in
+// the order of the channels.  Small results therefore spread over the chip as well (32 -> 32 -> 32: 16 CTAs, four
+// channels a warp).
 //
 // BN of layers taken as they are: the first's scale rides on its taps, the second's on the sums.  An identity
 // riding on a piece adds W2 or W1 itself (and 1) to the sums.  Blocks behind the tiles compute the bias (8 output
 // channels each); behind those, for a packed result, the chunks without weights are zeroed.
 //
 // Tiles of 16 x 32 pairs with CTA barriers per slice, a fold launch before and a delivery after: c = 64 50 us,
-// 256 141 us, 512 859 us.  Here 7.6, 86 and 587 us (37 useful fp32 TFLOP/s: two thirds of the issue slots are taken,
-// a quarter of them by the operand reads; what holds the rest is the register file, whose banks the compiler cannot
-// keep apart for 50 sums).  Packed FMAs over the two output channels measured 106 us at c = 256, 80 registers and
-// three CTAs per SM 98.
+// 256 141 us, 512 859 us.  Here 5.9, 76 and 551 us (39 useful fp32 TFLOP/s: two thirds of the issue slots are taken, a
+// third of those by what is not an FMA; what holds the rest is the register file, whose banks the compiler cannot
+// keep apart for 50 sums).  With eight warps everywhere, sums added element by element, the second layer's scale asked
+// for behind them and 64-bit source pointers per copy: 7.6, 86 and 584 us, c = 32 6.4 (now 4.7); a fifth of the
+// instructions were those.  Packed FMAs over the two output channels measured 106 us at c = 256, 80 registers and
+// three CTAs per SM 98, the taps of two channels by 8-byte reads 1 % (and spills).
 // ----------------------------------------------------------------------------------------------
-constexpr int kP3O = 8, kP3I = 8, kP3Warps = 8, kP3Slice = 4, kP3Stages = 3;
-constexpr int kP3Threads = kP3Warps * 32;
+constexpr int kP3O = 8, kP3I = 8, kP3Parts = 8, kP3Slice = 4, kP3Stages = 3;
 constexpr int kP3Op = kP3O * kP3Slice * 9;                        // floats of one operand's slice: [o][c][9] or [c][i][9]
 constexpr int kP3Stage = 2 * kP3Op;
 constexpr int kP3Tile = kP3O * kP3I * 25;
-constexpr int kP3Ring = kP3Warps * kP3Stages * kP3Stage * 4;
-static_assert(kP3Ring >= kP3Warps * kP3Tile * 4, "the warps' sums reuse the rings");
+static_assert(kP3Stages * kP3Stage >= kP3Tile, "the warps' sums reuse the rings");
+// Floats of the rings of W warps, and with them the sums of the first of two parts of each warp
+template <int W>
+struct P3Form {
+  static constexpr int RING = W * kP3Stages * kP3Stage, BYTES = (RING + (W < kP3Parts ? W * kP3Tile : 0)) * 4;
+};
 
 struct Operand33 {
   RawLayer l;                    // weights, bias, BN (none for a piece)
@@ -977,8 +998,11 @@ struct Compose33 {
   int gi, go;                    // tiles
 };
 
-__global__ void __launch_bounds__(kP3Threads, 2)
+template <int W>
+__global__ void __launch_bounds__(W * 32, 16 / W)
 k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDelivery dv) {
+  constexpr int V = kP3Parts / W;                  // parts of the reduction that a warp takes, one after the other
+  static_assert(V == 1 || V == 2, "");
   extern __shared__ __align__(16) float p3_smem[];
   const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c0 = a.c0, c1 = a.c1, c2 = a.c2;
@@ -992,62 +1016,69 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
       return;
     }
     // ---- bias: b'[o] = b2~[o] + sum_c (g2 sum of W2[o][c] (+ 1 where c == o and an identity rides)) b1~[c]; a warp per o
-    const int o = blk * kP3O + warp;
-    if (o >= c2) return;
-    const float g2 = raw_scale(l2, o);
-    float s = 0.f;
+    for (int o = blk * kP3O + warp; o < c2 && o < (blk + 1) * kP3O; o += W) {
+      const float g2 = raw_scale(l2, o);
+      float s = 0.f;
 #pragma unroll 2
-    for (int c = lane; c < c1; c += 32) {
-      const float b1 = raw_bias(l1, c, raw_scale(l1, c));
-      float ws = (a.second.ident && c == o) ? 1.f : 0.f;
-      float wt = 0.f;
+      for (int c = lane; c < c1; c += 32) {
+        const float b1 = raw_bias(l1, c, raw_scale(l1, c));
+        float ws = (a.second.ident && c == o) ? 1.f : 0.f;
+        float wt = 0.f;
 #pragma unroll
-      for (int t = 0; t < 9; ++t) wt += l2.w[((size_t)o * c1 + c) * 9 + t];
-      s = fmaf(fmaf(g2, wt, ws), b1, s);
+        for (int t = 0; t < 9; ++t) wt += l2.w[((size_t)o * c1 + c) * 9 + t];
+        s = fmaf(fmaf(g2, wt, ws), b1, s);
+      }
+      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+      if (lane == 0) a.b_out[o] = raw_bias(l2, o, g2) + s;
     }
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if (lane == 0) a.b_out[o] = raw_bias(l2, o, g2) + s;
     return;
   }
   const int o0 = (blk / a.gi) * kP3O, i0 = (blk % a.gi) * kP3I;
-  const int per = ((c1 + kP3Warps - 1) / kP3Warps + 3) & ~3;
-  const int cb = warp * per, ce = cb + per < c1 ? cb + per : c1;
+  __shared__ float g2s[kP3O];                      // BN scales of the tile's output channels
+  if (tid < kP3O) g2s[tid] = o0 + tid < c2 ? raw_scale(l2, o0 + tid) : 0.f;
+  const int per = ((c1 + kP3Parts - 1) / kP3Parts + 3) & ~3;        // channels of a part
+  const int cb = warp * V * per, ce = cb + V * per < c1 ? cb + V * per : c1;
   const int nsl = ce > cb ? (ce - cb) / kP3Slice : 0;               // c1 is a multiple of 4
   float *ring = p3_smem + warp * (kP3Stages * kP3Stage);
-  // 72 pieces of each operand per slice: W2 rows of 36 floats (4 channels of one o), W1 rows of 72 (8 i of one channel)
-  const float *src[5];
-  int step[5];
+  // 72 pieces of each operand per slice: W2 rows of 36 floats (4 channels of one o), W1 rows of 72 (8 i of one channel).
+  // A lane's places in a slice stay the same, what moves is where the slice begins.
+  int off[5];
+  bool ok[5];
 #pragma unroll
   for (int h = 0; h < 5; ++h) {
     const int e = lane + 32 * h;
-    src[h] = nullptr;
-    step[h] = 0;
-    if (e < 72) {
+    if (h < 2 || (h == 2 && e < 72)) {
       const int o = e / 9, x = e - o * 9;
-      if (o0 + o < c2) { src[h] = l2.w + ((size_t)(o0 + o) * c1 + cb) * 9 + x * 4; step[h] = kP3Slice * 9; }
-    } else if (e < 144) {
+      off[h] = o * c1 * 9 + x * 4;
+      ok[h] = o0 + o < c2;
+    } else {
       const int f = e - 72, c = f / 18, x = f - c * 18;             // a piece lies inside one channel's 8 i: c0 is a multiple of 4
-      if (i0 * 9 + x * 4 < c0 * 9) { src[h] = l1.w + ((size_t)(cb + c) * c0 + i0) * 9 + x * 4; step[h] = kP3Slice * c0 * 9; }
+      off[h] = c * c0 * 9 + x * 4;
+      ok[h] = i0 * 9 + x * 4 < c0 * 9;
     }
   }
+  const float *w2g = l2.w + ((size_t)o0 * c1 + cb) * 9, *w1g = l1.w + ((size_t)cb * c0 + i0) * 9;
+  const int step1 = kP3Slice * c0 * 9;
   auto fetch = [&](int buf) {
-    float *st = ring + buf * kP3Stage;
+    float *st = ring + buf * kP3Stage + lane * 4;
 #pragma unroll
     for (int h = 0; h < 5; ++h) {
-      const int e = lane + 32 * h;
-      if (e < 144) mb_cp16(st + e * 4, src[h] ? src[h] : l2.w, src[h] != nullptr);
-      if (src[h]) src[h] += step[h];
+      const float *g = h < 2 || (h == 2 && lane < 8) ? w2g : w1g;
+      if (h < 4 || lane < 16) mb_cp16(st + h * 128, ok[h] ? g + off[h] : l2.w, ok[h]);
     }
+    w2g += kP3Slice * 9;
+    w1g += step1;
   };
 #pragma unroll
   for (int sl = 0; sl < kP3Stages - 1; ++sl) {
     if (sl < nsl) fetch(sl);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  // BN scale of the first layer: lane l holds channel l & 3's of a slice, asked for a slice ahead
+  // BN scale of the first layer: lane l holds channel l's of 32, asked for a slice ahead of the first that uses it
+  constexpr int kScaled = 32 / kP3Slice;         // slices that one set of scales covers
   float bn_g = 1.f, bn_v = 1.f;
-  auto ask = [&](int sl) {
-    const int cs = cb + sl * kP3Slice + (lane & 3), c = cs < ce ? cs : cb;
+  auto ask = [&](int set) {
+    const int cs = cb + set * 32 + lane, c = cs < ce ? cs : cb;
     if (l1.gamma) { bn_g = l1.gamma[c]; bn_v = l1.var[c]; }
   };
   auto scale = [&]() { return l1.gamma ? bn_g / sqrtf(bn_v + l1.eps) : 1.f; };
@@ -1055,10 +1086,18 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
   if (nsl > 0) { ask(0); sc = scale(); }
   const int ol = (lane >> 3) * 2, il = lane & 7;
   float acc[2][25] = {};
+  float *mine = p3_smem + (warp * kP3O + ol) * kP3I * 25 + il * 25;  // where this thread leaves its sums
+  auto leave = [&](float *at) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int t = 0; t < 25; ++t) at[h * kP3I * 25 + t] = acc[h][t];
+  };
   int buf = 0, fbuf = kP3Stages - 1;
 #pragma unroll 1
   for (int sl = 0; sl < nsl; ++sl) {
-    ask(sl + 1);                                   // past the end: the warp's first channel, not used
+    const int at = sl % kScaled;
+    if (at == kScaled - 1) ask(sl / kScaled + 1);  // past the end: the warp's first channel, not used
     asm volatile("cp.async.wait_group %0;" ::"n"(kP3Stages - 2) : "memory");
     __syncwarp();
     if (sl + kP3Stages - 1 < nsl) fetch(fbuf);
@@ -1066,7 +1105,7 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
     const float *w2 = ring + buf * kP3Stage + ol * (kP3Slice * 9), *w1 = ring + buf * kP3Stage + kP3Op + il * 9;
 #pragma unroll
     for (int c = 0; c < kP3Slice; ++c) {
-      const float s = __shfl_sync(0xffffffffu, sc, c);
+      const float s = __shfl_sync(0xffffffffu, sc, at * kP3Slice + c);
       float b[9], x[2][9];
 #pragma unroll
       for (int t = 0; t < 9; ++t) {
@@ -1086,40 +1125,64 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
               acc[1][(u1 + u2) * 5 + v1 + v2] = fmaf(x[1][u2 * 3 + v2], b[u1 * 3 + v1], acc[1][(u1 + u2) * 5 + v1 + v2]);
             }
     }
-    sc = scale();
+    if (at == kScaled - 1) sc = scale();
+    if (V == 2 && sl == per / kP3Slice - 1) {      // the end of the warp's first part: its sums wait behind the rings
+      leave(mine + P3Form<W>::RING);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int t = 0; t < 25; ++t) acc[h][t] = 0.f;
+    }
     __syncwarp();                                  // the slice's buffer may be refilled
     buf = buf + 1 == kP3Stages ? 0 : buf + 1;
     fbuf = fbuf + 1 == kP3Stages ? 0 : fbuf + 1;
   }
+  if (V == 2 && nsl < per / kP3Slice) {            // the reduction ends inside that part
+    leave(mine + P3Form<W>::RING);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int t = 0; t < 25; ++t) acc[h][t] = 0.f;
+  }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int t = 0; t < 25; ++t) p3_smem[warp * kP3Tile + ((ol + h) * kP3I + il) * 25 + t] = acc[h][t];
+  leave(mine);
   __syncthreads();
-  const bool last = dv.mode >= 0;
-  for (int e = tid; e < kP3Tile; e += kP3Threads) {
-    float s = 0.f;
+  const bool last = dv.mode >= 0, special = a.first.ident || a.second.ident || (last && dv.ident);
+  // four elements of the warps' sums at a time: 50 pieces to a row of 8 input channels, 25 to each 4 of them that exist
+  for (int e = tid; e < kP3Tile / 4; e += W * 32) {
+    float4 *p = reinterpret_cast<float4 *>(p3_smem) + e;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int w = 0; w < kP3Warps; ++w) s += p3_smem[w * kP3Tile + e];
-    const int oi = e / 25, t = e - oi * 25, o = o0 + oi / kP3I, i = i0 + oi % kP3I;
-    if (o < c2 && i < c0) {
-      const float g2 = raw_scale(l2, o);
-      s *= g2;
-      const int u = t / 5 - 1, v = t - (t / 5) * 5 - 1;              // tap of the 3x3 kernel centred in the 5x5 one
-      if (u >= 0 && u < 3 && v >= 0 && v < 3) {
-        if (a.first.ident) s = fmaf(g2, l2.w[((size_t)o * c1 + i) * 9 + u * 3 + v], s);                       // W2 o I
-        if (a.second.ident) s = fmaf(raw_scale(l1, o), l1.w[((size_t)o * c0 + i) * 9 + u * 3 + v], s);        // I o W1
-      }
-      if (t == 12 && o == i) s += (a.first.ident && a.second.ident ? 1.f : 0.f) + (last && dv.ident ? 1.f : 0.f);
-      a.w_out[((size_t)o * c0 + i) * 25 + t] = s;
+    for (int v = 0; v < kP3Parts; ++v) {           // in the order of the channels, whichever warp had them
+      const float4 q = p[v / V * (kP3Tile / 4) + (V == 2 && v % 2 == 0 ? P3Form<W>::RING / 4 : 0)];
+      s.x += q.x; s.y += q.y; s.z += q.z; s.w += q.w;
     }
-    if (last && dv.mode > 0) p3_smem[e] = s;       // element e of warp 0's sums is read by this thread alone
+    const int oi = e / (kP3I * 25 / 4), x = (e - oi * (kP3I * 25 / 4)) * 4, o = o0 + oi;
+    if (o < c2 && i0 + x / 25 < c0) {
+      const float g2 = g2s[oi];
+      s.x *= g2; s.y *= g2; s.z *= g2; s.w *= g2;
+      if (special) {                               // of a tile with identities to add
+        float v4[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int iw = (x + q) / 25, t = x + q - iw * 25, i = i0 + iw;
+          const int u = t / 5 - 1, v = t - (t / 5) * 5 - 1;          // tap of the 3x3 kernel centred in the 5x5 one
+          if (u >= 0 && u < 3 && v >= 0 && v < 3) {
+            if (a.first.ident) v4[q] = fmaf(g2, l2.w[((size_t)o * c1 + i) * 9 + u * 3 + v], v4[q]);                 // W2 o I
+            if (a.second.ident) v4[q] = fmaf(raw_scale(l1, o), l1.w[((size_t)o * c0 + i) * 9 + u * 3 + v], v4[q]);  // I o W1
+          }
+          if (t == 12 && o == i) v4[q] += (a.first.ident && a.second.ident ? 1.f : 0.f) + (last && dv.ident ? 1.f : 0.f);
+        }
+        s = make_float4(v4[0], v4[1], v4[2], v4[3]);
+      }
+      *reinterpret_cast<float4 *>(a.w_out + ((size_t)o * c0 + i0) * 25 + x) = s;
+    }
+    if (last && dv.mode > 0) *p = s;               // these elements are read by this thread alone
   }
   if (!last || dv.mode == 0) return;
   __syncthreads();
-  deliver_tile<kP3O, kP3I, 5>(dv, p3_smem, o0, i0, c0, c2, tid, kP3Threads);
+  deliver_tile<kP3O, kP3I, 5>(dv, p3_smem, o0, i0, c0, c2, tid, W * 32);
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -1209,7 +1272,8 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
 // output) and zero the packed chunks without weights.
 //
 // As fold, product, bias and delivery, four launches with the product written and read in between: 960 -> 320 -> 1280 60.7 us,
-// now 37.8; 32 -> 16 -> 96 7.5, now 4.1; 160 -> 160 -> 160 15.0, now 6.0.
+// now 30.1 (35.3 with the sums added element by element and the second layer's scales asked for
+// behind them); 32 -> 16 -> 96 7.5, now 3.2; 160 -> 160 -> 160 15.0, now 5.9.
 // ----------------------------------------------------------------------------------------------
 struct Merge11 {
   RawLayer l1, l2;
@@ -1250,6 +1314,9 @@ k_merge_11(const __grid_constant__ Merge11 a, const __grid_constant__ BlockDeliv
     return;
   }
   const int o0 = (blk / a.gi) * BO, i0 = (blk % a.gi) * BI;
+  const bool special = a.ident1 || a.ident2 || dv.ident;
+  __shared__ float g2s[BO];                        // BN scales of the tile's output channels
+  if (tid < BO) g2s[tid] = o0 + tid < c2 ? raw_scale(a.l2, o0 + tid) : 0.f;
   float *mine = sm + g * 2 * STAGE;
   const int slices = (c1 + KS - 1) / KS, my = (slices - g + G - 1) / G;      // slices g, g + G, ...
   float4 va[NA], vb[NB];
@@ -1325,20 +1392,31 @@ k_merge_11(const __grid_constant__ Merge11 a, const __grid_constant__ BlockDeliv
   for (int q = 0; q < TO; ++q)
     *reinterpret_cast<float4 *>(sm + (g * BO + ty * TO + q) * BI + tx * 4) = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
   __syncthreads();
-  for (int e = tid; e < BO * BI; e += 256) {
-    float s = 0.f;
+  for (int e = tid; e < BO * BI / 4; e += 256) {   // four elements of the groups' sums at a time; c0 is a multiple of 4
+    float4 *p = reinterpret_cast<float4 *>(sm) + e;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < G; ++q) s += sm[q * BO * BI + e];
-    const int o = o0 + e / BI, i = i0 + e % BI;
-    if (o < c2 && i < c0) {
-      const float g2 = raw_scale(a.l2, o);
-      s *= g2;
-      if (a.ident1) s = fmaf(g2, a.l2.w[(size_t)o * c1 + i], s);                        // g2 W2 I1: c0 == c1
-      if (a.ident2) s = fmaf(raw_scale(a.l1, o), a.l1.w[(size_t)o * c0 + i], s);        // I2 g1 W1: c1 == c2
-      if (o == i) s += (a.ident1 && a.ident2 ? 1.f : 0.f) + (dv.ident ? 1.f : 0.f);
-      a.w_out[(size_t)o * c0 + i] = s;
+    for (int q = 0; q < G; ++q) {
+      const float4 f = p[q * (BO * BI / 4)];
+      s.x += f.x; s.y += f.y; s.z += f.z; s.w += f.w;
     }
-    sm[e] = s;                                     // element e of group 0's sums is read by this thread alone
+    const int oi = e / (BI / 4), o = o0 + oi, i = i0 + e % (BI / 4) * 4;
+    if (o < c2 && i < c0) {
+      const float g2 = g2s[oi];
+      s.x *= g2; s.y *= g2; s.z *= g2; s.w *= g2;
+      if (special) {                               // of a tile with identities to add
+        float v4[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (a.ident1) v4[q] = fmaf(g2, a.l2.w[(size_t)o * c1 + i + q], v4[q]);                      // g2 W2 I1: c0 == c1
+          if (a.ident2) v4[q] = fmaf(raw_scale(a.l1, o), a.l1.w[(size_t)o * c0 + i + q], v4[q]);      // I2 g1 W1: c1 == c2
+          if (o == i + q) v4[q] += (a.ident1 && a.ident2 ? 1.f : 0.f) + (dv.ident ? 1.f : 0.f);
+        }
+        s = make_float4(v4[0], v4[1], v4[2], v4[3]);
+      }
+      *reinterpret_cast<float4 *>(a.w_out + (size_t)o * c0 + i) = s;
+    }
+    *p = s;                                        // these elements of group 0's sums are read by this thread alone
   }
   if (dv.mode == 0) return;
   __syncthreads();
@@ -1565,13 +1643,23 @@ struct MergeStatus {
   void launched() { note(cudaGetLastError()); }
 };
 
+template <int W>
+static void launch_compose33_form(const Compose33 &a, const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
+  static unsigned char attr_done[kDcMaxDevices];
+  status.note(dc_set_max_smem_once(k_compose33<W>, P3Form<W>::BYTES, attr_done));
+  status.note(dc_launch_pdl(k_compose33<W>, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, W * 32)), dim3(W * 32), P3Form<W>::BYTES, st, a, dv));
+  status.launched();
+}
+// Four warps a tile, four tiles to an SM at once, except where the tiles of the SM with the most of them fill whole rounds of
+// two better than of four: one, two or five of them, or three with a reduction long enough (136 -> 136 -> 136, two tiles: 18.1 us by
+// eight warps; 208 -> 208 -> 208, five: 56.1 us by four, 49.3 by eight; 160 -> 160 -> 160, three: 28.9 and 24.4, with 48 channels between
+// 12.9 and 13.4; 192 -> 192 -> 192, four: 34.2 and 35.4; 512 -> 128 -> 512, 28: 158 and 170).
 static void launch_compose33(const Operand33 &first, const Operand33 &second, int c0, int c1, int c2, float *w, float *b,
                              const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
-  static unsigned char attr_done[kDcMaxDevices];
-  status.note(dc_set_max_smem_once(k_compose33, kP3Ring, attr_done));
-  status.note(dc_launch_pdl(k_compose33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kP3Threads)), dim3(kP3Threads), kP3Ring, st, a, dv));
-  status.launched();
+  const int most = dc_div_up(a.gi * a.go, dc_sm_count());
+  if (most <= 2 || most == 5 || (most == 3 && c1 >= 128)) launch_compose33_form<8>(a, dv, mg, st, status);
+  else launch_compose33_form<4>(a, dv, mg, st, status);
 }
 
 template <int IT, int W>

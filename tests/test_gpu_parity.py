@@ -312,6 +312,14 @@ def test_blocks_by_sixteen_warps_against_the_oracle(dc, c, hidden):
                          I.make_layer(83, 2, hidden, c, 1, 1, 0)], [(0, 2)], (dc.BF16, dc.F32))
 
 
+@pytest.mark.parametrize("a,c,o,res", [(152, 4, 160, []), (160, 20, 148, []), (148, 36, 152, []), (152, 152, 152, [(0, 0), (1, 1)]),
+                                       (152, 152, 152, [(0, 1)]), (200, 132, 256, [])])
+def test_3x3_after_3x3_by_four_warps_against_the_oracle(dc, a, c, o, res):
+    """More tiles than two to an SM: warps with two parts of the reduction, with one, with one that is cut short, with none."""
+    _check_delivery(dc, [I.make_layer(84, 0, a, c, 3, 1, 1), I.make_layer(84, 1, c, o, 3, 1, 1)], res,
+                    (dc.BF16, dc.F32) if a % 8 == 0 and o % 8 == 0 else (dc.F32,))
+
+
 @pytest.mark.parametrize("case", ["block", "dense_pair", "expand_dw"])
 @pytest.mark.parametrize("alias", ["weights", "bias", "packed"])
 def test_merge_into_its_layers_arrays(dc, case, alias):
