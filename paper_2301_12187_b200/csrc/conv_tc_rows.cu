@@ -37,6 +37,7 @@ constexpr int kEpiWarps = 8;
 constexpr int kConsumerThreads = (kMmaWarps + kEpiWarps) * 32;
 constexpr int kThreads = 32 + kConsumerThreads;
 constexpr int kBarConsumers = 7;                 // named barrier of all consumer warps
+constexpr int kMaxSplit = 8;                     // CTAs that share an item
 constexpr int kMaxBlocks = 2;                    // 128-row blocks per tile
 constexpr int kStagePitch = 64;                  // bytes per pixel in an epilogue warp's turn-around buffer (pieces XOR-swizzled)
 
@@ -119,7 +120,13 @@ struct Item {
 // SPLITK: a cluster of p.ksplit CTAs shares one work item, each taking a run of its (plane, tap row) steps, for layers
 // with fewer items than SMs whose reduction is long (384 -> 64 3x3 on one 14 x 14 image is one item of 432
 // instructions per block).  The partial sums meet in distributed shared memory -- in the rings' place, which nothing
-// reads any more -- and are added in rank order; every CTA finishes its share of the outputs.
+// reads any more -- and are added in rank order; every CTA finishes its share of the outputs.  What bounds it is a chain:
+// of the 11000 cycles of 960 -> 160 1x1 on one 7 x 7 image 1300 went into bias rows before the first instruction, 3000 into
+// the sums of the other CTAs (a lane read 16 of every 32 bytes of theirs, twice) and 1300 into a last meeting that waited for
+// the results to be stored.  Now one CTA fetches the bias, and only of its pass; a stage's first use waits for nothing;
+// lanes read neighbouring 16-byte pieces, all CTAs' before the first is added; the last meeting orders only reads.
+// 960 -> 160 6.3 -> 4.6 us, 960 -> 1280 9.9 -> 6.6, 384 -> 64 3x3 at 14 x 14 6.5 -> 5.4, 96 -> 144 5x5 of stride 2 at 56 x 56
+// 9.6 -> 7.6, 960 -> 160 on 20 images 9.5 -> 6.1 (shared only now).  The unsplit forms are faster without these (up to 8 %).
 //
 // S2: stride 2.  A plane of 64 channels is four sub-tiles of every second row and column of the patch (tensor map with
 // element strides 2, one load each), and tap (r, s) reads sub-tile (r & 1, s & 1) at row r >> 1, column s >> 1: each
@@ -180,6 +187,8 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
     else if (t == 96) { sh.abort = 0; mbar_init(&sh.b_all, 1); prefetch_tensormap(&map_a); did = true; }
     if (did) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  Item first;                                    // SPLITK: the CTA's item, worked out while the previous kernel ends
+  if (SPLITK) first.of(p, item0);
   dc_pdl_enter();                                // nothing above touched global memory; everything below may
   __syncthreads();
 
@@ -192,6 +201,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
       const char *wsrc = reinterpret_cast<const char *>(w_packed);
       int sa = 0, sb = 0;
       uint32_t pa = 0, pb = 0;
+      bool a_used = false, b_used = false;       // the rings have been filled once
       bool ok = true;
       if (RESIDENT && lane == 0) {               // the whole packed buffer once
         const uint32_t all = (uint32_t)(p.planes_all * p.n_tile * 16);
@@ -201,18 +211,19 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
 #pragma unroll 1
       for (int it = 0; it < nitems && ok; ++it) {
         Item q;
-        q.of(p, item0 + it);
+        if (SPLITK) q = first; else q.of(p, item0 + it);
 #pragma unroll 1
         for (int v = v_lo; v < v_hi && ok; ++v) {
           const Plane pl(p, v, S2);
-          if (!warp_wait(&sh.a_empty[sa], pa ^ 1, abort_flag, ws, 0x10000u | sa)) { ok = false; break; }
+          // (SPLITK: a stage's first use, often its only one, waits for nothing)
+          if ((!SPLITK || a_used) && !warp_wait(&sh.a_empty[sa], pa ^ 1, abort_flag, ws, 0x10000u | sa)) { ok = false; break; }
           if (lane == 0) {
             // channels past c_in, pixels outside the image and images past the batch arrive as zeros
             mbar_arrive_expect_tx(&sh.a_full[sa], (uint32_t)p.a_box_bytes);
             tma_load_4d(a_base0 + (uint32_t)(sa * p.a_stage_bytes + p.front), &map_a, &sh.a_full[sa], 64 * pl.g,
                         (S2 ? 2 : 1) * q.xt * p.tw - (p.share ? 0 : p.pad) + pl.px, (S2 ? 2 : 1) * q.ty * p.th - p.pad + pl.py, q.img0);
           }
-          if (++sa == p.sa) { sa = 0; pa ^= 1; }
+          if (++sa == p.sa) { sa = 0; pa ^= 1; a_used = true; }
           const int nsl = plane_steps(p, pl.g);
           const int nplanes = (PARTIAL ? 1 : pl.kc) * nsl * 2;     // chunk planes of one weight stage
           const int nstages = PARTIAL ? pl.kr * pl.kc : pl.kr;
@@ -221,7 +232,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
           size_t plane0 = (size_t)pl.g * p.k * p.k * 8 + (size_t)(pl.tap0 * nsl * 2) + (size_t)r_lo * nplanes;
 #pragma unroll 1
           for (int r = r_lo; r < r_hi && !RESIDENT; ++r, plane0 += nplanes) {
-            if (!warp_wait(&sh.b_empty[sb], pb ^ 1, abort_flag, ws, 0x20000u | sb)) { ok = false; break; }
+            if ((!SPLITK || b_used) && !warp_wait(&sh.b_empty[sb], pb ^ 1, abort_flag, ws, 0x20000u | sb)) { ok = false; break; }
             // the planes of a stage are contiguous in the packed weights, with several passes too (there a
             // pass's rows of all planes are stored together): one bulk copy
             if (lane == 0) {
@@ -230,13 +241,13 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
               bulk_load(b_base0 + (uint32_t)sb * (uint32_t)p.b_stage_bytes,
                         wsrc + ((size_t)q.nt * p.planes_all + plane0) * p.n_tile * 16, bytes, &sh.b_full[sb]);
             }
-            if (++sb == p.sb) { sb = 0; pb ^= 1; }
+            if (++sb == p.sb) { sb = 0; pb ^= 1; b_used = true; }
           }
         }
       }
     }
     __syncwarp();
-    if (SPLITK) { cluster_sync(); cluster_sync(); }
+    if (SPLITK) { cluster_sync(); cluster_meet_relaxed(); }
   } else {
     // ---- consumer preparation
     if (warp == kMmaWarp) {
@@ -253,8 +264,15 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
         const int r = t >> 3, c = t & 7;
         reinterpret_cast<uint4 *>(smem_ones)[t] = c == r ? bias_ones() : make_uint4(0u, 0u, 0u, 0u);
       }
-      for (int t = t0; t < p.n_pad + p.n_tile; t += kEpiWarps * 32)
-        reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && t < p.c_out ? bias[t] : 0.f);
+      if (SPLITK) {                              // the item's pass where it is added, and the zero rows
+        if (rank == 0)
+          for (int t = first.nt * p.n_tile + t0; t < (first.nt + 1) * p.n_tile; t += kEpiWarps * 32)
+            reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && t < p.c_out ? bias[t] : 0.f);
+        for (int t = t0; t < p.n_tile; t += kEpiWarps * 32) reinterpret_cast<uint4 *>(smem_bias)[p.n_pad + t] = make_uint4(0u, 0u, 0u, 0u);
+      } else {
+        for (int t = t0; t < p.n_pad + p.n_tile; t += kEpiWarps * 32)
+          reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && t < p.c_out ? bias[t] : 0.f);
+      }
       // zeros around the patches, which the loads never touch
       if (p.share) {
         const int per = (p.front + p.tail) >> 4;
@@ -300,7 +318,7 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
         {
           // bias first (needs no load): it also initialises the accumulators of this warp's blocks
           Item iq;
-          iq.of(p, item0 + it);
+          if (SPLITK) iq = first; else iq.of(p, item0 + it);
           // (with the reduction split, one CTA adds the bias and the others start from zero rows)
           const uint32_t bias_row = SPLITK && rank > 0 ? zero_row : bias_row0 + (uint32_t)(iq.nt * p.n_tile);
           const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)((bias_row & 0x3FFFu) | ((zero_row - bias_row) << 16));
@@ -406,11 +424,11 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
         tc_fence_after();
         const uint32_t part = smem_u32(smem_a);
 #pragma unroll 1
-        for (int b = par; b < p.mb; b += 2) {
+        for (int b = p.mb == 1 ? 0 : par; b < p.mb; b += 2) {   // one block: the two warps of a quadrant take its columns in turn
           const uint32_t row = part + (uint32_t)(b * 128 + q * 32 + lane) * (uint32_t)(p.part_pitch * 4);
           const uint32_t taddr = tmem_row + (uint32_t)(b * p.n_tile);
 #pragma unroll 1
-          for (int ch = 0; ch < p.n_tile; ch += 16) {
+          for (int ch = p.mb == 1 ? par * 16 : 0; ch < p.n_tile; ch += p.mb == 1 ? 32 : 16) {
             uint32_t v[16];
             tmem_ld16(taddr + (uint32_t)ch, v);
             tmem_ld_wait();
@@ -525,50 +543,50 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
     if (SPLITK) {
       cluster_sync();                              // every CTA's partial sums are written
       if (warp >= kFirstEpiWarp && !*abort_flag) {
-        Item iq;
-        iq.of(p, item0);
+        const Item iq = first;
         const int x0 = iq.xt * p.tw, y0 = iq.ty * p.th;
         const int tw_valid = p.wo - x0 < p.tw ? p.wo - x0 : p.tw;
         const int th_valid = p.ho - y0 < p.th ? p.ho - y0 : p.th;
         const int ch0 = iq.nt * p.n_tile;
-        const int chunks = (p.c_out - ch0 < p.n_tile ? p.c_out - ch0 : p.n_tile) >> 3;
+        const int quads = (p.c_out - ch0 < p.n_tile ? p.c_out - ch0 : p.n_tile) >> 2;
         const uint32_t part = smem_u32(smem_a);
         const bool relu6 = p.act == DC_ACT_RELU6;
-        // 8 channels of a pixel at a time, dealt out over the threads of the whole cluster
+        // 4 channels of a pixel at a time, dealt out over the threads of the whole cluster: lanes read 16 neighbouring bytes
 #pragma unroll 1
-        for (int u = rank * (kEpiWarps * 32) + (int)threadIdx.x - kFirstEpiWarp * 32; u < p.mb * 128 * chunks; u += p.ksplit * kEpiWarps * 32) {
-          const int pos = u / chunks, ch = (u - pos * chunks) * 8;
+        for (int u = rank * (kEpiWarps * 32) + (int)threadIdx.x - kFirstEpiWarp * 32; u < p.mb * 128 * quads; u += p.ksplit * kEpiWarps * 32) {
+          const int pos = u / quads, ch = (u - pos * quads) * 4;
           const int il = (int)(((uint32_t)pos * p.inv_lines) >> 20), rem = pos - il * p.lines_img;
           const int yy = (int)(((uint32_t)rem * p.inv_wbox) >> 20), xx = rem - yy * p.wbox;
           if (il >= p.ni || iq.img0 + il >= p.n_img || yy >= th_valid || xx >= tw_valid) continue;
           const uint32_t at = part + (uint32_t)(pos * p.part_pitch + ch) * 4u;
-          float f[8] = {};
-#pragma unroll 4
-          for (int r = 0; r < p.ksplit; ++r) {
-            const uint32_t remote = map_cluster(at, (uint32_t)r);
-            const uint4 lo = lds_cluster_u4(remote), hi = lds_cluster_u4(remote + 16u);
-            f[0] += __uint_as_float(lo.x); f[1] += __uint_as_float(lo.y); f[2] += __uint_as_float(lo.z); f[3] += __uint_as_float(lo.w);
-            f[4] += __uint_as_float(hi.x); f[5] += __uint_as_float(hi.y); f[6] += __uint_as_float(hi.z); f[7] += __uint_as_float(hi.w);
-          }
+          uint4 v[kMaxSplit];                      // all are asked for before the first is added
+#pragma unroll
+          for (int r = 0; r < kMaxSplit; ++r)
+            if (r < p.ksplit) v[r] = lds_cluster_u4(map_cluster(at, (uint32_t)r));
+          float f[4] = {};
+#pragma unroll
+          for (int r = 0; r < kMaxSplit; ++r)
+            if (r < p.ksplit) {
+              f[0] += __uint_as_float(v[r].x); f[1] += __uint_as_float(v[r].y);
+              f[2] += __uint_as_float(v[r].z); f[3] += __uint_as_float(v[r].w);
+            }
           const size_t o = ((size_t)((iq.img0 + il) * p.ho + (y0 + yy)) * p.wo + (x0 + xx)) * p.c_out + ch0 + ch;
           if (residual) {
-            const uint4 rv = *reinterpret_cast<const uint4 *>(residual + o);
+            const uint2 rv = *reinterpret_cast<const uint2 *>(residual + o);
             const __nv_bfloat162 *rb = reinterpret_cast<const __nv_bfloat162 *>(&rv);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 2; ++i) {
               const float2 rf = __bfloat1622float2(rb[i]);
               f[2 * i] += rf.x; f[2 * i + 1] += rf.y;
             }
           }
-          uint4 ov;
-          uint32_t *ow = reinterpret_cast<uint32_t *>(&ov);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            ow[i] = relu6 ? relu6_bf16x2(f[2 * i], f[2 * i + 1]) : pack_bf16x2(f[2 * i], f[2 * i + 1]);
-          *reinterpret_cast<uint4 *>(y + o) = ov;
+          uint2 ov;
+          ov.x = relu6 ? relu6_bf16x2(f[0], f[1]) : pack_bf16x2(f[0], f[1]);
+          ov.y = relu6 ? relu6_bf16x2(f[2], f[3]) : pack_bf16x2(f[2], f[3]);
+          *reinterpret_cast<uint2 *>(y + o) = ov;
         }
       }
-      cluster_sync();                              // nobody leaves while its sums may still be read
+      cluster_meet_relaxed();                      // nobody leaves while its sums may still be read
     }
     // ---- consumer teardown
     if (*abort_flag) {
@@ -628,7 +646,6 @@ int rows_fixed_bytes(const KOrder &ko, int *off_stage) {
 
 // Clusters of `size` CTAs (an SM's shared memory each) the current device runs at once: a property of its GPCs, asked for
 // once per device.  Without a device (planning on the host): a B200's.
-constexpr int kMaxSplit = 8;
 int max_clusters(int size) {
   static constexpr int kB200[kMaxSplit + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
   static int cached[kDcMaxDevices][kMaxSplit + 1];
@@ -688,13 +705,17 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
   // overlap in part, and a chain of waits; a shared item costs the meeting of its partial sums, which grows with the
   // CTAs and the bytes.  The constants are fitted to 41 layers timed in every tile and split considered here (1 to 128
   // images of 49 to 12544 pixels).  Timed again on 32 layers: the choice is 2 % above the best on
-  // average, 21 % at worst (160 -> 96 3x3 of stride 2, 64 images of 14 x 14).
+  // average, 21 % at worst (160 -> 96 3x3 of stride 2, 64 images of 14 x 14).  Whether a split beats the best tile by itself is
+  // asked with terms of its own, fitted to 237 layers of 1 to 128 images (20 to 6272 pixels) in up to nine tiles and splits:
+  // 1.2 % above the best of those on average, 1.19 times at worst, none more than 3 % slower than unsplit; with the one
+  // estimate that both shared before, fitted to a meeting of twice the time, 4.9 % and 1.64 times.
   // Candidates: every strip count that leaves rows of at most 256 pixels, with as many rows as give two blocks or
   // one, evened out over the height; whole small images several at a time.
   const int cyc = 36 + p->n_tile / 4 > p->n_tile / 2 ? 36 + p->n_tile / 4 : p->n_tile / 2;
   const double per_block = (double)g->k * g->k * dc_div_up(g->c_in, 16) * cyc;
   const double w_item = (double)ko.e_pad * p->n_tile * 16;
-  double best = 0.0;
+  double best = 0.0, best_shared = 0.0;          // of the best tile by itself; the same tile beside the shared ones
+  struct { double cost; int nxt, tw, th, ni, ksplit; } sp = {0.0, 0, 0, 0, 0, 1};      // the best shared one
   p->nxt = 0;
   p->ksplit = 1;
   const int fixed_part = kSmemBudget - 1024 - p->off_a;     // bytes of the rings, where partial sums would go
@@ -728,17 +749,28 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
     const long long whole = (long long)dc_round_up((size_t)(g->k * tap_bytes), 1024);
     const bool columns = S == 1 && g->k > 1 && 2048 + p->off_a + 2 * whole + 2 * stage_bytes(lines, ni, wbox, share) > kSmemBudget;
     const double waits = columns ? 150.0 * (double)per_cta * p->planes * g->k * g->k : 0.0;
-    for (int split = 1; split <= kMaxSplit; ++split) {
+    auto estimate = [&](int split, double more) {
+      const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
+      const double ctas = (double)(items * split < n_sm ? items * split : n_sm);
+      return (m > l ? m + 0.77 * l : l + 0.77 * m) + waits / split + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + more;
+    };
+    // Beside the shared items a step and a plane have a price of their own, and a shared one pays for the meeting: the CTAs
+    // that meet, the sums that each writes and reads and the results.
+    auto shared = [&](int split) {
+      const int steps = dc_div_up(p->planes * g->k * S, split), pl = dc_div_up(p->planes, split);
+      const double sums = p->n_tile * (0.5 * ni * th * tw + mb * 128 * (0.2 + 0.5 / split));
+      return estimate(split, (double)per_cta * (600.0 * steps + 800.0 * pl) + 3.9 * lines * ni + (split > 1 ? 500.0 + 200.0 * split + sums : 0.0));
+    };
+    const double alone = estimate(1, 0.0);
+    if (p->nxt == 0 || alone < best) { best = alone; best_shared = shared(1); p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; }
+    for (int split = 2; split <= kMaxSplit; ++split) {
       // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
       if (split == 7) continue;                  // no more clusters of seven than of eight run at once (15 each)
-      if (split > 1 && (items * split > n_sm || items > max_clusters(split) || p->planes * (S == 2 ? 4 : g->k) < split ||
-                        mb * 128 * (p->n_tile + 4) * 4 > fixed_part))
+      if (items * split > n_sm || items > max_clusters(split) || p->planes * (S == 2 ? 4 : g->k) < split ||
+          mb * 128 * (p->n_tile + 4) * 4 > fixed_part)
         break;
-      const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
-      const double meet = split > 1 ? 450.0 + 580.0 * split + (double)ni * th * tw * p->n_tile * 0.8 : 0.0;
-      const double ctas = (double)(items * split < n_sm ? items * split : n_sm);
-      const double cost = (m > l ? m + 0.77 * l : l + 0.77 * m) + waits / split + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + meet;
-      if (p->nxt == 0 || cost < best) { best = cost; p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->ksplit = split; }
+      const double cost = shared(split);
+      if (sp.ksplit == 1 || cost < sp.cost) sp = {cost, nxt, tw, th, ni, split};
     }
   };
   // The fewest strips whose tile of one output row is within the tensor map's box (256 pixels) and the activation ring
@@ -776,6 +808,7 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
       for (int ni = 2; ni <= 8 && ni <= n; ++ni) consider(wo, ho, ni);
   }
   if (p->nxt == 0) return false;
+  if (sp.ksplit > 1 && sp.cost < best_shared) { p->nxt = sp.nxt; p->tw = sp.tw; p->th = sp.th; p->ni = sp.ni; p->ksplit = sp.ksplit; }
   const int th = p->th;
   p->share = may_share && p->tw == wo;
   p->wbox = p->share ? p->tw + g->pad : p->tw + halo;

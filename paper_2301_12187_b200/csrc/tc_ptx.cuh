@@ -256,6 +256,11 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
+// the same, for a meeting that orders nothing but what this thread has read, and used, before
+__device__ __forceinline__ void cluster_meet_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+  asm volatile("barrier.cluster.wait;" ::: "memory");
+}
 // the address of this CTA's shared address `a` in CTA `rank` of the cluster, and a 16-byte read there
 __device__ __forceinline__ uint32_t map_cluster(uint32_t a, uint32_t rank) {
   uint32_t d;

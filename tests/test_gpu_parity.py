@@ -757,6 +757,19 @@ def test_rows_with_a_shared_reduction_against_the_oracle(dc, c_in, c_out, k, s, 
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
+    (960, 1280, 1, 1, 0, 1, 7, 7),       # passes of the widest tile: most sums to read, one block
+    (960, 1280, 1, 1, 0, 2, 15, 13),     # two blocks
+    (320, 40, 1, 1, 0, 2, 30, 29),       # five planes, a ragged last tile
+    (272, 328, 1, 1, 0, 2, 5, 5),        # a last pass with fewer channels than the tile, a plane of 16
+    (128, 64, 3, 1, 1, 20, 13, 13),      # few steps, many items
+    (1024, 40, 1, 1, 0, 1, 3, 3),        # few outputs: most threads have nothing to add
+    (720, 72, 5, 1, 2, 1, 9, 31),        # the rings go round several times
+])
+def test_shared_reductions_of_few_and_many_sums(dc, c_in, c_out, k, s, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
+
+
+@pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (96, 144, 5, 2, 2, 9, 57, 50),       # several tiles per image and per CTA, odd height
     (96, 144, 5, 2, 2, 1, 20, 20),       # the reduction shared by a cluster
     (40, 32, 3, 2, 1, 40, 28, 28),       # one image per tile, runs cut by blocks
