@@ -273,14 +273,14 @@ __device__ __forceinline__ void rows_body(const CUtensorMap &map_a, const RowsPa
         for (int t = t0; t < p.n_pad + p.n_tile; t += kEpiWarps * 32)
           reinterpret_cast<uint4 *>(smem_bias)[t] = bias_terms(bias && t < p.c_out ? bias[t] : 0.f);
       }
-      // zeros around the patches, which the loads never touch
+      // zeros around the patches, which the loads never touch, in the stages that this CTA fills
       if (p.share) {
-        const int per = (p.front + p.tail) >> 4;
-        for (int t = t0; t < p.sa * per; t += kEpiWarps * 32) {
-          const int st = t / per, e = t - st * per;
-          uint8_t *at = smem_a + st * p.a_stage_bytes + (e * 16 < p.front ? e * 16 : p.a_box_bytes + e * 16);
-          *reinterpret_cast<uint4 *>(at) = make_uint4(0u, 0u, 0u, 0u);
-        }
+        const int per = (p.front + p.tail) >> 4, fills = nitems * (v_hi - v_lo), used = fills < p.sa ? fills : p.sa;
+        for (int st = 0; st < used; ++st)
+          for (int e = t0; e < per; e += kEpiWarps * 32) {
+            uint8_t *at = smem_a + st * p.a_stage_bytes + (e * 16 < p.front ? e * 16 : p.a_box_bytes + e * 16);
+            *reinterpret_cast<uint4 *>(at) = make_uint4(0u, 0u, 0u, 0u);
+          }
       }
       fence_proxy_async();                       // all are read by the tensor core (async proxy)
     }
