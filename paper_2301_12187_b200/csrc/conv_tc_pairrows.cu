@@ -413,6 +413,12 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
     else if (t == 64) { mbar_init(&sh.weights, 1); sh.abort = 0; prefetch_tensormap(&map_a); did = true; }
     if (did) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // What comes between the start of the call and its first tile is time that nothing overlaps: where the first tile lies is
+  // worked out while the previous kernel ends, it is asked for before the weights, and a stage's first use waits for
+  // nothing: 24 -> 24, 64 images of 56 x 56 8.52 -> 8.16 us, 24 -> 32 of stride 2, 128 images 8.56 -> 8.27, 32 -> 32, 51 of 25 x 25
+  // 5.39 -> 5.26; 32 -> 32, 256 of 56 x 56 28.5 -> 28.8.
+  Walk first;
+  first.start(p, tile0);
   dc_pdl_enter();                                // nothing above touched global memory; everything below may
   __syncthreads();
 
@@ -434,6 +440,7 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
       }
     };
     if (lane == 0) {
+      request(first, 0);                         // the first tile comes from further away than the weights
       mbar_arrive_expect_tx(&sh.weights, (uint32_t)p.b_bytes);
       bulk_load(smem_u32(smem_b), w_packed, (uint32_t)p.b_bytes, &sh.weights);   // packed weights are the operand layout
     }
@@ -441,10 +448,9 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
     if (ODD) {
       // the whole warp: request tiles ahead, then finish the oldest one.  The stage asked for last belonged to
       // a tile that is finished already (inflight <= stages), so the waits below always end.
-      Walk ahead, t;
-      ahead.start(p, tile0);
-      t.start(p, tile0);
-      int asked = 0, sl = 0, s = 0;
+      Walk ahead = first, t = first;
+      ahead.step(p);
+      int asked = 1, sl = 1, s = 0;             // there are two stages at least
       uint32_t phl = 0, ph = 0;
       bool ok = true;
 #pragma unroll 1
@@ -475,13 +481,13 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
         if (++s == p.stages) { s = 0; ph ^= 1; }
       }
     } else if (lane == 0) {
-      Walk t;
-      t.start(p, tile0);
-      int s = 0;
+      Walk t = first;
+      t.step(p);
+      int s = 1;                                 // there are two stages at least
       uint32_t ph = 0;
 #pragma unroll 1
-      for (int it = 0; it < ntiles; ++it) {
-        if (!mbar_wait(&sh.empty[s], ph ^ 1, abort_flag, ws, 0x10000u | s)) break;
+      for (int it = 1; it < ntiles; ++it) {
+        if (it >= p.stages && !mbar_wait(&sh.empty[s], ph ^ 1, abort_flag, ws, 0x10000u | s)) break;
         // At most kInFlight tiles are on their way: every CTA starts at the same moment, and if
         // each asked for all its tiles at once the first tile (which the tensor core is waiting
         // for) would arrive together with the last.
@@ -547,8 +553,7 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
       // next block of this warp (warps beyond mma_warps take none, they only hand the stages back);
       // first block of the tile
       int next = mw < p.mma_warps ? mw : 0x40000000, c0 = 0;
-      Walk t;
-      t.start(p, tile0);
+      Walk t = first;
 #pragma unroll 1
       for (int it = 0; it < ntiles && ok; ++it) {
         const int nblk = t.nblk(p);
