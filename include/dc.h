@@ -252,6 +252,18 @@ dc_status dc_block_forward(const void *x, int n, int h, int w, const dc_block *b
                            dc_stream stream);
 
 /*
+ * Host only, launches nothing: how the one-launch kernel would run a DC_BF16 block of aligned, separate arrays, for reports and
+ * tests; DC_ERR_UNSUPPORTED where the block runs as three launches.
+ */
+typedef struct {
+  int tile_w, tile_h, tile_images, tiles;  /* outputs of a tile, tiles in all */
+  int chunks;                              /* of hidden channels, per tile */
+  int form, groups;                        /* form of the kernel, groups of warps that take the chunks in turn */
+  int operands, stages;                    /* buffers of the projection's operand, stages of the weights */
+} dc_block_plan;
+dc_status dc_block_plan_query(int n, int h, int w, const dc_block *blk, dc_dtype dtype, dc_block_plan *plan);
+
+/*
  * Synchronises `stream`, then returns the status latched in the first word of `workspace`
  * (DC_OK or DC_ERR_TIMEOUT) and clears it.
  */
@@ -277,6 +289,15 @@ dc_status dc_workspace_status_where(void *workspace, dc_stream stream, unsigned 
  */
 dc_status dc_selftest_bounded_wait(void *workspace, size_t workspace_bytes, unsigned int limit_us,
                                    dc_stream stream);
+
+/*
+ * Host only, launches nothing: what the block kernel's stencil waits for in front of its CTA's chunk number `chunk` with this many
+ * buffers of the projection's operand (1 or 2) and stages of weights (2..4), as the kernel itself works it out.
+ * waits[0..2]: the chunk's buffer, and the barrier and parity of its phase on both sides; then for each wait, in order: what for
+ * (0: that barrier says the operand is free, 1: the weights), the barrier's index, the parity.  Returns the number of waits,
+ * three at most (0: arguments out of range).
+ */
+int dc_selftest_block_waits(unsigned int chunk, int operands, int stages, unsigned int waits[12]);
 
 /*
  * Host only: the layout in which dc_chain_forward_host keeps a run's parameters on the device:

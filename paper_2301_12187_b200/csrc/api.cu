@@ -132,6 +132,13 @@ extern "C" dc_status dc_block_workspace_bytes(int n, int h, int w, const dc_bloc
   return DC_OK;
 }
 
+extern "C" dc_status dc_block_plan_query(int n, int h, int w, const dc_block *b, dc_dtype dtype, dc_block_plan *plan) {
+  dc_status s = check_block(n, h, w, b, dtype);
+  if (s != DC_OK) return s;
+  if (!plan) return DC_ERR_INVALID_ARG;
+  return dtype == DC_BF16 ? dc_block_tc_plan(n, h, w, b, plan) : DC_ERR_UNSUPPORTED;
+}
+
 // The one-launch block kernel reads its operands as long as it writes y, and 16 bytes at a time: pointers that are not
 // aligned (which the launches of the three layers report) and outputs that overlap an input go through the workspace.
 static bool one_launch_block(const void *x, int n, int h, int w, int ho, int wo, const dc_block *b, const void *y) {

@@ -486,6 +486,7 @@ bool dc_conv_stem_s2_supported(int n, int h, int w, const dc_geom *g);
 // a whole inverted-residual block (bf16); DC_ERR_UNSUPPORTED: outside its range, the three layers run one by one
 dc_status dc_launch_block_tc(const void *x, int n, int h, int w, const dc_block *b, void *y, void *workspace,
                              cudaStream_t stream);
+dc_status dc_block_tc_plan(int n, int h, int w, const dc_block *b, dc_block_plan *plan);
 bool dc_dwconv_stencil_supported(int n, int h, int w, int c, int k, int stride, int pad);
 dc_status dc_launch_dwconv_stencil(const void *x, int n, int h, int w, int c, int k, int stride, int pad, const float *wp,
                                    const float *bias, dc_act act, void *y, cudaStream_t st);

@@ -116,6 +116,27 @@ struct Ring {
   __device__ __forceinline__ void next(int n) { if (++s == n) { s = 0; ph ^= 1u; } }
 };
 
+// The waits in front of a chunk's stencil, in their order.  `use` counts the CTA's chunks, s and ph are its weight stage and the
+// parity of that stage's present use.  A barrier's wait tells two neighbouring phases apart and no more, so every phase
+// but the last must be known to be over where a wait begins.  (On the host as well: a test walks them through every order of events.)
+//
+// p_full and p_empty alternate between two barriers also where one buffer takes every chunk: the chunk three back, whose phase
+// comes before that of the chunk that the wait is for, is then one that the same group has waited for.  On one
+// barrier it would be the group's own last chunk, which nobody has waited for, and a wait that finds its phase still open
+// would return at once.
+enum : uint32_t { kOperandFree, kWeightsIn };
+struct StencilOperand {
+  uint32_t buffer, barrier, parity;              // where the chunk's result goes, its p_full and p_empty and their phase
+  __host__ __device__ __forceinline__ StencilOperand(uint32_t use, uint32_t np)
+      : buffer(np == 2 ? use & 1u : 0u), barrier(use & 1u), parity((use >> 1) & 1u) {}
+};
+#pragma nv_exec_check_disable
+template <typename Wait>
+__host__ __device__ __forceinline__ bool stencil_waits(uint32_t use, uint32_t np, uint32_t s, uint32_t ph, Wait wait) {
+  const StencilOperand last(use - np, np);       // the chunk that had the buffer (before the first ones: the phase before a barrier's first)
+  return wait(kWeightsIn, s, ph) && wait(kOperandFree, last.barrier, last.parity);
+}
+
 struct Tile {
   int img0, x0, y0;
   __device__ __forceinline__ Tile(const BlockParams &p, int t) {
@@ -318,12 +339,12 @@ k_block_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CU
 #pragma unroll 1
           for (Chunks c(p); i < p.nch && ok; ++i, c.next(p), ring.next(p.nw), ++p_use) {
             const int s = ring.s;
-            const uint32_t pb = p.np == 2 ? p_use & 1u : 0u, pph = p.np == 2 ? (p_use >> 1) & 1u : p_use & 1u;
-            ok = warp_wait(&sh.w3_full[s], ring.ph, abort_flag, ws, 0x33000u | s) && warp_wait(&sh.p_full[pb], pph, abort_flag, ws, 0x34000u | pb);
+            const StencilOperand o(p_use, (uint32_t)p.np);
+            ok = warp_wait(&sh.w3_full[s], ring.ph, abort_flag, ws, 0x33000u | s) && warp_wait(&sh.p_full[o.barrier], o.parity, abort_flag, ws, 0x34000u | o.barrier);
             if (!ok) break;
             tc_fence_after();
             if (leader) {
-              const uint32_t a0 = p_row + pb * (uint32_t)(p.p_bytes >> 4), w = w_row + (uint32_t)(s * (p.w3_bytes >> 4));
+              const uint32_t a0 = p_row + o.buffer * (uint32_t)(p.p_bytes >> 4), w = w_row + (uint32_t)(s * (p.w3_bytes >> 4));
 #pragma unroll 1
               for (int b = 0; b < p.mbp; ++b)
 #pragma unroll 1
@@ -333,7 +354,7 @@ k_block_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CU
             __syncwarp();
             if (leader) {
               umma_commit(&sh.w3_empty[s]);
-              umma_commit(&sh.p_empty[pb]);
+              umma_commit(&sh.p_empty[o.barrier]);
               if (i == p.nch - 1) umma_commit(&sh.y_full);
             }
           }
@@ -374,7 +395,8 @@ k_block_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CU
           // ---- convert: 16 columns of a block at a time
           ok = ok && warp_wait(&sh.e_full[grp], (use / G) & 1u, abort_flag, ws, 0x40000u | grp);
           bar_sync(kBarMath + (int)grp, kGroupThreads);        // the group's buffer is read by no one any more
-          const uint32_t s = (uint32_t)r3.s, pb = p.np == 2 ? use & 1u : 0u, pph = p.np == 2 ? (use >> 1) & 1u : use & 1u;
+          const uint32_t s = (uint32_t)r3.s;
+          const StencilOperand po(use, (uint32_t)p.np);
           if (ok) {
             tc_fence_after();
             const uint32_t te = tmem_e + tm_row + grp * (uint32_t)(p.mbe * p.ch);
@@ -409,11 +431,13 @@ k_block_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CU
           if (lane == 0) mbar_arrive(&sh.e_empty[grp]);
           bar_sync(kBarMath + (int)grp, kGroupThreads);
           // ---- depthwise
-          ok = ok && warp_wait(&sh.w3_full[s], r3.ph, abort_flag, ws, 0x41000u | s) &&
-               warp_wait(&sh.p_empty[pb], pph ^ 1u, abort_flag, ws, 0x42000u | pb);
+          ok = ok && stencil_waits(use, (uint32_t)p.np, s, r3.ph, [&](uint32_t kind, uint32_t at, uint32_t parity) {
+            return kind == kWeightsIn ? warp_wait(&sh.w3_full[at], parity, abort_flag, ws, 0x41000u | at)
+                                      : warp_wait(&sh.p_empty[at], parity, abort_flag, ws, 0x42000u | at);
+          });
           if (ok) {
             const uint32_t wdb = sm + (uint32_t)p.off_wd + s * (uint32_t)p.wd_bytes, ch4 = (uint32_t)p.ch * 4u;
-            const uint32_t pbuf = sm + (uint32_t)p.off_p + pb * (uint32_t)p.p_bytes;
+            const uint32_t pbuf = sm + (uint32_t)p.off_p + po.buffer * (uint32_t)p.p_bytes;
             const int ncg = chv >> 2;
             const uint32_t inv_ncg = p.inv_ncg[(chv >> 4) - 1];
             const int items = p.ni * p.th * p.strips * ncg;
@@ -469,7 +493,7 @@ k_block_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CU
             fence_proxy_async();
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(&sh.p_full[pb]);
+          if (lane == 0) mbar_arrive(&sh.p_full[po.barrier]);
         }
         // ---- read-out: 16 channels of 32 outputs at a time, turned around in the place of the group's hidden chunk (every
         // stencil of the tile is done when the sums are) so that two lanes store a pixel's 32 bytes
@@ -757,4 +781,25 @@ dc_status dc_launch_block_tc(const void *x, int n, int h, int w, const dc_block 
                                       map_x, map_w1, map_wd, p, b->b_expand, b->b_dw, b->w_project, b->b_project,
                                       (const __nv_bfloat16 *)x, (__nv_bfloat16 *)y, (DcWsHeader *)workspace);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+}
+
+dc_status dc_block_tc_plan(int n, int h, int w, const dc_block *b, dc_block_plan *plan) {
+  BlockParams p;
+  if (!block_plan(n, h, w, b, dc_sm_count(), &p)) return DC_ERR_UNSUPPORTED;
+  *plan = {p.tw, p.th, p.ni, p.tiles, p.nch, p.form, p.groups, p.np, p.nw};
+  return DC_OK;
+}
+
+extern "C" int dc_selftest_block_waits(unsigned int chunk, int operands, int stages, unsigned int waits[12]) {
+  if (operands < 1 || operands > 2 || stages < 2 || stages > kMaxW) return 0;
+  int n = 0;
+  auto note = [&](uint32_t kind, uint32_t at, uint32_t parity) {
+    waits[3 + 3 * n] = kind; waits[4 + 3 * n] = at; waits[5 + 3 * n] = parity;
+    ++n;
+    return true;
+  };
+  const StencilOperand o(chunk, (uint32_t)operands);
+  waits[0] = o.buffer; waits[1] = o.barrier; waits[2] = o.parity;
+  stencil_waits(chunk, (uint32_t)operands, chunk % (unsigned)stages, (chunk / (unsigned)stages) & 1u, note);
+  return n;
 }

@@ -52,6 +52,10 @@ class Block(C.Structure):
                 ("b_dw", C.c_void_p), ("w_project", C.c_void_p), ("b_project", C.c_void_p)]
 
 
+class BlockPlan(C.Structure):
+    _fields_ = [(name, C.c_int) for name in ("tile_w", "tile_h", "tile_images", "tiles", "chunks", "form", "groups", "operands", "stages")]
+
+
 EXPORTS = {
     "dc_status_string": (C.c_char_p, [C.c_int]),
     "dc_fold_bn": (C.c_int, [C.POINTER(Layer), C.c_void_p, C.c_void_p, C.c_void_p]),
@@ -95,9 +99,11 @@ EXPORTS = {
                                            C.POINTER(C.c_size_t)]),
     "dc_block_forward": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.POINTER(Block), C.c_void_p,
                                    C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]),
+    "dc_block_plan_query": (C.c_int, [C.c_int, C.c_int, C.c_int, C.POINTER(Block), C.c_int, C.POINTER(BlockPlan)]),
     "dc_workspace_status": (C.c_int, [C.c_void_p, C.c_void_p]),
     "dc_workspace_status_where": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(C.c_uint), C.POINTER(C.c_uint)]),
     "dc_selftest_bounded_wait": (C.c_int, [C.c_void_p, C.c_size_t, C.c_uint, C.c_void_p]),
+    "dc_selftest_block_waits": (C.c_int, [C.c_uint, C.c_int, C.c_int, C.POINTER(C.c_uint)]),
     "dc_chain_host_param_layout": (C.c_int, [C.POINTER(Layer), C.c_int, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]),
     "dc_chain_host_workspace_bytes": (C.c_int, [C.POINTER(Layer), C.c_int, C.POINTER(Residual), C.c_int,
                                                 C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_size_t)]),
@@ -432,6 +438,16 @@ def block_workspace_bytes(n, h, w, blk: Block, dtype: int) -> int:
     return int(nbytes.value)
 
 
+def block_plan(n, h, w, blk: Block, dtype: int) -> Optional[BlockPlan]:
+    """The plan of the one-launch block kernel, None where the block runs as three launches."""
+    plan = BlockPlan()
+    st = lib().dc_block_plan_query(n, h, w, C.byref(blk), dtype, C.byref(plan))
+    if st == ERR_UNSUPPORTED:
+        return None
+    _check(st, "dc_block_plan_query")
+    return plan
+
+
 def block_forward(x, blk: Block, y, workspace, stream=None):
     st = (_native or _load_native()).block(x, blk, y, workspace, stream)
     if st == OK:
@@ -458,6 +474,15 @@ def workspace_status_where(workspace, stream=None) -> Tuple[int, int, int]:
 def selftest_bounded_wait(workspace, limit_us: int, stream=None):
     _check(lib().dc_selftest_bounded_wait(_ptr(workspace), workspace.numel() * workspace.element_size(), int(limit_us),
                                           _stream(stream)), "dc_selftest_bounded_wait")
+
+
+def selftest_block_waits(chunk: int, operands: int, stages: int):
+    """((buffer, barrier, parity), [(what for, barrier, parity), ...]) of a chunk of the block kernel; see include/dc.h."""
+    out = (C.c_uint * 12)()
+    n = lib().dc_selftest_block_waits(chunk, operands, stages, out)
+    if n <= 0:
+        raise ValueError("operands or stages out of range")
+    return tuple(out[:3]), [tuple(out[3 + 3 * i:6 + 3 * i]) for i in range(n)]
 
 
 def host_layer_array(specs, pinned: bool = False) -> Tuple["C.Array", list]:

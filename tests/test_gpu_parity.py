@@ -916,6 +916,7 @@ def test_dwconv_stencil_tiles(dc, c, k, s, p, n, h, w):
     (16, 96, 24, 2, 1, 40, 112, True, True),     # several strips of columns
     (24, 144, 24, 1, 40, 20, 20, True, True),    # several tiles per CTA
     (32, 192, 32, 1, 77, 10, 10, False, True),   # several images per tile or tiles of one image, more of them than SMs
+    (40, 240, 40, 1, 64, 20, 20, True, True),    # two groups of warps, one buffer for the projection's operand
     (16, 96, 264, 1, 1, 12, 12, True, False),    # more than 256 outputs: three launches
     (24, 72, 24, 1, 1, 12, 12, True, False),     # hidden channels no multiple of 16: three launches
 ])
