@@ -124,6 +124,10 @@ struct Ring {
 // comes before that of the chunk that the wait is for, is then one that the same group has waited for.  On one
 // barrier it would be the group's own last chunk, which nobody has waited for, and a wait that finds its phase still open
 // would return at once.
+//
+// The operand comes first: with an odd number of weight stages a group meets a stage every second round only, and has not
+// waited for the round between.  But a free operand means that the chunk two back (with one buffer: the last one) is projected, which takes all
+// weights up to its own, and the round between has those of a chunk no later than that: there are two stages at least.
 enum : uint32_t { kOperandFree, kWeightsIn };
 struct StencilOperand {
   uint32_t buffer, barrier, parity;              // where the chunk's result goes, its p_full and p_empty and their phase
@@ -134,7 +138,7 @@ struct StencilOperand {
 template <typename Wait>
 __host__ __device__ __forceinline__ bool stencil_waits(uint32_t use, uint32_t np, uint32_t s, uint32_t ph, Wait wait) {
   const StencilOperand last(use - np, np);       // the chunk that had the buffer (before the first ones: the phase before a barrier's first)
-  return wait(kWeightsIn, s, ph) && wait(kOperandFree, last.barrier, last.parity);
+  return wait(kOperandFree, last.barrier, last.parity) && wait(kWeightsIn, s, ph);
 }
 
 struct Tile {

@@ -57,8 +57,9 @@ def walk(groups, operands, stages):
 
 
 @pytest.mark.parametrize("groups,operands,stages", [(g, o, s) for g in (1, 2) for o in (1, 2) for s in (2, 3, 4)])
-def test_no_stencil_writes_an_operand_that_is_still_read(groups, operands, stages):
-    assert not [f for f in walk(groups, operands, stages) if f[0] != "weights"]
+def test_no_stencil_runs_ahead_of_what_it_waits_for(groups, operands, stages):
+    """Neither writes an operand that is still read nor reads weights that have not landed; and no role waits for good."""
+    assert not walk(groups, operands, stages)
 
 
 def test_projection_and_stencil_name_the_same_phase():
