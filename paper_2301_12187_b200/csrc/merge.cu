@@ -1731,9 +1731,8 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       launch_compose33(operand(first), operand(second), first.c_in, first.c_out, second.c_out, w, b, dv ? *dv : piece,
                        mg ? *mg : dc_geom{}, st, status);
     } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k == 3 && first.c_in % 4 == 0 &&
-               first.c_out % 4 == 0 && first.c_out >= 32 && second.c_out < 65535) {
-      // From 32 intermediate channels on, a whole slice (96 -> 24 -> 24 inside a longer run took 2.3 us more here).  More output
-      // channels than 65534 are left to the kernel below, whose grid the runtime refuses.
+               first.c_out % 4 == 0 && first.c_out >= 32) {
+      // From 32 intermediate channels on, a whole slice (96 -> 24 -> 24 inside a longer run took 2.3 us more here).
       After11 a{first, second, w, b, dc_div_up(first.c_in, kA1I), dc_div_up(second.c_out, kA1O)};
       BlockDelivery piece{nullptr, -1, 0, KOrder{}};
       if (dv) { out.w = a.w_out = w_final; out.b = a.b_out = b_final; *delivered = true; piece = *dv; }

@@ -293,6 +293,11 @@ def test_3x3_after_1x1_against_the_oracle(dc, c0, c1, c2, s, res, tail):
     _check_delivery(dc, specs, res, (dc.BF16, dc.F32))
 
 
+def test_3x3_after_1x1_with_more_outputs_than_a_grid_has_rows(dc):
+    """65544 output channels: a grid with a row for each, as the kernel for fewer intermediate channels has, is refused."""
+    _check_delivery(dc, [I.make_layer(85, 0, 8, 32, 1, 1, 0), I.make_layer(85, 1, 32, 65544, 3, 1, 1)], [], (dc.BF16, dc.F32))
+
+
 def _check_delivery(dc, specs, res, codes):
     W, b, k, s, p = O.merge_formula(specs, res)
     for code in codes:
