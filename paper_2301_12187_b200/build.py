@@ -1,4 +1,4 @@
-"""Builds libdepthc.so (sm_100a, nvcc) and the Python module _dccall.so (gcc) next to this file.  `python -m paper_2301_12187_b200.build`."""
+"""Builds libdepthc.so (sm_100a, nvcc) and the Python module _dccall (gcc) next to this file.  `python -m paper_2301_12187_b200.build`."""
 from __future__ import annotations
 
 import glob
@@ -6,13 +6,14 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdepthc.so")
 CALL_SRC = os.path.join(CSRC, "dccall.c")
-CALL_LIB = os.path.join(HERE, "_dccall.so")     # marshals the forward calls of dc.py
+CALL_LIB = os.path.join(HERE, "_dccall" + sysconfig.get_config_var("EXT_SUFFIX"))     # marshals the forward calls of dc.py; one per Python ABI
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -42,7 +43,10 @@ def build_call(force: bool = False) -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    build_call(force)
+    try:
+        build_call(force)
+    except (OSError, subprocess.CalledProcessError) as e:          # no compiler or no headers of Python: ctypes makes those calls
+        warnings.warn("_dccall could not be built, calls are marshalled by ctypes: %r" % (e,))
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

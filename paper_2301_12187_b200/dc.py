@@ -1,6 +1,7 @@
 """ctypes binding of libdepthc (include/dc.h).  Argument marshalling only: every step of the
 path runs in the library's CUDA kernels.  torch is used for device memory and streams.  The three
-forward calls are marshalled natively (csrc/dccall.c); the ctypes form behind them takes what that does not read.
+forward calls are marshalled natively (csrc/dccall.c); the ctypes form behind them takes what that does not read, and
+everything where that module is missing.
 
 The functions carry the names of the C entry points without the `dc_` prefix.  Importing this
 module does not load the library; the first call does, and raises if it cannot.
@@ -144,15 +145,23 @@ def lib():
             fn = getattr(L, name)
             fn.restype = res
             fn.argtypes = args
-        import torch
-        from . import _dccall
-        at = lambda name: C.cast(getattr(L, name), C.c_void_p).value
-        _dccall.bind(at("dc_conv_forward_algo"), at("dc_dwconv_forward"), at("dc_block_forward"), torch.float32, torch.bfloat16,
-                     Geom, Block, getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device),
-                     getattr(torch._C, "_cuda_getCurrentRawStream", None))
-        _native = _dccall
+        try:
+            import torch
+            from . import _dccall
+            at = lambda name: C.cast(getattr(L, name), C.c_void_p).value
+            _dccall.bind(at("dc_conv_forward_algo"), at("dc_dwconv_forward"), at("dc_block_forward"), torch.float32, torch.bfloat16,
+                         Geom, Block, getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device),
+                         getattr(torch._C, "_cuda_getCurrentRawStream", None))
+            _native = _dccall
+        except ImportError:                      # not built for this Python
+            _native = _NoNative
         _lib = L
     return _lib
+
+
+class _NoNative:
+    """In the place of the native module: answers as it does for arguments it does not read."""
+    conv = dwconv = block = staticmethod(lambda *a: None)
 
 
 def _load_native():

@@ -246,3 +246,38 @@ def test_native_marshalling_reports_what_ctypes_reports(monkeypatch, change):
     native = outcomes()
     monkeypatch.setattr(dc, "_native", _NoNative)
     assert native == outcomes() and "returned" not in native
+
+
+def test_calls_work_without_the_native_marshalling(tmp_path):
+    """Neither a C compiler nor a built _dccall: the library is found and a forward call is made (and refused) through ctypes."""
+    import subprocess
+    import sys
+    code = """
+import sys, warnings
+sys.modules["paper_2301_12187_b200._dccall"] = None            # importing it raises ImportError
+from paper_2301_12187_b200 import build, dc
+build.CALL_LIB = sys.argv[1]
+with warnings.catch_warnings(record=True) as w:
+    warnings.simplefilter("always")
+    assert build.build() == build.LIB and any("_dccall" in str(x.message) for x in w)
+import torch
+class Stream:
+    cuda_stream = 0
+x = torch.zeros(1, 4, 4, 8, dtype=torch.bfloat16)
+try:
+    dc.conv_forward(x, dc.geom(8, 8, 1, 1, 1, 0), torch.zeros(64), None, 7, None, x, torch.zeros(256, dtype=torch.uint8), stream=Stream)
+except dc.DcError as e:
+    print("status", e.status)
+"""
+    env = dict(os.environ, CC=str(tmp_path / "no_compiler"), PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", code, str(tmp_path / "_dccall.so")], env=env, cwd=tmp_path, capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.split() == ["status", str(dc.ERR_INVALID_ARG)], r.stderr
+
+
+def test_native_module_carries_the_abi_of_this_python():
+    import importlib.machinery
+    from paper_2301_12187_b200 import build
+    dc.lib()
+    tag = os.path.basename(build.CALL_LIB)[len("_dccall"):]
+    assert tag in importlib.machinery.EXTENSION_SUFFIXES and tag != ".so" and os.path.exists(build.CALL_LIB)
+    assert dc._native.__file__ == build.CALL_LIB
