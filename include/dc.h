@@ -53,8 +53,9 @@ typedef enum {
 } dc_status;
 
 typedef enum { DC_F32 = 0, DC_BF16 = 1 } dc_dtype;
-/* DC_ACT_RELU6 is min(max(v, 0), 6).  A NaN becomes 0, except in k_conv_stem_s2 and in bf16 depthwise layers (a block's
- * too), where it becomes 6. */
+/* DC_ACT_RELU6 is min(max(v, 0), 6).  A NaN becomes 0, except in k_conv_stem_s2, in the bf16 depthwise stencil (3x3 or 5x5, stride 1
+ * or 2, channels in multiples of 8, maps no wider than about 250; other bf16 depthwise layers give 0) and in the
+ * depthwise layer of a block that runs as one launch, where it becomes 6. */
 typedef enum { DC_ACT_IDENTITY = 0, DC_ACT_RELU6 = 1 } dc_act;
 typedef enum { DC_ALGO_AUTO = 0, DC_ALGO_TCGEN05 = 1, DC_ALGO_SIMT = 2 } dc_algo;
 

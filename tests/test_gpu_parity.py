@@ -910,6 +910,20 @@ def test_dwconv_stencil_tiles(dc, c, k, s, p, n, h, w):
     test_dwconv(dc, "bf16", c, k, s, p, n, h, w)
 
 
+@pytest.mark.parametrize("c,k,w,becomes", [(16, 3, 9, 6.0), (40, 5, 9, 6.0), (16, 3, 300, 0.0), (12, 3, 9, 0.0), (16, 7, 9, 0.0)])
+def test_relu6_of_a_nan_in_depthwise_layers(dc, c, k, w, becomes):
+    """6 in the stencil, 0 in the kernels for what it does not take: wider maps, other channel counts, other kernel sizes."""
+    g = dc.geom(c, c, c, k, 1, k // 2)
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(torch.zeros(c, 1, k, k, device="cuda"), g, dc.F32, packed)
+    b = torch.ones(c, device="cuda")
+    b[1] = float("nan")
+    x, y = torch.zeros(2, 5, w, c, dtype=torch.bfloat16, device="cuda"), torch.empty(2, 5, w, c, dtype=torch.bfloat16, device="cuda")
+    dc.dwconv_forward(x, k, 1, k // 2, packed, b, dc.ACT_RELU6, y)
+    assert dc.dwconv_status() == dc.OK
+    assert bool((y[..., 1] == becomes).all()) and bool((y[..., 2:] == 1).all())
+
+
 @pytest.mark.parametrize("c_in,hidden,c_out,s,n,h,w,biases,one_launch", [
     (16, 96, 16, 1, 3, 9, 11, True, True),       # two groups of warps, a ragged map
     (64, 384, 64, 1, 5, 14, 14, True, True),     # six chunks of 64 hidden channels
