@@ -933,8 +933,8 @@ def test_relu6_of_a_nan_in_depthwise_layers(dc, c, k, w, becomes):
     (24, 80, 8, 1, 2, 13, 12, True, False),      # projection weights in groups of five chunks, padded to six: three launches
     (72, 432, 40, 1, 1, 33, 34, True, True),     # a last pass of hidden channels that is shorter than the others
     (16, 96, 24, 2, 1, 40, 112, True, True),     # several strips of columns
-    (24, 144, 24, 1, 40, 20, 20, True, True),    # several tiles per CTA
-    (32, 192, 32, 1, 77, 10, 10, False, True),   # several images per tile or tiles of one image, more of them than SMs
+    (24, 144, 24, 1, 40, 20, 20, True, True),    # tiles of 7 columns, three strips to an image
+    (32, 192, 32, 1, 77, 10, 10, False, True),   # a tile to each image
     (40, 240, 40, 1, 64, 20, 20, True, True),    # two groups of warps, one buffer for the projection's operand
     (16, 96, 264, 1, 1, 12, 12, True, False),    # more than 256 outputs: three launches
     (24, 72, 24, 1, 1, 12, 12, True, False),     # hidden channels no multiple of 16: three launches
@@ -962,6 +962,7 @@ def test_block_in_one_launch_against_the_oracle(dc, c_in, hidden, c_out, s, n, h
     gy.check("block output")
     gws.check("block workspace")
     assert (not bool(gws.t[256:].any())) == one_launch          # the hidden maps were never in the workspace
+    assert (dc.block_plan(n, h, w, blk, dc.BF16) is not None) == one_launch
     cur = x.transpose(0, 3, 1, 2).astype(np.float64)
     skip = cur
     for spec in specs:
@@ -969,6 +970,39 @@ def test_block_in_one_launch_against_the_oracle(dc, c_in, hidden, c_out, s, n, h
         cur = O.conv_direct(cur, Wf, bfo, spec.k, spec.stride, spec.pad, spec.groups)
         cur = O.relu6(cur) if spec.act == "relu6" else cur
     assert_close(nchw(gy.t), cur + skip if res else cur, 3 * TOL_BF16, scale=3.0)      # as for three launches: the same roundings
+
+
+# What a plan may have: form of the kernel (0 and 1: one group of warps), buffers of the projection's operand, weight stages, several
+# images in a tile, several tiles for a CTA.
+BLOCK_PLANS = [
+    # c_in, hidden, c_out, s, n, h, w, (form, operands, stages, images, tiles)
+    (24, 144, 24, 1, 40, 40, 40, (2, 1, 3, False, True)),
+    (24, 144, 24, 1, 78, 15, 14, (2, 2, 3, False, True)),
+    (24, 144, 32, 2, 40, 56, 56, (2, 2, 2, False, True)),
+    (16, 96, 216, 1, 320, 7, 7, (2, 2, 2, True, True)),
+    (24, 144, 24, 1, 300, 3, 3, (3, 2, 3, True, False)),
+    (24, 144, 24, 1, 153, 11, 11, (3, 1, 3, True, False)),
+    (24, 144, 224, 1, 162, 9, 11, (3, 2, 3, False, True)),
+    (16, 240, 16, 1, 300, 16, 16, (3, 1, 4, False, True)),
+    (16, 304, 136, 1, 84, 14, 11, (3, 2, 4, False, True)),
+    (32, 192, 32, 1, 64, 28, 28, (0, 1, 2, False, False)),
+    (16, 96, 152, 1, 94, 22, 25, (0, 2, 2, False, True)),
+    (16, 96, 24, 2, 20, 112, 112, (0, 2, 2, False, True)),
+    (16, 96, 16, 1, 156, 12, 12, (1, 1, 2, True, False)),
+    (16, 96, 88, 1, 283, 17, 17, (1, 1, 2, False, True)),
+    (16, 96, 176, 1, 19, 43, 43, (1, 2, 2, False, True)),
+]
+
+
+@pytest.mark.parametrize("c_in,hidden,c_out,s,n,h,w,plan", BLOCK_PLANS)
+def test_block_plans_against_the_oracle(dc, c_in, hidden, c_out, s, n, h, w, plan):
+    """Every form of the one-launch block kernel with what its loops carry from tile to tile and from image to image.  The plan is
+    asked for, so that a change of the choice between plans cannot take a case from here unseen."""
+    blk = dc.Block(c_in, hidden, c_out, 1, 3, s, 1, int(s == 1 and c_in == c_out), dc.ACT_RELU6, dc.ACT_RELU6, None, None, None, None, None, None)
+    p = dc.block_plan(n, h, w, blk, dc.BF16)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert (p.form, p.operands, p.stages, p.tile_images > 1, p.tiles > sms) == plan
+    test_block_in_one_launch_against_the_oracle(dc, c_in, hidden, c_out, s, n, h, w, True, True)
 
 
 def test_block_in_place(dc):
