@@ -715,21 +715,26 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
   const double per_block = (double)g->k * g->k * dc_div_up(g->c_in, 16) * cyc;
   const double w_item = (double)ko.e_pad * p->n_tile * 16;
   double best = 0.0, best_shared = 0.0;          // of the best tile by itself; the same tile beside the shared ones
-  struct { double cost; int nxt, tw, th, ni, ksplit; } sp = {0.0, 0, 0, 0, 0, 1};      // the best shared one
+  struct { double cost; int nxt, tw, th, ni, ksplit; bool halos; } sp = {0.0, 0, 0, 0, 0, 1, false};   // the best shared one
   p->nxt = 0;
   p->ksplit = 1;
+  p->share = 0;
   const int fixed_part = kSmemBudget - 1024 - p->off_a;     // bytes of the rings, where partial sums would go
   // Tiles of whole rows: the halo column right of a row is the one left of the next row (a load starts at column 0 and ends
   // pad columns past the last), and in tiles of several images the halo rows below one image are those above the next; the
   // zeros in front of the first and behind the last stand in shared memory and are never loaded over.  Of the 128 rows
   // that an instruction multiplies more are outputs, 98 instead of 74 for 3x3 at 7 x 7 (two images in 128 rows, before
-  // three in 256): 160 -> 960, 128 images 28.9 -> 20.8 us.
+  // three in 256): 160 -> 960, 128 images 28.9 -> 20.8 us.  Taken where the estimate is 8 % lower than that of the best tile with
+  // both halos.  Of two tiles alike but for that the shared one is up to 5 % slower (zeros to write, patches that no longer start on
+  // a swizzle's boundary), and where few blocks are saved the estimate cannot tell (160 -> 144 3x3, 16 images of 106 x
+  // 106: 89.4 us by 106 x 2 shared, 80.4 by 18 x 12; 144 -> 144 5x5, 41 of 41 x 41: 90.0 by 41 x 3, 79.8 by 14 x 14).  Of 180 layers
+  // timed in up to ten tiles the choice is 1.5 % above the best on average, none more than 2 % slower than without sharing; any line from 6
+  // to 10 % gives the same; without one 1.7 % and three.
   const bool may_share = S == 1 && g->pad > 0 && 2 * g->pad == g->k - 1 && g->pad <= 8;
   auto stage_bytes = [&](int lines, int ni, int wbox, bool share) {
     return (long long)dc_round_up((size_t)ni * lines * 128 + (share ? 1024 + (ni > 1 ? g->pad * wbox * 128 : 0) : 0), 1024);
   };
-  auto consider = [&](int tw, int th, int ni) {
-    const bool share = may_share && tw == wo;
+  auto consider_form = [&](int tw, int th, int ni, bool share) {
     const int wbox = share ? tw + g->pad : tw + halo, rbox = share && ni > 1 ? th + g->pad : th + halo;
     if (S * wbox > 256 || S * rbox > 256) return;
     const int lines = rbox * wbox;
@@ -749,10 +754,11 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
     const long long whole = (long long)dc_round_up((size_t)(g->k * tap_bytes), 1024);
     const bool columns = S == 1 && g->k > 1 && 2048 + p->off_a + 2 * whole + 2 * stage_bytes(lines, ni, wbox, share) > kSmemBudget;
     const double waits = columns ? 150.0 * (double)per_cta * p->planes * g->k * g->k : 0.0;
+    const double line = share ? 1.08 : 1.0;
     auto estimate = [&](int split, double more) {
       const double m = mma / split, one = (double)per_cta * bytes / split / 67.0, l = one > all ? one : all;
       const double ctas = (double)(items * split < n_sm ? items * split : n_sm);
-      return (m > l ? m + 0.77 * l : l + 0.77 * m) + waits / split + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + more;
+      return line * ((m > l ? m + 0.77 * l : l + 0.77 * m) + waits / split + 1700.0 * (double)per_cta + 1.1 * lines * ni + 30.0 * ctas + more);
     };
     // Beside the shared items a step and a plane have a price of their own, and a shared one pays for the meeting: the CTAs
     // that meet, the sums that each writes and reads and the results.
@@ -762,7 +768,7 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
       return estimate(split, (double)per_cta * (600.0 * steps + 800.0 * pl) + 3.9 * lines * ni + (split > 1 ? 500.0 + 200.0 * split + sums : 0.0));
     };
     const double alone = estimate(1, 0.0);
-    if (p->nxt == 0 || alone < best) { best = alone; best_shared = shared(1); p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; }
+    if (p->nxt == 0 || alone < best) { best = alone; best_shared = shared(1); p->nxt = nxt; p->tw = tw; p->th = th; p->ni = ni; p->share = share; }
     for (int split = 2; split <= kMaxSplit; ++split) {
       // A shared item: all clusters at once, at least one (plane, tap row) step per CTA, partial sums in the rings' place.
       if (split == 7) continue;                  // no more clusters of seven than of eight run at once (15 each)
@@ -770,8 +776,12 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
           mb * 128 * (p->n_tile + 4) * 4 > fixed_part)
         break;
       const double cost = shared(split);
-      if (sp.ksplit == 1 || cost < sp.cost) sp = {cost, nxt, tw, th, ni, split};
+      if (sp.ksplit == 1 || cost < sp.cost) sp = {cost, nxt, tw, th, ni, split, share};
     }
+  };
+  auto consider = [&](int tw, int th, int ni) {
+    consider_form(tw, th, ni, false);
+    if (may_share && tw == wo) consider_form(tw, th, ni, true);
   };
   // The fewest strips whose tile of one output row is within the tensor map's box (256 pixels) and the activation ring
   // (max_a, in whole kilobytes).  The ring is the tighter bound for 5x5 and 7x7 kernels, whose weight stages leave it
@@ -792,15 +802,17 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
   } else {
     for (int cand = nxt0; cand <= nxt0 + 5 && cand <= wo; ++cand) {
       const int tw = dc_div_up(wo, cand);
-      int last_th = 0;
-      for (int mb = kMaxBlocks; mb >= 1; --mb) {
-        if (mb * 128 < tw) break;
-        int th = (mb * 128 - tw) / (may_share && tw == wo ? tw + g->pad : tw + halo) + 1;
-        if (th > ho) th = ho;
-        if (th != last_th) consider(tw, th, 1);
-        last_th = th;
-        const int even = dc_div_up(ho, dc_div_up(ho, th));
-        if (even != th) consider(tw, even, 1);
+      for (int share = 0; share <= (may_share && tw == wo ? 1 : 0); ++share) {
+        int last_th = 0;
+        for (int mb = kMaxBlocks; mb >= 1; --mb) {
+          if (mb * 128 < tw) break;
+          int th = (mb * 128 - tw) / (tw + (share ? g->pad : halo)) + 1;
+          if (th > ho) th = ho;
+          if (th != last_th) consider_form(tw, th, 1, share != 0);
+          last_th = th;
+          const int even = dc_div_up(ho, dc_div_up(ho, th));
+          if (even != th) consider_form(tw, even, 1, share != 0);
+        }
       }
       if (p->nxt == 0) consider(tw, 1, 1);
     }
@@ -808,9 +820,11 @@ bool make_rows_plan(int n, int h, int w, const dc_geom *g, int n_sm, RowsParams 
       for (int ni = 2; ni <= 8 && ni <= n; ++ni) consider(wo, ho, ni);
   }
   if (p->nxt == 0) return false;
-  if (sp.ksplit > 1 && sp.cost < best_shared) { p->nxt = sp.nxt; p->tw = sp.tw; p->th = sp.th; p->ni = sp.ni; p->ksplit = sp.ksplit; }
+  // (a hundredth less: 144 -> 144 5x5, two images of 53 x 53, was split in two for a tenth of that, 15.7 us, 13.5 unsplit)
+  if (sp.ksplit > 1 && sp.cost < 0.99 * best_shared) {
+    p->nxt = sp.nxt; p->tw = sp.tw; p->th = sp.th; p->ni = sp.ni; p->ksplit = sp.ksplit; p->share = sp.halos;
+  }
   const int th = p->th;
-  p->share = may_share && p->tw == wo;
   p->wbox = p->share ? p->tw + g->pad : p->tw + halo;
   p->rbox = p->share && p->ni > 1 ? th + g->pad : th + halo;
   p->front = p->share ? 1024 : 0;

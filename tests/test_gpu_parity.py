@@ -738,12 +738,27 @@ def test_rows_tiles_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
-    (160, 136, 3, 1, 1, 131, 7, 7),      # two or four images per tile, a ragged last group
-    (64, 64, 5, 1, 2, 150, 5, 5),        # halo of two columns and rows
-    (72, 48, 7, 1, 3, 151, 4, 6),        # halo of three: as wide as half a map
-    (48, 144, 3, 1, 1, 153, 1, 3),       # one-row maps: every row between two images is halo
+    (160, 136, 3, 1, 1, 131, 7, 7),      # four images per tile, a ragged last group
+    (64, 64, 5, 1, 2, 150, 5, 5),        # too little to save: not shared
+    (72, 48, 7, 1, 3, 151, 4, 6),        # halo of three: as wide as half a map; the reduction shared as well
+    (48, 144, 3, 1, 1, 153, 1, 3),       # not shared
     (64, 64, 3, 1, 2, 150, 6, 6),        # padding that is not half the kernel: nothing is shared
-    (96, 64, 3, 1, 1, 40, 28, 28),       # whole rows of one image: halo columns only
+    (96, 64, 3, 1, 1, 40, 28, 28),       # not shared
+    (40, 48, 3, 1, 1, 88, 17, 6),        # several images, ...
+    (40, 104, 3, 1, 1, 75, 10, 10),      # ... with resident weights, ...
+    (152, 64, 3, 1, 1, 32, 1, 36),       # ... of one row, the reduction shared
+    (40, 56, 3, 1, 1, 15, 31, 31),       # whole rows of one image: halo columns only, ...
+    (48, 96, 3, 1, 1, 22, 27, 27),       # ... with resident weights
+    (40, 144, 5, 1, 2, 107, 1, 24),      # halo of two: one-row maps, every row between two images is halo, ...
+    (48, 128, 5, 1, 2, 181, 2, 37),      # ... with weights by tap columns, ...
+    (64, 184, 5, 1, 2, 11, 25, 25),      # ... the same with rows of one image, ...
+    (80, 48, 5, 1, 2, 17, 23, 8),        # ... and with the reduction shared
+    (56, 192, 7, 1, 3, 203, 2, 2),       # halo of three: wider than the map, ...
+    (56, 144, 7, 1, 3, 230, 4, 4),       # ... as wide as most of it, weights by tap columns, ...
+    (40, 72, 7, 1, 3, 29, 22, 22),       # ... and whole rows of one image
+    (176, 88, 3, 1, 1, 16, 63, 63),      # wide maps, where whole rows are not the best tiles
+    (160, 144, 3, 1, 1, 2, 106, 106),
+    (144, 144, 5, 1, 2, 3, 41, 41),
 ])
 def test_rows_with_shared_halos_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w):
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, w, "k_conv_tc_rows")
