@@ -627,20 +627,34 @@ bool block_layout(BlockParams *p) {
 // or its weights' way in from L2; a tile its patch's way in and the read-out.  The constants are fitted to 25 blocks (16 to 160
 // channels, maps of 7 to 112, 1 to 128 images) timed in every tile and form considered below, 5400 in all: 8 % off in the
 // root mean square; the choice is 2 % above the best on average, 10 % at worst (24 -> 144 -> 24, 64 images of 56 x 56).
-double plan_cycles(const BlockParams &p, int n_sm) {
-  const int warps = dc_div_up(p.ni * p.th * p.strips * (p.ch >> 2), 32), tasks = p.mbe * (p.ch >> 4), out = p.mbp * (p.n3 >> 4);
+double chunk_cycles(const BlockParams &p) {
+  const int warps = dc_div_up(p.ni * p.th * p.strips * (p.ch >> 2), 32), tasks = p.mbe * (p.ch >> 4);
   const double issue = (158.0 + 80.0 * p.tx) * warps / 4 + 211.0 * tasks;
   const double chain = (835.0 + 718.0 * dc_div_up(tasks * p.groups, 8) + 147.0 * p.tx * dc_div_up(warps * p.groups, kMathWarps)) / p.groups;
   const double weights = (double)(p.w1_bytes + p.wd_bytes + p.w3_bytes) / 24.4;
-  const double chunk = sqrt(sqrt(issue * issue * issue * issue + chain * chain * chain * chain + weights * weights * weights * weights));
-  return 6234.0 + dc_div_up(p.tiles, n_sm) * (3080.0 + 390.0 * out + 1.35 * p.planes * p.patch + p.nch * chunk);
+  return sqrt(sqrt(issue * issue * issue * issue + chain * chain * chain * chain + weights * weights * weights * weights));
+}
+double plan_cycles(const BlockParams &p, int n_sm) {
+  const int out = p.mbp * (p.n3 >> 4);
+  return 6234.0 + dc_div_up(p.tiles, n_sm) * (3080.0 + 390.0 * out + 1.35 * p.planes * p.patch + p.nch * chunk_cycles(p));
 }
 
-// The three launches' time, in cycles, fitted to 134 blocks: three launches, the hidden maps written and read, the weights.
-double three_launches_cycles(const BlockParams &p) {
+// What the chosen plan takes beside three launches, in cycles: the same terms fitted to the plans that are chosen for 499 blocks (16 to
+// 160 channels in, 8 to 320 out, maps of 3 to 112, 1 to 320 images), 6.5 % off in the root mean square (the estimate above,
+// fitted to good and bad plans alike, 7.4 %, and up to 26 % too high for wide outputs).
+double one_launch_cycles(const BlockParams &p, int n_sm) {
+  const int out = p.mbp * (p.n3 >> 4);
+  return 5239.0 + dc_div_up(p.tiles, n_sm) * (3207.0 + 239.0 * out + 2.75 * p.planes * p.patch + p.nch * (309.0 + 0.907 * chunk_cycles(p)));
+}
+
+// The three launches' time, in cycles: a start, the hidden maps written and read, the products.  A projection to fewer than 32
+// channels is not the rows kernel's and costs more, most of it a chain over the hidden channels.  Fitted to the same blocks: 7 % off
+// in the root mean square (19 % without the terms of the products and of narrow projections).
+double three_launches_cycles(const BlockParams &p, bool narrow) {
   const double hidden = (double)p.n_img * p.h * p.w * p.c_mid * 2e-6, thinned = (double)p.n_img * p.ho * p.wo * p.c_mid * 2e-6;
-  const double weights = (double)p.c_mid * (p.c_in + p.c_out) * 2e-6, flops = (double)p.n_img * p.h * p.w * p.ksteps * 16 * p.c_mid * 1e-9;
-  return 1900.0 * (11.9 + 0.359 * hidden + 0.585 * thinned + 4.28 * sqrt(weights) + 1.6 * flops);
+  const double expand = hidden * 8e-3 * p.ksteps, project = thinned * 5e-4 * p.n3;
+  return 1900.0 * (8.97 + 0.393 * hidden + 0.352 * thinned + 4.58e-3 * p.c_mid + 0.25 * expand + 3.18 * project +
+                   (narrow ? 0.71 * thinned + 27e-3 * p.c_mid : 0.0));
 }
 
 bool make_block_plan(int n, int h, int w, const dc_block *b, int n_sm, BlockParams *p) {
@@ -713,13 +727,12 @@ bool make_block_plan(int n, int h, int w, const dc_block *b, int n_sm, BlockPara
   for (int ni = 2; ni <= 8 && ni <= n; ++ni) consider(wo, ho, ni);
   if (!any) return false;
   *p = best;
-  // Taken where it is estimated to be faster than the three launches.  Those are underestimated for fewer than 32 input channels
-  // (measured 0.4 to 0.65 of their time here: a quarter to a half of each expansion's operand is padding) and this kernel where a CTA
-  // has several tiles in turn, so the line lies at 0.82 there: 80 channels on 44 maps of 35 x 35 are 2 % slower here, 112 on 10
-  // of 52 x 52 8 %, 32 on 128 of 28 x 28 7 % faster.  Long reductions of few pixels stay with the launches, whose reductions clusters share:
-  // 160 -> 960 -> 160 on one 7 x 7 map 22.4 us here, 14.1 there.
-  const double line = p->c_in < 32 ? 2.0 : (p->tiles > 2 * n_sm ? 0.82 : 1.0);
-  if (best_cost > line * three_launches_cycles(*p)) return false;
+  // Taken where it is estimated to be faster than the three launches.  The line lies where the 499 blocks together take least: at
+  // 1.03 where each tile has an SM of its own (0.756 of the three launches' time on average, as if the faster were always known to
+  // 0.3 %; five of 373 are more than 3 % slower than three launches, by 8 % at most), at 0.9 where a CTA has several tiles in turn (0.888;
+  // two of 126 by up to 5 %; at 0.95 0.886 but nine by up to 21 %: 32 -> 192 -> 32 on 30 maps of 51 x 48 37.1 us here, 30.7 in three).  Long reductions
+  // of few pixels stay with the launches, whose reductions clusters share: 160 -> 960 -> 160 on one 7 x 7 map 22.4 us here, 11.0 there.
+  if (one_launch_cycles(*p, n_sm) > (p->tiles > n_sm ? 0.9 : 1.03) * three_launches_cycles(*p, !k3.rows)) return false;
   p->inv_lines = inv20(p->lines_img); p->inv_wbox = inv20(p->wbox); p->inv_th = inv20(p->th);
   p->inv_strips = inv20(p->strips); p->inv_outs = inv20(p->th * p->tw); p->inv_tw = inv20(p->tw);
   p->inv_mbe = inv20(p->mbe); p->inv_mbp = inv20(p->mbp);

@@ -993,19 +993,21 @@ BLOCK_PLANS = [
     # c_in, hidden, c_out, s, n, h, w, (form, operands, stages, images, tiles)
     (24, 144, 24, 1, 40, 40, 40, (2, 1, 3, False, True)),
     (24, 144, 24, 1, 78, 15, 14, (2, 2, 3, False, True)),
-    (24, 144, 32, 2, 40, 56, 56, (2, 2, 2, False, True)),
-    (16, 96, 216, 1, 320, 7, 7, (2, 2, 2, True, True)),
+    (16, 96, 16, 1, 76, 18, 18, (2, 2, 2, False, True)),
+    (16, 96, 16, 2, 314, 13, 13, (2, 1, 2, True, True)),
     (24, 144, 24, 1, 300, 3, 3, (3, 2, 3, True, False)),
     (24, 144, 24, 1, 153, 11, 11, (3, 1, 3, True, False)),
-    (24, 144, 224, 1, 162, 9, 11, (3, 2, 3, False, True)),
+    (24, 144, 24, 1, 83, 15, 15, (3, 2, 3, False, True)),
     (16, 240, 16, 1, 300, 16, 16, (3, 1, 4, False, True)),
-    (16, 304, 136, 1, 84, 14, 11, (3, 2, 4, False, True)),
+    (16, 512, 16, 1, 82, 11, 11, (3, 2, 4, False, True)),
     (32, 192, 32, 1, 64, 28, 28, (0, 1, 2, False, False)),
-    (16, 96, 152, 1, 94, 22, 25, (0, 2, 2, False, True)),
+    (24, 144, 24, 1, 75, 32, 32, (0, 1, 3, False, True)),
+    (24, 144, 160, 1, 53, 17, 17, (0, 2, 3, False, False)),
     (16, 96, 24, 2, 20, 112, 112, (0, 2, 2, False, True)),
     (16, 96, 16, 1, 156, 12, 12, (1, 1, 2, True, False)),
-    (16, 96, 88, 1, 283, 17, 17, (1, 1, 2, False, True)),
-    (16, 96, 176, 1, 19, 43, 43, (1, 2, 2, False, True)),
+    (16, 96, 16, 1, 21, 64, 64, (1, 1, 2, False, True)),
+    (24, 144, 72, 1, 203, 11, 11, (1, 2, 3, True, False)),
+    (16, 96, 8, 2, 125, 38, 34, (1, 2, 2, False, True)),
 ]
 
 
