@@ -19,8 +19,6 @@
 //
 // The one wait (for the tile to land) is bounded like every wait of the library; a wait that runs
 // out sets a library-wide flag that dc_dwconv_status reports, and the CTA returns.
-#include <math.h>
-
 #include "tc_ptx.cuh"
 
 namespace {
@@ -234,23 +232,26 @@ bool make_stencil_plan(int n, int h, int w, int c, int k, int stride, int pad, S
   double best = 0.0;
   p->ct = 0;
   // Channels per tile (the last tile of a pixel may be partly filled), output rows per tile and per thread, images per tile:
-  // the least estimated time.  It goes with what the CTAs of the SM with most of them need of it (instructions, and bytes,
-  // of which the load unit moves fewer at a time in narrow tiles) and with the chain of one CTA (rounds of thread
-  // items, its patch's way in), as the product of powers 0.72 and 0.28 of the two: fitted to 26 layers (8 to 960 channels,
-  // 3x3 and 5x5, maps of 7 to 112, 1 to 128 images) timed in every tile considered here, 13 % off in the root mean
-  // square; the choice is 3 % above the best on average, 20 % at worst (384 channels, 20 maps of 13 x 13).
+  // the least estimated time, which is what the CTAs of the SM with most of them issue and what a CTA's chain takes (rounds of
+  // thread items, its patch's way in, of which the load unit moves fewer bytes at a time in narrow tiles, its weights, read 128
+  // at a time) as often as one follows the other in the four places of an SM.  Fitted to 303 layers (8 to 960 channels, 3x3 and
+  // 5x5, maps of 7 to 112, 1 to 128 images) timed in up to 24 tiles each, 6324 timings, for the choice: 3.4 % above the best on
+  // average, 27 % at worst (80 channels of stride 2, 31 maps of 13 x 13).  A product of powers of the two, without the weights and the
+  // places, fitted to 26 layers, chose tiles 8.8 % above the best, 64 % at worst: 304 channels 5x5, 35 maps of 7 x 7 5.6 us, now 4.4;
+  // 88 channels 5x5 of stride 2, 4 of 21 x 20 3.1, now 2.3; 192 channels, 121 of 9 x 10 5.8, now 5.0.
   auto consider = [&](int r, int ct, int rt, int ni) {
     const int rows = dc_div_up(rt, r) * r, in_rows = (rows - 1) * stride + k;
     const long long bytes = (long long)ni * in_rows * p->in_w * ct * 2;
     if (bytes > kTileBytes || in_rows > 256) return false;
     const int items = ni * dc_div_up(rt, r) * xtiles * (ct / kV);
     const long long ctas = (long long)dc_div_up(c, ct) * dc_div_up(ho, rt) * dc_div_up(n, ni);
-    const double item = (k == 5 ? 1.1 : 1.0) * (40 + k * k + ((r - 1) * stride + k) * nj * 5 + (2 * k * k + 7) * tx * r);   // instructions
-    const double moved = (double)bytes * (ct == 32 ? 1.0 : (stride == 2 ? (ct == 16 ? 1.7 : 3.0) : (ct == 16 ? 1.11 : 1.83)));
-    const double most = ctas <= 4ll * n_sm ? (double)((ctas + n_sm - 1) / n_sm) : (double)ctas / n_sm + 0.5;
-    const double sm = most * (62.5 + 0.069 * dc_div_up(items, 32) * item + moved / 120.0);
-    const double chain = (most > 4.0 ? most / 4.0 : 1.0) * (dc_div_up(items, kThreads) * item + moved / 223.0);
-    const double cost = sm * sm * sqrt(sm) * chain;
+    const int instructions = 40 + k * k + ((r - 1) * stride + k) * nj * 5 + (2 * k * k + 7) * tx * r;
+    const double item = instructions * (r == 1 ? 1.35 : 1.0) * (stride == 2 ? 2.3 : 1.0);
+    const double moved = (double)bytes * (ct == 32 ? 1.0 : (stride == 2 ? (ct == 16 ? 3.1 : 5.0) : (ct == 16 ? 1.6 : 3.2)));
+    const double per_sm = (double)ctas / n_sm, most = 0.77 * (double)((ctas + n_sm - 1) / n_sm) + 0.23 * per_sm;
+    const double places = 0.46 * (double)((ctas + 4 * n_sm - 1) / (4 * n_sm)) + 0.54 * (per_sm > 4.0 ? per_sm / 4.0 : 1.0);
+    const double chain = dc_div_up(items, kThreads) * item + moved / 10.3 + 635.0 * dc_div_up((k * k + 1) * ct, kThreads);
+    const double cost = most * (0.5 * dc_div_up(items, 32) * item + 45.0) + places * chain;
     if (p->ct == 0 || cost < best) { best = cost; p->rows = r; p->ct = ct; p->rt = rt; p->ni = ni; }
     return true;
   };

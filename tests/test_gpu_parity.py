@@ -910,15 +910,22 @@ def test_dwconv(dc, dtype, c, k, s, p, n, h, w):
 
 
 @pytest.mark.parametrize("c,k,s,p,n,h,w", [
-    (40, 3, 1, 1, 2, 9, 9),              # a partly filled last tile of channels
-    (72, 3, 2, 1, 3, 15, 13),            # the same, stride 2, odd sides
-    (8, 5, 1, 2, 1, 7, 7),               # eight channels, one tile
-    (152, 3, 1, 1, 1, 27, 24),           # one output row per thread
+    (40, 3, 1, 1, 2, 9, 9),              # small maps: tiles of eight channels and a row
+    (72, 3, 2, 1, 3, 15, 13),
+    (8, 5, 1, 2, 1, 7, 7),
+    (152, 3, 1, 1, 1, 27, 24),
+    (104, 5, 2, 2, 9, 21, 23),
     (360, 3, 1, 1, 70, 7, 7),            # two rows per thread of an odd height, several images per tile
     (48, 3, 1, 1, 32, 56, 56),           # two rows per thread, more tiles than CTAs at once
-    (104, 5, 2, 2, 9, 21, 23),           # 5x5 of stride 2
     (8, 5, 2, 2, 1, 6, 252),             # widest maps of the load unit's box: the last items read past their row
     (16, 3, 1, 1, 1, 5, 254),
+    (24, 3, 1, 1, 20, 12, 254),
+    # one row per thread: tiles of 16 and 32 channels, the last one partly filled, several images in some
+    (440, 3, 1, 1, 21, 6, 3), (360, 3, 1, 1, 38, 4, 4), (480, 3, 1, 1, 39, 3, 3), (152, 3, 2, 1, 25, 5, 11), (152, 3, 2, 1, 47, 3, 3),
+    (440, 5, 1, 2, 21, 4, 9), (408, 5, 2, 2, 21, 3, 3), (432, 5, 2, 2, 21, 6, 6),
+    # two rows per thread, odd heights: the same
+    (456, 3, 1, 1, 22, 5, 3), (176, 3, 1, 1, 28, 9, 8), (216, 3, 1, 1, 125, 3, 3), (40, 3, 2, 1, 62, 17, 17), (280, 3, 2, 1, 71, 5, 3),
+    (272, 5, 1, 2, 35, 6, 3), (104, 5, 1, 2, 23, 11, 11), (440, 5, 1, 2, 124, 5, 3), (440, 5, 2, 2, 11, 9, 9), (264, 5, 2, 2, 71, 6, 3),
 ])
 def test_dwconv_stencil_tiles(dc, c, k, s, p, n, h, w):
     test_dwconv_stencil_without_activation(dc, c, k, s, p, n, h, w)
