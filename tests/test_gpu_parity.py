@@ -792,6 +792,8 @@ def test_shared_reductions_of_few_and_many_sums(dc, c_in, c_out, k, s, p, n, h, 
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w", [
     (96, 144, 5, 2, 2, 9, 57, 50),       # several tiles per image and per CTA, odd height
     (96, 144, 5, 2, 2, 1, 20, 20),       # the reduction shared by a cluster
+    (64, 696, 3, 2, 1, 2, 12, 7),        # the same with one plane: CTAs with one or two of its six steps
+    (72, 216, 3, 2, 1, 20, 17, 12),      # the same with two planes, the second of eight channels
     (40, 32, 3, 2, 1, 40, 28, 28),       # one image per tile, runs cut by blocks
     (40, 48, 3, 2, 1, 160, 21, 21),      # weights resident, more items than CTAs
     (48, 64, 7, 2, 3, 2, 31, 44),        # 7x7: classes of 16, 12, 12 and 9 taps
