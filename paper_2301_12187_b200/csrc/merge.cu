@@ -666,21 +666,22 @@ __global__ void __launch_bounds__(kBlockThreads) k_merge_block(const __grid_cons
 //
 // For one hidden channel c the 3x3 kernel of a pair (o, i) grows by p = (W3[o][c] s[c]) W1[c][i] times
 // the nine taps D[c][.]: one multiplication and nine FMAs per pair, and W', with its 9 x c_hidden terms,
-// never exists in between.  A CTA owns 8 x 16 pairs, a thread of a warp 2 x 2 of them (36 sums); the
-// eight warps take an eighth of the hidden channels each, stage their own operands by cp.async four
+// never exists in between.  A CTA owns 8 x IT pairs, a thread of a warp 2 x IT/8 of them (36 or 54 sums);
+// its W warps take an equal part of the hidden channels each, stage their own operands by cp.async four
 // slices of 16 channels deep (no CTA barrier until the sums meet in shared memory, in warp order), so
-// that narrow blocks are short chains and wide ones fill the chip: 160 -> 960 -> 160 has 200 tiles.
-// BN scales s = g1 g2 ride on W3, g3 on the result.
+// that narrow blocks are short chains and wide ones fill the chip.  8 x 16 pairs by eight warps; for long
+// reductions sixteen warps, in tiles of 8 x 16 or 8 x 24 (see the rule at the launch): 160 -> 960 -> 160 has 140 tiles of
+// 8 x 24.  BN scales s = g1 g2 ride on W3, g3 on the result.
 //
 // Blocks behind the tiles compute the bias (8 output channels each); behind those, for a packed
 // result, the chunks of the packed copy that hold no weight are zeroed.
 //
-// Before, with one CTA per output channel that read every operand, then a delivery launch: 24 -> 144 -> 24
-// 9.4 us, 64 -> 384 -> 64 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  With eight warps 6.5, 9.0 and 25.9 us (200 tiles
-// of 8 x 16 on 148 SMs: 52 of them had two, the others eight warps with no second tile to hide their latency); by sixteen warps in 140 tiles of 8 x 24 20.7
-// us, 120 -> 720 -> 120 (120 tiles) 19.0 -> 12.9, 88 -> 528 -> 88 15.0 -> 11.3.  With the sums added 16 bytes at a time and the third
-// layer's scales asked for in front (behind the sums they were a chain of their own) 24 -> 144 -> 24 6.4 -> 6.0, 160 -> 960 -> 160 19.7.  Halved runs of the sums are nearer to 64 bits as well
-// (160 channels: 1.6e-7 -> 1.35e-7).
+// Before, with one CTA per output channel that read every operand, then a delivery launch: 24 -> 144 -> 24 9.4 us, 64 -> 384 -> 64
+// 29.5 us; 160 -> 960 -> 160, step by step, 103 us.  With eight warps 6.5, 9.0 and 25.9 us (200 tiles of 8 x 16 on 148 SMs: 52 of
+// them had two, the others eight warps with no second tile to hide their latency); by sixteen warps in 140 tiles of 8 x 24 20.7
+// us, 120 -> 720 -> 120 (120 tiles) 19.0 -> 12.9, 88 -> 528 -> 88 15.0 -> 11.3.  With the sums added 16 bytes at a time and the
+// third layer's scales asked for in front (behind the sums they were a chain of their own) 24 -> 144 -> 24 6.4 -> 6.0, 160 -> 960
+// -> 160 19.7.  Halved runs of the sums are nearer to 64 bits as well (160 channels: 1.6e-7 -> 1.35e-7).
 // ----------------------------------------------------------------------------------------------
 constexpr int kMbO = 8, kMbI = 16, kMbSlice = 16, kMbStages = 4;
 constexpr int kMbThreads = 256;
@@ -810,7 +811,7 @@ k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ 
     }
     return;
   }
-  // ---- 8 x 16 pairs
+  // ---- 8 x IT pairs
   const int o0 = (blk / gi) * kMbO, i0 = (blk % gi) * IT;
   __shared__ float g3s[kMbO];                      // BN scales of the tile's output channels
   if (tid < kMbO) g3s[tid] = o0 + tid < c2 ? raw_scale(a.l3, o0 + tid) : 0.f;
@@ -1650,15 +1651,16 @@ static void launch_compose33_form(const Compose33 &a, const BlockDelivery &dv, c
   status.note(dc_launch_pdl(k_compose33<W>, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, W * 32)), dim3(W * 32), P3Form<W>::BYTES, st, a, dv));
   status.launched();
 }
-// Four warps a tile, four tiles to an SM at once, except where the tiles of the SM with the most of them fill whole rounds of
-// two better than of four: one, two or five of them, or three with a reduction long enough (136 -> 136 -> 136, two tiles: 18.1 us by
-// eight warps; 208 -> 208 -> 208, five: 56.1 us by four, 49.3 by eight; 160 -> 160 -> 160, three: 28.9 and 24.4, with 48 channels between
-// 12.9 and 13.4; 192 -> 192 -> 192, four: 34.2 and 35.4; 512 -> 128 -> 512, 28: 158 and 170).
+// Four warps a tile, four tiles to an SM at once, except where the tiles of the SM with the most of them fill whole rounds of two
+// better than of four: one or two of them (136 -> 136 -> 136: 25.6 us by four warps, 17.8 by eight), or three or five with a
+// reduction long enough to matter (160 -> 160 -> 160, three: 29.1 and 24.1, with 48 channels between 12.7 and 13.2; 208 -> 208 ->
+// 208, five: 55.0 and 49.0, with 48 20.9 and 21.3).  Timed in both forms at 1 to 16 tiles, 48 or as many channels between as
+// outside: four tiles and from six on four warps are the faster ones, by up to 30 % with 48 channels between, or within 1.5 %.
 static void launch_compose33(const Operand33 &first, const Operand33 &second, int c0, int c1, int c2, float *w, float *b,
                              const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
   const int most = dc_div_up(a.gi * a.go, dc_sm_count());
-  if (most <= 2 || most == 5 || (most == 3 && c1 >= 128)) launch_compose33_form<8>(a, dv, mg, st, status);
+  if (most <= 2 || ((most == 3 || most == 5) && c1 >= 128)) launch_compose33_form<8>(a, dv, mg, st, status);
   else launch_compose33_form<4>(a, dv, mg, st, status);
 }
 
