@@ -18,12 +18,14 @@
 // so the tensor core works on the next chunk's expansion while the warps are at this chunk's stencil.  The roundings are
 // those of the three launches: hidden maps to bf16 after their ReLU6, everything else in fp32.
 //
-// What bounds it is the stencil, 4.5 packed FMAs and 7 other instructions per hidden value, and shared memory, which feeds
-// the stencil (13 bytes read per hidden value) and both products.  64 -> 384 -> 64, 128 images of 14 x 14: 21.5 us, 26.5 as
-// three launches; one image 9.6 and 12.4; 24 -> 144 -> 24, 64 images of 56 x 56 60 and 112; 16 -> 96 -> 16, 20 images of 9 x 9 6.5
-// and 14.8.  Measured and not kept: two rows of outputs per thread (fewer instructions, but more than the 96 registers that 19
-// warps leave: 10 % slower), both products issued by one warp, a bulk copy for every 8-channel chunk of the weights (80
-// cycles each to issue: 3 us a chunk of hidden channels).
+// What bounds it is a chunk's chain in a group of warps: its accumulators, their way out of tensor memory, conversion, a barrier,
+// the stencil, the hand-over.  Half of the cycles issue nothing (64 -> 384 -> 64, 128 images of 14 x 14: issue slots 48 % taken,
+// FMA pipe 19 %, the largest stall is on what memory returns), and of the 11.9 thousand warp instructions of a chunk the stencil,
+// 4.5 packed FMAs and 7 others per hidden value, has 4.5.  That block takes 20.2 us, 25.1 as three launches; one image 9.4 and
+// 10.1; 24 -> 144 -> 24, 64 images of 56 x 56 60 and 111; 16 -> 96 -> 16, 20 images of 9 x 9 6.4 and 13.9.  Measured and not kept:
+// two rows of outputs per thread (fewer instructions, but more than the 96 registers that 19 warps leave: 10 % slower), both
+// products issued by one warp, a bulk copy for every 8-channel chunk of the weights (80 cycles each to issue: 3 us a chunk of
+// hidden channels).
 //
 // Roles (608 threads): warp 0 loads (a chunk's weights, several stages ahead), warps 1 and 2 issue the tensor-core
 // instructions of the two products, warps 3-18 convert, run the stencil and read out.  All waits are bounded
@@ -729,9 +731,10 @@ bool make_block_plan(int n, int h, int w, const dc_block *b, int n_sm, BlockPara
   *p = best;
   // Taken where it is estimated to be faster than the three launches.  The line lies where the 499 blocks together take least: at
   // 1.03 where each tile has an SM of its own (0.756 of the three launches' time on average, as if the faster were always known to
-  // 0.3 %; five of 373 are more than 3 % slower than three launches, by 8 % at most), at 0.9 where a CTA has several tiles in turn (0.888;
-  // two of 126 by up to 5 %; at 0.95 0.886 but nine by up to 21 %: 32 -> 192 -> 32 on 30 maps of 51 x 48 37.1 us here, 30.7 in three).  Long reductions
-  // of few pixels stay with the launches, whose reductions clusters share: 160 -> 960 -> 160 on one 7 x 7 map 22.4 us here, 11.0 there.
+  // 0.3 %; five of 373 are more than 3 % slower than three launches, by 8 % at most), at 0.9 where a CTA has several tiles in turn
+  // (0.888; two of 126 by up to 5 %; at 0.95 0.886 but nine by up to 21 %: 32 -> 192 -> 32 on 30 maps of 51 x 48 37.1 us here,
+  // 30.7 in three).  Long reductions of few pixels stay with the launches, whose reductions clusters share: 160 -> 960 -> 160 on
+  // one 7 x 7 map 22.4 us here, 11.0 there.
   if (one_launch_cycles(*p, n_sm) > (p->tiles > n_sm ? 0.9 : 1.03) * three_launches_cycles(*p, !k3.rows)) return false;
   p->inv_lines = inv20(p->lines_img); p->inv_wbox = inv20(p->wbox); p->inv_th = inv20(p->th);
   p->inv_strips = inv20(p->strips); p->inv_outs = inv20(p->th * p->tw); p->inv_tw = inv20(p->tw);

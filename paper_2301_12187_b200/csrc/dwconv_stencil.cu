@@ -6,16 +6,17 @@
 // so the stencil itself has no border cases.  Threads then compute from shared memory: a thread owns
 // 4 channels of TX neighbouring outputs of R rows (two where the tiles give every thread enough, one otherwise), so that an
 // input is read and unpacked once for all the outputs it feeds -- 9 instructions per output value of a 3x3 layer with 7 x
-// 2 outputs, 13 with the 8 channels x 7 x 1 of before -- with fp32 weights and fp32 accumulation, and writes 8-byte pieces (neighbouring threads write neighbouring pieces of a pixel: whole 32-byte
-// sectors).  Depthwise layers are bound by HBM (1.8-4.5 FLOP/B):
+// 2 outputs, 13 with the 8 channels x 7 x 1 of before -- with fp32 weights and fp32 accumulation, and writes 8-byte pieces
+// (neighbouring threads write neighbouring pieces of a pixel: whole 32-byte sectors).  Depthwise layers are bound by HBM (1.8-4.5
+// FLOP/B):
 // the tile is read from HBM once (neighbouring tiles share only their halo rows), and several CTAs
 // per SM overlap one tile's load with another's arithmetic and stores.  No tensor cores.
 //
 // Channels come in tiles of 32, 16 or 8, the last one of a pixel partly filled where that is cheaper than narrow tiles (with 8
 // channels a line the load unit moves half as many bytes).  All three are compile-time: every shared-memory offset of the
-// stencil is an immediate.  Inputs from HBM: 144 channels, 64 images of 56 x 56 28.8 -> 25.2 us, of stride 2 23.1 -> 16.7, one
-// image 4.5 -> 2.5; 40 channels, 32 images 14.1 -> 7.5; 96 channels of stride 2, 20 images of 100 x 100 14.3 -> 11.6; 240
-// channels 5x5, 64 images of 28 x 28 27.7 -> 24.2.
+// stencil is an immediate.  Inputs from HBM, against the 8 channels x 7 x 1: 144 channels, 64 images of 56 x 56 28.8 -> 25.6 us, of
+// stride 2 23.1 -> 16.3, one image 4.9 -> 3.0; 40 channels, 32 images 14.3 -> 6.8; 96 channels of stride 2, 20 images of 100 x 100
+// 14.6 -> 12.0; 240 channels 5x5, 64 images of 28 x 28 27.6 -> 24.6.
 //
 // The one wait (for the tile to land) is bounded like every wait of the library; a wait that runs
 // out sets a library-wide flag that dc_dwconv_status reports, and the CTA returns.
@@ -238,7 +239,7 @@ bool make_stencil_plan(int n, int h, int w, int c, int k, int stride, int pad, S
   // 5x5, maps of 7 to 112, 1 to 128 images) timed in up to 24 tiles each, 6324 timings, for the choice: 3.4 % above the best on
   // average, 27 % at worst (80 channels of stride 2, 31 maps of 13 x 13).  A product of powers of the two, without the weights and the
   // places, fitted to 26 layers, chose tiles 8.8 % above the best, 64 % at worst: 304 channels 5x5, 35 maps of 7 x 7 5.6 us, now 4.4;
-  // 88 channels 5x5 of stride 2, 4 of 21 x 20 3.1, now 2.3; 192 channels, 121 of 9 x 10 5.8, now 5.0.
+  // 88 channels 5x5 of stride 2, 4 of 21 x 20 3.1, now 2.4; 192 channels, 121 of 9 x 10 5.8, now 5.0.
   auto consider = [&](int r, int ct, int rt, int ni) {
     const int rows = dc_div_up(rt, r) * r, in_rows = (rows - 1) * stride + k;
     const long long bytes = (long long)ni * in_rows * p->in_w * ct * 2;
