@@ -74,6 +74,7 @@ struct PairParams {
   int mb, mb_last;             // blocks of a full tile / of a strip's last (shorter) tile
   int a_stage_bytes, a_box_bytes, a_plane_bytes, b_bytes;   // stride 2: a stage is two planes (even / odd rows)
   int stages, slots, groups, mma_warps, act, bulk_out, out_buf_bytes;
+  int tile_first;              // the first tile is asked for before the weights
   int off_b, off_bias, off_out, off_a, smem_bytes;
   int tmem_cols;
   int nmma;
@@ -414,9 +415,7 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
     if (did) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // What comes between the start of the call and its first tile is time that nothing overlaps: where the first tile lies is
-  // worked out while the previous kernel ends, and a stage's first use waits for nothing.  180 layers take 0.982 of the time
-  // without that on average, one 3 % more; with the first tile asked for before the weights 0.990, nine 3 to 6 % more (24 -> 32 of
-  // stride 2, 128 images of 56 x 56 7.1 us, 6.95 this way).
+  // worked out while the previous kernel ends, and a stage's first use waits for nothing.
   Walk first;
   first.start(p, tile0);
   dc_pdl_enter();                                // nothing above touched global memory; everything below may
@@ -440,9 +439,10 @@ k_conv_tc_pairrows(const __grid_constant__ CUtensorMap map_a, const __grid_const
       }
     };
     if (lane == 0) {
+      if (p.tile_first) request(first, 0);
       mbar_arrive_expect_tx(&sh.weights, (uint32_t)p.b_bytes);
       bulk_load(smem_u32(smem_b), w_packed, (uint32_t)p.b_bytes, &sh.weights);   // packed weights are the operand layout
-      request(first, 0);
+      if (!p.tile_first) request(first, 0);
     }
     const int inflight = p.stages < kInFlight ? p.stages : kInFlight;   // never more than there are stages
     if (ODD) {
@@ -732,6 +732,11 @@ bool make_pair_plan(int n, int h, int w, const dc_geom *g, int n_sm, PairParams 
   p->stages = stages;
   p->off_out = p->off_a + stages * p->a_stage_bytes;
   p->smem_bytes = (int)total_bytes(th, stages);
+  // The first tile is asked for before the weights where the input is large and may come from HBM, behind them where it is small.
+  // Of 95 layers with inputs from HBM those of 1.3 MB and more are up to 4.5 % faster that way (32 -> 32 5x5, 128 images of 28 x 28 13.4 ->
+  // 12.8 us; with inputs from L2 up to 6 % slower, 24 -> 32 of stride 2, 128 of 56 x 56 6.95 -> 7.1), smaller ones up to 7 % slower
+  // wherever they come from (24 -> 24, one 56 x 56 image 3.31 -> 3.55).
+  p->tile_first = (long long)n * h * w * g->c_in * 2 >= 1280 * 1024;
   // one instruction per (tap row r, pair shift t, 32-byte K step): where its operand starts in a stage
   int j = 0;
   for (int r = 0; r < g->k; ++r)
