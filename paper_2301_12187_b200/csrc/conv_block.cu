@@ -20,7 +20,7 @@
 //
 // What bounds it is a chunk's chain in a group of warps: its accumulators, their way out of tensor memory, conversion, a barrier,
 // the stencil, the hand-over.  Half of the cycles issue nothing (64 -> 384 -> 64, 128 images of 14 x 14: issue slots 48 % taken,
-// FMA pipe 19 %, the largest stall is on what memory returns), and of the 11.9 thousand warp instructions of a chunk the stencil,
+// FMA pipe 19 %, the largest stall is on what memory returns), and of the 11.8 thousand warp instructions of a chunk the stencil,
 // 4.5 packed FMAs and 7 others per hidden value, has 4.5.  That block takes 20.2 us, 25.1 as three launches; one image 9.4 and
 // 10.1; 24 -> 144 -> 24, 64 images of 56 x 56 60 and 111; 16 -> 96 -> 16, 20 images of 9 x 9 6.4 and 13.9.  Measured and not kept:
 // two rows of outputs per thread (fewer instructions, but more than the 96 registers that 19 warps leave: 10 % slower), both
