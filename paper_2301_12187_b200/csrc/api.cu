@@ -23,6 +23,7 @@ extern "C" size_t dc_conv_workspace_bytes(void) { return sizeof(DcWsHeader); }
 
 extern "C" const char *dc_conv_kernel_name(int n, int h, int w, const dc_geom *g, dc_dtype dtype) {
   if (dc_validate_geom(g) != DC_OK || g->groups != 1 || n <= 0 || h <= 0 || w <= 0) return nullptr;
+  if (dtype == DC_F32 && dc_conv_f32_tc_supported(n, h, w, g)) return "k_conv_f32_tc";
   if (dtype == DC_F32) return dc_conv_f32_supported(n, h, w, g) ? "k_conv_dense_f32" : "k_conv_dense_f32_any";
   if (dtype != DC_BF16) return nullptr;
   if (dc_conv_pairrows_supported(n, h, w, g)) return "k_conv_tc_pairrows";
@@ -71,6 +72,10 @@ extern "C" dc_status dc_conv_forward_algo(const void *x, int n, int h, int w, co
     }
   }
   if (algo == DC_ALGO_TCGEN05) return DC_ERR_UNSUPPORTED;
+  if (dtype == DC_F32 && algo == DC_ALGO_AUTO) {
+    s = dc_launch_conv_f32_tc(x, n, h, w, g, w_packed, bias, act, residual, y, workspace, st);
+    if (s != DC_ERR_UNSUPPORTED) return s;
+  }
   return dc_launch_conv_simt(x, n, h, w, g, w_packed, bias, act, residual, y, dtype, st);
 }
 

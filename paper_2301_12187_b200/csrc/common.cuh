@@ -458,6 +458,11 @@ dc_status dc_launch_conv_simt(const void *x, int n, int h, int w, const dc_geom 
 bool dc_conv_f32_supported(int n, int h, int w, const dc_geom *g);
 dc_status dc_launch_conv_f32(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                              const float *bias, dc_act act, const void *residual, void *y, cudaStream_t stream);
+double dc_conv_f32_estimate_us(int n, int h, int w, const dc_geom *g);
+// fp32 by three bf16 terms on the tensor core; false and DC_ERR_UNSUPPORTED: outside its range, or slower there than the kernel above
+bool dc_conv_f32_tc_supported(int n, int h, int w, const dc_geom *g);
+dc_status dc_launch_conv_f32_tc(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed, const float *bias,
+                                dc_act act, const void *residual, void *y, void *workspace, cudaStream_t stream);
 dc_status dc_launch_conv_tc(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                             const float *bias, dc_act act, const void *residual, void *y,
                             void *workspace, cudaStream_t stream);

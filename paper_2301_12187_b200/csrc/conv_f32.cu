@@ -326,6 +326,20 @@ bool f32_plan(int n, int h, int w, const dc_geom *g, int n_sm, F32Plan *p) {
 
 }  // namespace
 
+// Estimated time, fitted to 300 layers as this plan runs them (13 % off; the plan's own cost ranks tiles and splits of one layer and is up
+// to three times off from one layer to another).  0: outside the kernel's range.
+double dc_conv_f32_estimate_us(int n, int h, int w, const dc_geom *g) {
+  F32Plan pl;
+  const int n_sm = dc_sm_count();
+  if (!f32_plan(n, h, w, g, n_sm, &pl)) return 0.0;
+  const F32Config &c = kF32Configs[pl.config];
+  const int area = c.tm * c.tn, resident = f32_resident(area);
+  const double on_sm = (double)(((long long)pl.p.m_tiles * pl.p.n_tiles * pl.p.split + n_sm - 1) / n_sm);
+  const double rounds = (double)((long long)(on_sm + resident - 1) / resident);
+  const double fma = on_sm * (28.6 * area + 180.0), chain = rounds * (16.4 * area + 560.0);
+  return (4000.0 + pl.p.slices_per * (fma > chain ? fma : chain) + on_sm * c.bm * (0.33 * c.bn + 3.5) + (pl.p.split > 1 ? 3500.0 : 0.0)) / 1900.0;
+}
+
 bool dc_conv_f32_supported(int n, int h, int w, const dc_geom *g) {
   F32Plan pl;
   return f32_plan(n, h, w, g, dc_sm_count(), &pl);

@@ -111,6 +111,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t sdst, const CUtensorMap *ma
       ::"r"(sdst), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t sdst, const CUtensorMap *map, uint64_t *bar, int c0, int c1, int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+      ::"r"(sdst), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
 // 4-D tile: the innermost coordinate times the element size must be a multiple of 16 bytes
 __device__ __forceinline__ void tma_load_4d(uint32_t sdst, const CUtensorMap *map, uint64_t *bar, int c0, int c1, int c2,
                                             int c3) {

@@ -1184,3 +1184,57 @@ def test_empty_and_degenerate_inputs_are_rejected_or_handled(dc):
         dc.conv_forward(torch.zeros((1, 2, 2, 8), dtype=torch.bfloat16, device="cuda"), dc.geom(8, 8, 1, 5, 1, 0),
                         packed, None, 0, None, y, new_ws(dc))
     assert e.value.status == dc.ERR_SHAPE
+
+
+# n, h, w, c_in, c_out, k, stride, pad: runs of 256 and 128 lines, 16 to 80 outputs a tile, reductions shared by 2 to 8 CTAs, loads of
+# rows, of several and of whole images, odd sides, odd channel groups, outputs that end inside a tile, both strides, more and less
+# padding than "same", shallow rings
+F32_TC_SHAPES = [(32, 28, 28, 32, 32, 5, 1, 2), (3, 52, 52, 48, 128, 3, 1, 1), (1, 44, 44, 192, 72, 5, 1, 2), (3, 97, 97, 160, 72, 3, 2, 1),
+                 (2, 41, 43, 96, 112, 5, 2, 2), (78, 15, 15, 328, 56, 1, 1, 0), (20, 31, 31, 20, 36, 5, 1, 2), (2, 60, 60, 24, 24, 7, 1, 3),
+                 (4, 61, 59, 64, 96, 3, 1, 0), (4, 61, 59, 64, 96, 3, 1, 2), (2, 33, 250, 64, 64, 3, 1, 1), (12, 43, 43, 64, 16, 5, 1, 2),
+                 (40, 11, 11, 96, 96, 3, 1, 1), (1, 37, 37, 208, 72, 5, 1, 2), (2, 7, 7, 512, 512, 3, 1, 1), (8, 14, 14, 384, 64, 3, 1, 1)]
+
+
+@pytest.mark.parametrize("shape", F32_TC_SHAPES)
+def test_fp32_conv_by_bf16_terms(dc, shape):
+    """fp32 on the tensor core against torch in 64 bits: at most as far from it as the FMA kernel (which the smaller shapes of this
+    file hold to the oracle) and within 4e-7 of the result (2-norm; short sums of exact products, then fp32 additions of at most
+    225 of them: 225 ** 0.5 * 2 ** -25), with bias, skip input and ReLU6 and without; guarded output; an infinity and a NaN in the
+    input and in the weights come out as in the FMA kernel."""
+    n, h, w, ci, co, k, s, p = shape
+    g = dc.geom(ci, co, 1, k, s, p)
+    assert dc.conv_kernel_name(n, h, w, g, dc.F32) == "k_conv_f32_tc"
+    gen = torch.Generator("cuda")
+    gen.manual_seed(ci * 1000 + co)
+    rnd = lambda *d: torch.randn(d, generator=gen, device="cuda")
+    x, wf = rnd(n, h, w, ci), rnd(co, ci, k, k) * (ci * k * k) ** -0.5
+    ho, wo = (h + 2 * p - k) // s + 1, (w + 2 * p - k) // s + 1
+    bias, res = rnd(co), rnd(n, ho, wo, co)
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(wf, g, dc.F32, packed)
+    ws = torch.zeros(dc.conv_workspace_bytes(), dtype=torch.uint8, device="cuda")
+
+    def run(algo, full=False):
+        y = Guarded(torch, (n, ho, wo, co), torch.float32, fill=float("nan"))
+        dc.conv_forward(x, g, packed, bias if full else None, dc.ACT_RELU6 if full else dc.ACT_IDENTITY, res if full else None, y.t, ws,
+                        algo=algo)
+        y.check("output")
+        return y.t
+
+    ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), wf.double(), None, s, p).permute(0, 2, 3, 1)
+    err = lambda y, r: ((y.double() - r).norm() / r.norm()).item()
+    worst = lambda y, r: ((y.double() - r).abs().max() / r.square().mean().sqrt()).item()
+    y = run(dc.ALGO_AUTO)
+    assert err(y, ref) <= min(4e-7, 1.02 * err(run(dc.ALGO_SIMT), ref)) and worst(y, ref) <= 1e-5
+    full = (ref + bias.double() + res.double()).clamp(0, 6)
+    y = run(dc.ALGO_AUTO, full=True)
+    assert err(y, full) <= 4e-7 and worst(y, full) <= 1e-5
+    assert dc.workspace_status(ws) == dc.OK
+    # what is not finite
+    x[0, 0, 0, 0], x[n - 1, h - 1, w - 1, ci - 1], x[0, h // 2, w // 2, ci // 2] = float("inf"), float("nan"), 3.4e38
+    view = packed.view(torch.float32)[:k * k * ci * co].view(k, k, ci, co)
+    view[k // 2, k // 2, ci - 1, 0], view[0, 0, 0, co - 1] = float("-inf"), float("nan")
+    a, b = run(dc.ALGO_AUTO), run(dc.ALGO_SIMT)
+    same = (a == b) | (torch.isnan(a) & torch.isnan(b))
+    close = (a - b).abs() <= 1e-5 * b.abs().clamp(min=1.0)
+    assert bool((same | (close & torch.isfinite(b))).all()) and bool((~torch.isfinite(b)).any())
