@@ -125,7 +125,8 @@ dc_status dc_packed_bytes(const dc_geom *g, dc_dtype dtype, size_t *bytes);
  * Outputs (device): w_merged fp32 [c_out][c_in][k'][k'], b_merged fp32 [c_out]; if w_packed is
  * not NULL also the packed copy for packed_dtype (size from dc_packed_bytes).  workspace: device,
  * at least the bytes dc_merge_query reports; it overlaps nothing else.  The outputs may overlap the
- * layers' arrays (which then do not survive the call), not one another.  fp32 FMA arithmetic throughout.
+ * layers' arrays (which then do not survive the call), not one another.  fp32 arithmetic: FMAs, or on the tensor
+ * core products of exact bf16 terms of fp32 values, added up in fp32.
  */
 dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
                          float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,
@@ -231,9 +232,9 @@ dc_status dc_dwconv_forward(const void *x, int n, int h, int w, int c, int k, in
                             dc_dtype dtype, dc_stream stream);
 
 /*
- * Synchronises `stream`, then returns DC_ERR_TIMEOUT if the bounded wait of a depthwise launch
- * (which takes no workspace to latch it in) ran out on the current device since the last call,
- * DC_OK otherwise; clears the flag.
+ * Synchronises `stream`, then returns DC_ERR_TIMEOUT if a bounded wait of a depthwise launch or of a
+ * merge on the tensor core (which take no workspace to latch it in) ran out on the current device
+ * since the last call, DC_OK otherwise; clears the flag.
  */
 dc_status dc_dwconv_status(dc_stream stream);
 

@@ -36,7 +36,7 @@
 // 1x1, 78 of 15 x 15 36 -> 19.
 //
 // On the way (first layer): weights and activations through cp.async slots and a wait for each step of weights 41.7 us; by TMA the same; waits
-// and commits by chunks 27.8; two issuing warps 24.4; two runs of lines 19.8.  conversions (cvt.rn.bf16x2) instead of the integer
+// and commits by chunks 27.8; two issuing warps 24.4; two runs of lines 19.8.  Terms by integer rounding
 // rounding in cut2 the same.
 #include "tc_ptx.cuh"
 
@@ -74,31 +74,6 @@ struct Params {
   unsigned char tap_uv[kMaxTaps + 32];         // tap row * k + tap column, by planes
   unsigned short tap_line[kMaxTaps + kFlush];       // lines that the tap is further on
 };
-
-// The bf16 terms of two values, high, middle and low: the first two rounded to nearest (halves up in magnitude, by an addition below
-// the cut, which costs no conversion), what is left then has 8 bits.  Cut off instead of rounded, the dropped products all
-// have the sign of the kept ones: 12 -> 100 1x1 0.75e-7 instead of 0.33e-7 from 64 bits.
-__device__ __forceinline__ void cut2(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l) {
-  uint32_t x = __float_as_uint(a) + 0x8000u, z = __float_as_uint(b) + 0x8000u;
-  h = __byte_perm(x, z, 0x7632);
-  a -= __uint_as_float(x & 0xFFFF0000u);
-  b -= __uint_as_float(z & 0xFFFF0000u);
-  x = __float_as_uint(a) + 0x8000u;
-  z = __float_as_uint(b) + 0x8000u;
-  m = __byte_perm(x, z, 0x7632);
-  l = __byte_perm(__float_as_uint(a - __uint_as_float(x & 0xFFFF0000u)), __float_as_uint(b - __uint_as_float(z & 0xFFFF0000u)), 0x7632);
-}
-__device__ __forceinline__ void cut8(const float *v, uint4 &h, uint4 &m, uint4 &l) {
-  cut2(v[0], v[1], h.x, m.x, l.x);
-  cut2(v[2], v[3], h.y, m.y, l.y);
-  cut2(v[4], v[5], h.z, m.z, l.z);
-  cut2(v[6], v[7], h.w, m.w, l.w);
-}
-__device__ __forceinline__ float lds_f(uint32_t a) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
-}
 
 __device__ __forceinline__ void store4(const Params &p, const float *bias, const float *residual, float *y, int pix, int o, float4 s) {
   if (bias) {
@@ -349,8 +324,8 @@ k_conv_f32_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
             const float v1[8] = {__uint_as_float(u2.x), __uint_as_float(u2.y), __uint_as_float(u2.z), __uint_as_float(u2.w),
                                  __uint_as_float(u3.x), __uint_as_float(u3.y), __uint_as_float(u3.z), __uint_as_float(u3.w)};
             uint4 h0, m0, l0, h1, m1, l1;
-            cut8(v0, h0, m0, l0);
-            cut8(v1, h1, m1, l1);
+            bf16_terms8(v0, h0, m0, l0);
+            bf16_terms8(v1, h1, m1, l1);
             sts_u4(d0, h0);
             sts_u4(d0 + 2 * chunk_a, m0);
             sts_u4(d0 + 4 * chunk_a, l0);
@@ -401,8 +376,8 @@ k_conv_f32_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
 #pragma unroll
             for (int j = 0; j < 8; ++j) v1[j] = lds_f(f1 + (uint32_t)(j * NT * 4));
             uint4 h0, m0, l0, h1, m1, l1;
-            cut8(v0, h0, m0, l0);
-            cut8(v1, h1, m1, l1);
+            bf16_terms8(v0, h0, m0, l0);
+            bf16_terms8(v1, h1, m1, l1);
             sts_u4(d0, h0);
             sts_u4(d0 + NT * 16u, m0);
             sts_u4(d0 + NT * 32u, l0);

@@ -20,6 +20,7 @@
 //
 // The one wait (for the tile to land) is bounded like every wait of the library; a wait that runs
 // out sets a library-wide flag that dc_dwconv_status reports, and the CTA returns.
+#include "merge_parts.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
@@ -357,7 +358,9 @@ extern "C" dc_status dc_dwconv_status(dc_stream stream) {
   if (st != 0) {
     const unsigned int zero = 0;
     DC_CUDA_OK(cudaMemcpyToSymbol(g_dw_status, &zero, sizeof(zero)));
-    return DC_ERR_TIMEOUT;
   }
-  return DC_OK;
+  bool merge = false;
+  const dc_status s = dc_merge_tc_status(&merge);
+  if (s != DC_OK) return s;
+  return st != 0 || merge ? DC_ERR_TIMEOUT : DC_OK;
 }

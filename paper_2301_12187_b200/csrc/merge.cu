@@ -1,9 +1,9 @@
 // BN folding, composition of a run of convolutions into one convolution, and weight repacking.
-// fp32 FMA arithmetic on CUDA cores: the merged weights must match an fp64 evaluation of the
-// same formula to 1e-5 relative, which rules out reduced-precision tensor-core math.
+// fp32 FMA arithmetic on CUDA cores (the merged weights must match an fp64 evaluation of the same formula to 1e-5 relative; large
+// 3x3 pairs go to the tensor core in exact terms, merge_tc.cu).
 #include <vector>
 
-#include "common.cuh"
+#include "merge_parts.cuh"
 
 // ----------------------------------------------------------------------------------------------
 // kernels
@@ -565,10 +565,6 @@ __global__ void k_deliver(Piece acc, float *w_merged, float *b_merged, void *pac
 // elements those waits are the whole cost.  One CTA per output channel o; the raw layer weights are
 // read once per CTA (they sit in L2), `chunk` hidden channels at a time.
 // ----------------------------------------------------------------------------------------------
-struct RawLayer {
-  const float *w, *b, *gamma, *beta, *mean, *var;
-  float eps;
-};
 struct BlockArgs {
   RawLayer l1, l2, l3;
   int c0, c1, c2, k;      // input, hidden, output channels; depthwise kernel size
@@ -577,14 +573,6 @@ struct BlockArgs {
 };
 constexpr int kBlockThreads = 256;
 constexpr int kBlockMaxPerThread = 8;       // outputs per thread: c0 * k * k <= 2048
-
-__device__ __forceinline__ float raw_scale(const RawLayer &L, int o) {
-  return L.gamma ? L.gamma[o] / sqrtf(L.var[o] + L.eps) : 1.f;
-}
-__device__ __forceinline__ float raw_bias(const RawLayer &L, int o, float g) {
-  const float b = L.b ? L.b[o] : 0.f;
-  return L.gamma ? fmaf(b - L.mean[o], g, L.beta[o]) : b;
-}
 
 // Up to kBlockBatch blocks of one run go out in one launch (blockIdx.y picks the block): they depend
 // on the raw layers only, not on one another.
@@ -701,76 +689,6 @@ struct TiledBlocks {
   int first[kBlockBatch + 1];    // first CTA of each block's tiles and bias groups
   int n;
 };
-struct BlockDelivery {           // of a run that is one block; mode < 0: the block is a piece of a longer run
-  void *packed;
-  int mode;                      // 0: no packed copy, 1: fp32, 2: bf16 chunks
-  int ident;
-  KOrder ko;
-};
-
-__device__ __forceinline__ void mb_cp16(float *dst, const float *src, bool ok) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst), n = ok ? 16u : 0u;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n));
-}
-
-// true when chunk `idx8` of the packed bf16 copy holds weights (c_in is a multiple of 8: all of them or none)
-__device__ __forceinline__ bool packed_chunk_live(const KOrder &ko, int idx8, int c_out) {
-  int plane, o, pc, ccg, r, s;
-  dc_packed_unchunk(ko, idx8, &plane, &o);
-  const int grp = plane / ko.e_pad, e = plane - grp * ko.e_pad;
-  if (!dc_korder_decode(ko, e, &pc, &ccg, &r, &s)) return false;
-  if (ko.fold) {
-    s = o / ko.co8;
-    return s < ko.k && o - s * ko.co8 < c_out;
-  }
-  if (ko.pair >= 2) {
-    int px = 0;
-    if (ko.pair == 2) { px = o / ko.co8; o -= px * ko.co8; }
-    s = 2 * s + (ccg >= ko.cch ? 1 : 0) - (ko.pair == 2 ? px : (ko.pad & 1));
-    return px < 2 && o < c_out && s >= 0 && s < ko.k;
-  }
-  return o < c_out && (grp * ko.cg + ccg) * 8 < ko.c_in;
-}
-
-// The packed copy of a tile of OT output x IT input channels whose K x K kernels lie in shared memory as
-// [o][i][tap].  fp32: [tap][i][o].  bf16: one chunk of 8 input channels per (output channel, chunk, tap), written
-// where the forward kernels' K order wants it; pair rows hold every chunk twice, the second copy one pixel further on.
-template <int OT, int IT, int K>
-__device__ __forceinline__ void deliver_tile(const BlockDelivery &dv, const float *sums, int o0, int i0, int c0, int c2,
-                                             int tid, int threads) {
-  constexpr int KK = K * K;
-  if (dv.mode == 1) {
-    float *out = reinterpret_cast<float *>(dv.packed);
-    for (int e = tid; e < OT * IT * KK; e += threads) {
-      const int ow = e % OT, rest = e / OT, iw = rest % IT, t = rest / IT;
-      if (o0 + ow < c2 && i0 + iw < c0) out[((size_t)t * c0 + i0 + iw) * c2 + o0 + ow] = sums[(ow * IT + iw) * KK + t];
-    }
-    return;
-  }
-  uint4 *out = reinterpret_cast<uint4 *>(dv.packed);
-  for (int e = tid; e < OT * (IT / 8) * KK; e += threads) {
-    const int ow = e % OT, rest = e / OT, hf = rest % (IT / 8), t = rest / (IT / 8), o = o0 + ow, ch = i0 + hf * 8;
-    if (o >= c2 || ch >= c0) continue;
-    __align__(16) __nv_bfloat16 v8[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(sums[(ow * IT + hf * 8 + q) * KK + t]);
-    const uint4 v = *reinterpret_cast<const uint4 *>(v8);
-    const int r = t / K, sx = t - K * r;
-    out[dc_packed_chunk(dv.ko, dc_korder_encode(dv.ko, ch >> 3, r, sx), dc_korder_row(dv.ko, sx, o))] = v;
-    if (dv.ko.pair == 2) {
-      const int plane = (r * dv.ko.ns[0] + ((sx + 1) >> 1)) * 2 * dv.ko.cch + ((sx + 1) & 1) * dv.ko.cch + (ch >> 3);
-      out[dc_packed_chunk(dv.ko, plane, dv.ko.co8 + o)] = v;
-    }
-  }
-}
-
-// zeroes the chunks of the packed bf16 copy that hold no weight; CTA `cta` of `ctas`
-__device__ __forceinline__ void zero_dead_chunks(const BlockDelivery &dv, int c_out, int cta, int ctas) {
-  const int total8 = dv.ko.ng * dv.ko.e_pad * dv.ko.n_pad;
-  for (int e = cta * (int)blockDim.x + (int)threadIdx.x; e < total8; e += ctas * (int)blockDim.x)
-    if (!packed_chunk_live(dv.ko, e, c_out)) reinterpret_cast<uint4 *>(dv.packed)[e] = make_uint4(0u, 0u, 0u, 0u);
-}
-
 template <int IT, int W>
 __global__ void __launch_bounds__(W * 32, W == 8 ? 2 : 1)
 k_merge_block33(const __grid_constant__ TiledBlocks tb, const __grid_constant__ BlockDelivery dv) {
@@ -988,17 +906,6 @@ struct P3Form {
   static constexpr int RING = W * kP3Stages * kP3Stage, BYTES = (RING + (W < kP3Parts ? W * kP3Tile : 0)) * 4;
 };
 
-struct Operand33 {
-  RawLayer l;                    // weights, bias, BN (none for a piece)
-  int ident;                     // the identity kernel is added
-};
-struct Compose33 {
-  Operand33 first, second;
-  int c0, c1, c2;
-  float *w_out, *b_out;
-  int gi, go;                    // tiles
-};
-
 template <int W>
 __global__ void __launch_bounds__(W * 32, 16 / W)
 k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDelivery dv) {
@@ -1018,19 +925,7 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
     }
     // ---- bias: b'[o] = b2~[o] + sum_c (g2 sum of W2[o][c] (+ 1 where c == o and an identity rides)) b1~[c]; a warp per o
     for (int o = blk * kP3O + warp; o < c2 && o < (blk + 1) * kP3O; o += W) {
-      const float g2 = raw_scale(l2, o);
-      float s = 0.f;
-#pragma unroll 2
-      for (int c = lane; c < c1; c += 32) {
-        const float b1 = raw_bias(l1, c, raw_scale(l1, c));
-        float ws = (a.second.ident && c == o) ? 1.f : 0.f;
-        float wt = 0.f;
-#pragma unroll
-        for (int t = 0; t < 9; ++t) wt += l2.w[((size_t)o * c1 + c) * 9 + t];
-        s = fmaf(fmaf(g2, wt, ws), b1, s);
-      }
-      for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-      if (lane == 0) a.b_out[o] = raw_bias(l2, o, g2) + s;
+      compose33_bias(a, o, lane);
     }
     return;
   }
@@ -1166,15 +1061,7 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
       if (special) {                               // of a tile with identities to add
         float v4[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int iw = (x + q) / 25, t = x + q - iw * 25, i = i0 + iw;
-          const int u = t / 5 - 1, v = t - (t / 5) * 5 - 1;          // tap of the 3x3 kernel centred in the 5x5 one
-          if (u >= 0 && u < 3 && v >= 0 && v < 3) {
-            if (a.first.ident) v4[q] = fmaf(g2, l2.w[((size_t)o * c1 + i) * 9 + u * 3 + v], v4[q]);                 // W2 o I
-            if (a.second.ident) v4[q] = fmaf(raw_scale(l1, o), l1.w[((size_t)o * c0 + i) * 9 + u * 3 + v], v4[q]);  // I o W1
-          }
-          if (t == 12 && o == i) v4[q] += (a.first.ident && a.second.ident ? 1.f : 0.f) + (last && dv.ident ? 1.f : 0.f);
-        }
+        for (int q = 0; q < 4; ++q) v4[q] = compose33_ident(a, last && dv.ident, g2, v4[q], o, i0 + (x + q) / 25, (x + q) % 25);
         s = make_float4(v4[0], v4[1], v4[2], v4[3]);
       }
       *reinterpret_cast<float4 *>(a.w_out + ((size_t)o * c0 + i0) * 25 + x) = s;
@@ -1651,6 +1538,19 @@ static void launch_compose33_form(const Compose33 &a, const BlockDelivery &dv, c
   status.note(dc_launch_pdl(k_compose33<W>, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, W * 32)), dim3(W * 32), P3Form<W>::BYTES, st, a, dv));
   status.launched();
 }
+// By estimates of both in microseconds, fitted to 82 pairs of 32 to 512 channels timed on either side (on the tensor core 3 % off, by
+// FMAs 13 %): of the 82 this line sends 31 there, together 0.90 of the time on (geometric) average (always the faster one: 0.89), none
+// slower; a line at 1.05 sends 36, two of them 3 % slower.  There a CTA's first tile takes 6.4 us and 0.6 for every 16 channels
+// between, a further one 4.7 us or more: many output and input channels, and enough between them, go there.
+static bool compose33_on_tensor_core(int c0, int c1, int c2) {
+  const int n_sm = dc_sm_count(), steps = dc_div_up(c1, 64) * 4, tiles = dc_div_up(c0, 8) * dc_div_up(c2, 8), most = dc_div_up(tiles, n_sm);
+  const double further = steps > 16 ? 0.57 * steps : (steps > 7 ? 2.5 + 0.3 * steps : 4.7);
+  const double tc = 6.4 + 0.6 * steps + (dc_div_up(dc_div_up(c2, 14) * dc_div_up(c0, 8), n_sm) - 1) * further;
+  const double fma = 4.0 + most * c1 * (most > 1 || 2 * tiles <= n_sm ? 0.042 : 0.063);
+  return tc < 0.95 * fma;
+}
+
+
 // Four warps a tile, four tiles to an SM at once, except where the tiles of the SM with the most of them fill whole rounds of two
 // better than of four: one or two of them (136 -> 136 -> 136: 25.6 us by four warps, 17.8 by eight), or three or five with a
 // reduction long enough to matter (160 -> 160 -> 160, three: 29.1 and 24.1, with 48 channels between 12.7 and 13.2; 208 -> 208 ->
@@ -1659,6 +1559,10 @@ static void launch_compose33_form(const Compose33 &a, const BlockDelivery &dv, c
 static void launch_compose33(const Operand33 &first, const Operand33 &second, int c0, int c1, int c2, float *w, float *b,
                              const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
+  if (compose33_on_tensor_core(c0, c1, c2)) {
+    status.note(dc_launch_compose33_tc(a, dv, st));
+    return;
+  }
   const int most = dc_div_up(a.gi * a.go, dc_sm_count());
   if (most <= 2 || ((most == 3 || most == 5) && c1 >= 128)) launch_compose33_form<8>(a, dv, mg, st, status);
   else launch_compose33_form<4>(a, dv, mg, st, status);

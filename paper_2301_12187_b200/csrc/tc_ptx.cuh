@@ -212,6 +212,25 @@ __device__ __forceinline__ uint4 bias_terms(float b) {
 }
 // the constant operand's row for them: 1.0 in its first three K elements
 __device__ __forceinline__ uint4 bias_ones() { return make_uint4(0x3F803F80u, 0x3F80u, 0u, 0u); }
+// The three bf16 terms of fp32 values, high, middle and low: the first two rounded to nearest, what is left then has 8 bits.  (Cut
+// off instead of rounded, the products of terms that a sum leaves out all have the sign of the kept ones: a fp32 1x1 convolution
+// of 12 channels is 0.75e-7 instead of 0.33e-7 from 64 bits.)  An infinity, a NaN and what lies beyond the largest bf16 leave a NaN
+// among their terms.
+__device__ __forceinline__ void bf16_terms2(float a, float b, uint32_t &h, uint32_t &m, uint32_t &l) {
+  h = pack_bf16x2(a, b);
+  a -= __uint_as_float(h << 16);
+  b -= __uint_as_float(h & 0xFFFF0000u);
+  m = pack_bf16x2(a, b);
+  a -= __uint_as_float(m << 16);
+  b -= __uint_as_float(m & 0xFFFF0000u);
+  l = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+__device__ __forceinline__ void bf16_terms8(const float *v, uint4 &h, uint4 &m, uint4 &l) {
+  bf16_terms2(v[0], v[1], h.x, m.x, l.x);
+  bf16_terms2(v[2], v[3], h.y, m.y, l.y);
+  bf16_terms2(v[4], v[5], h.z, m.z, l.z);
+  bf16_terms2(v[6], v[7], h.w, m.w, l.w);
+}
 // min of packed bf16 pairs
 __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
   uint32_t d;
@@ -239,6 +258,11 @@ __device__ __forceinline__ void sts_u4(uint32_t a, uint4 v) {
 __device__ __forceinline__ uint4 lds_u4(uint32_t a) {
   uint4 v;
   asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float lds_f(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ void bar_sync(int id, int count) {

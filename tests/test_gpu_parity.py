@@ -1238,3 +1238,54 @@ def test_fp32_conv_by_bf16_terms(dc, shape):
     same = (a == b) | (torch.isnan(a) & torch.isnan(b))
     close = (a - b).abs() <= 1e-5 * b.abs().clamp(min=1.0)
     assert bool((same | (close & torch.isfinite(b))).all()) and bool((~torch.isfinite(b)).any())
+
+
+@pytest.mark.parametrize("a,c,o,res,codes", [
+    (104, 208, 136, [], "both"),               # a round of tiles and a bit
+    (40, 120, 192, [], "both"),                # a tile a CTA, 8 of the last step's 64 channels
+    (256, 256, 256, [], "both"),               # runs of tiles that change columns
+    (196, 132, 250, [], "f32"),                # nothing a multiple of a tile or a step
+    (168, 168, 168, [(0, 0)], "both"), (168, 168, 168, [(0, 0), (1, 1)], "both"), (168, 168, 168, [(0, 1)], "both"),
+    (160, 320, 160, [], "both"),               # columns' terms cut again for every tile
+    (24, 1216, 40, [], "both"),                # a packed order that holds pixels in its rows
+])
+def test_3x3_after_3x3_by_bf16_terms_against_the_oracle(dc, a, c, o, res, codes):
+    specs = [I.make_layer(86, 0, a, c, 3, 1, 1), I.make_layer(86, 1, c, o, 3, 1, 1)]
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
+    assert dc.dwconv_status() == dc.OK
+    if c >= 192 and not res:
+        # sums of 128 products in the tensor core, cut below 2 ** -24 of the largest, then fp32 additions: 1.7e-7 measured at most; one
+        # chain of FMAs over that many channels is 2.05e-7 or more away (so this also tells that it was not taken)
+        W = O.merge_formula(specs, res)[0]
+        _, wm, _, _ = run_merge(dc, specs, res, packed_dtype=dc.F32)
+        assert O.rel_l2(wm.cpu().numpy(), W) <= 1.95e-7
+
+
+def test_3x3_after_3x3_by_bf16_terms_as_a_piece(dc):
+    _check_delivery(dc, [I.make_layer(87, 0, 120, 200, 3, 1, 1), I.make_layer(87, 1, 200, 136, 3, 1, 1), I.make_layer(87, 2, 136, 16, 1, 1, 0)], [],
+                    (dc.BF16, dc.F32))
+
+
+def test_3x3_after_3x3_by_bf16_terms_of_what_is_not_finite(dc):
+    """An infinity, a NaN and a value beyond the largest bf16 among the weights: infinities and NaN where 64 bits have them."""
+    specs = [I.make_layer(88, 0, 104, 208, 3, 1, 1, with_bn=False), I.make_layer(88, 1, 208, 136, 3, 1, 1, with_bn=False)]
+    w1, w2 = specs[0].weight, specs[1].weight
+    w1[5, 7, 0, 1], w1[200, 103, 2, 2], w2[9, 11, 1, 1] = np.inf, np.nan, 3.4e38
+    w1[11] *= 2.0 ** -20                           # the products of the largest value stay finite
+    layers = [dc.DeviceLayer(s) for s in specs]
+    g, ws_bytes = dc.merge_query(layers, [])
+    wm, bm = torch.zeros(g.c_out, g.c_in, 5, 5, device="cuda"), torch.empty(g.c_out, device="cuda")
+    dc.merge_chain(layers, [], wm, bm, None, dc.F32, torch.empty(ws_bytes, dtype=torch.uint8, device="cuda"))
+    t1, t2 = (torch.from_numpy(w).double().cuda() for w in (w1, w2))
+    ref = torch.zeros(136, 104, 5, 5, dtype=torch.float64, device="cuda")
+    for u in range(3):
+        for v in range(3):
+            for p in range(3):
+                for q in range(3):
+                    ref[:, :, u + p, v + q] += (t2[:, :, u, v, None] * t1[None, :, :, p, q]).sum(1)
+    wm = wm.double()
+    assert torch.equal(torch.isnan(wm), torch.isnan(ref)) and torch.equal(torch.isinf(wm), torch.isinf(ref))
+    fin = torch.isfinite(ref)
+    big = ref.abs() > 1e20
+    assert bool((wm[fin & big] / ref[fin & big] - 1).abs().max() < 1e-5) and int((fin & big).sum()) > 0
+    assert ((wm - ref)[fin & ~big].norm() / ref[fin & ~big].norm()).item() <= 3e-7
