@@ -192,8 +192,17 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
       return;
     }
   }
-  if (g->groups == 1 && g->stride == 1 && g->k >= 3 && g->k <= 7 && ko->cch <= 8 && ko->co8 <= 32 &&
-      g->c_in % 8 == 0 && g->c_out % 8 == 0) {
+  // Fewer than 32 outputs from 40 channels or more go by rows too, like the wider layers below: neither the general kernel's gather nor
+  // the fold kernel's repacking keeps up with their instructions, and the fold kernel has no room for 5x5 on maps wider than about 40,
+  // which then ran on the CUDA cores.  144 -> 24 1x1, 128 images of 56 x 56 99 us there, 25 by rows; 72 -> 24, 32 of 77 x 80 31 and 12;
+  // 112 -> 16 3x3, 104 of 9 x 9 22 and 6; 136 -> 24 5x5, 20 of 69 x 66 87 and 39; 48 -> 24 5x5, one of 44 x 44 58 and 4.9.  Over 97 such
+  // layers 0.31 of the time on (geometric) average, one slower, by 2 %.  3x3 layers of 24 outputs and 1x1 layers of 8 keep the
+  // kernels they have, though they would gain as much (152 -> 24 3x3, 50 of 28 x 28 121 and 12): which kernels read their packed
+  // order is held by tests.
+  const bool narrow_rows = g->groups == 1 && g->stride == 1 && g->k <= 7 && ko->cch >= 5 && g->c_out < 32 &&
+                           (g->k == 1 ? g->c_out >= 16 : g->k != 3 || g->c_out <= 16) && g->c_in % 8 == 0 && g->c_out % 8 == 0;
+  if (g->groups == 1 && g->stride == 1 && g->k >= 3 && ko->cch >= 5 && ko->cch <= 8 && (g->c_out == 24 || g->c_out == 32) &&
+      !narrow_rows && g->c_in % 8 == 0) {
     const int n_pad = (int)dc_round_up((size_t)(g->k * ko->co8), 16);
     if ((size_t)ko->cch * g->k * n_pad * 16 <= 64 * 1024) {
       ko->fold = 1;
@@ -214,7 +223,7 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   // column they read, class by class, so that one class reads one sub-tile of every second row and column.
   const bool rows_s2 = g->stride == 2 && g->k >= 3 && ko->cch >= 2;
   if (g->groups == 1 && g->k <= 7 && (g->stride == 1 || rows_s2) &&
-      (rows_s2 || (ko->cch >= 5 ? g->c_out >= 32
+      (rows_s2 || (ko->cch >= 5 ? g->c_out >= 32 || narrow_rows
                     : ((g->k == 1 && ko->cch >= 2 && g->c_out >= 48) || (g->k >= 3 && ko->cch >= 2 && ko->co8 > 128)))) &&
       g->c_in % 8 == 0 && g->c_out % 8 == 0) {
     const int n16 = (int)dc_round_up((size_t)g->c_out, 16);

@@ -649,9 +649,11 @@ double one_launch_cycles(const BlockParams &p, int n_sm) {
   return 5239.0 + dc_div_up(p.tiles, n_sm) * (3207.0 + 239.0 * out + 2.75 * p.planes * p.patch + p.nch * (309.0 + 0.907 * chunk_cycles(p)));
 }
 
-// The three launches' time, in cycles: a start, the hidden maps written and read, the products.  A projection to fewer than 32
-// channels is not the rows kernel's and costs more, most of it a chain over the hidden channels.  Fitted to the same blocks: 7 % off
-// in the root mean square (19 % without the terms of the products and of narrow projections).
+// The three launches' time, in cycles: a start, the hidden maps written and read, the products.  The terms of narrow projections are
+// those of the general kernel, a chain over the hidden channels.  Fitted to the same blocks: 7 % off in the root mean square (19 %
+// without the terms of the products and of narrow projections).  Projections to 16 and 24 channels, by rows, no longer cost that much,
+// but the choice is right with them all the same: over 60 blocks one launch takes 0.78 of the three's time, seven of them more, by up
+// to 9 % (16 -> 96 -> 24 on 23 maps of 103 x 103 51.6 us here, 47.3 in three; 24 -> 144 -> 24 on 9 maps of 12 x 12 7.4 and 10.4).
 double three_launches_cycles(const BlockParams &p, bool narrow) {
   const double hidden = (double)p.n_img * p.h * p.w * p.c_mid * 2e-6, thinned = (double)p.n_img * p.ho * p.wo * p.c_mid * 2e-6;
   const double expand = hidden * 8e-3 * p.ksteps, project = thinned * 5e-4 * p.n3;
@@ -735,7 +737,7 @@ bool make_block_plan(int n, int h, int w, const dc_block *b, int n_sm, BlockPara
   // (0.888; two of 126 by up to 5 %; at 0.95 0.886 but nine by up to 21 %: 32 -> 192 -> 32 on 30 maps of 51 x 48 37.1 us here,
   // 30.7 in three).  Long reductions of few pixels stay with the launches, whose reductions clusters share: 160 -> 960 -> 160 on
   // one 7 x 7 map 22.4 us here, 11.0 there.
-  if (one_launch_cycles(*p, n_sm) > (p->tiles > n_sm ? 0.9 : 1.03) * three_launches_cycles(*p, !k3.rows)) return false;
+  if (one_launch_cycles(*p, n_sm) > (p->tiles > n_sm ? 0.9 : 1.03) * three_launches_cycles(*p, !k3.rows || b->c_out < 32)) return false;
   p->inv_lines = inv20(p->lines_img); p->inv_wbox = inv20(p->wbox); p->inv_th = inv20(p->th);
   p->inv_strips = inv20(p->strips); p->inv_outs = inv20(p->th * p->tw); p->inv_tw = inv20(p->tw);
   p->inv_mbe = inv20(p->mbe); p->inv_mbp = inv20(p->mbp);

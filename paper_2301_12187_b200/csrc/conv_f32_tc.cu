@@ -36,8 +36,7 @@
 // 1x1, 78 of 15 x 15 36 -> 19.
 //
 // On the way (first layer): weights and activations through cp.async slots and a wait for each step of weights 41.7 us; by TMA the same; waits
-// and commits by chunks 27.8; two issuing warps 24.4; two runs of lines 19.8.  Terms by integer rounding
-// rounding in cut2 the same.
+// and commits by chunks 27.8; two issuing warps 24.4; two runs of lines 19.8; terms by integer rounding the same.
 #include "tc_ptx.cuh"
 
 namespace {

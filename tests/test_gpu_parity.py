@@ -617,6 +617,24 @@ def test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, s, p, n, h, 
     assert_close(nchw(y), O.relu6(lin + r.transpose(0, 3, 1, 2)), TOL_BF16)
 
 
+@pytest.mark.parametrize("c_in,c_out,k,p,n,h,w", [
+    (40, 16, 1, 0, 1, 3, 5),         # the fewest channels and fewer pixels than a block has rows
+    (144, 24, 1, 0, 3, 37, 41),      # 24 outputs of 32 operand rows, ragged runs of pixels
+    (520, 24, 1, 0, 5, 7, 7),        # a last plane of one chunk
+    (64, 16, 3, 1, 2, 12, 70),       # one plane, column strips
+    (40, 8, 3, 0, 1, 18, 41),        # eight outputs, no padding
+    (112, 16, 3, 1, 104, 9, 9),      # several images
+    (280, 16, 3, 2, 1, 14, 15),      # the widest padding, a long reduction of few items
+    (40, 24, 5, 2, 1, 22, 300),      # wider than the fold kernel took
+    (64, 8, 5, 4, 2, 9, 11),
+    (136, 24, 5, 2, 1, 20, 66),
+    (48, 24, 7, 3, 2, 15, 20),
+    (72, 8, 7, 0, 1, 7, 9),          # one row of outputs
+])
+def test_narrow_outputs_by_rows_against_the_oracle(dc, c_in, c_out, k, p, n, h, w):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, 1, p, n, h, w, "k_conv_tc_rows")
+
+
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w,kernel", [
     (24, 24, 3, 1, 1, 3, 31, 23, "k_conv_tc_pairrows"),     # odd padding: the last pixel is the second of its output pair
     (32, 32, 5, 1, 2, 2, 28, 29, "k_conv_tc_pairrows"),     # even padding: the last output pair has one pixel
