@@ -359,8 +359,9 @@ extern "C" dc_status dc_dwconv_status(dc_stream stream) {
     const unsigned int zero = 0;
     DC_CUDA_OK(cudaMemcpyToSymbol(g_dw_status, &zero, sizeof(zero)));
   }
-  bool merge = false;
-  const dc_status s = dc_merge_tc_status(&merge);
+  bool merge = false, product = false;
+  dc_status s = dc_merge_tc_status(&merge);
+  if (s == DC_OK) s = dc_merge_product_tc_status(&product);
   if (s != DC_OK) return s;
-  return st != 0 || merge ? DC_ERR_TIMEOUT : DC_OK;
+  return st != 0 || merge || product ? DC_ERR_TIMEOUT : DC_OK;
 }

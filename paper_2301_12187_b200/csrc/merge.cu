@@ -1586,6 +1586,18 @@ static void launch_block33_form(TiledBlocks &tb, const BlockDelivery &dv, const 
   status.note(dc_launch_pdl(k_merge_block33<IT, W>, dim3(grid), dim3(W * 32), grid <= dc_sm_count() ? alone : ring, st, tb, dv));
   status.launched();
 }
+// A single block goes to the tensor core where an estimate says so: of 250 drawn blocks of 40 to 320 channels in and 160 to 1280 hidden
+// ones 130, in 0.74 of the time on (geometric) average, none slower.  (The line: of the 67 that the estimates were fitted to it sends
+// 33, none slower, at 1.0 36, one of them 9 % slower.)  160 -> 960 -> 160 20.0 us and
+// 13.9, 200 -> 928 -> 200 39.4 and 17.5, 64 -> 1168 -> 64 17.5 and 10.7, 96 -> 576 -> 96 11.1 and 9.9; what 24 -> 144 -> 24 takes there,
+// 8.2 us, most of it the start and the end of a launch, is more than here, 6.1.
+static bool block33_on_tensor_core(int c0, int c1, int c2, int run, int most16, int most24, int form) {
+  const double fma = form == 0   ? 4.07 + 1.69 * (most16 - 1) + c1 / 8.0 * (0.0692 * most16 + 0.0306 * dc_div_up(most16, 2))
+                     : form == 1 ? 4.6 + 0.1757 * c1 / 16.0
+                                 : 5.69 + 0.248 * most24 * c1 / 16.0;
+  const double tc = dc_merge_product_tc_us(kProductBlock, c0, c1, c2, run);
+  return tc != 0.0 && tc < 0.95 * fma;
+}
 // Tiles of 8 x 16 pairs by eight warps; by sixteen, one CTA to an SM, for long reductions: of 8 x 16 where that gives no SM a
 // second tile, of 8 x 24 where it leaves the SM with the most pairs fewer of them.
 static void launch_block33(TiledBlocks &tb, const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
@@ -1595,10 +1607,16 @@ static void launch_block33(TiledBlocks &tb, const BlockDelivery &dv, const dc_ge
     tiles24 += dc_div_up(tb.blk[i].c0, 24) * dc_div_up(tb.blk[i].c2, kMbO);
     if (tb.blk[i].c1 > hidden) hidden = tb.blk[i].c1;
   }
-  const int n_sm = dc_sm_count(), most16 = dc_div_up(tiles16, n_sm) * 16, most24 = dc_div_up(tiles24, n_sm) * 24;
-  if (hidden < 320) launch_block33_form<16, 8>(tb, dv, mg, st, status);
-  else if (tiles16 <= n_sm) launch_block33_form<16, 16>(tb, dv, mg, st, status);
-  else if (most24 < most16) launch_block33_form<24, 16>(tb, dv, mg, st, status);
+  const int n_sm = dc_sm_count(), most16 = dc_div_up(tiles16, n_sm), most24 = dc_div_up(tiles24, n_sm);
+  const int form = hidden < 320 ? 0 : tiles16 <= n_sm ? 1 : most24 * 24 < most16 * 16 ? 2 : 0;
+  const BlockArgs &b = tb.blk[0];
+  const int run = hidden / (hidden < 320 ? 8 : 16);          // channels of a warp's sums, at least
+  if (tb.n == 1 && block33_on_tensor_core(b.c0, b.c1, b.c2, run, most16, most24, form)) {
+    status.note(dc_launch_merge_product_tc(kProductBlock, Product{b.l1, b.l2, b.l3, 0, 0, b.c0, b.c1, b.c2, b.w_out, b.b_out}, dv, run, st));
+    return;
+  }
+  if (form == 1) launch_block33_form<16, 16>(tb, dv, mg, st, status);
+  else if (form == 2) launch_block33_form<24, 16>(tb, dv, mg, st, status);
   else launch_block33_form<16, 8>(tb, dv, mg, st, status);
 }
 
@@ -1808,6 +1826,18 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     }
     a.gi = dc_div_up(a.c0, bi);
     a.go = dc_div_up(a.c2, bo);
+    // The tensor core by estimates as well: of 131 drawn pairs of 40 to 1280 channels 50, in 0.63 of the time on (geometric) average, one
+    // slower, by 3 %.
+    // 960 -> 320 -> 1280 30.7 us here and 21.7 there, 320 -> 1280 -> 320 25.4 and 13.9, 1024 -> 256 -> 1024 31.4 and 17.4.
+    const int most = dc_div_up(a.gi * a.go, n_sm), run = a.c1 / 4;           // channels of a group's sums, at most half of them
+    const double fma = bo == 64   ? 4.82 + a.c1 * (0.0185 * most + 0.0705 * dc_div_up(most, 3))
+                       : bo == 48 ? 5.2 + a.c1 * (0.0072 * most + 0.06 * dc_div_up(most, 3))
+                                  : 3.07 + a.c1 * (0.0136 * most + 0.0023 * dc_div_up(most, 3));
+    const double tc = dc_merge_product_tc_us(kProductPair, a.c0, a.c1, a.c2, run);
+    if (tc != 0.0 && tc < 0.95 * fma) {
+      status.note(dc_launch_merge_product_tc(kProductPair, Product{a.l1, RawLayer{}, a.l2, a.ident1, a.ident2, a.c0, a.c1, a.c2, a.w_out, a.b_out}, dv, run, st));
+      return status.s;
+    }
     const dim3 grid(a.gi * a.go + dc_div_up(a.c2, 8) + zero_ctas(dv, mg, 256));
     if (bo == 64) status.note(dc_launch_pdl(k_merge_11<64, 64, 8, 2>, grid, dim3(256), 0, st, a, dv));
     else if (bo == 48) status.note(dc_launch_pdl(k_merge_11<48, 64, 6, 2>, grid, dim3(256), 0, st, a, dv));

@@ -46,9 +46,33 @@ __device__ __forceinline__ bool packed_chunk_live(const KOrder &ko, int idx8, in
   return o < c_out && (grp * ko.cg + ccg) * 8 < ko.c_in;
 }
 
-// The packed copy of a tile of OT output x IT input channels whose K x K kernels lie in shared memory as
-// [o][i][tap].  fp32: [tap][i][o].  bf16: one chunk of 8 input channels per (output channel, chunk, tap), written
-// where the forward kernels' K order wants it; pair rows hold every chunk twice, the second copy one pixel further on.
+// Tap t of 8 input channels i .. i + 7 of output channel o, which lie KK floats apart, in the packed copy.  fp32: [tap][i][o].  bf16: one
+// chunk, written where the forward kernels' K order wants it; pair rows hold every chunk twice, the second copy one pixel
+// further on.
+template <int KK>
+__device__ __forceinline__ void deliver_chunk(const BlockDelivery &dv, const float *f, int o, int i, int t, int c0, int c2) {
+  constexpr int K = KK == 1 ? 1 : KK == 9 ? 3 : 5;
+  if (dv.mode == 1) {
+    float *out = reinterpret_cast<float *>(dv.packed);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (i + q < c0) out[((size_t)t * c0 + i + q) * c2 + o] = f[q * KK];
+    return;
+  }
+  uint4 *out = reinterpret_cast<uint4 *>(dv.packed);
+  __align__(16) __nv_bfloat16 v8[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(f[q * KK]);
+  const uint4 v = *reinterpret_cast<const uint4 *>(v8);
+  const int r = t / K, sx = t - K * r;
+  out[dc_packed_chunk(dv.ko, dc_korder_encode(dv.ko, i >> 3, r, sx), dc_korder_row(dv.ko, sx, o))] = v;
+  if (dv.ko.pair == 2) {
+    const int plane = (r * dv.ko.ns[0] + ((sx + 1) >> 1)) * 2 * dv.ko.cch + ((sx + 1) & 1) * dv.ko.cch + (i >> 3);
+    out[dc_packed_chunk(dv.ko, plane, dv.ko.co8 + o)] = v;
+  }
+}
+
+// The packed copy of a tile of OT output x IT input channels whose K x K kernels lie in shared memory as [o][i][tap].
 template <int OT, int IT, int K>
 __device__ __forceinline__ void deliver_tile(const BlockDelivery &dv, const float *sums, int o0, int i0, int c0, int c2,
                                              int tid, int threads) {
@@ -61,20 +85,10 @@ __device__ __forceinline__ void deliver_tile(const BlockDelivery &dv, const floa
     }
     return;
   }
-  uint4 *out = reinterpret_cast<uint4 *>(dv.packed);
   for (int e = tid; e < OT * (IT / 8) * KK; e += threads) {
     const int ow = e % OT, rest = e / OT, hf = rest % (IT / 8), t = rest / (IT / 8), o = o0 + ow, ch = i0 + hf * 8;
     if (o >= c2 || ch >= c0) continue;
-    __align__(16) __nv_bfloat16 v8[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(sums[(ow * IT + hf * 8 + q) * KK + t]);
-    const uint4 v = *reinterpret_cast<const uint4 *>(v8);
-    const int r = t / K, sx = t - K * r;
-    out[dc_packed_chunk(dv.ko, dc_korder_encode(dv.ko, ch >> 3, r, sx), dc_korder_row(dv.ko, sx, o))] = v;
-    if (dv.ko.pair == 2) {
-      const int plane = (r * dv.ko.ns[0] + ((sx + 1) >> 1)) * 2 * dv.ko.cch + ((sx + 1) & 1) * dv.ko.cch + (ch >> 3);
-      out[dc_packed_chunk(dv.ko, plane, dv.ko.co8 + o)] = v;
-    }
+    deliver_chunk<KK>(dv, sums + (ow * IT + hf * 8) * KK + t, o, ch, t, c0, c2);
   }
 }
 
@@ -134,3 +148,18 @@ __device__ __forceinline__ float compose33_ident(const Compose33 &a, bool whole,
 dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, cudaStream_t st);
 // whether a bounded wait of such a launch ran out on the current device since the last call; clears the flag
 dc_status dc_merge_tc_status(bool *ran_out);
+
+// What a dense 1x1 layer l1 is composed with, as one product on the tensor core (merge_product_tc.cu): the rest of an inverted-residual
+// block (mid: the 3x3 depthwise layer, l2: the last one), or a 1x1 layer l2.  c0 and c1 are multiples of 4.
+enum { kProductBlock, kProductPair };
+struct Product {
+  RawLayer l1, mid, l2;
+  int ident1, ident2;            // identity kernels riding on l1 and l2 (not of a block)
+  int c0, c1, c2;
+  float *w_out, *b_out;
+};
+// DC_ERR_UNSUPPORTED: outside its range, nothing was launched.  `run`: see make_plan there
+dc_status dc_launch_merge_product_tc(int kind, const Product &a, const BlockDelivery &dv, int run, cudaStream_t st);
+// its estimated time; 0: outside its range
+double dc_merge_product_tc_us(int kind, int c0, int c1, int c2, int run);
+dc_status dc_merge_product_tc_status(bool *ran_out);

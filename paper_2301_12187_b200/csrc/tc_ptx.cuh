@@ -302,6 +302,18 @@ __device__ __forceinline__ uint4 lds_cluster_u4(uint32_t a) {
   asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
   return v;
 }
+// contiguous copy from this CTA's shared memory to another's of the cluster (cluster addresses `dst` and `bar`, 16-byte aligned, bytes a
+// multiple of 16); the bytes are reported to the mbarrier there as they land
+__device__ __forceinline__ void bulk_send(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ float lds_cluster_f(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // 16-byte asynchronous copy global -> shared without the zero-fill operand
 __device__ __forceinline__ void cp_async16_full(uint32_t dst, const void *src) {

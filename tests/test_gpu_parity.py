@@ -1307,3 +1307,62 @@ def test_3x3_after_3x3_by_bf16_terms_of_what_is_not_finite(dc):
     big = ref.abs() > 1e20
     assert bool((wm[fin & big] / ref[fin & big] - 1).abs().max() < 1e-5) and int((fin & big).sum()) > 0
     assert ((wm - ref)[fin & ~big].norm() / ref[fin & ~big].norm()).item() <= 3e-7
+
+
+@pytest.mark.parametrize("a,c,o,res,codes", [
+    (160, 960, 160, [(0, 2)], "both"),         # two tiles of columns, twelve steps in eleven slots, the tile shared by five CTAs
+    (96, 576, 96, [(0, 2)], "both"),           # shared by eight, the last with fewer steps
+    (112, 672, 192, [], "both"),               # four sums of the products of the high terms
+    (252, 700, 300, [], "f32"),                # the same; nothing a multiple of a tile or a step, slots used twice
+    (36, 700, 250, [], "f32"),                 # columns and rows of the last tile that are not there
+    (24, 1264, 40, [], "both"),                # packed orders that hold pixels, and taps, in their rows
+    (40, 816, 24, [], "both"),
+])
+def test_blocks_by_bf16_terms_against_the_oracle(dc, a, c, o, res, codes):
+    specs = [I.make_layer(90, 0, a, c, 1, 1, 0), I.make_layer(90, 1, c, c, 3, 1, 1, depthwise=True), I.make_layer(90, 2, c, o, 1, 1, 0)]
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
+    _check_delivery(dc, specs + [I.make_layer(90, 3, o, 16, 1, 1, 0)], res, (dc.F32,))         # as a piece
+    assert dc.dwconv_status() == dc.OK
+
+
+@pytest.mark.parametrize("a,c,o,res,codes", [
+    (960, 320, 1280, [], "both"),              # a tile a CTA, twenty steps in ten slots
+    (320, 1280, 320, [], "both"),              # shared by eight
+    (332, 604, 333, [], "f32"),                # nothing a multiple of a tile or a step
+    (72, 1500, 72, [], "both"),
+    (504, 504, 504, [(0, 0)], "both"), (504, 504, 504, [(0, 0), (1, 1)], "both"), (504, 504, 504, [(0, 1)], "both"),
+])
+def test_1x1_pairs_by_bf16_terms_against_the_oracle(dc, a, c, o, res, codes):
+    specs = [I.make_layer(91, 0, a, c, 1, 1, 0), I.make_layer(91, 1, c, o, 1, 1, 0)]
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
+    assert dc.dwconv_status() == dc.OK
+    if not res:
+        # sums of at most 128 products in the tensor core, then fp32 additions: 1.5e-7 measured at most; FMAs in runs of half or a quarter
+        # of so many channels are 2.05e-7 or more away (so this also tells that they were not taken)
+        _, wm, _, _ = run_merge(dc, specs, res, packed_dtype=dc.F32)
+        assert O.rel_l2(wm.cpu().numpy(), O.merge_formula(specs, res)[0]) <= 1.9e-7
+
+
+@pytest.mark.parametrize("block", [True, False])
+def test_products_by_bf16_terms_of_what_is_not_finite(dc, block):
+    """An infinity, a NaN and a value beyond the largest bf16 among the weights: infinities and NaN where 64 bits have them."""
+    a, c, o = (96, 576, 96) if block else (320, 1280, 320)
+    specs = [I.make_layer(92, 0, a, c, 1, 1, 0, with_bn=False), I.make_layer(92, 1, c, c, 3, 1, 1, depthwise=True, with_bn=False),
+             I.make_layer(92, 2, c, o, 1, 1, 0, with_bn=False)]
+    w1, wd, w2 = (s.weight for s in specs)
+    w1[5, 7, 0, 0], w1[c - 1, a - 1, 0, 0], w2[9, 11, 0, 0] = np.inf, np.nan, 3.4e38
+    w1[11] *= 2.0 ** -20                           # the products of the largest value stay finite
+    specs = specs if block else specs[::2]
+    layers = [dc.DeviceLayer(s) for s in specs]
+    g, ws_bytes = dc.merge_query(layers, [])
+    wm, bm = torch.zeros(g.c_out, g.c_in, g.k, g.k, device="cuda"), torch.empty(g.c_out, device="cuda")
+    dc.merge_chain(layers, [], wm, bm, None, dc.F32, torch.empty(ws_bytes, dtype=torch.uint8, device="cuda"))
+    t1, td, t2 = (torch.from_numpy(w).double().cuda() for w in (w1, wd, w2))
+    taps = td[:, 0].reshape(c, 9) if block else torch.ones(c, 1, dtype=torch.float64, device="cuda")
+    ref = torch.stack([((t2[:, :, 0, 0] * taps[:, t])[:, :, None] * t1[None, :, :, 0, 0]).sum(1) for t in range(taps.shape[1])], 2).reshape(wm.shape)
+    wm = wm.double()
+    assert torch.equal(torch.isnan(wm), torch.isnan(ref)) and torch.equal(torch.isinf(wm), torch.isinf(ref))
+    fin = torch.isfinite(ref)
+    big = ref.abs() > 1e20
+    assert bool((wm[fin & big] / ref[fin & big] - 1).abs().max() < 1e-5) and int((fin & big).sum()) > 0
+    assert ((wm - ref)[fin & ~big].norm() / ref[fin & ~big].norm()).item() <= 4e-7
