@@ -1077,10 +1077,14 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
 // A dense 1x1 and a 3x3 depthwise layer, in either order, as a run of its own: every element of the result is one
 // product, W'[o][i][t] = W~[o][i] D~[c][t] with c = o (1x1 first) or c = i (depthwise first), so the run is bound by
 // writing its result (160 -> 960: 5.5 MB and its packed copy) and by its launches.  One launch reads the layers as they
-// are and delivers tiles of 8 x 16 channel pairs; blocks behind the tiles compute the bias (a warp per output channel)
-// and zero the packed chunks without weights.  As fold, composition and delivery, three launches with the result
-// written and read in between: 160 -> 960 then depthwise 27.6 us, depthwise then 576 -> 96 27.1, 384 -> 64 17.3; here
-// 9.6, 7.6 and 5.3 us.
+// are and delivers tiles of 8 x 16 channel pairs, or of 8 x 32 or 8 x 64 where those are two to an SM; blocks behind the tiles compute the
+// bias (a warp per output channel) and zero the packed chunks without weights.  As fold, composition and delivery, three launches with the
+// result written and read in between: 160 -> 960 then depthwise 27.6 us, depthwise then 576 -> 96 27.1, 384 -> 64 17.3; here 8.6, 4.6 and
+// 3.9 us.
+//
+// Before: 9.3, 7.2 and 5.1 us; 320 -> 1920 20.2, now 17.6, depthwise then 1152 -> 192 16.9, now 10.1.  After a depthwise layer the bias
+// blocks were the longest: each warp worked out every channel's factor for itself.  Then each chunk's place in the packed copy,
+// divisions all, and in large results the tiles' starts.  (The smallest, 2.7 us, take 0.1 more.)
 // ----------------------------------------------------------------------------------------------
 struct Outer33 {
   RawLayer dense, dw;
@@ -1091,9 +1095,12 @@ struct Outer33 {
   int gi, go;
 };
 
+template <int IT>
 __global__ void __launch_bounds__(kMbThreads)
 k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ BlockDelivery dv) {
-  __shared__ float wv[kMbO * kMbI], dd[kMbI * 9], out[kMbTile];
+  constexpr int kBias = 1024;                      // channels whose bias factors a CTA holds at a time
+  __shared__ float wv[kMbO * IT > kBias ? kMbO * IT : kBias], dd[IT * 9], out[IT == 16 ? kMbO * IT * 9 : 1];
+  __shared__ size_t row_s[kMbO], plane_s[IT / 8 * 9];              // where channels and taps are in the packed copy
   const int tid = (int)threadIdx.x, lane = tid & 31;
   const int c0 = a.c0, c2 = a.c2;
   int blk = (int)blockIdx.x;
@@ -1105,18 +1112,35 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
       return;
     }
     const int o = blk * kMbO + (tid >> 5);
-    if (o >= c2) return;
     float s = 0.f;
-    if (a.dw_first) {                              // b2~ + sum_c W~[o][c] b1~[c]
-      const float g2 = raw_scale(a.dense, o);
-#pragma unroll 4
-      for (int c = lane; c < c0; c += 32) {
-        const float w = fmaf(g2, a.dense.w[(size_t)o * c0 + c], a.ident_dense && c == o ? 1.f : 0.f);
-        s = fmaf(w, raw_bias(a.dw, c, raw_scale(a.dw, c)), s);
+    if (a.dw_first) {                              // b2~ + sum_c W~[o][c] b1~[c], b1~ by all of the CTA
+      const int ol = o < c2 ? o : 0;
+      const RawNumbers n2(a.dense, ol);
+      const float *w = a.dense.w + (size_t)ol * c0;
+      const float g2 = n2.scale(a.dense);
+      float *b1 = wv;
+#pragma unroll 1
+      for (int cs = 0; cs < c0; cs += kBias) {
+        const int n = c0 - cs < kBias ? c0 - cs : kBias;
+        __syncthreads();
+        for (int c = tid; c < n; c += kMbThreads) {
+          const RawNumbers n1(a.dw, cs + c);
+          b1[c] = n1.bias(a.dw, n1.scale(a.dw));
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int c = lane; c < n; c += 256) {      // eight weights on their way at once
+          float x[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) x[q] = c + 32 * q < n ? w[cs + c + 32 * q] : 0.f;
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if (c + 32 * q < n) s = fmaf(fmaf(g2, x[q], a.ident_dense && cs + c + 32 * q == o ? 1.f : 0.f), b1[c + 32 * q], s);
+        }
       }
       for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-      if (lane == 0) a.b_out[o] = raw_bias(a.dense, o, g2) + s;
-    } else {                                       // b2~ + (sum_t D~[o][t]) b1~[o]
+      if (lane == 0 && o < c2) a.b_out[o] = n2.bias(a.dense, g2) + s;
+    } else if (o < c2) {                           // b2~ + (sum_t D~[o][t]) b1~[o]
       const float g2 = raw_scale(a.dw, o);
       s = lane < 9 ? g2 * a.dw.w[(size_t)o * 9 + lane] : 0.f;
       for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
@@ -1125,27 +1149,83 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
     }
     return;
   }
-  const int o0 = (blk / a.gi) * kMbO, i0 = (blk % a.gi) * kMbI;
-  if (tid < kMbO * kMbI) {
-    const int o = o0 + tid / kMbI, i = i0 + tid % kMbI;
-    wv[tid] = o < c2 && i < c0 ? fmaf(raw_scale(a.dense, o), a.dense.w[(size_t)o * c0 + i], a.ident_dense && o == i ? 1.f : 0.f) : 0.f;
+  const int o0 = (blk / a.gi) * kMbO, i0 = (blk % a.gi) * IT;
+  for (int e = tid; e < kMbO * IT; e += kMbThreads) {
+    const int o = o0 + e / IT, i = i0 + e % IT;
+    wv[e] = o < c2 && i < c0 ? fmaf(raw_scale(a.dense, o), a.dense.w[(size_t)o * c0 + i], a.ident_dense && o == i ? 1.f : 0.f) : 0.f;
   }
-  const int d0 = a.dw_first ? i0 : o0, nd = a.dw_first ? kMbI : kMbO, cd = a.dw_first ? c0 : c2;
-  if (tid < nd * 9) {
-    const int c = d0 + tid / 9, t = tid % 9;
-    dd[tid] = c < cd ? fmaf(raw_scale(a.dw, c), a.dw.w[(size_t)c * 9 + t], a.ident_dw && t == 4 ? 1.f : 0.f) : 0.f;
+  const int d0 = a.dw_first ? i0 : o0, nd = a.dw_first ? IT : kMbO, cd = a.dw_first ? c0 : c2;
+  for (int e = tid; e < nd * 9; e += kMbThreads) {
+    const int c = d0 + e / 9, t = e % 9;
+    dd[e] = c < cd ? fmaf(raw_scale(a.dw, c), a.dw.w[(size_t)c * 9 + t], a.ident_dw && t == 4 ? 1.f : 0.f) : 0.f;
+  }
+  // Where a bf16 chunk goes: rows of a tap's chunk plane, except in orders that hold taps or pixels in the rows.  Worked out once a
+  // CTA: the divisions are most of what a chunk costs.
+  const bool by_rows = dv.mode == 2 && !dv.ko.fold && !dv.ko.pair;
+  const int per = dv.ko.rows && dv.ko.nnt > 1 ? dv.ko.n_tile : dv.ko.n_pad;
+  if (by_rows) {
+    const int e = tid - (kMbThreads - IT / 8 * 9), r = tid - 32;
+    if (e >= 0) plane_s[e] = (size_t)dc_korder_encode(dv.ko, (i0 >> 3) + e / 9, e % 9 / 3, e % 3) * per;
+    if (r >= 0 && r < kMbO) row_s[r] = dc_packed_chunk(dv.ko, 0, o0 + r);
   }
   __syncthreads();
-  for (int e = tid; e < kMbTile; e += kMbThreads) {
-    const int oi = e / 9, t = e - oi * 9, ow = oi / kMbI, iw = oi % kMbI, o = o0 + ow, i = i0 + iw;
-    float v = wv[oi] * dd[(a.dw_first ? iw : ow) * 9 + t];
-    if (dv.ident && o == i && t == 4) v += 1.f;
-    if (o < c2 && i < c0) a.w_out[((size_t)o * c0 + i) * 9 + t] = v;
-    out[e] = v;
+  auto value = [&](int ow, int iw, int t) {
+    const float v = wv[ow * IT + iw] * dd[(a.dw_first ? iw : ow) * 9 + t];
+    return dv.ident && t == 4 && o0 + ow == i0 + iw ? v + 1.f : v;
+  };
+  if (IT == 16) {                                  // small results: each once, for the result and its packed copy
+    for (int e = tid; e < kMbO * IT * 9; e += kMbThreads) {
+      const int ow = e / (IT * 9), x = e - ow * (IT * 9);
+      const float v = value(ow, x / 9, x % 9);
+      if (o0 + ow < c2 && i0 + x / 9 < c0) a.w_out[((size_t)(o0 + ow) * c0 + i0) * 9 + x] = v;
+      out[e] = v;
+    }
+    if (dv.mode == 0) return;
+    __syncthreads();
+    if (!by_rows) {
+      deliver_tile<kMbO, IT, 3>(dv, out, o0, i0, c0, c2, tid, kMbThreads);
+      return;
+    }
+  } else if (c0 % 4 == 0) {                        // four neighbouring results at a time: rows are whole pieces then
+    for (int e = tid; e < kMbO * IT * 9 / 4; e += kMbThreads) {
+      const int ow = e / (IT * 9 / 4), x = (e - ow * (IT * 9 / 4)) * 4;
+      if (o0 + ow >= c2 || i0 + x / 9 >= c0) continue;
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = value(ow, (x + j) / 9, (x + j) % 9);
+      *reinterpret_cast<float4 *>(a.w_out + ((size_t)(o0 + ow) * c0 + i0) * 9 + x) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+  } else {
+    for (int e = tid; e < kMbO * IT * 9; e += kMbThreads) {
+      const int ow = e / (IT * 9), x = e - ow * (IT * 9);
+      if (o0 + ow < c2 && i0 + x / 9 < c0) a.w_out[((size_t)(o0 + ow) * c0 + i0) * 9 + x] = value(ow, x / 9, x % 9);
+    }
   }
   if (dv.mode == 0) return;
-  __syncthreads();
-  deliver_tile<kMbO, kMbI, 3>(dv, out, o0, i0, c0, c2, tid, kMbThreads);
+  if (dv.mode == 1) {
+    float *to = reinterpret_cast<float *>(dv.packed);
+    for (int e = tid; e < kMbO * IT * 9; e += kMbThreads) {
+      const int ow = e % kMbO, rest = e / kMbO, iw = rest % IT, t = rest / IT;
+      if (o0 + ow < c2 && i0 + iw < c0) to[((size_t)t * c0 + i0 + iw) * c2 + o0 + ow] = value(ow, iw, t);
+    }
+    return;
+  }
+  auto two = [](float lo, float hi) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&p);
+  };
+  for (int e = tid; e < kMbO * (IT / 8) * 9; e += kMbThreads) {
+    const int ow = e % kMbO, rest = e / kMbO, hf = rest % (IT / 8), t = rest / (IT / 8), o = o0 + ow, i = i0 + hf * 8;
+    if (o >= c2 || i >= c0) continue;
+    float v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = IT == 16 ? out[(ow * IT + hf * 8 + q) * 9 + t] : value(ow, hf * 8 + q, t);
+    if (by_rows)
+      reinterpret_cast<uint4 *>(dv.packed)[row_s[ow] + plane_s[hf * 9 + t]] =
+          make_uint4(two(v[0], v[1]), two(v[2], v[3]), two(v[4], v[5]), two(v[6], v[7]));
+    else
+      deliver_chunk<9, 1>(dv, v, o, i, t, c0, c2);
+  }
 }
 
 // ----------------------------------------------------------------------------------------------
@@ -1568,6 +1648,13 @@ static void launch_compose33(const Operand33 &first, const Operand33 &second, in
   else launch_compose33_form<4>(a, dv, mg, st, status);
 }
 
+template <int IT>
+static void launch_outer33(Outer33 a, const BlockDelivery &dv, int zero, cudaStream_t st, MergeStatus &status) {
+  a.gi = dc_div_up(a.c0, IT);
+  status.note(dc_launch_pdl(k_merge_outer33<IT>, dim3(a.gi * a.go + a.go + zero), dim3(kMbThreads), 0, st, a, dv));
+  status.launched();
+}
+
 template <int IT, int W>
 static void launch_block33_form(TiledBlocks &tb, const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   tb.first[0] = 0;
@@ -1794,11 +1881,13 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
         if (res[g].first != res[g].last) whole = 1;
         else id[res[g].first] = 1;
       }
-      const Outer33 a{raw_of(de), raw_of(dw), id[dw_first ? 1 : 0], id[dw_first ? 0 : 1], dw_first ? 1 : 0, mg.c_in, mg.c_out,
-                      w_merged, b_merged, dc_div_up(mg.c_in, kMbI), dc_div_up(mg.c_out, kMbO)};
+      Outer33 a{raw_of(de), raw_of(dw), id[dw_first ? 1 : 0], id[dw_first ? 0 : 1], dw_first ? 1 : 0, mg.c_in, mg.c_out,
+                      w_merged, b_merged, 0, dc_div_up(mg.c_out, kMbO)};
       const BlockDelivery dv{w_packed, mode, whole, ko};
-      status.note(dc_launch_pdl(k_merge_outer33, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, kMbThreads)), dim3(kMbThreads), 0, st, a, dv));
-      status.launched();
+      const int n_sm = dc_sm_count(), zero = zero_ctas(dv, mg, kMbThreads);
+      if (a.go * dc_div_up(mg.c_in, 64) >= 2 * n_sm) launch_outer33<64>(a, dv, zero, st, status);
+      else if (a.go * dc_div_up(mg.c_in, 32) >= 2 * n_sm) launch_outer33<32>(a, dv, zero, st, status);
+      else launch_outer33<16>(a, dv, zero, st, status);
       return status.s;
     }
   }

@@ -15,6 +15,19 @@ __device__ __forceinline__ float raw_bias(const RawLayer &L, int o, float g) {
   return L.gamma ? fmaf(b - L.mean[o], g, L.beta[o]) : b;
 }
 
+static __device__ __noinline__ float bn_scale(float gamma, float var) { return gamma / sqrtf(var); }
+// BN and bias of a channel as they are read: asked for at once, used later
+struct RawNumbers {
+  float gamma, var, mean, beta, b;
+  __device__ __forceinline__ RawNumbers(const RawLayer &l, int c) {
+    gamma = 1.f; var = mean = beta = b = 0.f;
+    if (l.gamma) { gamma = l.gamma[c]; var = l.var[c]; mean = l.mean[c]; beta = l.beta[c]; }
+    if (l.b) b = l.b[c];
+  }
+  __device__ __forceinline__ float scale(const RawLayer &l) const { return l.gamma ? bn_scale(gamma, var + l.eps) : 1.f; }
+  __device__ __forceinline__ float bias(const RawLayer &l, float g) const { return l.gamma ? fmaf(b - mean, g, beta) : b; }
+};
+
 struct BlockDelivery {           // of a run that is one block; mode < 0: the block is a piece of a longer run
   void *packed;
   int mode;                      // 0: no packed copy, 1: fp32, 2: bf16 chunks
@@ -46,23 +59,23 @@ __device__ __forceinline__ bool packed_chunk_live(const KOrder &ko, int idx8, in
   return o < c_out && (grp * ko.cg + ccg) * 8 < ko.c_in;
 }
 
-// Tap t of 8 input channels i .. i + 7 of output channel o, which lie KK floats apart, in the packed copy.  fp32: [tap][i][o].  bf16: one
+// Tap t of KK of 8 input channels i .. i + 7 of output channel o, which lie STRIDE floats apart, in the packed copy.  fp32: [tap][i][o].  bf16: one
 // chunk, written where the forward kernels' K order wants it; pair rows hold every chunk twice, the second copy one pixel
 // further on.
-template <int KK>
+template <int KK, int STRIDE = KK>
 __device__ __forceinline__ void deliver_chunk(const BlockDelivery &dv, const float *f, int o, int i, int t, int c0, int c2) {
   constexpr int K = KK == 1 ? 1 : KK == 9 ? 3 : 5;
   if (dv.mode == 1) {
     float *out = reinterpret_cast<float *>(dv.packed);
 #pragma unroll
     for (int q = 0; q < 8; ++q)
-      if (i + q < c0) out[((size_t)t * c0 + i + q) * c2 + o] = f[q * KK];
+      if (i + q < c0) out[((size_t)t * c0 + i + q) * c2 + o] = f[q * STRIDE];
     return;
   }
   uint4 *out = reinterpret_cast<uint4 *>(dv.packed);
   __align__(16) __nv_bfloat16 v8[8];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(f[q * KK]);
+  for (int q = 0; q < 8; ++q) v8[q] = __float2bfloat16_rn(f[q * STRIDE]);
   const uint4 v = *reinterpret_cast<const uint4 *>(v8);
   const int r = t / K, sx = t - K * r;
   out[dc_packed_chunk(dv.ko, dc_korder_encode(dv.ko, i >> 3, r, sx), dc_korder_row(dv.ko, sx, o))] = v;

@@ -35,19 +35,6 @@ constexpr int kMaxSlots = 16, kMaxSplit = 8;
 constexpr int kSmemMax = 225 * 1024;             // asked for always: a CTA holds all of its SM's tensor memory, and clusters that did so
                                                  // beside one another on an SM could wait for each other's
 
-__device__ __noinline__ float bn_scale(float gamma, float var) { return gamma / sqrtf(var); }
-// BN and bias of a channel as they are read: asked for at once, used later
-struct RawNumbers {
-  float gamma, var, mean, beta, b;
-  __device__ __forceinline__ RawNumbers(const RawLayer &l, int c) {
-    gamma = 1.f; var = mean = beta = b = 0.f;
-    if (l.gamma) { gamma = l.gamma[c]; var = l.var[c]; mean = l.mean[c]; beta = l.beta[c]; }
-    if (l.b) b = l.b[c];
-  }
-  __device__ __forceinline__ float scale(const RawLayer &l) const { return l.gamma ? bn_scale(gamma, var + l.eps) : 1.f; }
-  __device__ __forceinline__ float bias(const RawLayer &l, float g) const { return l.gamma ? fmaf(b - mean, g, beta) : b; }
-};
-
 __host__ __device__ constexpr int threads_of(int nt) { return 2 * (8 + nt / 16) * 32 + 64; }      // two teams that cut, two warps that issue
 
 template <int KIND>

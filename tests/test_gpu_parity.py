@@ -1366,3 +1366,20 @@ def test_products_by_bf16_terms_of_what_is_not_finite(dc, block):
     big = ref.abs() > 1e20
     assert bool((wm[fin & big] / ref[fin & big] - 1).abs().max() < 1e-5) and int((fin & big).sum()) > 0
     assert ((wm - ref)[fin & ~big].norm() / ref[fin & ~big].norm()).item() <= 4e-7
+
+
+@pytest.mark.parametrize("dw_first,a,o,res,codes", [
+    (False, 160, 960, [], "both"),             # tiles of 64 input channels, the last one half filled
+    (False, 72, 800, [], "both"),              # of 32
+    (False, 150, 1000, [], "f32"),             # rows that are no whole 16-byte pieces
+    (False, 24, 1600, [], "both"),             # a packed order that holds pixels in its rows
+    (True, 1100, 180, [], "f32"),              # bias factors in two parts, tiles of 64
+    (True, 1032, 48, [], "both"),              # the same, tiles of 16
+    (True, 48, 24, [], "both"),                # taps in the rows
+    (True, 400, 400, [(0, 0), (1, 1)], "both"), (False, 400, 400, [(0, 1)], "both"),
+])
+def test_1x1_and_depthwise_pairs_against_the_oracle(dc, dw_first, a, o, res, codes):
+    mk = I.make_layer
+    c = a if dw_first else o
+    pair = [mk(93, 0, c, c, 3, 1, 1, depthwise=True), mk(93, 1, a, o, 1, 1, 0)]
+    _check_delivery(dc, pair if dw_first else pair[::-1], res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
