@@ -2,7 +2,7 @@
 //
 // W'[o][i][t] = sum_c sum_{t1 + t2 = t} W2[o][c][t2] W1~[c][i][t1]: the product Z of the matrix W2 with rows (o, t2) and the matrix W1
 // with columns (i, t1), reduction over c, has none of the structural zeros that a gathered product has, and the 25 taps of a pair
-// are sums of its 81 elements Z[o, t2][i, t1].  A tile is 14 output channels (126 of 128 rows) x 8 input channels (72 of 80 columns).
+// are sums of its 81 elements Z[o, t2][i, t1].  A tile is 14 output channels (126 of 128 rows) x 8 input channels (72 columns).
 // A value is three bf16 terms, six products of them are above 2^-24, and they are three instructions a step of 16 channels (A_h x [h m l],
 // A_m x [h m], A_l x [h], sums of hh, hm + mh and the rest in column groups of their own) as in conv_f32_tc.cu; every eight steps the
 // sums are read out and added in fp32.  Error against 64 bits (2-norm) 256 channels: 1.0e-7, by FMAs 2.3e-7.
@@ -11,15 +11,17 @@
 // steps' time for one: a warp alone on its scheduler needs it), one issues, four add up, take the 25 taps together through shared
 // memory and deliver the result while the next tile is multiplied.  The terms of a tile's columns stay in shared memory for all tiles
 // below one another where they fit (256 channels between); CTAs own runs of such tiles.  The warps that cut compute the bias
-// behind their last tile.  What bounds it is shared memory: of a step's 256 cycles of instructions 216 fetch operands, and the
-// cuts read and write another 200.
+// behind their last tile.  What bounds it is no unit (256 channels: tensor pipe 0.25, issue slots 0.42, shared memory 0.48 and the
+// instructions' operands) but the way of a step through its pair of warps: operands there, read, cut, slot free, written, multiplied,
+// 2.7 thousand cycles with four on their way at once, and a slot of operands and terms more has no room beside the columns' terms.
 //
 // An infinity or a NaN among the weights makes NaN of results: such a result is computed again by FMAs.
 //
-// 256 -> 256 -> 256 75.6 us by FMAs (k_compose33), here 46; 512 551 -> 290; 200 -> 248 -> 80 23.6 -> 22.0; 64 6.7 -> 8.3 (left to FMAs).
+// 256 -> 256 -> 256 75.6 us by FMAs (k_compose33), here 46; 512 551 -> 288; 200 -> 248 -> 80 23.6 -> 21.6; 64 6.7 -> 8.3 (left to FMAs).
 // A tile of 256 channels takes 12 thousand cycles: the taps, the scale, the result and its packed copy 9 of them in the adding warps (they run
 // once a tile, from a cold instruction cache), its sixteen steps 8.6.  On the way: cut by nine warps together 76, by pairs 54, operands
-// asked for again before they are cut 47, one issuing warp that waits for two steps side by side 45.
+// asked for again before they are cut 47, one issuing warp that waits for two steps side by side 45.  80 columns a term instead of 72 0.5 to 0.9 %
+// more; eight adding warps 44.6, but 512 channels 296; steps cut by four warps 51, by two teams with two slots each 53.
 #include "merge_parts.cuh"
 #include "tc_ptx.cuh"
 
@@ -28,11 +30,12 @@ using namespace tc;
 
 __device__ unsigned int g_merge_status;          // DC_ERR_TIMEOUT once a wait of this kernel ran out
 
-constexpr int kO = 14, kI = 8, kRows = kO * 9, kCols = kI * 9, NT = 80;
+constexpr int kO = 14, kI = 8, kRows = kO * 9, kCols = kI * 9;
+constexpr int kRowsB = 224;                      // of the columns' terms of 8 channels: 72 of each, and 8 that only make up the instruction's 224 columns
 constexpr int kWarpsAcc = 4, kPairs = 4, kWarpsCut = 2 * kPairs, kLoad = kWarpsAcc + kWarpsCut, kIssue = kLoad + 1, kThreads = (kIssue + 1) * 32;
 constexpr int kChunk = 8;                        // steps of 16 channels between two read-outs
 constexpr int kPitchA = 128 * 16;                // bytes between the halves of a step's 16 channels
-constexpr int kStepA = 6 * kPitchA, kStepB = NT * 96, kRawA = kO * 144 * 4;
+constexpr int kStepA = 6 * kPitchA, kStepB = 2 * kRowsB * 16, kRawA = kO * 144 * 4;
 constexpr int kPitchZ = kCols / 2 + 1;           // floats of a row of Z, four input channels at a time
 constexpr int kZ = (kRows * kPitchZ * 4 + 127) / 128 * 128;
 constexpr int kMaxB = 16;                        // steps whose columns' terms are there at once
@@ -144,10 +147,10 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
 #pragma unroll
         for (int c = 0; c < kCols; c += 8) {
           uint32_t v0[8], v1[8], v2[8];
-          const uint32_t at = drow + b * (3 * NT) + c;
+          const uint32_t at = drow + b * kRowsB + c;
           tmem_ld8(at, v0);
-          tmem_ld8(at + NT, v1);
-          tmem_ld8(at + 2 * NT, v2);
+          tmem_ld8(at + kCols, v1);
+          tmem_ld8(at + 2 * kCols, v2);
           tmem_ld_wait();
 #pragma unroll
           for (int j = 0; j < 8; ++j) acc[c + j] += __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + __uint_as_float(v2[j]));
@@ -239,7 +242,7 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
     if (!ok && tid == 0) atomicExch(&g_merge_status, (unsigned int)DC_ERR_TIMEOUT);
   } else if (warp < kLoad) {
     // ---------------------------------------------------------------- operands into terms: a pair of warps takes every fourth step
-    const int cw = warp - kWarpsAcc, ct = tid - kWarpsAcc * 32, pair = cw >> 1, w1 = cw & 1, hf = lane >> 4;
+    const int cw = warp - kWarpsAcc, ct = tid - kWarpsAcc * 32, pair = cw >> 1, w1 = cw & 1;
     float *g1s = reinterpret_cast<float *>(smem + p.off_scale);
     for (int c = ct; c < p.steps * 16; c += kWarpsCut * 32) g1s[c] = c < c1 ? raw_scale(a.first.l, c) : 0.f;
     bar_sync(2, kWarpsCut * 32);
@@ -268,9 +271,9 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
           float vb[3][8];
 #pragma unroll
           for (int t = 0; t < 3; ++t) {
-            const int e = (t * 2 + w1) * 32 + hf * 16, half = e >= NT ? 1 : 0, n = e - half * NT + (lane & 15), c = at * 16 + half * 8;
-            const bool in = e < 2 * NT && n0 + n < c0 * 9;
-            db[t] = (uint32_t)(half * (NT * 48) + n * 16);
+            const int e = (t * 2 + w1) * 32 + lane, half = e >= kCols ? 1 : 0, n = e - half * kCols, c = at * 16 + half * 8;
+            const bool in = e < 2 * kCols && n0 + n < c0 * 9;
+            db[t] = (uint32_t)(half * (kRowsB * 16) + n * 16);
 #pragma unroll
             for (int j = 0; j < 8; ++j) vb[t][j] = in && c + j < c1 ? a.first.l.w[(size_t)(c + j) * c0 * 9 + n0 + n] : 0.f;
           }
@@ -278,16 +281,16 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
           if (!(ok = wait(kBEmpty + slot, pb))) break;
 #pragma unroll
           for (int t = 0; t < 3; ++t) {
-            const int e = (t * 2 + w1) * 32 + hf * 16, half = e >= NT ? 1 : 0, c = at * 16 + half * 8;
-            if (e >= 2 * NT) continue;
+            const int e = (t * 2 + w1) * 32 + lane, half = e >= kCols ? 1 : 0, c = at * 16 + half * 8;
+            if (e >= 2 * kCols) continue;
 #pragma unroll
             for (int j = 0; j < 8; ++j) vb[t][j] *= g1s[c + j];
             uint4 h, mi, l;
             bf16_terms8(vb[t], h, mi, l);
             const uint32_t d = sm + (uint32_t)(p.off_b + slot * kStepB) + db[t];
             sts_u4(d, h);
-            sts_u4(d + NT * 16u, mi);
-            sts_u4(d + NT * 32u, l);
+            sts_u4(d + kCols * 16u, mi);
+            sts_u4(d + kCols * 32u, l);
           }
           fence_proxy_async();
           __syncwarp();
@@ -361,9 +364,9 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
   } else {
     // ---------------------------------------------------------------- issue: two steps at a time, their barriers waited for side by side
     const uint32_t id0 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
-    constexpr uint32_t i3 = (3 * NT / 8) << 17, i2 = (2 * NT / 8) << 17, i1 = (NT / 8) << 17;
+    constexpr uint32_t i3 = (kRowsB / 8) << 17, i2 = (2 * kCols / 8) << 17, i1 = (80 / 8) << 17;
     const uint64_t hi = (uint64_t)((128u >> 4) | (1u << 14)) << 32;
-    const uint64_t a_hi = hi | ((uint64_t)(kPitchA >> 4) << 16), b_hi = hi | ((uint64_t)(3 * NT) << 16);
+    const uint64_t a_hi = hi | ((uint64_t)(kPitchA >> 4) << 16), b_hi = hi | ((uint64_t)kRowsB << 16);
     const uint32_t sm16 = sm >> 4, b16 = (sm + (uint32_t)p.off_b) >> 4;
     int as = 0, bs = 0;
     uint32_t pa = 0, pb = 0, fl = 0;
@@ -374,7 +377,7 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
 #pragma unroll 1
       for (int s = 0; s < p.steps; s += 2) {
         const bool opens = s % kChunk == 0, closes = s % kChunk == kChunk - 2 || s + 2 == p.steps;
-        const uint32_t buf = fl & 1u, d = tmem + buf * (3 * NT);
+        const uint32_t buf = fl & 1u, d = tmem + buf * kRowsB;
         int b = kAFull + as + (lane & 1);
         uint32_t parity = pa;
         if (first && (lane & 2)) { b = kBFull + bs + (lane & 1); parity = pb; }
@@ -390,8 +393,8 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
             const uint64_t bd = b_hi | (uint64_t)((bt + q * (kStepB >> 4)) & 0x3FFFu);
             const uint32_t aq = at + q * (kStepA >> 4);
             umma_bf16(d, a_hi | (uint64_t)(aq & 0x3FFFu), bd, id0 | i3, opens && q == 0 ? 0u : 1u);
-            umma_bf16(d + NT, a_hi | (uint64_t)((aq + (2 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i2, 1u);
-            umma_bf16(d + 2 * NT, a_hi | (uint64_t)((aq + (4 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i1, 1u);
+            umma_bf16(d + kCols, a_hi | (uint64_t)((aq + (2 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i2, 1u);
+            umma_bf16(d + 2 * kCols, a_hi | (uint64_t)((aq + (4 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i1, 1u);
             umma_commit(&bar[kAEmpty + as + q]);
             if (last) umma_commit(&bar[kBEmpty + bs + q]);
           }
