@@ -453,7 +453,7 @@ def measure_network(args, peaks, peak_src):
     return {
         "config": {"workload": "cfg4_mbv2_full_batch128", "launch_groups": len(cn.ops), "kernel_launches": n_launch,
                    "merged_spans": sum(1 for op in cn.ops if op.merged), "plan_seed": 0, "plan": plan_name,
-                   "step": "all dc_merge_chain calls + forward in one graph (a launch group waits for the merge of its own span only)",
+                   "step": "all dc_merge_chain calls + forward in one graph (the forward waits for its first merged span, then for all others)",
                    "l2": "activation maps (0.1-0.6 GB each) exceed L2"},
         "value": 128 / (step["median"] * 1e-6), "unit": "images/s",
         "ms_per_step": step["median"] * 1e-3,
