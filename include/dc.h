@@ -134,7 +134,8 @@ dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual
 
 /*
  * How dc_merge_chain walks a run.  DC_MERGE_STEPS: fold every layer, then compose the pieces
- * pairwise and deliver (a launch per step; the last composition of two 3x3 kernels delivers itself).
+ * pairwise and deliver (a launch per step; the last composition of two 3x3 kernels, the second dense or
+ * depthwise, delivers itself).
  * DC_MERGE_AUTO (what dc_merge_chain uses): as above, except that runs and parts of runs of these
  * kinds are merged straight from the raw layers, BN folded on the fly, in one launch:
  *   - an inverted-residual block -- dense 1x1 with stride 1, depthwise k x k, dense 1x1 with

@@ -356,6 +356,85 @@ __global__ void k_compose_diag(Piece first, Piece second, float *out, float *b_o
   }
 }
 
+// ----------------------------------------------------------------------------------------------
+// A 3x3 depthwise layer as the last one of a longer run, after a dense 3x3 piece with stride 1: composition and delivery in one launch.
+// A CTA owns 8 output x 16 input channels, a thread a pair's 25 results (18 weights, 81 FMAs, in the order of k_compose_diag); they
+// meet in shared memory and leave as the result and the packed copy.  Small kernels of a chain: launches and their starts bound it.
+// 96 -> 24 -> (144) -> 24 -> 144 -> depthwise: six launches 33.0 us, the last two (a thread per result, found out of its index by divisions, and a
+// delivery that read them again) 17 of them; now five, 19.5 us, the same bits.
+// ----------------------------------------------------------------------------------------------
+constexpr int kDwO = 8, kDwI = 16, kDwThreads = kDwO * kDwI;
+__global__ void __launch_bounds__(kDwThreads)
+k_compose_dw33(const Piece first, const Piece second, float *w_out, float *b_out, const __grid_constant__ BlockDelivery dv, int gi, int tiles) {
+  __shared__ __align__(16) float out[kDwThreads * 25];
+  __shared__ size_t row_s[kDwO], plane_s[kDwI / 8 * 25];
+  const int tid = (int)threadIdx.x, c0 = first.c_in, c2 = second.c_out;
+  dc_pdl_enter();
+  if ((int)blockIdx.x >= tiles) {
+    zero_dead_chunks(dv, c2, (int)blockIdx.x - tiles, (int)gridDim.x - tiles);
+    return;
+  }
+  const int o0 = (int)blockIdx.x / gi * kDwO, i0 = (int)blockIdx.x % gi * kDwI, o = o0 + tid / kDwI, i = i0 + tid % kDwI;
+  if (o < c2 && i < c0) {
+    float w1[9], w2[9], r[25] = {};
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      w1[t] = piece_dense_at(first, o, i, t / 3, t % 3);
+      w2[t] = piece_diag_at(second, o, t / 3, t % 3);
+    }
+#pragma unroll
+    for (int t2 = 0; t2 < 9; ++t2)
+#pragma unroll
+      for (int t1 = 0; t1 < 9; ++t1) {
+        float &x = r[(t2 / 3 + t1 / 3) * 5 + t2 % 3 + t1 % 3];
+        x = fmaf(w2[t2], w1[t1], x);
+      }
+#pragma unroll
+    for (int t = 0; t < 25; ++t) out[tid * 25 + t] = r[t];
+    if (i == 0) {                                  // b2~ + (sum of the taps) b1~
+      float ws = second.ident ? 1.f : 0.f;
+#pragma unroll
+      for (int t = 0; t < 9; ++t) ws += second.w[(size_t)o * 9 + t];
+      b_out[o] = second.b[o] + __fmul_rn(ws, first.b[o]);
+    }
+  }
+  const bool by_rows = dv.mode == 2 && !dv.ko.fold && !dv.ko.pair;
+  const int per = dv.ko.rows && dv.ko.nnt > 1 ? dv.ko.n_tile : dv.ko.n_pad;
+  if (by_rows) {                                   // as in k_merge_outer33
+    const int e = tid - (kDwThreads - kDwI / 8 * 25);
+    if (e >= 0) plane_s[e] = (size_t)dc_korder_encode(dv.ko, (i0 >> 3) + e / 25, e % 25 / 5, e % 5) * per;
+    if (tid < kDwO) row_s[tid] = dc_packed_chunk(dv.ko, 0, o0 + tid);
+  }
+  __syncthreads();
+  for (int e = tid; e < kDwThreads * 25 / 4; e += kDwThreads) {
+    const int ow = e / (kDwI * 25 / 4), x = (e - ow * (kDwI * 25 / 4)) * 4;
+    if (o0 + ow >= c2) continue;
+    float *to = w_out + ((size_t)(o0 + ow) * c0 + i0) * 25 + x;
+    const float *from = out + ow * (kDwI * 25) + x;
+    if (c0 % 4 == 0) {
+      if (i0 + x / 25 < c0) *reinterpret_cast<float4 *>(to) = *reinterpret_cast<const float4 *>(from);
+    } else {
+      for (int j = 0; j < 4; ++j)
+        if (i0 + (x + j) / 25 < c0) to[j] = from[j];
+    }
+  }
+  if (dv.mode == 0) return;
+  if (!by_rows) {
+    deliver_tile<kDwO, kDwI, 5>(dv, out, o0, i0, c0, c2, tid, kDwThreads);
+    return;
+  }
+  auto two = [](float lo, float hi) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&p);
+  };
+  for (int e = tid; e < kDwO * (kDwI / 8) * 25; e += kDwThreads) {
+    const int ow = e % kDwO, rest = e / kDwO, hf = rest % (kDwI / 8), t = rest / (kDwI / 8);
+    if (o0 + ow >= c2 || i0 + hf * 8 >= c0) continue;
+    const float *f = out + (ow * kDwI + hf * 8) * 25 + t;
+    reinterpret_cast<uint4 *>(dv.packed)[row_s[ow] + plane_s[hf * 25 + t]] = make_uint4(two(f[0], f[25]), two(f[50], f[75]), two(f[100], f[125]), two(f[150], f[175]));
+  }
+}
+
 // fp32 [o][i][u][v] -> fp32 [u][v][i][o]
 __global__ void k_pack_f32(const float *w, float *out, int c_out, int c_in, int k) {
   int total = c_out * c_in * k * k;
@@ -673,7 +752,6 @@ __global__ void __launch_bounds__(kBlockThreads) k_merge_block(const __grid_cons
 // ----------------------------------------------------------------------------------------------
 constexpr int kMbO = 8, kMbI = 16, kMbSlice = 16, kMbStages = 4;
 constexpr int kMbThreads = 256;
-constexpr int kMbTile = kMbO * kMbI * 9;                          // sums of a CTA of 8 x 16 pairs
 // A form of the kernel: IT input channels of a tile, W warps that share the hidden channels.
 template <int IT, int W>
 struct MbForm {
@@ -1741,6 +1819,10 @@ static Piece compose(const Piece &first, const Piece &second, Bump &bump, bool g
       if (dv) { out.w = w = w_final; out.b = b = b_final; *delivered = true; }
       launch_compose33(operand(first), operand(second), first.c_in, first.c_out, second.c_out, w, b, dv ? *dv : piece,
                        mg ? *mg : dc_geom{}, st, status);
+    } else if (dv && !first.diag && second.diag && first.k == 3 && first.stride == 1 && second.k == 3) {
+      const int gi = dc_div_up(first.c_in, kDwI), tiles = gi * dc_div_up(second.c_out, kDwO);
+      out.w = w_final; out.b = b_final; *delivered = true;
+      status.note(dc_launch_pdl(k_compose_dw33, dim3(tiles + zero_ctas(*dv, *mg, kDwThreads)), dim3(kDwThreads), 0, st, first, second, w_final, b_final, *dv, gi, tiles));
     } else if (!first.diag && !second.diag && first.k == 1 && first.stride == 1 && second.k == 3 && first.c_in % 4 == 0 &&
                first.c_out % 4 == 0 && first.c_out >= 32) {
       // From 32 intermediate channels on, a whole slice (96 -> 24 -> 24 inside a longer run took 2.3 us more here).

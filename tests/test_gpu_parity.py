@@ -1383,3 +1383,19 @@ def test_1x1_and_depthwise_pairs_against_the_oracle(dc, dw_first, a, o, res, cod
     c = a if dw_first else o
     pair = [mk(93, 0, c, c, 3, 1, 1, depthwise=True), mk(93, 1, a, o, 1, 1, 0)]
     _check_delivery(dc, pair if dw_first else pair[::-1], res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
+
+
+@pytest.mark.parametrize("before,a,c,s,res,codes", [
+    ([], 96, 144, 2, [], "both"),
+    ([], 24, 16, 1, [], "both"),               # packed orders that hold pixels in their rows
+    ([], 48, 24, 1, [], "both"),               # and that do not
+    ([], 50, 30, 1, [], "f32"), ([], 20, 12, 2, [], "f32"),        # rows that are no whole 16-byte pieces; tiles partly filled
+    ([], 40, 40, 1, [(0, 0)], "both"), ([], 40, 40, 1, [(0, 0), (1, 1)], "both"), ([], 40, 40, 1, [(0, 1)], "both"),
+    ([72, 24], 24, 144, 2, [], "both"),        # behind other layers
+])
+def test_3x3_then_depthwise_at_the_end_of_a_run(dc, before, a, c, s, res, codes):
+    mk = I.make_layer
+    chan = before + ([] if before and before[-1] == a else [a])
+    specs = [mk(94, i, chan[i], chan[i + 1], 1, 1, 0) for i in range(len(chan) - 1)]
+    specs += [mk(94, 7, a, c, 3, 1, 1), mk(94, 8, c, c, 3, s, 1, depthwise=True)]
+    _check_delivery(dc, specs, res, (dc.BF16, dc.F32) if codes == "both" else (dc.F32,))
