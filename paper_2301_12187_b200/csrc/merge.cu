@@ -1157,10 +1157,10 @@ k_compose33(const __grid_constant__ Compose33 a, const __grid_constant__ BlockDe
 // writing its result (160 -> 960: 5.5 MB and its packed copy) and by its launches.  One launch reads the layers as they
 // are and delivers tiles of 8 x 16 channel pairs, or of 8 x 32 or 8 x 64 where those are two to an SM; blocks behind the tiles compute the
 // bias (a warp per output channel) and zero the packed chunks without weights.  As fold, composition and delivery, three launches with the
-// result written and read in between: 160 -> 960 then depthwise 27.6 us, depthwise then 576 -> 96 27.1, 384 -> 64 17.3; here 8.6, 4.6 and
+// result written and read in between: 160 -> 960 then depthwise 27.6 us, depthwise then 576 -> 96 27.1, 384 -> 64 17.3; here 7.3, 4.6 and
 // 3.9 us.
 //
-// Before: 9.3, 7.2 and 5.1 us; 320 -> 1920 20.2, now 17.6, depthwise then 1152 -> 192 16.9, now 10.1.  After a depthwise layer the bias
+// Before: 9.3, 7.2 and 5.1 us; 320 -> 1920 20.2, now 13.7, depthwise then 1152 -> 192 16.9, now 8.9.  After a depthwise layer the bias
 // blocks were the longest: each warp worked out every channel's factor for itself.  Then each chunk's place in the packed copy,
 // divisions all, and in large results the tiles' starts.  (The smallest, 2.7 us, take 0.1 more.)
 // ----------------------------------------------------------------------------------------------
@@ -1269,8 +1269,12 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
       const int ow = e / (IT * 9 / 4), x = (e - ow * (IT * 9 / 4)) * 4;
       if (o0 + ow >= c2 || i0 + x / 9 >= c0) continue;
       float v[4];
+      int iw = x / 9, t = x - iw * 9;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = value(ow, (x + j) / 9, (x + j) % 9);
+      for (int j = 0; j < 4; ++j) {
+        v[j] = value(ow, iw, t);
+        if (++t == 9) { t = 0; ++iw; }
+      }
       *reinterpret_cast<float4 *>(a.w_out + ((size_t)(o0 + ow) * c0 + i0) * 9 + x) = make_float4(v[0], v[1], v[2], v[3]);
     }
   } else {
@@ -1292,17 +1296,23 @@ k_merge_outer33(const __grid_constant__ Outer33 a, const __grid_constant__ Block
     const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&p);
   };
-  for (int e = tid; e < kMbO * (IT / 8) * 9; e += kMbThreads) {
-    const int ow = e % kMbO, rest = e / kMbO, hf = rest % (IT / 8), t = rest / (IT / 8), o = o0 + ow, i = i0 + hf * 8;
+  // a thread to three taps of a chunk's channels, whose weights it reads once; in small results to one
+  constexpr int TAPS = IT == 16 ? 1 : 3;
+  for (int e = tid; e < kMbO * (IT / 8) * (9 / TAPS); e += kMbThreads) {
+    const int ow = e % kMbO, rest = e / kMbO, hf = rest % (IT / 8), o = o0 + ow, i = i0 + hf * 8;
+    int t = rest / (IT / 8) * TAPS;
     if (o >= c2 || i >= c0) continue;
-    float v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = IT == 16 ? out[(ow * IT + hf * 8 + q) * 9 + t] : value(ow, hf * 8 + q, t);
-    if (by_rows)
-      reinterpret_cast<uint4 *>(dv.packed)[row_s[ow] + plane_s[hf * 9 + t]] =
-          make_uint4(two(v[0], v[1]), two(v[2], v[3]), two(v[4], v[5]), two(v[6], v[7]));
-    else
-      deliver_chunk<9, 1>(dv, v, o, i, t, c0, c2);
+    for (int n = 0; n < TAPS; ++n, ++t) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = IT == 16 ? out[(ow * IT + hf * 8 + q) * 9 + t] : value(ow, hf * 8 + q, t);
+      if (by_rows)
+        reinterpret_cast<uint4 *>(dv.packed)[row_s[ow] + plane_s[hf * 9 + t]] =
+            make_uint4(two(v[0], v[1]), two(v[2], v[3]), two(v[4], v[5]), two(v[6], v[7]));
+      else
+        deliver_chunk<9, 1>(dv, v, o, i, t, c0, c2);
+    }
   }
 }
 
