@@ -303,6 +303,15 @@ dc_status dc_selftest_bounded_wait(void *workspace, size_t workspace_bytes, unsi
 int dc_selftest_block_waits(unsigned int chunk, int operands, int stages, unsigned int waits[12]);
 
 /*
+ * Host only, launches nothing: what the merges on the tensor core (blocks and 1x1 pairs) wait for at step `step` of a reduction whose
+ * terms go through `slots` slots, as the kernel itself works it out.  Then for each wait, in order, the barrier's index and the parity:
+ * first the waits of a warp that cuts the step's terms (waits[0] of them), then those of the warp that multiplies them.  Barriers below
+ * waits[1] say that the terms of a slot are there, waits[1] and above that those of slot (index - waits[1]) are multiplied.  Returns
+ * the number of waits, three at most (0: arguments out of range).
+ */
+int dc_selftest_product_waits(int step, int slots, unsigned int waits[8]);
+
+/*
  * Host only: the layout in which dc_chain_forward_host keeps a run's parameters on the device:
  * offsets[6 * i + j] is the byte offset of array j of layer i (j = 0 weight, 1 bias, 2 bn_gamma,
  * 3 bn_beta, 4 bn_mean, 5 bn_var; each rounded up to 256 bytes), total the size of the block.

@@ -37,6 +37,25 @@ constexpr int kSmemMax = 225 * 1024;             // asked for always: a CTA hold
 
 __host__ __device__ constexpr int threads_of(int nt) { return 2 * (8 + nt / 16) * 32 + 64; }      // two teams that cut, two warps that issue
 
+// The waits of a step on its slot, which a plan uses twice at most.  A barrier's wait tells two neighbouring phases apart and no more, so
+// every phase but the last must be known to be over where a wait begins.  (On the host as well: a test walks them through every order of
+// events.)
+//
+// Terms of a second use are the second phase of their barrier, and a wait for that one returns at once while the first is still open.
+// The warp that issues need not have met the first one: with an odd number of slots and two sums that was the other warp's step, and
+// the teams that cut are not ordered against each other.  So it waits first until the first use is multiplied, as those that cut do.  Of
+// that barrier no second phase can be over before this warp has issued the step.
+#pragma nv_exec_check_disable
+template <typename Wait>
+__host__ __device__ __forceinline__ bool cut_waits(int step, int slots, Wait wait) {
+  return step < slots || wait(kMaxSlots + step - slots, 0u);
+}
+#pragma nv_exec_check_disable
+template <typename Wait>
+__host__ __device__ __forceinline__ bool issue_waits(int step, int slots, Wait wait) {
+  return step < slots ? wait(step, 0u) : wait(kMaxSlots + step - slots, 0u) && wait(step - slots, 1u);
+}
+
 template <int KIND>
 struct Shape {
   static constexpr int T = KIND == kProductPair ? 1 : 9, OT = KIND == kProductPair ? 128 : 14, ROWS = OT * T;
@@ -197,7 +216,8 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
       uint4 h, mi, l;
       bf16_terms8(v, h, mi, l);
       const int slot = s < p.slots ? s : s - p.slots;
-      if (s >= p.slots && !(ok = warp_wait(&bar[kMaxSlots + slot], 0u, abort_flag, nullptr, 0u))) break;
+      ok = cut_waits(s, p.slots, [&](int b, uint32_t parity) { return warp_wait(&bar[b], parity, abort_flag, nullptr, 0u); });
+      if (!ok) break;
       const uint32_t d = sm + to + (uint32_t)(slot * kStep);
       sts_u4(d, h);
       sts_u4(d + plane, mi);
@@ -234,8 +254,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
     const uint32_t sm16 = (sm >> 4) & 0x3FFFu;   // a CTA's own addresses name its rank in a cluster
     const int odd = warp - kIssue;
     auto ready = [&](int mine) {
-      const bool again = mine >= p.slots;
-      ok = mbar_wait(&bar[again ? mine - p.slots : mine], again ? 1u : 0u, abort_flag, nullptr, 0u);
+      ok = issue_waits(mine, p.slots, [&](int b, uint32_t parity) { return mbar_wait(&bar[b], parity, abort_flag, nullptr, 0u); });
       __syncwarp();
       ok = __all_sync(0xffffffffu, ok) != 0;
       tc_fence_after();
@@ -532,4 +551,20 @@ dc_status dc_merge_product_tc_status(bool *ran_out) {
     DC_CUDA_OK(cudaMemcpyToSymbol(g_product_status, &zero, sizeof(zero)));
   }
   return DC_OK;
+}
+
+extern "C" int dc_selftest_product_waits(int step, int slots, unsigned int waits[8]) {
+  if (slots < 1 || slots > kMaxSlots || step < 0 || step >= 2 * slots) return 0;
+  int n = 0;
+  auto note = [&](int at, uint32_t parity) {
+    waits[2 + 2 * n] = (unsigned int)at;
+    waits[3 + 2 * n] = parity;
+    ++n;
+    return true;
+  };
+  cut_waits(step, slots, note);
+  waits[0] = (unsigned int)n;
+  issue_waits(step, slots, note);
+  waits[1] = (unsigned int)kMaxSlots;
+  return n;
 }

@@ -105,6 +105,7 @@ EXPORTS = {
     "dc_workspace_status_where": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(C.c_uint), C.POINTER(C.c_uint)]),
     "dc_selftest_bounded_wait": (C.c_int, [C.c_void_p, C.c_size_t, C.c_uint, C.c_void_p]),
     "dc_selftest_block_waits": (C.c_int, [C.c_uint, C.c_int, C.c_int, C.POINTER(C.c_uint)]),
+    "dc_selftest_product_waits": (C.c_int, [C.c_int, C.c_int, C.POINTER(C.c_uint)]),
     "dc_chain_host_param_layout": (C.c_int, [C.POINTER(Layer), C.c_int, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]),
     "dc_chain_host_workspace_bytes": (C.c_int, [C.POINTER(Layer), C.c_int, C.POINTER(Residual), C.c_int,
                                                 C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_size_t)]),
@@ -492,6 +493,17 @@ def selftest_block_waits(chunk: int, operands: int, stages: int):
     if n <= 0:
         raise ValueError("operands or stages out of range")
     return tuple(out[:3]), [tuple(out[3 + 3 * i:6 + 3 * i]) for i in range(n)]
+
+
+def selftest_product_waits(step: int, slots: int):
+    """What a step of a merge on the tensor core waits for where it is cut and where it is multiplied, as two lists of (multiplied,
+    slot, parity): that slot's terms are multiplied, or (0) are there; see include/dc.h."""
+    out = (C.c_uint * 8)()
+    n = lib().dc_selftest_product_waits(step, slots, out)
+    if n <= 0:
+        raise ValueError("step or slots out of range")
+    waits = [(out[2 + 2 * i] // out[1], out[2 + 2 * i] % out[1], out[3 + 2 * i]) for i in range(n)]
+    return waits[:out[0]], waits[out[0]:]
 
 
 def host_layer_array(specs, pinned: bool = False) -> Tuple["C.Array", list]:
