@@ -1728,8 +1728,8 @@ static void launch_compose33(const Operand33 &first, const Operand33 &second, in
                              const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
   if (compose33_on_tensor_core(c0, c1, c2)) {
-    status.note(dc_launch_compose33_tc(a, dv, st));
-    return;
+    const dc_status s = dc_launch_compose33_tc(a, dv, st);
+    if (s != DC_ERR_UNSUPPORTED) { status.note(s); return; }       // beyond its range (4096 channels between): the FMAs have none
   }
   const int most = dc_div_up(a.gi * a.go, dc_sm_count());
   if (most <= 2 || ((most == 3 || most == 5) && c1 >= 128)) launch_compose33_form<8>(a, dv, mg, st, status);

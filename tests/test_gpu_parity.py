@@ -1284,6 +1284,21 @@ def test_3x3_after_3x3_by_bf16_terms_as_a_piece(dc):
                     (dc.BF16, dc.F32))
 
 
+@pytest.mark.parametrize("algo", ["auto", "steps", "piece"])
+@pytest.mark.parametrize("a,c,o", [(64, 4104, 64), (128, 4100, 130)])
+def test_3x3_after_3x3_with_more_channels_between_than_the_tensor_core_takes(dc, algo, a, c, o):
+    specs = [I.make_layer(89, 0, a, c, 3, 1, 1), I.make_layer(89, 1, c, o, 3, 1, 1)]
+    if algo == "piece":                            # in the middle of a run, whose end reads what the composition wrote
+        specs.append(I.make_layer(89, 2, o, 8, 1, 1, 0))
+    W, b, k, s, p = O.merge_formula(specs, [])
+    g, wm, bm, packed = run_merge(dc, specs, [], packed_dtype=dc.F32, algo=dc.MERGE_STEPS if algo == "steps" else dc.MERGE_AUTO)
+    assert (g.k, g.stride, g.pad) == (k, s, p)
+    assert O.rel_l2(wm.cpu().numpy(), W) <= TOL_W and O.rel_l2(bm.cpu().numpy(), b) <= TOL_W
+    again = torch.full_like(packed, 7)
+    dc.pack_weights(wm, g, dc.F32, again)
+    assert torch.equal(packed, again)
+
+
 def test_3x3_after_3x3_by_bf16_terms_of_what_is_not_finite(dc):
     """An infinity, a NaN and a value beyond the largest bf16 among the weights: infinities and NaN where 64 bits have them."""
     specs = [I.make_layer(88, 0, 104, 208, 3, 1, 1, with_bn=False), I.make_layer(88, 1, 208, 136, 3, 1, 1, with_bn=False)]
