@@ -199,12 +199,20 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   // layers 0.31 of the time on (geometric) average, one slower, by 2 %.  3x3 layers of 24 outputs and 1x1 layers of 8 keep the
   // kernels they have, though they would gain as much (152 -> 24 3x3, 50 of 28 x 28 121 and 12): which kernels read their packed
   // order is held by tests.
-  const bool narrow_rows = g->groups == 1 && g->stride == 1 && g->k <= 7 && ko->cch >= 5 && g->c_out < 32 &&
+  // 7x7 layers of 24 and 32 channels to at most 24 outputs, which the pair rows do not take either: the fold kernel runs 24 -> 8 at any width,
+  // and faster where there is much to do (128 images of 28 x 28 14.2 us there, 25.6 by rows, 31.3 by the general kernel; of 56 x 56 32, 78
+  // and 53; one of 14 x 14 6.6, 4.7 and 6.6).  Wider ones go by rows: beyond some width (44 for 32 -> 16) the fold kernel has no room
+  // beside their weights, the general one has none for some sizes at any width (24 -> 24 on 128 maps of 56 x 56, on the CUDA cores 6035 us,
+  // by rows 77), and over 72 sizes rows take 0.84 of the fold kernel's time on (geometric) average where that runs and 0.74 of the general
+  // one's (24 -> 16 on 128 maps of 28 x 28 25.6 us by rows, 16.7 and 31.5; on 128 of 14 x 14 9.0, 9.6 and 21.0).
+  const size_t fold_bytes = (size_t)ko->cch * g->k * dc_round_up((size_t)(g->k * ko->co8), 16) * 16;
+  const bool narrow7 = g->k == 7 && ko->cch < 5 && fold_bytes <= 64 * 1024, fold7 = narrow7 && fold_bytes <= 24 * 1024;
+  const bool narrow_rows = g->groups == 1 && g->stride == 1 && g->k <= 7 && (ko->cch >= 5 || (narrow7 && !fold7)) && g->c_out < 32 &&
                            (g->k == 1 ? g->c_out >= 16 : g->k != 3 || g->c_out <= 16) && g->c_in % 8 == 0 && g->c_out % 8 == 0;
-  if (g->groups == 1 && g->stride == 1 && g->k >= 3 && ko->cch >= 5 && ko->cch <= 8 && (g->c_out == 24 || g->c_out == 32) &&
-      !narrow_rows && g->c_in % 8 == 0) {
+  if (g->groups == 1 && g->stride == 1 && g->k >= 3 && (fold7 || (ko->cch >= 5 && ko->cch <= 8 && (g->c_out == 24 || g->c_out == 32))) &&
+      !narrow_rows && g->c_in % 8 == 0 && g->c_out % 8 == 0) {
     const int n_pad = (int)dc_round_up((size_t)(g->k * ko->co8), 16);
-    if ((size_t)ko->cch * g->k * n_pad * 16 <= 64 * 1024) {
+    if (fold_bytes <= 64 * 1024) {
       ko->fold = 1;
       ko->n_pad = n_pad;
       ko->ns[0] = g->k; ko->ns[1] = 0; ko->s0[0] = 0; ko->s0[1] = 0;
@@ -223,7 +231,7 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   // column they read, class by class, so that one class reads one sub-tile of every second row and column.
   const bool rows_s2 = g->stride == 2 && g->k >= 3 && ko->cch >= 2;
   if (g->groups == 1 && g->k <= 7 && (g->stride == 1 || rows_s2) &&
-      (rows_s2 || (ko->cch >= 5 ? g->c_out >= 32 || narrow_rows
+      (rows_s2 || narrow_rows || (ko->cch >= 5 ? g->c_out >= 32
                     : ((g->k == 1 && ko->cch >= 2 && g->c_out >= 48) || (g->k >= 3 && ko->cch >= 2 && ko->co8 > 128)))) &&
       g->c_in % 8 == 0 && g->c_out % 8 == 0) {
     const int n16 = (int)dc_round_up((size_t)g->c_out, 16);

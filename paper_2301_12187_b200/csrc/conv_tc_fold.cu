@@ -499,7 +499,8 @@ k_conv_tc_fold(const __grid_constant__ FoldParams p, const __nv_bfloat16 *__rest
         if (++s == p.stages) { s = 0; ph ^= 1; a_row = a_row0; }
       }
     } else {
-      if (p.co8 == 24) epilogue_dispatch<24>(p, sh, ws, bias_s, xch, smem_out, residual, y, tile0, ntiles);
+      if (p.co8 == 8) epilogue_dispatch<8>(p, sh, ws, bias_s, xch, smem_out, residual, y, tile0, ntiles);
+      else if (p.co8 == 24) epilogue_dispatch<24>(p, sh, ws, bias_s, xch, smem_out, residual, y, tile0, ntiles);
       else epilogue_dispatch<32>(p, sh, ws, bias_s, xch, smem_out, residual, y, tile0, ntiles);
     }
     // ---- consumer teardown

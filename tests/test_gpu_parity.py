@@ -635,6 +635,28 @@ def test_narrow_outputs_by_rows_against_the_oracle(dc, c_in, c_out, k, p, n, h, 
     test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, k, 1, p, n, h, w, "k_conv_tc_rows")
 
 
+@pytest.mark.parametrize("c_in,c_out,p,n,h,w,kernel", [
+    (24, 8, 3, 2, 14, 14, "k_conv_tc_fold"),
+    (24, 8, 0, 1, 7, 9, "k_conv_tc_fold"),           # one row of outputs
+    (24, 8, 6, 1, 9, 300, "k_conv_tc_fold"),         # the widest padding, column strips
+    (24, 16, 3, 1, 7, 8, "k_conv_tc_rows"),          # a plane of three chunks, fewer pixels than a block has rows
+    (24, 16, 3, 1, 20, 260, "k_conv_tc_rows"),
+    (24, 24, 3, 16, 28, 28, "k_conv_tc_rows"),       # 24 outputs of 32 operand rows
+    (24, 24, 0, 3, 33, 41, "k_conv_tc_rows"),
+    (32, 8, 2, 2, 15, 70, "k_conv_tc_rows"),
+    (32, 16, 6, 5, 9, 11, "k_conv_tc_rows"),
+    (32, 24, 3, 2, 14, 14, "k_conv_tc"),             # weights beyond the line for either
+])
+def test_7x7_of_few_channels_to_few_against_the_oracle(dc, c_in, c_out, p, n, h, w, kernel):
+    test_each_forward_kernel_against_the_oracle(dc, c_in, c_out, 7, 1, p, n, h, w, kernel)
+
+
+@pytest.mark.parametrize("c_in,c_out", [(24, 8), (24, 16), (24, 24), (32, 8)])
+def test_three_3x3_layers_to_few_outputs_in_the_packed_order(dc, c_in, c_out):
+    _check_delivery(dc, [I.make_layer(95, 0, c_in, 24, 3, 1, 1), I.make_layer(95, 1, 24, 40, 3, 1, 1), I.make_layer(95, 2, 40, c_out, 3, 1, 1)], [],
+                    (dc.BF16, dc.F32))
+
+
 @pytest.mark.parametrize("c_in,c_out,k,s,p,n,h,w,kernel", [
     (24, 24, 3, 1, 1, 3, 31, 23, "k_conv_tc_pairrows"),     # odd padding: the last pixel is the second of its output pair
     (32, 32, 5, 1, 2, 2, 28, 29, "k_conv_tc_pairrows"),     # even padding: the last output pair has one pixel
