@@ -286,7 +286,7 @@ class ChainBench:
             conv = replay_stats(self.g_conv, self.stream, self.slots)
             merge = replay_stats(self.g_merge, self.stream, self.MERGES_PER_GRAPH)
             step = replay_stats(self.g_round, self.stream, self.slots)
-        if self.dc.workspace_status(self.conv_ws, self.stream) != self.dc.OK:
+        if self.dc.workspace_status(self.conv_ws, self.stream) != self.dc.OK or self.dc.async_status(self.stream) != self.dc.OK:
             raise RuntimeError("device-side wait timed out during the benchmark (%s)" % self.name)
         n = self.case.x_shape[0]
         roof = roofline_entry(self.flops, self.abytes, conv["median"] * 1e-6, peaks, peak_src)

@@ -22,11 +22,12 @@
  *   - Ownership: the caller owns every buffer, workspaces included.  The library never
  *     allocates or frees device memory.
  *   - Every call enqueues work on `stream` and returns without synchronising, except
- *     dc_workspace_status and the *_host entry points, which say so.
+ *     dc_workspace_status, dc_async_status and the *_host entry points, which say so.
  *   - Errors: a dc_status is returned; argument and shape errors are detected on the host
  *     before anything is launched.  Device-side waits are bounded; a wait that runs out
  *     latches DC_ERR_TIMEOUT in the first word of the caller's workspace (read it with
- *     dc_workspace_status) and the kernel returns without hanging.
+ *     dc_workspace_status) -- or, of depthwise layers and merges, in a flag of the device (read
+ *     it with dc_async_status) -- and the kernel returns without hanging; its output is not valid then.
  */
 #ifndef DC_H_
 #define DC_H_
@@ -126,7 +127,8 @@ dc_status dc_packed_bytes(const dc_geom *g, dc_dtype dtype, size_t *bytes);
  * not NULL also the packed copy for packed_dtype (size from dc_packed_bytes).  workspace: device,
  * at least the bytes dc_merge_query reports; it overlaps nothing else.  The outputs may overlap the
  * layers' arrays (which then do not survive the call), not one another.  fp32 arithmetic: FMAs, or on the tensor
- * core products of exact bf16 terms of fp32 values, added up in fp32.
+ * core products of exact bf16 terms of fp32 values, added up in fp32.  DC_OK says that everything was launched;
+ * merges on the tensor core have bounded waits, and dc_async_status tells whether one ran out.
  */
 dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
                          float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,
@@ -233,10 +235,13 @@ dc_status dc_dwconv_forward(const void *x, int n, int h, int w, int c, int k, in
                             dc_dtype dtype, dc_stream stream);
 
 /*
- * Synchronises `stream`, then returns DC_ERR_TIMEOUT if a bounded wait of a depthwise launch or of a
- * merge on the tensor core (which take no workspace to latch it in) ran out on the current device
- * since the last call, DC_OK otherwise; clears the flag.
+ * Synchronises `stream`, then returns DC_ERR_TIMEOUT if a bounded wait of a launch that has no workspace
+ * header to latch it in -- dc_dwconv_forward, dc_block_forward's depthwise layers, dc_merge_chain,
+ * dc_merge_chain_algo, dc_merge_chain_static -- ran out on the current device since the last call, DC_OK
+ * otherwise; clears what it reports.  (The host-buffer entry points' merges latch in their workspace.)
+ * dc_dwconv_status is the same call by its older name.  Not while a stream of the thread is being captured.
  */
+dc_status dc_async_status(dc_stream stream);
 dc_status dc_dwconv_status(dc_stream stream);
 
 /* Host only: workspace bytes dc_block_forward needs for this input size. */
@@ -292,6 +297,13 @@ dc_status dc_workspace_status_where(void *workspace, dc_stream stream, unsigned 
  */
 dc_status dc_selftest_bounded_wait(void *workspace, size_t workspace_bytes, unsigned int limit_us,
                                    dc_stream stream);
+
+/*
+ * The same for launches that report through dc_async_status: enqueues a one-CTA kernel that waits, with the library's own wait
+ * routine, on a barrier that nothing completes, gives up after limit_us microseconds (1..100000) and sets the flag of `which`: 0 the
+ * depthwise stencil, 1 merges of 3x3 pairs on the tensor core, 2 merges of blocks and 1x1 pairs there.
+ */
+dc_status dc_selftest_flagged_wait(int which, unsigned int limit_us, dc_stream stream);
 
 /*
  * Host only, launches nothing: what the block kernel's stencil waits for in front of its CTA's chunk number `chunk` with this many

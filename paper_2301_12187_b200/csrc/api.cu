@@ -105,6 +105,32 @@ extern "C" dc_status dc_workspace_status(void *workspace, dc_stream stream) {
   return dc_workspace_status_where(workspace, stream, nullptr, nullptr);
 }
 
+dc_status dc_async_flag(int which, unsigned int **flag) {
+  static constexpr cudaError_t (*kFlags[kDcAsyncFlags])(unsigned int **) = {dc_dwconv_flag, dc_merge_tc_flag, dc_merge_product_tc_flag};
+  DC_CUDA_OK(kFlags[which](flag));
+  return DC_OK;
+}
+
+// All flags are read before any is cleared, so that an error on the way loses none.
+extern "C" dc_status dc_async_status(dc_stream stream) {
+  DC_CUDA_OK(cudaStreamSynchronize((cudaStream_t)stream));
+  unsigned int *flag[kDcAsyncFlags], set[kDcAsyncFlags];
+  for (int i = 0; i < kDcAsyncFlags; ++i) {
+    const dc_status s = dc_async_flag(i, &flag[i]);
+    if (s != DC_OK) return s;
+    DC_CUDA_OK(cudaMemcpy(&set[i], flag[i], sizeof(set[i]), cudaMemcpyDeviceToHost));
+  }
+  dc_status s = DC_OK;
+  for (int i = 0; i < kDcAsyncFlags; ++i)
+    if (set[i] != 0) {
+      s = DC_ERR_TIMEOUT;
+      if (cudaMemset(flag[i], 0, sizeof(set[i])) != cudaSuccess) (void)cudaGetLastError();        // it is reported again
+    }
+  return s;
+}
+
+extern "C" dc_status dc_dwconv_status(dc_stream stream) { return dc_async_status(stream); }
+
 // ----------------------------------------------------------------------------------------------
 // unmerged inverted-residual block: three launches sharing the caller's workspace
 //   [status header][expand output n*h*w*c_hidden][depthwise output n*ho*wo*c_hidden]
@@ -328,8 +354,8 @@ extern "C" dc_status dc_chain_forward_host_async(const dc_layer *layers, int n_l
   char *dx = take(hp.x_bytes);
   char *dy = take(hp.y_bytes);
   DC_CUDA_OK(cudaMemcpyAsync(dx, x_host, hp.x_bytes, cudaMemcpyHostToDevice, st));
-  s = dc_merge_chain(dev.data(), n_layers, res, n_res, w_merged, b_merged, packed, dtype, merge_ws, hp.merge_ws,
-                     stream);
+  s = dc_merge_chain_ws(dev.data(), n_layers, res, n_res, w_merged, b_merged, packed, dtype, merge_ws, hp.merge_ws, stream, DC_MERGE_AUTO,
+                        (DcWsHeader *)workspace);
   if (s != DC_OK) return s;
   s = dc_conv_forward(dx, n, h, w, &hp.mg, packed, b_merged, act, nullptr, dy, dtype, workspace, sizeof(DcWsHeader),
                       stream);

@@ -475,6 +475,18 @@ dc_status dc_launch_conv_simt(const void *x, int n, int h, int w, const dc_geom 
 bool dc_conv_f32_supported(int n, int h, int w, const dc_geom *g);
 dc_status dc_launch_conv_f32(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                              const float *bias, dc_act act, const void *residual, void *y, cudaStream_t stream);
+// dc_merge_chain_algo whose launches latch a bounded wait that runs out in `ws`
+dc_status dc_merge_chain_ws(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res, float *w_merged, float *b_merged,
+                            void *w_packed, dc_dtype packed_dtype, void *workspace, size_t workspace_bytes, dc_stream stream,
+                            dc_merge_algo algo, DcWsHeader *ws);
+// Device addresses of the flags that kernels without a workspace header set when a bounded wait runs out: the depthwise stencil, merges of
+// 3x3 pairs and merges as a product on the tensor core.
+cudaError_t dc_dwconv_flag(unsigned int **flag);
+cudaError_t dc_merge_tc_flag(unsigned int **flag);
+cudaError_t dc_merge_product_tc_flag(unsigned int **flag);
+constexpr int kDcAsyncFlags = 3;
+dc_status dc_async_flag(int which, unsigned int **flag);     // one of them
+
 double dc_conv_f32_estimate_us(int n, int h, int w, const dc_geom *g);
 // fp32 by three bf16 terms on the tensor core; false and DC_ERR_UNSUPPORTED: outside its range, or slower there than the kernel above
 bool dc_conv_f32_tc_supported(int n, int h, int w, const dc_geom *g);

@@ -19,8 +19,7 @@
 // 14.6 -> 12.0; 240 channels 5x5, 64 images of 28 x 28 27.6 -> 24.6.
 //
 // The one wait (for the tile to land) is bounded like every wait of the library; a wait that runs
-// out sets a library-wide flag that dc_dwconv_status reports, and the CTA returns.
-#include "merge_parts.cuh"
+// out sets a library-wide flag that dc_async_status reports, and the CTA returns.
 #include "tc_ptx.cuh"
 
 namespace {
@@ -351,17 +350,4 @@ dc_status dc_launch_dwconv_stencil(const void *x, int n, int h, int w, int c, in
   return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }
 
-extern "C" dc_status dc_dwconv_status(dc_stream stream) {
-  DC_CUDA_OK(cudaStreamSynchronize((cudaStream_t)stream));
-  unsigned int st = 0;
-  DC_CUDA_OK(cudaMemcpyFromSymbol(&st, g_dw_status, sizeof(st)));
-  if (st != 0) {
-    const unsigned int zero = 0;
-    DC_CUDA_OK(cudaMemcpyToSymbol(g_dw_status, &zero, sizeof(zero)));
-  }
-  bool merge = false, product = false;
-  dc_status s = dc_merge_tc_status(&merge);
-  if (s == DC_OK) s = dc_merge_product_tc_status(&product);
-  if (s != DC_OK) return s;
-  return st != 0 || merge || product ? DC_ERR_TIMEOUT : DC_OK;
-}
+cudaError_t dc_dwconv_flag(unsigned int **flag) { return cudaGetSymbolAddress((void **)flag, g_dw_status); }

@@ -1694,6 +1694,7 @@ static bool compose33_ok(int c_in, int c_mid, int k1, int s1, int k2) {
 // convolution asks, and clears, it too; a run whose refused launch was followed by one of those returned DC_OK).
 struct MergeStatus {
   dc_status s = DC_OK;
+  DcWsHeader *ws = nullptr;      // where a bounded wait of its launches is latched (null: in the device's flags)
   void note(dc_status t) { if (s == DC_OK) s = t; }
   void note(cudaError_t e) { note(e == cudaSuccess ? DC_OK : DC_ERR_CUDA); }
   void launched() { note(cudaGetLastError()); }
@@ -1728,7 +1729,7 @@ static void launch_compose33(const Operand33 &first, const Operand33 &second, in
                              const BlockDelivery &dv, const dc_geom &mg, cudaStream_t st, MergeStatus &status) {
   const Compose33 a{first, second, c0, c1, c2, w, b, dc_div_up(c0, kP3I), dc_div_up(c2, kP3O)};
   if (compose33_on_tensor_core(c0, c1, c2)) {
-    const dc_status s = dc_launch_compose33_tc(a, dv, st);
+    const dc_status s = dc_launch_compose33_tc(a, dv, status.ws, st);
     if (s != DC_ERR_UNSUPPORTED) { status.note(s); return; }       // beyond its range (4096 channels between): the FMAs have none
   }
   const int most = dc_div_up(a.gi * a.go, dc_sm_count());
@@ -1787,7 +1788,7 @@ static void launch_block33(TiledBlocks &tb, const BlockDelivery &dv, const dc_ge
   const BlockArgs &b = tb.blk[0];
   const int run = hidden / (hidden < 320 ? 8 : 16);          // channels of a warp's sums, at least
   if (tb.n == 1 && block33_on_tensor_core(b.c0, b.c1, b.c2, run, most16, most24, form)) {
-    status.note(dc_launch_merge_product_tc(kProductBlock, Product{b.l1, b.l2, b.l3, 0, 0, b.c0, b.c1, b.c2, b.w_out, b.b_out}, dv, run, st));
+    status.note(dc_launch_merge_product_tc(kProductBlock, Product{b.l1, b.l2, b.l3, 0, 0, b.c0, b.c1, b.c2, b.w_out, b.b_out}, dv, run, status.ws, st));
     return;
   }
   if (form == 1) launch_block33_form<16, 16>(tb, dv, mg, st, status);
@@ -1931,13 +1932,14 @@ static bool writes_into_layers(const dc_layer *layers, int n, const float *w, si
 static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *res, int n_res,
                             float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,
                             void *workspace, cudaStream_t st, bool go, dc_geom *merged, size_t *need,
-                            dc_merge_algo algo = DC_MERGE_AUTO) {
+                            dc_merge_algo algo = DC_MERGE_AUTO, DcWsHeader *ws = nullptr) {
   dc_geom mg;
   dc_status s = check_chain(layers, n, res, n_res, &mg);
   if (s != DC_OK) return s;
   if (merged) *merged = mg;
   Bump bump{go ? (char *)workspace : nullptr, 0};
   MergeStatus status;
+  status.ws = ws;
 
   // What the last launch delivers.  A run that is one block of the tiled kind, or two dense 3x3 layers, needs no launch of
   // its own for that (nor, in the second case, for the BN): the kernel that merges it reads the layers as they are and
@@ -2016,7 +2018,7 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
                                   : 3.07 + a.c1 * (0.0136 * most + 0.0023 * dc_div_up(most, 3));
     const double tc = dc_merge_product_tc_us(kProductPair, a.c0, a.c1, a.c2, run);
     if (tc != 0.0 && tc < 0.95 * fma) {
-      status.note(dc_launch_merge_product_tc(kProductPair, Product{a.l1, RawLayer{}, a.l2, a.ident1, a.ident2, a.c0, a.c1, a.c2, a.w_out, a.b_out}, dv, run, st));
+      status.note(dc_launch_merge_product_tc(kProductPair, Product{a.l1, RawLayer{}, a.l2, a.ident1, a.ident2, a.c0, a.c1, a.c2, a.w_out, a.b_out}, dv, run, status.ws, st));
       return status.s;
     }
     const dim3 grid(a.gi * a.go + dc_div_up(a.c2, 8) + zero_ctas(dv, mg, 256));
@@ -2200,10 +2202,9 @@ extern "C" dc_status dc_merge_query(const dc_layer *layers, int n_layers, const 
   return merge_need(layers, n_layers, res, n_res, merged, workspace_bytes);
 }
 
-extern "C" dc_status dc_merge_chain_algo(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
-                                         float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,
-                                         void *workspace, size_t workspace_bytes, dc_stream stream,
-                                         dc_merge_algo algo) {
+dc_status dc_merge_chain_ws(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res, float *w_merged, float *b_merged,
+                            void *w_packed, dc_dtype packed_dtype, void *workspace, size_t workspace_bytes, dc_stream stream,
+                            dc_merge_algo algo, DcWsHeader *ws) {
   if (!w_merged || !b_merged) return DC_ERR_INVALID_ARG;
   if (packed_dtype != DC_F32 && packed_dtype != DC_BF16) return DC_ERR_INVALID_ARG;
   if (algo != DC_MERGE_AUTO && algo != DC_MERGE_STEPS) return DC_ERR_INVALID_ARG;
@@ -2217,7 +2218,15 @@ extern "C" dc_status dc_merge_chain_algo(const dc_layer *layers, int n_layers, c
   for (int i = 0; i < n_layers; ++i)
     if (!dc_aligned16(layers[i].weight)) return DC_ERR_ALIGNMENT;
   return merge_walk(layers, n_layers, res, n_res, w_merged, b_merged, w_packed, packed_dtype, workspace,
-                    (cudaStream_t)stream, true, nullptr, nullptr, algo);
+                    (cudaStream_t)stream, true, nullptr, nullptr, algo, ws);
+}
+
+extern "C" dc_status dc_merge_chain_algo(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
+                                         float *w_merged, float *b_merged, void *w_packed, dc_dtype packed_dtype,
+                                         void *workspace, size_t workspace_bytes, dc_stream stream,
+                                         dc_merge_algo algo) {
+  return dc_merge_chain_ws(layers, n_layers, res, n_res, w_merged, b_merged, w_packed, packed_dtype, workspace, workspace_bytes, stream, algo,
+                           nullptr);
 }
 
 extern "C" dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,

@@ -157,10 +157,9 @@ __device__ __forceinline__ float compose33_ident(const Compose33 &a, bool whole,
   return s;
 }
 
-// the same composition on the tensor core (merge_tc.cu); DC_ERR_UNSUPPORTED: outside its range, nothing was launched
-dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, cudaStream_t st);
-// whether a bounded wait of such a launch ran out on the current device since the last call; clears the flag
-dc_status dc_merge_tc_status(bool *ran_out);
+// The same composition on the tensor core (merge_tc.cu); DC_ERR_UNSUPPORTED: outside its range, nothing was launched.  A wait that runs
+// out is latched in `ws` where there is one, else in the device's flag of these kernels.
+dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, DcWsHeader *ws, cudaStream_t st);
 
 // What a dense 1x1 layer l1 is composed with, as one product on the tensor core (merge_product_tc.cu): the rest of an inverted-residual
 // block (mid: the 3x3 depthwise layer, l2: the last one), or a 1x1 layer l2.  c0 and c1 are multiples of 4.
@@ -171,8 +170,7 @@ struct Product {
   int c0, c1, c2;
   float *w_out, *b_out;
 };
-// DC_ERR_UNSUPPORTED: outside its range, nothing was launched.  `run`: see make_plan there
-dc_status dc_launch_merge_product_tc(int kind, const Product &a, const BlockDelivery &dv, int run, cudaStream_t st);
+// DC_ERR_UNSUPPORTED: outside its range, nothing was launched.  `run`: see make_plan there; `ws` as above
+dc_status dc_launch_merge_product_tc(int kind, const Product &a, const BlockDelivery &dv, int run, DcWsHeader *ws, cudaStream_t st);
 // its estimated time; 0: outside its range
 double dc_merge_product_tc_us(int kind, int c0, int c1, int c2, int run);
-dc_status dc_merge_product_tc_status(bool *ran_out);

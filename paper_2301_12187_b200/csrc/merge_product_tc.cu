@@ -27,7 +27,7 @@
 namespace {
 using namespace tc;
 
-__device__ unsigned int g_product_status;        // DC_ERR_TIMEOUT once a wait of this kernel ran out
+__device__ unsigned int g_product_status;        // DC_ERR_TIMEOUT once a wait of this kernel ran out in a launch without a workspace header
 
 constexpr int kPitchA = 128 * 16;                // bytes between the halves of a step's 16 channels
 constexpr int kStepA = 6 * kPitchA;
@@ -95,7 +95,7 @@ __device__ __forceinline__ float add_ident(const Product &a, bool whole, float g
 
 template <int KIND, int NT>
 __global__ void __launch_bounds__(threads_of(NT), 1)
-k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ BlockDelivery dv, const __grid_constant__ Plan p) {
+k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ BlockDelivery dv, const __grid_constant__ Plan p, DcWsHeader *ws) {
   using S = Shape<KIND>;
   constexpr int T = S::T, OT = S::OT, UNIT = S::UNIT, kStep = kStepA + NT * 96;
   constexpr int kTeam = 8 + NT / 16, kWarpsCut = 2 * kTeam, kIssue = kWarpsCut, kCutThreads = kWarpsCut * 32, kThreads = threads_of(NT);
@@ -216,7 +216,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
       uint4 h, mi, l;
       bf16_terms8(v, h, mi, l);
       const int slot = s < p.slots ? s : s - p.slots;
-      ok = cut_waits(s, p.slots, [&](int b, uint32_t parity) { return warp_wait(&bar[b], parity, abort_flag, nullptr, 0u); });
+      ok = cut_waits(s, p.slots, [&](int b, uint32_t parity) { return warp_wait(&bar[b], parity, abort_flag, ws, 0x220000u | (uint32_t)b); });
       if (!ok) break;
       const uint32_t d = sm + to + (uint32_t)(slot * kStep);
       sts_u4(d, h);
@@ -254,7 +254,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
     const uint32_t sm16 = (sm >> 4) & 0x3FFFu;   // a CTA's own addresses name its rank in a cluster
     const int odd = warp - kIssue;
     auto ready = [&](int mine) {
-      ok = issue_waits(mine, p.slots, [&](int b, uint32_t parity) { return mbar_wait(&bar[b], parity, abort_flag, nullptr, 0u); });
+      ok = issue_waits(mine, p.slots, [&](int b, uint32_t parity) { return mbar_wait(&bar[b], parity, abort_flag, ws, 0x230000u | (uint32_t)b); });
       __syncwarp();
       ok = __all_sync(0xffffffffu, ok) != 0;
       tc_fence_after();
@@ -310,7 +310,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
   }
   // ---------------------------------------------------------------- sums: the warps that can read the same 32 rows take 8 columns in turn
   if (warp < kWarpsCut) {
-    ok = warp_wait(&bar[2 * kMaxSlots], 0u, abort_flag, nullptr, 0u) && ok;
+    ok = warp_wait(&bar[2 * kMaxSlots], 0u, abort_flag, ws, 0x240000u) && ok;
     tc_fence_after();
     const int quarter = warp & 3, m = quarter * 32 + lane, ow = m / T;
     const uint32_t drow = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -345,7 +345,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
     }
     tc_fence_before();
   }
-  if (!ok) atomicExch(&g_product_status, (unsigned int)DC_ERR_TIMEOUT);
+  if (!ok && !ws) atomicExch(&g_product_status, (unsigned int)DC_ERR_TIMEOUT);
   // ---------------------------------------------------------------- each CTA takes a share of the tile: units of 8 input channels of an output channel
   constexpr int kPieces = 2 * T, kAll = OT * (NT / 8);
   const int per = (kAll + p.split - 1) / p.split, u0 = rank * per, left = kAll - u0, cnt = left < 0 ? 0 : (left < per ? left : per);
@@ -362,7 +362,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
                   (uint32_t)(n * UNIT * 4), map_cluster(smem_u32(&bar[2 * kMaxSlots + 1]), (uint32_t)q));
       }
     __syncwarp();
-    if (cnt > 0 && !warp_wait(&bar[2 * kMaxSlots + 1], 0u, abort_flag, nullptr, 0u))
+    if (cnt > 0 && !warp_wait(&bar[2 * kMaxSlots + 1], 0u, abort_flag, ws, 0x250000u) && !ws)
       atomicExch(&g_product_status, (unsigned int)DC_ERR_TIMEOUT);
   } else {
     __syncthreads();
@@ -512,28 +512,28 @@ double make_plan(int c0, int c1, int c2, int run, Plan *best, int *best_nt) {
 }
 
 template <int KIND, int NT>
-dc_status launch(const Product &a, const BlockDelivery &dv, const Plan &p, cudaStream_t st) {
+dc_status launch(const Product &a, const BlockDelivery &dv, const Plan &p, DcWsHeader *ws, cudaStream_t st) {
   static unsigned char attr_done[kDcMaxDevices];
   DC_CUDA_OK(dc_set_max_smem_once(k_merge_product_tc<KIND, NT>, kSmemMax, attr_done));
   const int grid = dc_div_up(a.c2, Shape<KIND>::OT) * p.n_tiles * p.split;
-  const cudaError_t e = dc_launch_pdl_cluster(k_merge_product_tc<KIND, NT>, dim3((unsigned)grid), dim3(threads_of(NT)), (size_t)kSmemMax, st, p.split, a, dv, p);
+  const cudaError_t e = dc_launch_pdl_cluster(k_merge_product_tc<KIND, NT>, dim3((unsigned)grid), dim3(threads_of(NT)), (size_t)kSmemMax, st, p.split, a, dv, p, ws);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }
 
 template <int KIND>
-dc_status launch_kind(const Product &a, const BlockDelivery &dv, int run, cudaStream_t st) {
+dc_status launch_kind(const Product &a, const BlockDelivery &dv, int run, DcWsHeader *ws, cudaStream_t st) {
   Plan p{};
   int nt = 0;
   if (make_plan<KIND>(a.c0, a.c1, a.c2, run, &p, &nt) == 0.0) return DC_ERR_UNSUPPORTED;
-  if (nt == 48) return launch<KIND, 48>(a, dv, p, st);
-  if (nt == 64) return launch<KIND, 64>(a, dv, p, st);
-  return launch<KIND, 80>(a, dv, p, st);
+  if (nt == 48) return launch<KIND, 48>(a, dv, p, ws, st);
+  if (nt == 64) return launch<KIND, 64>(a, dv, p, ws, st);
+  return launch<KIND, 80>(a, dv, p, ws, st);
 }
 
 }  // namespace
 
-dc_status dc_launch_merge_product_tc(int kind, const Product &a, const BlockDelivery &dv, int run, cudaStream_t st) {
-  return kind == kProductBlock ? launch_kind<kProductBlock>(a, dv, run, st) : launch_kind<kProductPair>(a, dv, run, st);
+dc_status dc_launch_merge_product_tc(int kind, const Product &a, const BlockDelivery &dv, int run, DcWsHeader *ws, cudaStream_t st) {
+  return kind == kProductBlock ? launch_kind<kProductBlock>(a, dv, run, ws, st) : launch_kind<kProductPair>(a, dv, run, ws, st);
 }
 
 double dc_merge_product_tc_us(int kind, int c0, int c1, int c2, int run) {
@@ -542,16 +542,7 @@ double dc_merge_product_tc_us(int kind, int c0, int c1, int c2, int run) {
   return kind == kProductBlock ? make_plan<kProductBlock>(c0, c1, c2, run, &p, &nt) : make_plan<kProductPair>(c0, c1, c2, run, &p, &nt);
 }
 
-dc_status dc_merge_product_tc_status(bool *ran_out) {
-  unsigned int s = 0;
-  DC_CUDA_OK(cudaMemcpyFromSymbol(&s, g_product_status, sizeof(s)));
-  *ran_out = s != 0;
-  if (s != 0) {
-    const unsigned int zero = 0;
-    DC_CUDA_OK(cudaMemcpyToSymbol(g_product_status, &zero, sizeof(zero)));
-  }
-  return DC_OK;
-}
+cudaError_t dc_merge_product_tc_flag(unsigned int **flag) { return cudaGetSymbolAddress((void **)flag, g_product_status); }
 
 extern "C" int dc_selftest_product_waits(int step, int slots, unsigned int waits[8]) {
   if (slots < 1 || slots > kMaxSlots || step < 0 || step >= 2 * slots) return 0;

@@ -28,7 +28,7 @@
 namespace {
 using namespace tc;
 
-__device__ unsigned int g_merge_status;          // DC_ERR_TIMEOUT once a wait of this kernel ran out
+__device__ unsigned int g_merge_status;          // DC_ERR_TIMEOUT once a wait of this kernel ran out in a launch without a workspace header
 
 constexpr int kO = 14, kI = 8, kRows = kO * 9, kCols = kI * 9;
 constexpr int kRowsB = 224;                      // of the columns' terms of 8 channels: 72 of each, and 8 that only make up the instruction's 224 columns
@@ -79,7 +79,7 @@ __device__ __noinline__ float sum_by_fma(const Compose33 &a, int o, int i, int t
 
 __global__ void __launch_bounds__(kThreads, 1)
 k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ Compose33 a,
-               const __grid_constant__ BlockDelivery dv, const __grid_constant__ Params33 p) {
+               const __grid_constant__ BlockDelivery dv, const __grid_constant__ Params33 p, DcWsHeader *ws) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t bar[kBars];
   __shared__ size_t row_s[kO];                   // where the tile's output channels, and its taps, are in the packed copy
@@ -112,7 +112,7 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
     tc_fence_after();
   }
   const uint32_t tmem = tmem_s;
-  auto wait = [&](int b, uint32_t parity) { return warp_wait(&bar[b], parity, abort_flag, nullptr, 0u); };
+  auto wait = [&](int b, uint32_t parity) { return warp_wait(&bar[b], parity, abort_flag, ws, 0x200000u | (uint32_t)b); };
   // the first and the last of a CTA's tiles that use the same columns' terms
   auto first_of = [&](int item) { return !p.resident || item == begin || item % p.m_tiles == 0; };
   auto last_of = [&](int item) { return !p.resident || item + 1 == end || (item + 1) % p.m_tiles == 0; };
@@ -239,7 +239,7 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
       }
       bar_sync(3, 128);
     }
-    if (!ok && tid == 0) atomicExch(&g_merge_status, (unsigned int)DC_ERR_TIMEOUT);
+    if (!ok && !ws && tid == 0) atomicExch(&g_merge_status, (unsigned int)DC_ERR_TIMEOUT);
   } else if (warp < kLoad) {
     // ---------------------------------------------------------------- operands into terms: a pair of warps takes every fourth step
     const int cw = warp - kWarpsAcc, ct = tid - kWarpsAcc * 32, pair = cw >> 1, w1 = cw & 1;
@@ -382,7 +382,7 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
         uint32_t parity = pa;
         if (first && (lane & 2)) { b = kBFull + bs + (lane & 1); parity = pb; }
         if (opens && lane == 4) { b = kDEmpty + (int)buf; parity = ((fl >> 1) & 1u) ^ 1u; }
-        ok = mbar_wait(&bar[b], parity, abort_flag, nullptr, 0u);
+        ok = mbar_wait(&bar[b], parity, abort_flag, ws, 0x210000u | (uint32_t)b);
         __syncwarp();
         if (!(ok = __all_sync(0xffffffffu, ok) != 0)) break;
         tc_fence_after();
@@ -465,7 +465,7 @@ bool matrix_map(CUtensorMap *map, EncodeTiledFn encode, const float *w, long lon
 
 }  // namespace
 
-dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, cudaStream_t st) {
+dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, DcWsHeader *ws, cudaStream_t st) {
   Params33 p{};
   if (!plan33(a.c0, a.c1, a.c2, &p)) return DC_ERR_UNSUPPORTED;
   EncodeTiledFn encode = get_encode_fn();
@@ -475,18 +475,8 @@ dc_status dc_launch_compose33_tc(const Compose33 &a, const BlockDelivery &dv, cu
   DC_CUDA_OK(dc_set_max_smem_once(k_compose33_tc, kSmemMax, attr_done));
   const int n_sm = dc_sm_count();
   const cudaError_t e = dc_launch_pdl(k_compose33_tc, dim3((unsigned)(p.items < n_sm ? p.items : n_sm)), dim3(kThreads),
-                                      (size_t)p.smem_bytes, st, map_w2, a, dv, p);
+                                      (size_t)p.smem_bytes, st, map_w2, a, dv, p, ws);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }
 
-// whether a wait of these kernels ran out on the current device since the last call; clears the flag
-dc_status dc_merge_tc_status(bool *ran_out) {
-  unsigned int s = 0;
-  DC_CUDA_OK(cudaMemcpyFromSymbol(&s, g_merge_status, sizeof(s)));
-  *ran_out = s != 0;
-  if (s != 0) {
-    const unsigned int zero = 0;
-    DC_CUDA_OK(cudaMemcpyToSymbol(g_merge_status, &zero, sizeof(zero)));
-  }
-  return DC_OK;
-}
+cudaError_t dc_merge_tc_flag(unsigned int **flag) { return cudaGetSymbolAddress((void **)flag, g_merge_status); }

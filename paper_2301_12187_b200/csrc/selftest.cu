@@ -34,6 +34,20 @@ __global__ void __launch_bounds__(64, 1) k_wait_probe(DcWsHeader *ws, unsigned l
   if (threadIdx.x == 0) ws->pad[0] = gave_up;   // both roles must have left their wait
 }
 
+// the same for kernels that report in a flag of the device
+__global__ void __launch_bounds__(32, 1) k_flag_probe(unsigned int *flag, unsigned long long limit_ns) {
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ uint32_t abort_word;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    abort_word = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const bool ok = warp_wait(&bar, 0, &abort_word, nullptr, 0u, limit_ns);
+  if (!ok) atomicExch(flag, (unsigned int)DC_ERR_TIMEOUT);
+}
+
 }  // namespace
 
 extern "C" dc_status dc_selftest_bounded_wait(void *workspace, size_t workspace_bytes, unsigned int limit_us,
@@ -43,5 +57,14 @@ extern "C" dc_status dc_selftest_bounded_wait(void *workspace, size_t workspace_
   if (!dc_aligned16(workspace)) return DC_ERR_ALIGNMENT;
   if (limit_us == 0 || limit_us > 100000u) return DC_ERR_INVALID_ARG;
   k_wait_probe<<<1, 64, 0, (cudaStream_t)stream>>>((DcWsHeader *)workspace, 1000ull * limit_us);
+  return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
+}
+
+extern "C" dc_status dc_selftest_flagged_wait(int which, unsigned int limit_us, dc_stream stream) {
+  if (which < 0 || which >= kDcAsyncFlags || limit_us == 0 || limit_us > 100000u) return DC_ERR_INVALID_ARG;
+  unsigned int *flag = nullptr;
+  const dc_status s = dc_async_flag(which, &flag);
+  if (s != DC_OK) return s;
+  k_flag_probe<<<1, 32, 0, (cudaStream_t)stream>>>(flag, 1000ull * limit_us);
   return cudaGetLastError() == cudaSuccess ? DC_OK : DC_ERR_CUDA;
 }

@@ -95,6 +95,7 @@ EXPORTS = {
                                        C.c_size_t, C.c_void_p, C.c_int]),
     "dc_dwconv_forward": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                     C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_void_p]),
+    "dc_async_status": (C.c_int, [C.c_void_p]),
     "dc_dwconv_status": (C.c_int, [C.c_void_p]),
     "dc_block_workspace_bytes": (C.c_int, [C.c_int, C.c_int, C.c_int, C.POINTER(Block), C.c_int,
                                            C.POINTER(C.c_size_t)]),
@@ -104,6 +105,7 @@ EXPORTS = {
     "dc_workspace_status": (C.c_int, [C.c_void_p, C.c_void_p]),
     "dc_workspace_status_where": (C.c_int, [C.c_void_p, C.c_void_p, C.POINTER(C.c_uint), C.POINTER(C.c_uint)]),
     "dc_selftest_bounded_wait": (C.c_int, [C.c_void_p, C.c_size_t, C.c_uint, C.c_void_p]),
+    "dc_selftest_flagged_wait": (C.c_int, [C.c_int, C.c_uint, C.c_void_p]),
     "dc_selftest_block_waits": (C.c_int, [C.c_uint, C.c_int, C.c_int, C.POINTER(C.c_uint)]),
     "dc_selftest_product_waits": (C.c_int, [C.c_int, C.c_int, C.POINTER(C.c_uint)]),
     "dc_chain_host_param_layout": (C.c_int, [C.POINTER(Layer), C.c_int, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]),
@@ -437,6 +439,11 @@ def dwconv_forward(x, k, stride, pad, w_packed, bias, act, y, stream=None):
                                    _ptr(y), dtype_code(x.dtype), _stream(stream)), "dc_dwconv_forward")
 
 
+def async_status(stream=None) -> int:
+    """ERR_TIMEOUT if a bounded wait of a depthwise layer or a merge ran out on this device since the last call; clears it."""
+    return int(lib().dc_async_status(_stream(stream)))
+
+
 def dwconv_status(stream=None) -> int:
     return int(lib().dc_dwconv_status(_stream(stream)))
 
@@ -484,6 +491,10 @@ def workspace_status_where(workspace, stream=None) -> Tuple[int, int, int]:
 def selftest_bounded_wait(workspace, limit_us: int, stream=None):
     _check(lib().dc_selftest_bounded_wait(_ptr(workspace), workspace.numel() * workspace.element_size(), int(limit_us),
                                           _stream(stream)), "dc_selftest_bounded_wait")
+
+
+def selftest_flagged_wait(which: int, limit_us: int, stream=None):
+    _check(lib().dc_selftest_flagged_wait(int(which), int(limit_us), _stream(stream)), "dc_selftest_flagged_wait")
 
 
 def selftest_block_waits(chunk: int, operands: int, stages: int):

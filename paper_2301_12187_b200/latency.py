@@ -146,7 +146,7 @@ def measure_latency_table(net, unit_us: float = 1.0, reps: int = 10, max_span: i
                     e1.record(stream)
                     stream.synchronize()
                     t_us = e0.elapsed_time(e1) * 1e3 / reps
-            if dc.workspace_status(conv_ws) != dc.OK:
+            if dc.workspace_status(conv_ws) != dc.OK or dc.async_status() != dc.OK:
                 raise RuntimeError("device-side wait timed out while timing span (%d, %d)" % (i, j))
             us[i][j] = t_us
             T[i][j] = max(1, int(math.ceil(t_us / unit_us)))

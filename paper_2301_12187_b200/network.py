@@ -301,8 +301,9 @@ class CompressedNetwork:
         return self.graph
 
     def status(self):
-        """DC_OK unless a bounded device-side wait ran out in any launch so far."""
-        st = dc.workspace_status(self.conv_ws)
+        """DC_OK unless a bounded device-side wait ran out in any launch so far.  (Merges and depthwise layers have no workspace of
+        their own to say so: a wait of theirs counts from wherever on this device it was launched.)"""
+        st = max(dc.workspace_status(self.conv_ws), dc.async_status())
         for op in self.ops:
             if op.kind == "block":
                 st = max(st, dc.workspace_status(op.ws))

@@ -57,6 +57,30 @@ def test_a_wait_that_runs_out_is_reported_once_and_the_workspace_stays_usable():
     assert_close(y.float().cpu().numpy().astype(np.float64).transpose(0, 3, 1, 2), ref, 2e-2)
 
 
+@pytest.mark.parametrize("which", [0, 1, 2])       # depthwise stencil, merges of 3x3 pairs, merges as a product
+def test_a_wait_that_runs_out_without_a_workspace_is_reported_once(which):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_12187_b200 import dc
+    from paper_2301_12187_b200.network import CompressedNetwork
+    net = I.mobilenet_v2(seed=0, batch=1)
+    cn = CompressedNetwork(net, *I.plan_spans(net, seed=0))
+    assert dc.async_status() == dc.OK and cn.status() == dc.OK
+    dc.selftest_flagged_wait(which, 2000)
+    assert dc.async_status() == dc.ERR_TIMEOUT
+    assert dc.async_status() == dc.OK and dc.dwconv_status() == dc.OK             # reported once, then clear
+    dc.selftest_flagged_wait(which, 2000)
+    dc.selftest_flagged_wait((which + 1) % 3, 2000)                               # both are told at once
+    assert cn.status() == dc.ERR_TIMEOUT
+    assert cn.status() == dc.OK
+    cn.merge()
+    assert cn.status() == dc.OK
+    for bad, limit in ((3, 1000), (-1, 1000), (which, 0), (which, 100001)):
+        with pytest.raises(dc.DcError) as e:
+            dc.selftest_flagged_wait(bad, limit)
+        assert e.value.status == dc.ERR_INVALID_ARG
+
+
 def test_selftest_argument_errors():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
