@@ -304,15 +304,6 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
         for (int t = 0; t < 4; ++t)
 #pragma unroll
           for (int j = 0; j < 8; ++j) v[t][j] = lds_f(f[t] + (uint32_t)(j * 36));
-        // The next load comes while these are cut.  Nothing keeps the compiler from moving a read behind an arrival (it did, some of
-        // the last ones, and one run in three had sums with the next step's values), so who arrives depends on all of them.
-        uint32_t all = 0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) all ^= __float_as_uint(v[t][j]);
-        const bool odd = __ballot_sync(0xffffffffu, all == 0x9E3779B9u) == 0xffffffffu;
-        if (lane == (odd ? 1 : 0)) mbar_arrive(&bar[kREmpty + pair]);
         // half is cut before the slot is free (all of it would spill): what is behind the wait stands between two steps' instructions
         uint4 h[2], mi[2], l[2];
         bf16_terms8(v[0], h[0], mi[0], l[0]);
@@ -331,7 +322,10 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
         }
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bar[kAFull + pair]);
+        // The operands' slot is given back here, behind the stores that need what was read from it.  Given back before the cut, with
+        // the values in registers, it was read too late: the compiler reads shared memory again where a value is used, or moves a
+        // read behind the arrival, __syncwarp() or not (single channels of the next step in some rows, of a CTA's later tiles).
+        if (lane < 2) mbar_arrive(&bar[lane ? kREmpty + pair : kAFull + pair]);
       }
       if (p.resident && last_of(item)) pb ^= 1u;
     }

@@ -1306,6 +1306,70 @@ def test_3x3_after_3x3_by_bf16_terms_as_a_piece(dc):
                     (dc.BF16, dc.F32))
 
 
+def whole_numbers(seed, shape, top):
+    return np.random.default_rng(seed).integers(-top, top + 1, shape).astype(np.float32)
+
+
+@pytest.mark.parametrize("kind,a,c,o", [
+    ("33", 256, 256, 256),                     # 3x3 pairs: up to five tiles a CTA, columns' terms that stay
+    ("33", 320, 384, 256),                     # columns' terms cut again for every tile
+    ("33", 168, 168, 168),                     # two tiles a CTA
+    ("block", 160, 960, 160),                  # a slot's second use is the other team's step
+    ("block", 200, 928, 200), ("block", 252, 700, 300), ("block", 96, 576, 96),
+    ("pair", 960, 320, 1280), ("pair", 320, 1280, 320), ("pair", 72, 1500, 72),
+])
+def test_merges_by_bf16_terms_of_whole_numbers_are_exact_every_time(dc, kind, a, c, o):
+    """Sums of whole numbers below 2 ** 24 are exact in any order, so one operand that a step reads too early, too late or from another
+    step shows, however small its share.  Many runs, with other kernels between them."""
+    mk = I.make_layer
+    if kind == "33":
+        specs = [mk(96, 0, a, c, 3, 1, 1, with_bn=False), mk(96, 1, c, o, 3, 1, 1, with_bn=False)]
+    else:
+        specs = [mk(96, 0, a, c, 1, 1, 0, with_bn=False), mk(96, 2, c, o, 1, 1, 0, with_bn=False)]
+        if kind == "block":
+            specs.insert(1, mk(96, 1, c, c, 3, 1, 1, depthwise=True, with_bn=False))
+    for i, s in enumerate(specs):
+        s.weight[...] = whole_numbers(a + i, s.weight.shape, 8)
+    layers = [dc.DeviceLayer(s) for s in specs]
+    g, ws_bytes = dc.merge_query(layers, [])
+    wm, bm = torch.empty((g.c_out, g.c_in, g.k, g.k), device="cuda"), torch.empty(g.c_out, device="cuda")
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
+    w1, w2 = layers[0].weight.double(), layers[-1].weight.double()
+    if kind == "33":
+        ref = torch.zeros(wm.shape, dtype=torch.float64, device="cuda")
+        for t in range(9):
+            u, v = t // 3, t % 3
+            ref[:, :, u:u + 3, v:v + 3] += torch.einsum("oc,cixy->oixy", w2[:, :, u, v], w1)
+    else:
+        taps = layers[1].weight.double().reshape(c, 9) if kind == "block" else torch.ones(c, 1, dtype=torch.float64, device="cuda")
+        ref = torch.einsum("oc,ct,ci->oit", w2[:, :, 0, 0], taps, w1[:, :, 0, 0]).reshape(wm.shape)
+    assert ref.abs().max() < 2 ** 24
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(60):
+        wm.fill_(-0.5)
+        dc.merge_chain(layers, [], wm, bm, None, dc.F32, ws)
+        wrong += (wm.double() != ref).sum()
+    assert int(wrong) == 0 and dc.async_status() == dc.OK
+
+
+@pytest.mark.parametrize("n,h,w,ci,co,k,s", [(32, 28, 28, 32, 32, 5, 1), (3, 97, 97, 160, 72, 3, 2), (4, 61, 59, 64, 96, 3, 1), (128, 14, 14, 576, 96, 1, 1),
+                                             (8, 14, 14, 384, 64, 3, 1), (2, 41, 43, 96, 112, 5, 2)])
+def test_fp32_convs_by_bf16_terms_of_whole_numbers_are_exact_every_time(dc, n, h, w, ci, co, k, s):
+    g = dc.geom(ci, co, 1, k, s, k // 2)
+    assert dc.conv_kernel_name(n, h, w, g, dc.F32) == "k_conv_f32_tc"
+    x, wf = (torch.from_numpy(whole_numbers(ci, d, 12)).cuda() for d in ((n, h, w, ci), (co, ci, k, k)))
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(wf, g, dc.F32, packed)
+    ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), wf.double(), None, s, k // 2).permute(0, 2, 3, 1)
+    ws, y = torch.zeros(dc.conv_workspace_bytes(), dtype=torch.uint8, device="cuda"), torch.empty(ref.shape, device="cuda")
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(60):
+        y.fill_(-0.5)
+        dc.conv_forward(x, g, packed, None, dc.ACT_IDENTITY, None, y, ws)
+        wrong += (y.double() != ref).sum()
+    assert int(wrong) == 0 and dc.workspace_status(ws) == dc.OK
+
+
 @pytest.mark.parametrize("algo", ["auto", "steps", "piece"])
 @pytest.mark.parametrize("a,c,o", [(64, 4104, 64), (128, 4100, 130)])
 def test_3x3_after_3x3_with_more_channels_between_than_the_tensor_core_takes(dc, algo, a, c, o):
