@@ -1,6 +1,6 @@
 // BN folding, composition of a run of convolutions into one convolution, and weight repacking.
-// fp32 FMA arithmetic on CUDA cores (the merged weights must match an fp64 evaluation of the same formula to 1e-5 relative; large
-// 3x3 pairs go to the tensor core in exact terms, merge_tc.cu).
+// fp32 arithmetic (the merged weights must match an fp64 evaluation of the same formula to 1e-5 relative): FMAs on CUDA cores here; large 3x3
+// pairs (merge_tc.cu), blocks and 1x1 pairs (merge_product_tc.cu) as products on the tensor core, operands in exact bf16 terms.
 #include <vector>
 
 #include "merge_parts.cuh"
@@ -1707,18 +1707,19 @@ static void launch_compose33_form(const Compose33 &a, const BlockDelivery &dv, c
   status.note(dc_launch_pdl(k_compose33<W>, dim3(a.gi * a.go + a.go + zero_ctas(dv, mg, W * 32)), dim3(W * 32), P3Form<W>::BYTES, st, a, dv));
   status.launched();
 }
-// By estimates of both in microseconds, fitted to 82 pairs of 32 to 512 channels timed on either side (on the tensor core 3 % off, by
-// FMAs 13 %): of the 82 this line sends 31 there, together 0.90 of the time on (geometric) average (always the faster one: 0.89), none
-// slower; a line at 1.05 sends 36, two of them 3 % slower.  There a CTA's first tile takes 6.4 us and 0.6 for every 16 channels
-// between, a further one 4.7 us or more: many output and input channels, and enough between them, go there.
+// By estimates of both in microseconds, fitted to 93 pairs of 32 to 1024 channels timed on either side (on the tensor core 4 % off, by
+// FMAs 13 %): of the 93 this line sends 35 there, together 0.891 of the time on (geometric) average over all (always the faster one:
+// 0.881), none slower; a line at 1.0 sends 40, two of them up to 8 % slower.  There a CTA's first tile takes 6.5 us and 0.6 for every 16
+// channels between, a further one 4.9 us or more: many output and input channels, and enough between them, go there.  64 channels between
+// and fewer stay: chains of FMAs so short are nearer to 64 bits for weights of one sign (0.76e-7, there up to 1.17e-7; the one pair of the 93
+// that loses time by it: 144 -> 64 -> 200, 13.6 us there and 15.2 here).
 static bool compose33_on_tensor_core(int c0, int c1, int c2) {
   const int n_sm = dc_sm_count(), steps = dc_div_up(c1, 64) * 4, tiles = dc_div_up(c0, 8) * dc_div_up(c2, 8), most = dc_div_up(tiles, n_sm);
-  const double further = steps > 16 ? 0.57 * steps : (steps > 7 ? 2.5 + 0.3 * steps : 4.7);
-  const double tc = 6.4 + 0.6 * steps + (dc_div_up(dc_div_up(c2, 14) * dc_div_up(c0, 8), n_sm) - 1) * further;
+  const double further = steps > 16 ? 0.58 * steps : (steps > 7 ? 2.4 + 0.33 * steps : 4.9);
+  const double tc = 6.5 + 0.585 * steps + (dc_div_up(dc_div_up(c2, 14) * dc_div_up(c0, 8), n_sm) - 1) * further;
   const double fma = 4.0 + most * c1 * (most > 1 || 2 * tiles <= n_sm ? 0.042 : 0.063);
-  return tc < 0.95 * fma;
+  return c1 > 64 && tc < 0.95 * fma;
 }
-
 
 // Four warps a tile, four tiles to an SM at once, except where the tiles of the SM with the most of them fill whole rounds of two
 // better than of four: one or two of them (136 -> 136 -> 136: 25.6 us by four warps, 17.8 by eight), or three or five with a
@@ -1762,10 +1763,9 @@ static void launch_block33_form(TiledBlocks &tb, const BlockDelivery &dv, const 
   status.note(dc_launch_pdl(k_merge_block33<IT, W>, dim3(grid), dim3(W * 32), grid <= dc_sm_count() ? alone : ring, st, tb, dv));
   status.launched();
 }
-// A single block goes to the tensor core where an estimate says so: of 250 drawn blocks of 40 to 320 channels in and 160 to 1280 hidden
-// ones 130, in 0.74 of the time on (geometric) average, none slower.  (The line: of the 67 that the estimates were fitted to it sends
-// 33, none slower, at 1.0 36, one of them 9 % slower.)  160 -> 960 -> 160 20.0 us and
-// 13.9, 200 -> 928 -> 200 39.4 and 17.5, 64 -> 1168 -> 64 17.5 and 10.7, 96 -> 576 -> 96 11.1 and 9.9; what 24 -> 144 -> 24 takes there,
+// A single block goes to the tensor core where an estimate says so: of 166 drawn blocks of 40 to 320 channels in and 160 to 1280 hidden
+// ones 102, in 0.72 of the time on (geometric) average, two slower, by 2 and 5 %.  160 -> 960 -> 160 20.0 us and
+// 14.3, 200 -> 928 -> 200 39.4 and 17.4, 64 -> 1168 -> 64 17.5 and 11.5, 96 -> 576 -> 96 11.2 and 10.5; what 24 -> 144 -> 24 takes there,
 // 8.2 us, most of it the start and the end of a launch, is more than here, 6.1.
 static bool block33_on_tensor_core(int c0, int c1, int c2, int run, int most16, int most24, int form) {
   const double fma = form == 0   ? 4.07 + 1.69 * (most16 - 1) + c1 / 8.0 * (0.0692 * most16 + 0.0306 * dc_div_up(most16, 2))
@@ -2009,9 +2009,8 @@ static dc_status merge_walk(const dc_layer *layers, int n, const dc_residual *re
     }
     a.gi = dc_div_up(a.c0, bi);
     a.go = dc_div_up(a.c2, bo);
-    // The tensor core by estimates as well: of 131 drawn pairs of 40 to 1280 channels 50, in 0.63 of the time on (geometric) average, one
-    // slower, by 3 %.
-    // 960 -> 320 -> 1280 30.7 us here and 21.7 there, 320 -> 1280 -> 320 25.4 and 13.9, 1024 -> 256 -> 1024 31.4 and 17.4.
+    // The tensor core by estimates as well: of 57 drawn pairs of 40 to 1280 channels 29, in 0.63 of the time on (geometric) average, none
+    // slower.  960 -> 320 -> 1280 30.5 us here and 22.0 there, 320 -> 1280 -> 320 24.9 and 14.3, 1024 -> 256 -> 1024 30.9 and 17.7.
     const int most = dc_div_up(a.gi * a.go, n_sm), run = a.c1 / 4;           // channels of a group's sums, at most half of them
     const double fma = bo == 64   ? 4.82 + a.c1 * (0.0185 * most + 0.0705 * dc_div_up(most, 3))
                        : bo == 48 ? 5.2 + a.c1 * (0.0072 * most + 0.06 * dc_div_up(most, 3))

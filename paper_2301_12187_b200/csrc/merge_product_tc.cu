@@ -15,9 +15,10 @@
 //
 // An infinity or a NaN among the weights makes NaN of results: such a result is computed again by FMAs.
 //
-// 160 -> 960 -> 160 19.7 us by FMAs (k_merge_block33), here 13.9; 200 -> 928 -> 200 39.4 -> 17.5; 960 -> 320 -> 1280 30.4 us (k_merge_11) ->
-// 21.7; 320 -> 1280 -> 320 25.4 -> 13.9; small ones are left to the FMAs (24 -> 144 -> 24 6.1, here 8.2).  Of 160 channels' 20 thousand
-// cycles the first weights and scales take 3, the twelve steps 8, their instructions 2 more, the meeting 3 and the shares 2.
+// 160 -> 960 -> 160 19.7 us by FMAs (k_merge_block33), here 14.3; 200 -> 928 -> 200 39.4 -> 17.4; 960 -> 320 -> 1280 30.4 us (k_merge_11) ->
+// 22.0; 320 -> 1280 -> 320 25.4 -> 14.3; small ones are left to the FMAs (24 -> 144 -> 24 6.1, here 8.2).  Of 160 channels' 20 thousand
+// cycles the first weights and scales take 3, the twelve steps 8, their instructions 2 more, the meeting 3 and the shares 2 (with two
+// sums of the products of the high terms, 13.9).
 // Everything that runs once costs its instructions' way from memory: a third of the warps' time goes to that and to
 // branches.  On the way: shares of a step dealt out over the warps by number 16.2, the same rows for each warp 14.3, one team (two steps at a time) 13.9,
 // the others' sums read from their shared memory instead of sent 14.3; terms by packed subtractions the same.
@@ -35,6 +36,8 @@ constexpr int kMaxSlots = 16, kMaxSplit = 8;
 constexpr int kSmemMax = 225 * 1024;             // asked for always: a CTA holds all of its SM's tensor memory, and clusters that did so
                                                  // beside one another on an SM could wait for each other's
 
+// sums of the products of the high terms in the fine form: what tensor memory holds beside those of the other products
+__host__ __device__ constexpr int sums_of(int nt) { return 512 / nt - 2; }
 __host__ __device__ constexpr int threads_of(int nt) { return 2 * (8 + nt / 16) * 32 + 64; }      // two teams that cut, two warps that issue
 
 // The waits of a step on its slot, which a plan uses twice at most.  A barrier's wait tells two neighbouring phases apart and no more, so
@@ -65,7 +68,7 @@ struct Shape {
 struct Plan {
   int n_tiles, split, steps, total_steps, slots; // a CTA's steps of 16 channels, all steps
   int off_d, off_q, off_parts;
-  int fine;                                      // four sums of the products of the high terms instead of two
+  int fine;                                      // the products of the high terms in sums_of() sums instead of two
 };
 
 // one result by FMAs, before the last layer's scale: where the terms gave NaN
@@ -98,6 +101,7 @@ __global__ void __launch_bounds__(threads_of(NT), 1)
 k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ BlockDelivery dv, const __grid_constant__ Plan p, DcWsHeader *ws) {
   using S = Shape<KIND>;
   constexpr int T = S::T, OT = S::OT, UNIT = S::UNIT, kStep = kStepA + NT * 96;
+  constexpr int kSums = sums_of(NT);
   constexpr int kTeam = 8 + NT / 16, kWarpsCut = 2 * kTeam, kIssue = kWarpsCut, kCutThreads = kWarpsCut * 32, kThreads = threads_of(NT);
   static_assert(NT % 16 == 0 && 6 * NT <= 512, "tile");
   extern __shared__ __align__(128) uint8_t smem[];
@@ -282,7 +286,7 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
         }
         __syncwarp();
       }
-    } else {                                     // one warp issues h h, every fourth step into the same sums, the other the rest
+    } else {                                     // one warp issues h h, every kSums-th step into the same sums, the other the rest
 #pragma unroll 1
       for (int s = 0; s < steps; s += 4) {
         const int mine = s + (lane & 3);
@@ -294,11 +298,11 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
           const uint64_t ad = a_hi | at, bd = b_hi | (at + (kStepA >> 4));
           if (elect_one()) {
             if (odd == 0) {
-              umma_bf16(tmem + (uint32_t)((st - s) * NT), ad, bd, i1, s > 0);
+              umma_bf16(tmem + (uint32_t)(st % kSums * NT), ad, bd, i1, st >= kSums);
             } else {
-              umma_bf16(tmem + 4 * NT, ad, bd + NT, i2, st > 0);
-              umma_bf16(tmem + 4 * NT, ad + (2 * kPitchA >> 4), bd, i2, 1u);
-              umma_bf16(tmem + 5 * NT, ad + (4 * kPitchA >> 4), bd, i1, 1u);
+              umma_bf16(tmem + kSums * NT, ad, bd + NT, i2, st > 0);
+              umma_bf16(tmem + kSums * NT, ad + (2 * kPitchA >> 4), bd, i2, 1u);
+              umma_bf16(tmem + (kSums + 1) * NT, ad + (4 * kPitchA >> 4), bd, i1, 1u);
             }
             umma_commit(&bar[kMaxSlots + slot]);
             if (st + 1 == steps) umma_commit(&bar[2 * kMaxSlots]);
@@ -318,19 +322,32 @@ k_merge_product_tc(const __grid_constant__ Product a, const __grid_constant__ Bl
 #pragma unroll 1
     for (int col = (warp >> 2) * 8; col < NT && ok; col += (kWarpsCut - quarter + 3) / 4 * 8) {
       float sum[8] = {};
+      if (p.fine) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        uint32_t x[3][8];
+        for (int h = 0; h < kSums + 2; h += 2) {
+          uint32_t x[2][8];
+          tmem_ld8(drow + (uint32_t)(h * NT + col), x[0]);
+          tmem_ld8(drow + (uint32_t)((h + 1) * NT + col), x[1]);
+          tmem_ld_wait();
 #pragma unroll
-        for (int g = 0; g < 3; ++g) tmem_ld8(drow + (uint32_t)((3 * h + g) * NT + col), x[g]);
-        tmem_ld_wait();
+          for (int g = 0; g < 2; ++g)            // a sum of no step holds anything
+            if (h + g < kSums && h + g >= steps)
 #pragma unroll
-        for (int g = 0; g < 3; ++g)              // a sum of no step holds anything
-          if (p.fine ? 3 * h + g < 4 && 3 * h + g >= steps : h > 0 && steps == 1)
+              for (int j = 0; j < 8; ++j) x[g][j] = 0u;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) x[g][j] = 0u;
+          for (int j = 0; j < 8; ++j) sum[j] += __uint_as_float(x[0][j]) + __uint_as_float(x[1][j]);
+        }
+      } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) sum[j] += __uint_as_float(x[0][j]) + (__uint_as_float(x[1][j]) + __uint_as_float(x[2][j]));
+        for (int h = 0; h < 2; ++h) {
+          uint32_t x[3][8];
+#pragma unroll
+          for (int g = 0; g < 3; ++g) tmem_ld8(drow + (uint32_t)((3 * h + g) * NT + col), x[g]);
+          tmem_ld_wait();
+          if (h > 0 && steps == 1) break;        // nor has the second warp any here
+#pragma unroll
+          for (int j = 0; j < 8; ++j) sum[j] += __uint_as_float(x[0][j]) + (__uint_as_float(x[1][j]) + __uint_as_float(x[2][j]));
+        }
       }
       if (m < S::ROWS) {
         float *unit = to + col / 8 * (OT * UNIT);
@@ -475,9 +492,12 @@ double estimate_us(int nt, int split, int steps, int fine, int rounds, double bu
 }
 
 // The columns of a tile and the parts of its reduction with the smallest estimate, in us; 0: outside the range.  `run`: channels that
-// one sum of the FMA kernel goes through.  A sum of the tensor core's takes a tenth as many steps at most: its error is then
-// the smaller one (2-norm against 64 bits, of 130 drawn blocks 0.96 of the FMAs' at most and 0.82 on average, of 50 pairs 0.64 and
-// 0.49; with an eighth one block in a hundred was above, up to 1.11).
+// one sum of the FMA kernel goes through.  The tensor core cuts its sums instead of rounding them, so a sum of products of high terms
+// takes a tenth as many steps at most, and from five steps on there are as many sums as tensor memory holds (0.3 to 0.8 us for 0.6 to
+// 0.9 of the error).  Against 64 bits (2-norm), of 166 drawn blocks and 57 pairs the 102 and 29 that go there: weights of both
+// signs 0.73 of the FMAs' error on average and 0.87 at most, pairs 0.42 and 0.60; weights of one sign, where what is cut off adds up, 1.19 and
+// 1.79 (1.56e-7 at most; FMAs have up to 2.5e-7 for weights of both signs), pairs 0.66 and 0.90.  At most three steps a sum would be 1.44
+// instead of 1.79, for 0.757 instead of 0.716 of the FMAs' time.
 template <int KIND>
 double make_plan(int c0, int c1, int c2, int run, Plan *best, int *best_nt) {
   using S = Shape<KIND>;
@@ -489,8 +509,8 @@ double make_plan(int c0, int c1, int c2, int run, Plan *best, int *best_nt) {
     for (int split = 1; split <= kMaxSplit; ++split) {
       const int steps = dc_div_up(total, split), step_bytes = kStepA + nt * 96;
       if ((split - 1) * steps >= total || steps > 2 * (8 + nt / 16)) continue;                     // a thread to a channel
-      const int fine = dc_div_up(steps, 2) * 10 > run;
-      if (fine && dc_div_up(steps, 4) * 10 > run) continue;
+      const int fine = steps > 4;
+      if (dc_div_up(steps, fine ? sums_of(nt) : 2) * 10 > run) continue;
       const int scales = steps * 16 * 4 * (KIND == kProductBlock ? 9 : 1), sums = S::ROWS * nt * 4;
       const int parts = split > 1 ? split * dc_div_up(S::OT * (nt / 8), split) * S::UNIT * 4 : 0;
       int slots = (kSmemMax - 256 - scales - steps * 64) / step_bytes;

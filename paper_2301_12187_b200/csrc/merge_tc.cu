@@ -3,25 +3,29 @@
 // W'[o][i][t] = sum_c sum_{t1 + t2 = t} W2[o][c][t2] W1~[c][i][t1]: the product Z of the matrix W2 with rows (o, t2) and the matrix W1
 // with columns (i, t1), reduction over c, has none of the structural zeros that a gathered product has, and the 25 taps of a pair
 // are sums of its 81 elements Z[o, t2][i, t1].  A tile is 14 output channels (126 of 128 rows) x 8 input channels (72 columns).
-// A value is three bf16 terms, six products of them are above 2^-24, and they are three instructions a step of 16 channels (A_h x [h m l],
-// A_m x [h m], A_l x [h], sums of hh, hm + mh and the rest in column groups of their own) as in conv_f32_tc.cu; every eight steps the
-// sums are read out and added in fp32.  Error against 64 bits (2-norm) 256 channels: 1.0e-7, by FMAs 2.3e-7.
+// A value is three bf16 terms, six products of them are above 2^-24, and they are four instructions a step of 16 channels: A_h x h into
+// sums of hh, A_h x [m l], A_m x [h m] and A_l x h into sums of hm + mh and of the rest.  The tensor core cuts its sums instead of
+// rounding them, so those of hh are read out every four steps and added in fp32; the others, 2^8 times smaller, every sixteen.
+// Error against 64 bits (2-norm), 256 channels between: weights of both signs 1.2e-7, by FMAs 2.3e-7; of one sign, where what is cut off adds up,
+// 1.2e-7 and 0.96e-7.  (512 channels 1.3e-7 and 3.2e-7, 1.2e-7 and 1.2e-7.)
 //
 // Warps: one loads the second layer by TMA, eight cut operands into terms, in four pairs that take the steps in turn (a pair has four
 // steps' time for one: a warp alone on its scheduler needs it), one issues, four add up, take the 25 taps together through shared
-// memory and deliver the result while the next tile is multiplied.  The terms of a tile's columns stay in shared memory for all tiles
-// below one another where they fit (256 channels between); CTAs own runs of such tiles.  The warps that cut compute the bias
-// behind their last tile.  What bounds it is no unit (256 channels: tensor pipe 0.25, issue slots 0.42, shared memory 0.48 and the
-// instructions' operands) but the way of a step through its pair of warps: operands there, read, cut, slot free, written, multiplied,
-// 2.7 thousand cycles with four on their way at once, and a slot of operands and terms more has no room beside the columns' terms.
+// memory and deliver the result while the next tile is multiplied: the four sums of hh hold sixteen steps.  The terms of a tile's columns stay in
+// shared memory for all tiles below one another where they fit (256 channels between); CTAs own runs of such tiles.  The warps that cut
+// compute the bias behind their last tile.  What bounds it is no unit (the counters are in profiles/) but the way of a step through its
+// pair of warps: operands there, read, cut, slot free, written, multiplied, 2.7 thousand cycles with four on their way at once, and a
+// slot of operands and terms more has no room beside the columns' terms.
 //
 // An infinity or a NaN among the weights makes NaN of results: such a result is computed again by FMAs.
 //
-// 256 -> 256 -> 256 75.6 us by FMAs (k_compose33), here 46; 512 551 -> 288; 200 -> 248 -> 80 23.6 -> 21.6; 64 6.7 -> 8.3 (left to FMAs).
-// A tile of 256 channels takes 12 thousand cycles: the taps, the scale, the result and its packed copy 9 of them in the adding warps (they run
-// once a tile, from a cold instruction cache), its sixteen steps 8.6.  On the way: cut by nine warps together 76, by pairs 54, operands
-// asked for again before they are cut 47, one issuing warp that waits for two steps side by side 45.  80 columns a term instead of 72 0.5 to 0.9 %
-// more; eight adding warps 44.6, but 512 channels 296; steps cut by four warps 51, by two teams with two slots each 53.
+// 256 -> 256 -> 256 75.6 us by FMAs (k_compose33), here 47; 512 551 -> 289; 104 -> 208 -> 136 21.0 -> 16.1; 64 6.7 -> 9.0 (left to FMAs).
+// The taps, the scale, the result and its packed copy take 9 thousand cycles a tile in the adding warps (they run once a tile, from a cold
+// instruction cache).  On the way: cut by nine warps together 76, by pairs 54, operands asked for again before they are cut 47 (not sound, see
+// there; without, no slower any more), one issuing warp that waits for two steps side by side 45.  80 columns a term instead of 72 0.5 to
+// 0.9 % more; eight adding warps 44.6, but 512 channels 296; steps cut by four warps 51, by two teams with two slots each 53.  All sums read
+// out every eight steps, two sets of them: 45.0, 512 channels 279, but errors of 1.6e-7 and, for weights of one sign, 2.0e-7; those of
+// hh every two steps: 53.2 and 298, errors of 1.1e-7 and 0.9e-7 (the adding warps then fall behind: four such sums hold half a tile).
 #include "merge_parts.cuh"
 #include "tc_ptx.cuh"
 
@@ -31,9 +35,11 @@ using namespace tc;
 __device__ unsigned int g_merge_status;          // DC_ERR_TIMEOUT once a wait of this kernel ran out in a launch without a workspace header
 
 constexpr int kO = 14, kI = 8, kRows = kO * 9, kCols = kI * 9;
-constexpr int kRowsB = 224;                      // of the columns' terms of 8 channels: 72 of each, and 8 that only make up the instruction's 224 columns
+constexpr int kRowsB = 3 * kCols;                // of the columns' terms of 8 channels
 constexpr int kWarpsAcc = 4, kPairs = 4, kWarpsCut = 2 * kPairs, kLoad = kWarpsAcc + kWarpsCut, kIssue = kLoad + 1, kThreads = (kIssue + 1) * 32;
-constexpr int kChunk = 8;                        // steps of 16 channels between two read-outs
+constexpr int kChunk = 4, kLong = 16;            // steps of 16 channels between two read-outs of the sums of hh, and of the others
+constexpr int kSums = 4, kPitchSum = 80;         // sums of hh and their columns (8 of them only make up an instruction); then those of the others
+constexpr int kColM = kSums * kPitchSum, kColR = kColM + kCols;
 constexpr int kPitchA = 128 * 16;                // bytes between the halves of a step's 16 channels
 constexpr int kStepA = 6 * kPitchA, kStepB = 2 * kRowsB * 16, kRawA = kO * 144 * 4;
 constexpr int kPitchZ = kCols / 2 + 1;           // floats of a row of Z, four input channels at a time
@@ -50,7 +56,7 @@ struct Params33 {
 
 // a pair of warps owns a slot of operands (R), of terms (A) and, of the columns' terms (B), every fourth
 enum { kRFull = 0, kREmpty = kPairs, kAFull = 2 * kPairs, kAEmpty = 3 * kPairs, kBFull = 4 * kPairs, kBEmpty = kBFull + kMaxB,
-       kDFull = kBEmpty + kMaxB, kDEmpty = kDFull + 2, kBars = kDEmpty + 2 };
+       kDFull = kBEmpty + kMaxB, kMFull = kDFull + kSums, kDEmpty = kMFull + 1, kMEmpty = kDEmpty + kSums, kBars = kMEmpty + 1 };
 
 // a load that stays where it is written
 __device__ __forceinline__ float ask(const float *p) {
@@ -120,13 +126,12 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
   if (warp < kWarpsAcc) {
     // ---------------------------------------------------------------- sums, taps, delivery
     const uint32_t drow = tmem + ((uint32_t)(warp * 32) << 16);
-    const int chunks = (p.steps + kChunk - 1) / kChunk;
     float *z = reinterpret_cast<float *>(smem + p.off_z);
     const bool last = dv.mode >= 0, special = a.first.ident || a.second.ident || (last && dv.ident);
     // where a bf16 chunk goes: rows of a tap's chunk plane, except in orders that hold taps or pixels in the rows
     const bool rows = dv.mode == 2 && !dv.ko.fold && !dv.ko.pair;
     const int po = (tid & 63) >> 2, pi = tid & 3, side = tid >> 6;               // this thread's pair of channels, when taps are summed
-    uint32_t fl = 0;
+    uint32_t fl = 0, ml = 0;
     bool ok = true;
 #pragma unroll 1
     for (int item = begin; item < end && ok; ++item) {
@@ -140,24 +145,44 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
 #pragma unroll
       for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
 #pragma unroll 1
-      for (int s = 0; s < chunks; ++s, ++fl) {
-        const uint32_t b = fl & 1u;
-        if (!(ok = wait(kDFull + (int)b, (fl >> 1) & 1u))) break;
+      for (int s = 0; s < p.steps; s += kChunk, ++fl) {
+        const uint32_t b = fl % kSums;
+        if (!(ok = wait(kDFull + (int)b, (fl / kSums) & 1u))) break;
         tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < kCols; c += 8) {
+        for (int c = 0; c < kCols; c += 24) {
           uint32_t v0[8], v1[8], v2[8];
-          const uint32_t at = drow + b * kRowsB + c;
+          const uint32_t at = drow + b * kPitchSum + c;
           tmem_ld8(at, v0);
-          tmem_ld8(at + kCols, v1);
-          tmem_ld8(at + 2 * kCols, v2);
+          tmem_ld8(at + 8, v1);
+          tmem_ld8(at + 16, v2);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[c + j] += __uint_as_float(v0[j]) + (__uint_as_float(v1[j]) + __uint_as_float(v2[j]));
+          for (int j = 0; j < 8; ++j) {
+            acc[c + j] += __uint_as_float(v0[j]);
+            acc[c + 8 + j] += __uint_as_float(v1[j]);
+            acc[c + 16 + j] += __uint_as_float(v2[j]);
+          }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bar[kDEmpty + b]);
+        if (s % kLong != kLong - kChunk && s + kChunk < p.steps) continue;
+        if (!(ok = wait(kMFull, ml & 1u))) break;
+        ++ml;
+        tc_fence_after();
+#pragma unroll
+        for (int c = 0; c < kCols; c += 8) {
+          uint32_t v0[8], v1[8];
+          tmem_ld8(drow + kColM + c, v0);
+          tmem_ld8(drow + kColR + c, v1);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[c + j] += __uint_as_float(v0[j]) + __uint_as_float(v1[j]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar[kMEmpty]);
       }
       if (!(ok = bar_all(3, 128, ok))) break;    // the four warps agree before they meet below
       if (rows) {                                // read behind the barriers below
@@ -358,24 +383,26 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
   } else {
     // ---------------------------------------------------------------- issue: two steps at a time, their barriers waited for side by side
     const uint32_t id0 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
-    constexpr uint32_t i3 = (kRowsB / 8) << 17, i2 = (2 * kCols / 8) << 17, i1 = (80 / 8) << 17;
+    constexpr uint32_t i2 = (2 * kCols / 8) << 17, i1 = (kPitchSum / 8) << 17;
     const uint64_t hi = (uint64_t)((128u >> 4) | (1u << 14)) << 32;
     const uint64_t a_hi = hi | ((uint64_t)(kPitchA >> 4) << 16), b_hi = hi | ((uint64_t)kRowsB << 16);
     const uint32_t sm16 = sm >> 4, b16 = (sm + (uint32_t)p.off_b) >> 4;
     int as = 0, bs = 0;
-    uint32_t pa = 0, pb = 0, fl = 0;
+    uint32_t pa = 0, pb = 0, fl = 0, ml = 0;
     bool ok = true;
 #pragma unroll 1
     for (int item = begin; item < end && ok; ++item) {
       const bool first = first_of(item), last = last_of(item);
 #pragma unroll 1
       for (int s = 0; s < p.steps; s += 2) {
-        const bool opens = s % kChunk == 0, closes = s % kChunk == kChunk - 2 || s + 2 == p.steps;
-        const uint32_t buf = fl & 1u, d = tmem + buf * kRowsB;
+        const bool opens_h = s % kChunk == 0, closes_h = s % kChunk == kChunk - 2;
+        const bool opens = s % kLong == 0, closes = s % kLong == kLong - 2 || s + 2 == p.steps;
+        const uint32_t buf = fl % kSums, d = tmem + buf * kPitchSum;
         int b = kAFull + as + (lane & 1);
         uint32_t parity = pa;
         if (first && (lane & 2)) { b = kBFull + bs + (lane & 1); parity = pb; }
-        if (opens && lane == 4) { b = kDEmpty + (int)buf; parity = ((fl >> 1) & 1u) ^ 1u; }
+        if (opens_h && lane == 4) { b = kDEmpty + (int)buf; parity = ((fl / kSums) & 1u) ^ 1u; }
+        if (opens && lane == 5) { b = kMEmpty; parity = (ml & 1u) ^ 1u; }
         ok = mbar_wait(&bar[b], parity, abort_flag, ws, 0x210000u | (uint32_t)b);
         __syncwarp();
         if (!(ok = __all_sync(0xffffffffu, ok) != 0)) break;
@@ -386,16 +413,20 @@ k_compose33_tc(const __grid_constant__ CUtensorMap map_w2, const __grid_constant
           for (int q = 0; q < 2; ++q) {
             const uint64_t bd = b_hi | (uint64_t)((bt + q * (kStepB >> 4)) & 0x3FFFu);
             const uint32_t aq = at + q * (kStepA >> 4);
-            umma_bf16(d, a_hi | (uint64_t)(aq & 0x3FFFu), bd, id0 | i3, opens && q == 0 ? 0u : 1u);
-            umma_bf16(d + kCols, a_hi | (uint64_t)((aq + (2 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i2, 1u);
-            umma_bf16(d + 2 * kCols, a_hi | (uint64_t)((aq + (4 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i1, 1u);
+            const uint64_t bm = b_hi | (uint64_t)((bt + q * (kStepB >> 4) + kCols) & 0x3FFFu);       // from the middle terms on
+            umma_bf16(d, a_hi | (uint64_t)(aq & 0x3FFFu), bd, id0 | i1, opens_h && q == 0 ? 0u : 1u);
+            umma_bf16(tmem + kColM, a_hi | (uint64_t)(aq & 0x3FFFu), bm, id0 | i2, opens && q == 0 ? 0u : 1u);
+            umma_bf16(tmem + kColM, a_hi | (uint64_t)((aq + (2 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i2, 1u);
+            umma_bf16(tmem + kColR, a_hi | (uint64_t)((aq + (4 * kPitchA >> 4)) & 0x3FFFu), bd, id0 | i1, 1u);
             umma_commit(&bar[kAEmpty + as + q]);
             if (last) umma_commit(&bar[kBEmpty + bs + q]);
           }
-          if (closes) umma_commit(&bar[kDFull + buf]);
+          if (closes_h) umma_commit(&bar[kDFull + buf]);
+          if (closes) umma_commit(&bar[kMFull]);
         }
         __syncwarp();
-        if (closes) ++fl;
+        if (closes_h) ++fl;
+        if (closes) ++ml;
         as += 2;
         if (as == kPairs) { as = 0; pa ^= 1u; }
         bs += 2;

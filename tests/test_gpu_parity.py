@@ -1301,9 +1301,60 @@ def test_3x3_after_3x3_by_bf16_terms_against_the_oracle(dc, a, c, o, res, codes)
         assert O.rel_l2(wm.cpu().numpy(), W) <= 1.95e-7
 
 
+@pytest.mark.parametrize("kind,a,c,o", [("33", 64, 136, 152), ("33", 256, 256, 256), ("33", 104, 208, 136), ("block", 160, 960, 160),
+                                        ("block", 96, 576, 96), ("block", 200, 928, 200), ("pair", 320, 1280, 320), ("pair", 504, 504, 504)])
+def test_merges_by_bf16_terms_of_weights_of_one_sign(dc, kind, a, c, o):
+    """The tensor core cuts its sums, which adds up where all products have one sign: L steps of a sum lose (L + 1) / 2 x 2 ** -24 of it at
+    0.7 on average over a binade, 1.1e-7 for the four of a 3x3 pair and 1.3e-7 for the five of the widest block here; beside the
+    roundings of FMA kernels, 1e-7.  Weights of both signs: at most 1.7e-7 measured, and 3x3 pairs 1.3e-7 (1.85e-7 or more by FMAs)."""
+    mk = I.make_layer
+    if kind == "33":
+        specs = [mk(97, 0, a, c, 3, 1, 1), mk(97, 1, c, o, 3, 1, 1)]
+    else:
+        specs = [mk(97, 0, a, c, 1, 1, 0), mk(97, 2, c, o, 1, 1, 0)]
+        if kind == "block":
+            specs.insert(1, mk(97, 1, c, c, 3, 1, 1, depthwise=True))
+    for sign in (False, True):
+        if sign:
+            for s in specs:
+                s.weight[...] = np.abs(s.weight)
+        _, wm, _, _ = run_merge(dc, specs, [], packed_dtype=dc.F32)
+        err = O.rel_l2(wm.cpu().numpy(), O.merge_formula(specs, [])[0])
+        assert err <= (1.8e-7 if sign else 1.5e-7 if kind == "33" else 1.9e-7), (sign, err)
+
+
 def test_3x3_after_3x3_by_bf16_terms_as_a_piece(dc):
     _check_delivery(dc, [I.make_layer(87, 0, 120, 200, 3, 1, 1), I.make_layer(87, 1, 200, 136, 3, 1, 1), I.make_layer(87, 2, 136, 16, 1, 1, 0)], [],
                     (dc.BF16, dc.F32))
+
+
+@pytest.mark.parametrize("shape", F32_TC_SHAPES[:8])
+def test_fp32_conv_by_bf16_terms_of_one_sign_and_of_small_values(dc, shape):
+    """Maps behind ReLU6 under weights of one sign, where what the tensor core cuts off adds up: four steps of a sum lose 2.5 x 2 ** -24 x 0.7 =
+    1e-7 of it at most, so no further from 64 bits than FMAs' 0.7e-7 or more by a tenth.  And values as small as terms reach: exact
+    from 2 ** -110 on, below it to within 2 ** -133."""
+    n, h, w, ci, co, k, s, p = shape
+    g = dc.geom(ci, co, 1, k, s, p)
+    assert dc.conv_kernel_name(n, h, w, g, dc.F32) == "k_conv_f32_tc"
+    gen = torch.Generator("cuda")
+    gen.manual_seed(ci * 1000 + co + 1)
+    rnd = lambda *d: torch.randn(d, generator=gen, device="cuda")
+    x, wf = rnd(n, h, w, ci), rnd(co, ci, k, k) * (ci * k * k) ** -0.5
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(dc.conv_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    y = torch.empty((n, (h + 2 * p - k) // s + 1, (w + 2 * p - k) // s + 1, co), device="cuda")
+
+    def err(x, wf, algo):
+        dc.pack_weights(wf, g, dc.F32, packed)
+        dc.conv_forward(x, g, packed, None, dc.ACT_IDENTITY, None, y, ws, algo=algo)
+        ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), wf.double(), None, s, p).permute(0, 2, 3, 1)
+        return ((y.double() - ref).norm() / ref.norm()).item()
+
+    sign = (x * 2).clamp(0, 6), wf.abs()
+    assert err(*sign, dc.ALGO_AUTO) <= min(1.2e-7, 1.1 * err(*sign, dc.ALGO_SIMT))
+    assert err(x * 2.0 ** -104, wf * 2.0 ** 104, dc.ALGO_AUTO) <= 4e-7           # a thousandth of the values is below 2 ** -114
+    assert err(x * 2.0 ** -120, wf * 2.0 ** 104, dc.ALGO_AUTO) <= 2.0 ** -13
+    assert dc.workspace_status(ws) == dc.OK
 
 
 def whole_numbers(seed, shape, top):
