@@ -1357,6 +1357,23 @@ def test_fp32_conv_by_bf16_terms_of_one_sign_and_of_small_values(dc, shape):
     assert dc.workspace_status(ws) == dc.OK
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_fp32_conv_by_bf16_terms_of_maps_that_are_not_finite(dc, value):
+    n, h, w, ci, co, k, s, p = F32_TC_SHAPES[0]
+    g = dc.geom(ci, co, 1, k, s, p)
+    x = torch.full((n, h, w, ci), value, device="cuda")
+    x[1] = 1.0                                     # one image is
+    wf = torch.full((co, ci, k, k), 0.5, device="cuda")
+    wf[3] = -0.5
+    packed = torch.empty(dc.packed_bytes(g, dc.F32), dtype=torch.uint8, device="cuda")
+    dc.pack_weights(wf, g, dc.F32, packed)
+    ws = torch.zeros(dc.conv_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    a, b = (torch.empty((n, h, w, co), device="cuda") for _ in range(2))
+    dc.conv_forward(x, g, packed, None, dc.ACT_IDENTITY, None, a, ws)
+    dc.conv_forward(x, g, packed, None, dc.ACT_IDENTITY, None, b, ws, algo=dc.ALGO_SIMT)
+    assert torch.equal(a.nan_to_num(7.0), b.nan_to_num(7.0)) and bool(torch.isfinite(a[1]).all()) and not bool(torch.isfinite(a[0]).any())
+
+
 def whole_numbers(seed, shape, top):
     return np.random.default_rng(seed).integers(-top, top + 1, shape).astype(np.float32)
 
