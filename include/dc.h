@@ -127,7 +127,9 @@ dc_status dc_packed_bytes(const dc_geom *g, dc_dtype dtype, size_t *bytes);
  * not NULL also the packed copy for packed_dtype (size from dc_packed_bytes).  workspace: device,
  * at least the bytes dc_merge_query reports; it overlaps nothing else.  The outputs may overlap the
  * layers' arrays (which then do not survive the call), not one another.  fp32 arithmetic: FMAs, or on the tensor
- * core products of exact bf16 terms of fp32 values, added up in fp32.  DC_OK says that everything was launched;
+ * core six of the nine products of three bf16 terms of each value (exact from 2^-110 on, smaller values to within 2^-133; what is
+ * left out is below 2^-24 of a product), added up in fp32, short sums of them cut instead of rounded: for weights of both signs the
+ * error against 64 bits is below the FMAs', for weights of one sign up to 1.8 times it, 1.6e-7 of the result (2-norm).  DC_OK says that everything was launched;
  * merges on the tensor core have bounded waits, and dc_async_status tells whether one ran out.
  */
 dc_status dc_merge_chain(const dc_layer *layers, int n_layers, const dc_residual *res, int n_res,
@@ -212,14 +214,18 @@ const char *dc_conv_kernel_name(int n, int h, int w, const dc_geom *g, dc_dtype 
  * `dtype`; w_packed from dc_merge_chain / dc_pack_weights for the same dtype; bias fp32 [c_out]
  * or NULL.  DC_BF16 runs as an implicit GEMM on the tensor cores (fp32 accumulate) when the
  * shape allows (c_in, c_out multiples of 8, stride 1 or 2, ...), else on CUDA cores; DC_F32
- * runs on CUDA cores in fp32.  workspace: device, >= dc_conv_workspace_bytes(), zeroed once by
- * the caller.
+ * runs in fp32 FMAs on CUDA cores or, where that is faster (channels in multiples of 4, stride 1 or 2, k <= 7, enough work),
+ * on the tensor core as products of bf16 terms, as described at dc_merge_chain; infinities and NaN come out as FMAs give
+ * them.  workspace: device, >= dc_conv_workspace_bytes(), zeroed once by the caller.
  */
 dc_status dc_conv_forward(const void *x, int n, int h, int w, const dc_geom *g, const void *w_packed,
                           const float *bias, dc_act act, const void *residual, void *y,
                           dc_dtype dtype, void *workspace, size_t workspace_bytes, dc_stream stream);
 
-/* As dc_conv_forward with the kernel family forced; DC_ERR_UNSUPPORTED if it cannot run the shape. */
+/*
+ * As dc_conv_forward with the kernel family forced; DC_ERR_UNSUPPORTED if it cannot run the shape.  DC_ALGO_TCGEN05 is for DC_BF16;
+ * fp32 layers reach the tensor core through DC_ALGO_AUTO alone, and DC_ALGO_SIMT keeps them on FMAs.
+ */
 dc_status dc_conv_forward_algo(const void *x, int n, int h, int w, const dc_geom *g,
                                const void *w_packed, const float *bias, dc_act act,
                                const void *residual, void *y, dc_dtype dtype, void *workspace,

@@ -197,8 +197,8 @@ static inline void dc_korder_init(KOrder *ko, const dc_geom *g) {
   // which then ran on the CUDA cores.  144 -> 24 1x1, 128 images of 56 x 56 99 us there, 25 by rows; 72 -> 24, 32 of 77 x 80 31 and 12;
   // 112 -> 16 3x3, 104 of 9 x 9 22 and 6; 136 -> 24 5x5, 20 of 69 x 66 87 and 39; 48 -> 24 5x5, one of 44 x 44 58 and 4.9.  Over 97 such
   // layers 0.31 of the time on (geometric) average, one slower, by 2 %.  3x3 layers of 24 outputs and 1x1 layers of 8 keep the
-  // kernels they have, though they would gain as much (152 -> 24 3x3, 50 of 28 x 28 121 and 12): which kernels read their packed
-  // order is held by tests.
+  // kernels they have, though they would gain as much (152 -> 24 3x3, 50 of 28 x 28 121 and 12), and so does 40 -> 32 5x5, which the fold
+  // kernel leaves to the CUDA cores from maps of about 44 x 44 on: which kernels read their packed order is held by tests.
   // 7x7 layers of 24 and 32 channels to at most 24 outputs, which the pair rows do not take either: the fold kernel runs 24 -> 8 at any width,
   // and faster where there is much to do (128 images of 28 x 28 14.2 us there, 25.6 by rows, 31.3 by the general kernel; of 56 x 56 32, 78
   // and 53; one of 14 x 14 6.6, 4.7 and 6.6).  Wider ones go by rows: beyond some width (44 for 32 -> 16) the fold kernel has no room

@@ -1,12 +1,14 @@
 // Dense convolution in fp32 on the tensor core, by operands cut into bf16 terms.
 //
-// An fp32 value is exactly three bf16 terms of 8 significant bits each, so a product of two values is nine products of terms, of
-// which six are above 2^-24: hh, hm, mh, hl, mm, lh.
+// An fp32 value of 2^-110 or more is exactly three bf16 terms of 8 significant bits each (smaller ones are to within 2^-133: the smallest
+// bf16 ends there), so a product of two values is nine products of terms, of which six are above 2^-24: hh, hm, mh, hl, mm, lh.
 // tcgen05.mma multiplies bf16 terms exactly; its fp32 sums are cut instead of rounded, which over a long reduction would cost
 // more than fp32 FMAs do (2.7e-6 of the result after 800 products).  So the sums are kept short and apart: hh, hm + mh and
 // hl + mm + lh have accumulators of their own, and after at most kFlush steps of 16 products they are read out and added to the
 // outputs' sums in registers by ordinary fp32 additions.  Measured against 64 bits on normal values (2-norm): 288 products
-// 0.8e-7, 800 1.0e-7, 2400 1.35e-7, where one chain of FMAs has 3.0e-7, 5.1e-7 and 8.7e-7, eight chains 1.2e-7, 1.9e-7, 3.2e-7.
+// 0.8e-7, 800 1.0e-7, 2400 1.35e-7, where one chain of FMAs has 3.0e-7, 5.1e-7 and 8.7e-7, eight chains 1.2e-7, 1.9e-7, 3.2e-7.  Where all
+// products have one sign, what is cut off adds up: maps behind ReLU6 under weights of one sign, 19 layers, 0.6 to 0.9e-7, 0.28 to 0.84 of
+// k_conv_dense_f32's error, one of them 1.06 of it (20 -> 36 5x5, 0.72e-7).
 //
 // The three groups cost no instruction of their own: the B operand of a step holds the terms of NT output channels one behind
 // the other, [h | m | l], and A_h x [h m l], A_m x [h m], A_l x [h] are three instructions of 3 NT, 2 NT and NT columns whose
@@ -156,8 +158,7 @@ k_conv_f32_tc(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   } else if (tid >= 64 && tid < 64 + n_chunks) {
     const int c = tid - 64;
-    const uint32_t line[4] = {0u, 0u, 0u, 0u};
-    uint4 e = make_uint4((uint32_t)p.chunk_tap[c] << 16, line[0], line[1], line[2]);
+    uint4 e = make_uint4((uint32_t)p.chunk_tap[c] << 16, 0u, 0u, 0u);
     if (p.taps > 1) {
       const unsigned short *l = p.tap_line + p.chunk_tap[c];
       e.x |= (uint32_t)(p.chunk_tap[c + 1] - p.chunk_tap[c]);
@@ -639,10 +640,7 @@ bool grid_of(int n, int h, int w, const dc_geom *g, int nt, int tn, int split, P
   while (p->tmem_cols < 6 * nt * tn) p->tmem_cols *= 2;
   return true;
 }
-int smem_bytes(const Params &p, int nt) {
-  (void)nt;
-  return p.off_a + p.stages_a * p.pitch * 96 * p.per_stage;
-}
+int smem_bytes(const Params &p) { return p.off_a + p.stages_a * p.pitch * 96 * p.per_stage; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -670,7 +668,7 @@ struct Plan {
 // its cuts of activations, whichever is most, and its read-out beside the next one's; shallow rings make them wait for one
 // another.  Of the start-up, 3.5 us, most is a cold instruction cache in every role.
 double estimate_us(const Params &p, int nt, int tn, int n_sm) {
-  static constexpr int kClusters[kMaxSplit + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};    // of that many CTAs that run at once
+  static constexpr int kClusters[kMaxSplit + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};    // of that many CTAs that run at once, on 148 SMs
   const double steps = p.units_per * (p.taps > 1 ? p.taps : p.per_stage), chunks = p.units_per * p.plane_first[p.planes],
                stages = p.units_per * p.planes, turns = steps * nt / 16 / (kWarpsCut - p.warps_a);
   const double issue = steps * tn * (20 + 5.75 * nt) + chunks * 690, cut_w = chunks * 710 + (chunks > turns ? chunks : turns) * 390,
@@ -732,7 +730,7 @@ cudaError_t launch(const Params &p, const float *x, const float *w, const float 
       return cudaErrorNotSupported;
   }
   const int grid = p.split > 1 ? p.items * p.split : (p.items < n_sm ? p.items : n_sm);
-  return dc_launch_pdl_cluster(k_conv_f32_tc<NT, T>, dim3((unsigned)grid), dim3(kThreads), (size_t)smem_bytes(p, NT), st, p.split, map_x, map_w, x, w, bias, residual, y, p, ws);
+  return dc_launch_pdl_cluster(k_conv_f32_tc<NT, T>, dim3((unsigned)grid), dim3(kThreads), (size_t)smem_bytes(p), st, p.split, map_x, map_w, x, w, bias, residual, y, p, ws);
 }
 
 }  // namespace

@@ -1766,7 +1766,9 @@ static void launch_block33_form(TiledBlocks &tb, const BlockDelivery &dv, const 
 // A single block goes to the tensor core where an estimate says so: of 166 drawn blocks of 40 to 320 channels in and 160 to 1280 hidden
 // ones 102, in 0.72 of the time on (geometric) average, two slower, by 2 and 5 %.  160 -> 960 -> 160 20.0 us and
 // 14.3, 200 -> 928 -> 200 39.4 and 17.4, 64 -> 1168 -> 64 17.5 and 11.5, 96 -> 576 -> 96 11.2 and 10.5; what 24 -> 144 -> 24 takes there,
-// 8.2 us, most of it the start and the end of a launch, is more than here, 6.1.
+// 8.2 us, most of it the start and the end of a launch, is more than here, 6.1.  These are merges repeated; a run's first one finds
+// neither weights nor code in L2.  Timed so, between events (5 us more each), 160 -> 960 -> 160 25.5 and 19.4, 200 -> 928 -> 200 45.0 and 23.5,
+// 64 -> 1168 -> 64 22.4 and 16.5, 96 -> 576 -> 96 15.9 and 16.4, 120 -> 720 -> 120 17.4 and 18.4: what is near the line loses a little.
 static bool block33_on_tensor_core(int c0, int c1, int c2, int run, int most16, int most24, int form) {
   const double fma = form == 0   ? 4.07 + 1.69 * (most16 - 1) + c1 / 8.0 * (0.0692 * most16 + 0.0306 * dc_div_up(most16, 2))
                      : form == 1 ? 4.6 + 0.1757 * c1 / 16.0

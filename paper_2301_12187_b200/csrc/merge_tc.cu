@@ -54,7 +54,8 @@ struct Params33 {
   int off_raw, off_b, off_z, off_scale, smem_bytes;
 };
 
-// a pair of warps owns a slot of operands (R), of terms (A) and, of the columns' terms (B), every fourth
+// A pair of warps owns a slot of operands (R), of terms (A) and, of the columns' terms (B), every fourth; D are the sums of hh, M those of
+// the other products.  Every role waits for every phase of its barriers in order, so a phase's bit tells it from the one before.
 enum { kRFull = 0, kREmpty = kPairs, kAFull = 2 * kPairs, kAEmpty = 3 * kPairs, kBFull = 4 * kPairs, kBEmpty = kBFull + kMaxB,
        kDFull = kBEmpty + kMaxB, kMFull = kDFull + kSums, kDEmpty = kMFull + 1, kMEmpty = kDEmpty + kSums, kBars = kMEmpty + 1 };
 
