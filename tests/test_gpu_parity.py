@@ -1283,6 +1283,7 @@ def test_fp32_conv_by_bf16_terms(dc, shape):
 @pytest.mark.parametrize("a,c,o,res,codes", [
     (104, 208, 136, [], "both"),               # a round of tiles and a bit
     (40, 120, 192, [], "both"),                # a tile a CTA, 8 of the last step's 64 channels
+    (64, 200, 152, [], "both"),                # the same, a few tiles fewer than CTAs (the one above may go to the FMAs)
     (256, 256, 256, [], "both"),               # runs of tiles that change columns
     (196, 132, 250, [], "f32"),                # nothing a multiple of a tile or a step
     (168, 168, 168, [(0, 0)], "both"), (168, 168, 168, [(0, 0), (1, 1)], "both"), (168, 168, 168, [(0, 1)], "both"),
