@@ -1,10 +1,10 @@
 """The waits of the merges on the tensor core (blocks and 1x1 pairs), in every order of events (no GPU).
 
-Two teams of warps cut the steps of a reduction into terms in turn, into slots that are used twice at most; two warps multiply them: each
-every second step ("two sums"), or both every step ("four sums").  A wait on a barrier only tells the phase with one parity from
-the phase with the other, so it means what it should only where the earlier phases are known to be over.  The walk below takes the
-waits from the library, in the order in which the kernel makes them, lets every warp move whenever its waits allow, lets products end
-when they like, and looks at what each step finds."""
+Two teams of warps cut the steps of a reduction into terms in turn, into slots that are used twice at most; two warps multiply them:
+each every second step (two sums of the products of high terms), or both every step (as many sums as there is room for).  A wait on
+a barrier only tells the phase with one parity from the phase with the other, so it means what it should only where the earlier
+phases are known to be over.  The walk below takes the waits from the library, in the order in which the kernel makes them, lets
+every warp move whenever its waits allow, lets products end when they like, and looks at what each step finds."""
 import pytest
 
 from paper_2301_12187_b200 import dc
@@ -12,12 +12,12 @@ from paper_2301_12187_b200 import dc
 MULTIPLIED = 1
 
 
-def walk(steps, slots, four_sums, warps=1, waits=dc.selftest_product_waits):
+def walk(steps, slots, both, warps=1, waits=dc.selftest_product_waits):
     """Visits every reachable state; returns the faults found, ("terms" | "slot" | "stuck", step)."""
     sites = [waits(s, slots) for s in range(steps)]
     passes = lambda phases_over, parity: (phases_over & 1) != parity
     # the steps of an issuing warp, those that it waits for side by side together
-    if four_sums:
+    if both:
         turns = [[list(range(s, min(s + 4, steps))) for s in range(0, steps, 4)]] * 2
     else:
         turns = [[[t for t in (s, s + 2) if t < steps] for s in range(odd, steps, 4)] for odd in (0, 1)]
@@ -33,14 +33,14 @@ def walk(steps, slots, four_sums, warps=1, waits=dc.selftest_product_waits):
         multiplied = lambda s: sum(s in mine[w][:over[w]] for w in range(2))
         def phases(what, slot):
             uses = [s for s in (slot, slot + slots) if s < steps]
-            return sum(multiplied(s) for s in uses) // (2 if four_sums else 1) if what == MULTIPLIED else sum(has_cut(s) for s in uses) // warps
+            return sum(multiplied(s) for s in uses) // (2 if both else 1) if what == MULTIPLIED else sum(has_cut(s) for s in uses) // warps
         moves = []
         for team in range(2):
             for i, k in enumerate(cut[team]):
                 s = 2 * k + team
                 if s >= steps or not all(passes(phases(what, slot), parity) for what, slot, parity in sites[s][0]):
                     continue
-                if s >= slots and multiplied(s - slots) < (2 if four_sums else 1):
+                if s >= slots and multiplied(s - slots) < (2 if both else 1):
                     faults.add(("slot", s))
                 team_cut = tuple(sorted(cut[team][:i] + (k + 1,) + cut[team][i + 1:]))
                 moves.append(((team_cut, cut[1]) if team == 0 else (cut[0], team_cut), issue, over))
@@ -70,14 +70,14 @@ def walk(steps, slots, four_sums, warps=1, waits=dc.selftest_product_waits):
 
 
 # every number of slots that 225 KB hold (ten at 80 columns with long reductions, 13 at 48), odd and even, and small ones with every reuse
-@pytest.mark.parametrize("steps,slots,four_sums,warps", [
+@pytest.mark.parametrize("steps,slots,both,warps", [
     (12, 11, False, 1), (13, 11, False, 1), (16, 11, False, 1), (12, 10, False, 1), (14, 13, False, 1), (16, 12, False, 1),
     (10, 5, False, 1), (14, 7, False, 1), (12, 6, False, 1), (7, 5, False, 2), (8, 5, False, 2), (7, 4, False, 2),
     (10, 5, True, 1), (8, 4, True, 1), (7, 5, True, 2), (11, 7, True, 1),
 ])
-def test_no_step_is_multiplied_before_its_terms_are_there(steps, slots, four_sums, warps):
+def test_no_step_is_multiplied_before_its_terms_are_there(steps, slots, both, warps):
     """Nor does one write a slot that is still read; and no warp waits for good."""
-    assert not walk(steps, slots, four_sums, warps)
+    assert not walk(steps, slots, both, warps)
 
 
 def test_the_walk_finds_a_wait_for_a_second_phase_alone():
